@@ -192,6 +192,7 @@ class Engine:
                 self.ctx = C.c_void_p(None)
             raise VlaError(rc, msg)
         self.head_passes = max(1, int(head_passes))
+        self._frames_done = [0] * self.n_streams     # frames of each stream whose chunk has been polled
         self.chunk_shape = (model.horizon, model.act_dim) if self.head_passes == 1 else (self.head_passes, model.horizon, model.act_dim)
 
     # ---- thin wrappers -------------------------------------------------------------
@@ -261,6 +262,7 @@ class Engine:
         if rc == VLA_ERR_NOT_READY:
             return None
         self._check(rc)
+        self._frames_done[stream] = fid.value + 1
         return out, fid.value
 
     def hold_launches(self, on):
@@ -274,8 +276,6 @@ class Engine:
         """frames[r][n] -> chunks[r][n]; submits as fast as the rings accept and polls in frame order."""
         import time
         R = len(frames)
-        if not hasattr(self, "_frames_done"):
-            self._frames_done = [0] * self.n_streams
         base = list(self._frames_done)
         nxt = [0] * R
         got = [[None] * len(frames[r]) for r in range(R)]
@@ -296,7 +296,6 @@ class Engine:
                         break
                     chunk, fid = res
                     got[r][fid - base[r]] = chunk
-                    self._frames_done[r] += 1
                     remaining -= 1
                     progressed = True
             if not progressed:
