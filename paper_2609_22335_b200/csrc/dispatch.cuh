@@ -10,7 +10,7 @@ constexpr unsigned CTRL_EXITING = 0x80000000u;
 constexpr uint32_t TRACE_ADMIT_NODE = 0xFFFFFFFFu;   // node id of the trace record that marks a frame's admission
 constexpr int MAX_WORKERS = 3;
 constexpr int SM_CTL_BYTES = 1024;       // per-worker control block (mbarriers, row scales) handed to the tile bodies
-constexpr int SM_STATE_BASE = 2048;      // dispatcher state of the SM
+constexpr int SM_STATE_BASE = 4096;      // dispatcher state of the SM
 constexpr int SM_STATE_BYTES = SM_STATE_BASE + MAX_WORKERS * SM_CTL_BYTES;   // then the tile slab, 1024-byte aligned
 
 __device__ __forceinline__ uint64_t gtimer() {
@@ -80,17 +80,18 @@ __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t cols) {
 // Pushing tiles is split in three so a whole warp can fill the entries in parallel:
 // reserve (one thread), fill (any threads, entry i of the range), commit (one thread, after a barrier).
 // The ring is sized for every tile of every frame slot, so a reservation can never overrun the head.
-// One entry = one 64-bit word: generation (12 bits, never 0 for a written entry of the current lap... the lap count + 1)
-// | node (20) | frame slot (9) | tile (12) | and the node's per-tile resource need in units so that a claim needs no
-// second load: shared memory (6) and tensor memory (5).
-constexpr int QW_NODE_BITS = 20, QW_INST_BITS = 9, QW_TILE_BITS = 12, QW_SMEM_BITS = 6, QW_TMEM_BITS = 5, QW_GEN_BITS = 12;
-static_assert(QW_NODE_BITS + QW_INST_BITS + QW_TILE_BITS + QW_SMEM_BITS + QW_TMEM_BITS + QW_GEN_BITS == 64, "queue word layout");
+// One entry = one 64-bit word: generation (11 bits, never 0 for a written entry of the current lap... the lap count + 1)
+// | node (20) | frame slot (9) | tile (12) | the node's per-tile resource need in units so that a claim needs no
+// second load: shared memory (6) and tensor memory (5) | and whether the tile was queued before its node's release (1).
+constexpr int QW_NODE_BITS = 20, QW_INST_BITS = 9, QW_TILE_BITS = 12, QW_SMEM_BITS = 6, QW_TMEM_BITS = 5, QW_GEN_BITS = 11;
+static_assert(QW_NODE_BITS + QW_INST_BITS + QW_TILE_BITS + QW_SMEM_BITS + QW_TMEM_BITS + 1 + QW_GEN_BITS == 64, "queue word layout");
+constexpr uint32_t RES_EARLY = 1u << (QW_SMEM_BITS + QW_TMEM_BITS);      // in the resource field of an entry being written
 __device__ __forceinline__ unsigned long long queue_gen(const DeviceCtx& ctx, unsigned long long ticket) {
   return ((ticket >> ctx.q_shift) + 1ull) & ((1ull << QW_GEN_BITS) - 1ull);
 }
 __device__ __forceinline__ unsigned long long queue_word(const DeviceCtx& ctx, unsigned long long ticket, uint32_t inst,
                                                          uint32_t node, uint32_t tile, uint32_t res_units) {
-  // res_units = smem units | tmem units << QW_SMEM_BITS
+  // res_units = smem units | tmem units << QW_SMEM_BITS (| RES_EARLY)
   return (queue_gen(ctx, ticket) << (64 - QW_GEN_BITS)) | ((unsigned long long)res_units << (QW_NODE_BITS + QW_INST_BITS + QW_TILE_BITS)) |
          ((unsigned long long)tile << (QW_NODE_BITS + QW_INST_BITS)) | ((unsigned long long)inst << QW_NODE_BITS) | (unsigned long long)node;
 }
@@ -107,6 +108,7 @@ __device__ inline void queue_fill(const DeviceCtx& ctx, int cls, unsigned long l
                                   uint32_t res_units, int first, int count, int stride) {
   const unsigned long long mask = (unsigned long long)ctx.q_capacity - 1;
   QueueEntry* ent = ctx.q_entries + (size_t)cls * ctx.q_capacity;
+#pragma unroll 1
   for (int i = first; i < count; i += stride)
     *reinterpret_cast<volatile unsigned long long*>(ent + ((base + i) & mask)) = queue_word(ctx, base + i, inst, node, (uint32_t)i, res_units);
 }
@@ -150,7 +152,6 @@ __device__ inline bool queue_try_pop(const DeviceCtx& ctx, int cls, QueueEntry& 
 }
 
 // ------------------------------------------------------------------ per-SM state of the persistent kernel
-constexpr int MAX_READY = 6;
 constexpr int DISPATCH_THREADS = 64;     // two service warps per SM (claim, retire), after the worker groups
 constexpr long long PRIO_WINDOW_NS = 8000;   // an action-head tile may be claimed for a worker this close to the end of its tile
 constexpr int PREFETCH_MIN_TOTAL = 600;   // tiles are claimed ahead of need only while this many VLM tiles are queued in all
@@ -159,19 +160,19 @@ constexpr int HELD_DEPTH = 1;            // claimed tiles a worker may have wait
 constexpr unsigned CLAIM_NAP_NS = 60, CLAIM_NAP_MAX_NS = 240;   // claim warp, while a worker of its SM has nothing to run
 constexpr unsigned CLAIM_SLEEP_NS = 2000;    // claim warp, every worker busy: longest sleep without a ring
 constexpr unsigned RETIRE_SLEEP_NS = 4000;   // retire warp: longest sleep without a ring
+// With no more tiles queued or running than the GPU has SMs, tiles are spread one per SM (two per SM up to twice as many) and
+// take the pipeline depth that leaves room for; an SM that has its share leaves the queue to the others for a moment.
+constexpr unsigned long long SPREAD_WAIT_NS = 1000;
+// A node whose predecessors' tiles have all been taken may be queued before they finish (its workers wait holding their
+// weights) as long as everything queued or running still fits one tile per SM.
+constexpr int EARLY_MAX_TILES = 148;
 constexpr unsigned long long HEAD_WAIT_NS = 1500;   // an action-head tile nobody took for this long may go to a running worker
-
-struct ReadyItem {
-  unsigned long long base;   // reserved queue range
-  uint32_t node, res_units;
-  int n_tiles, cls;
-};
 
 struct WorkerTile {
   uint32_t inst, node, tile;
   int cls;
   int smem_unit0, smem_units, tmem_unit0, tmem_units;
-  int succ_begin, succ_count, op, pad_;     // of the tile's node, filled in by the worker for the retire warp
+  int succ_begin, succ_count, op, early;    // of the tile's node, filled in by the worker for the retire warp; queued before the release
   uint64_t t0, t1, frame;
 };
 
@@ -182,15 +183,17 @@ struct WorkerSlot {
   volatile int leave;            // claim warp -> worker: go home
   volatile int done_state;       // 0 empty, 1 finished tile posted for the retire warp
   volatile int busy;             // the worker is running a tile (set and cleared by the worker)
-  int pad_;
+  int turn;                      // which half of SmState::cur holds the running tile
+  uint32_t bell_parity;
+  volatile int start_state;      // 1: the worker took the last tile of (start_inst, start_node): its successors may be queued early
+  uint32_t start_inst, start_node;
   volatile unsigned prio_tail, prio_head;   // one-deep slot for an action-head tile that goes ahead of the held VLM tiles
   volatile unsigned long long t_busy;       // when the running tile was taken (worker), for the claim warp's estimate of its end
-  WorkerTile done, fin, held[HELD_DEPTH], prio;
-  int n_ready;
-  ReadyItem ready[MAX_READY];
+  WorkerTile done, held[HELD_DEPTH], prio;
 };
 
-struct SmState {
+static_assert(sizeof(NodeDesc) % 16 == 0 && sizeof(NodeDesc) <= 512, "a node's description is copied by one warp, 16 bytes a lane");
+struct __align__(16) SmState {
   unsigned long long smem_mask;    // bit i set = shared-memory unit i in use
   unsigned tmem_mask;              // bit i set = tensor-memory unit i in use
   int n_smem_units, n_tmem_units;
@@ -200,12 +203,20 @@ struct SmState {
   int smem_promised, tmem_promised;  // units of tiles handed to free workers that have not allocated them yet
   unsigned room_wait;              // a worker waiting for room right now: smem units | tmem units << 8 | (worker + 1) << 16, else 0
                                    // (the latest one when two wait); the claim warp keeps that room out of its offers
+  volatile int outstanding;        // tiles queued or running on the whole GPU when the claim warp last looked
   volatile int ema_ns[N_CLASSES];  // running mean of tile durations per class on this SM (retire warp)
-  int tau_tab[N_CLASSES * 3];      // the classes' intensity tags (read by the workers when a tile ends)
+  // per class: intensity tags, pick group, tiles queued (-G score), largest need of a tile in units, R_k of the -R score
+  int tau_tab[N_CLASSES * 3];
+  unsigned group_mask[N_CLASSES];
+  int grid[N_CLASSES], smem_units[N_CLASSES], tmem_units[N_CLASSES], res[N_CLASSES];
   unsigned long long bell_claim;   // rung by a worker that took a claimed tile or ran out of work
   unsigned long long bell_retire;  // rung by a worker that posted a finished tile
   unsigned long long bell_worker[MAX_WORKERS];   // rung by the claim warp when it hands worker w a tile or sends it home
-  WorkerTile cur[MAX_WORKERS];     // the tile each worker is running (written by its leader)
+  WorkerTile cur[MAX_WORKERS][2];  // the tile each worker is running and the one before it (written by its leader in turn): what the
+                                   // end of a tile needs is read back from here instead of living in registers through the tile body
+  TileCtx tc[MAX_WORKERS];         // context of the running tile ...
+  NodeDesc node[MAX_WORKERS];      // ... and the description of its node, copied here: the tile body's arguments
+  volatile int cur_cls[MAX_WORKERS];   // class of the running tile, for the claim warp
   WorkerSlot slot[MAX_WORKERS];
 };
 static_assert(sizeof(SmState) <= SM_STATE_BASE, "SM state too large");
@@ -217,6 +228,7 @@ __device__ __forceinline__ int find_free(unsigned long long mask, int need, int 
   if (need == 0) return 0;
   if (need > total) return -1;
   unsigned long long run = ~mask & unit_bits(total);
+#pragma unroll 1
   for (int k = 1; k < need;) {
     const int step = min(k, need - k);
     run &= run >> step;
@@ -236,6 +248,12 @@ __device__ inline void write_trace(const DeviceCtx& ctx, uint32_t inst, uint32_t
   ctx.trace[idx] = r;
 }
 
+// Release count that a node of the frame now in slot `inst` reaches when it is released.
+__device__ __forceinline__ unsigned release_count(const DeviceCtx& ctx, uint32_t inst) {
+  const uint64_t frame = *reinterpret_cast<const volatile uint64_t*>(ctx.inst_frame + inst);
+  return (unsigned)(frame / (unsigned)ctx.ring_depth + 1u) & 0x7FFFFFFFu;
+}
+
 // A frame became ready (its inputs are in HBM): take its admission record and queue its root tiles.
 __device__ inline void try_admit(const DeviceCtx& ctx) {
   Control* ctl = ctx.control;
@@ -243,6 +261,7 @@ __device__ inline void try_admit(const DeviceCtx& ctx) {
   const unsigned long long tail = ld_volatile_u64(&ctl->admit_tail);
   if (head >= tail) return;
   unsigned old = ld_volatile_u32(&ctl->ctrl);
+#pragma unroll 1
   for (int tries = 0; tries < 8; ++tries) {
     if (old & CTRL_EXITING) return;
     unsigned prev = atomicCAS(&ctl->ctrl, old, old + 1u);
@@ -263,63 +282,35 @@ __device__ inline void try_admit(const DeviceCtx& ctx) {
     write_trace(ctx, inst, TRACE_ADMIT_NODE, 0, 0, 0xFF, frame, now, now);
   }
   __threadfence();
+#pragma unroll 1
   for (int i = 0; i < ctx.n_roots; ++i) {
     int r = ctx.roots[i];
     queue_push(ctx, ctx.nodes[r].cls, inst, (uint32_t)r, ctx.nodes[r].n_tiles);
   }
 }
 
-// Global side of a finished tile: every successor node's counter (which counts its predecessors' tiles)
-// goes down by one; a counter reaching zero re-arms itself and releases that node, whose queue range is
-// reserved here and returned in `slot` for the warp to fill.
-__device__ inline void complete_tile(const DeviceCtx& ctx, const WorkerTile& f, WorkerSlot* slot) {
-  const uint32_t inst = f.inst;
-  slot->n_ready = 0;
-  __threadfence();
-  const int n_succ = f.succ_count, succ0 = f.succ_begin;      // carried by the tile's record: no load of its node here
-  for (int i0 = 0; i0 < n_succ; i0 += 4) {
-    // up to four successors per pass: one 16-byte load each, then their counters are decremented by independent
-    // atomics in flight together
-    SuccInfo si[4];
-    int left[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      si[j].node = -1;
-      if (i0 + j < n_succ) {
-        const int4 v = __ldg(reinterpret_cast<const int4*>(ctx.succ + succ0 + i0 + j));
-        si[j].node = v.x; si[j].n_tiles = v.y; si[j].cls_res = v.z; si[j].n_pred = v.w;
-      }
-    }
-#pragma unroll
-    for (int j = 0; j < 4; ++j) left[j] = si[j].node >= 0 ? atomicSub(ctx.dep_count + (size_t)inst * ctx.n_nodes + si[j].node, 1) - 1 : 1;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      if (left[j] != 0) continue;
-      ctx.dep_count[(size_t)inst * ctx.n_nodes + si[j].node] = si[j].n_pred;
-      const int s_cls = si[j].cls_res & 0xFF;
-      const uint32_t s_res = (uint32_t)si[j].cls_res >> 8;
-      if (slot->n_ready < MAX_READY) {
-        ReadyItem& it = slot->ready[slot->n_ready++];
-        it.base = queue_reserve(ctx, s_cls, si[j].n_tiles);
-        it.node = (uint32_t)si[j].node; it.n_tiles = si[j].n_tiles; it.cls = s_cls;
-        it.res_units = s_res;
-      } else {
-        queue_push(ctx, s_cls, inst, (uint32_t)si[j].node, si[j].n_tiles);
-      }
-    }
-  }
-  if (slot->n_ready > 0) __threadfence();   // acquire side of the counters just read, before the entries are published
-  if (f.op == OP_EMIT) atomicSub(&ctx.control->ctrl, 1u);
+__device__ __forceinline__ SuccInfo load_succ(const DeviceCtx& ctx, int i) {
+  const int4 v = __ldg(reinterpret_cast<const int4*>(ctx.succ + i));
+  return SuccInfo{v.x, v.y, v.z, v.w};
 }
 
-// u[x] += sign * tau[cls][x] on the SM's utilisation counters, with `cls` known only at run time: the class is matched
-// against loop-constant positions so that the tag table stays in registers.
-__device__ __forceinline__ void tau_add(int* u, const int* tau, int cls, int sign) {
-  int t0 = 0, t1 = 0, t2 = 0;
-#pragma unroll
-  for (int c = 0; c < N_CLASSES; ++c)
-    if (c == cls) { t0 = tau[c * 3]; t1 = tau[c * 3 + 1]; t2 = tau[c * 3 + 2]; }
-  atomicAdd(u + 0, sign * t0); atomicAdd(u + 1, sign * t1); atomicAdd(u + 2, sign * t2);
+// Queues the node each `ready` lane holds (whole warp): the lanes reserve their ranges at once, the warp writes the entries.
+__device__ __forceinline__ void push_nodes(const DeviceCtx& ctx, bool ready, uint32_t inst, const SuccInfo& si, uint32_t early, int lane) {
+  unsigned m = __ballot_sync(0xffffffffu, ready);
+  if (m == 0u) return;
+  const int cls = si.cls_res & 0xFF;
+  const uint32_t res = (((uint32_t)si.cls_res >> 8) & (RES_EARLY - 1u)) | early;
+  const unsigned long long base = ready ? queue_reserve(ctx, cls, si.n_tiles) : 0ull;
+  queue_fill_fence();
+#pragma unroll 1
+  for (; m != 0u; m &= m - 1u) {
+    const int src = __ffs((int)m) - 1;
+    queue_fill(ctx, __shfl_sync(0xffffffffu, cls, src), __shfl_sync(0xffffffffu, base, src), __shfl_sync(0xffffffffu, inst, src),
+               (uint32_t)__shfl_sync(0xffffffffu, si.node, src), __shfl_sync(0xffffffffu, res, src), lane,
+               __shfl_sync(0xffffffffu, si.n_tiles, src), 32);
+  }
+  __syncwarp();
+  if (ready) queue_commit(ctx, cls, si.n_tiles);
 }
 
 // ------------------------------------------------------------------ the two service warps of an SM
@@ -328,50 +319,99 @@ __device__ __forceinline__ void tau_add(int* u, const int* tau, int cls, int sig
 //   * the CLAIM warp (lane w serves worker w) claims tiles under the pick policy -- for a busy worker one
 //     tile ahead -- and hands a claimed tile over as soon as its worker is free and its exact
 //     shared/tensor-memory need fits;
-//   * the RETIRE warp (lane w serves worker w) takes a finished tile, frees its memory at once, then does
-//     the global bookkeeping (node counter, successors' dependency counters, queue pushes; the whole warp
-//     fills the released successors' entries).
+//   * the RETIRE warp (eight lanes serve one worker) takes a finished tile and does the global bookkeeping
+//     (successors' dependency counters, queue pushes; the whole warp fills the released successors' entries).
 // Per-SM state is shared-memory words updated with shared-memory atomics by these two warps only.
-__device__ inline void retire_loop(const DeviceCtx& ctx, SmState* sm, int n_workers) {
-  const int lane = threadIdx.x & 31;
-  const bool serving = lane < n_workers;
-  WorkerSlot* slot = sm->slot + (serving ? lane : 0);
+// Eight lanes serve one worker, a successor of its tile's node each, so the counter round trips of all workers and
+// successors run at the same time.
+constexpr int RETIRE_LANES = 8;
+static_assert(RETIRE_LANES * MAX_WORKERS <= 32, "the retire warp has lanes for every worker");
+__device__ __forceinline__ void retire_loop(const DeviceCtx& ctx, SmState* sm, int n_workers) {
+  const int lane = threadIdx.x & 31, w = lane / RETIRE_LANES, sub = lane % RETIRE_LANES;
+  const bool serving = w < n_workers;
+  WorkerSlot* slot = sm->slot + (serving ? w : 0);
   uint32_t bell_parity = 0;
   for (;;) {
-    bool have_fin = false;
-    if (serving && slot->done_state == 1) {
-      slot->fin = slot->done;
-      __threadfence_block();
-      slot->done_state = 0;
-      have_fin = true;
-      const WorkerTile& f = slot->fin;
-      sm->ema_ns[f.cls] = (3 * sm->ema_ns[f.cls] + (int)(f.t1 - f.t0)) >> 2;
-      write_trace(ctx, f.inst, f.node, f.tile, lane, f.cls, f.frame, f.t0, f.t1);
-      complete_tile(ctx, f, slot);
-    } else if (serving) {
-      slot->n_ready = 0;
-    }
+    // (the flags are read in this order and handled in the other: a tile's start is announced before its end is)
+    const bool ended = serving && slot->done_state == 1;
+    __threadfence_block();
+    const bool started = serving && slot->start_state == 1;
     __syncwarp();
-    const bool any = __any_sync(0xffffffffu, have_fin);
-    if (any) {
-      bool fenced = false;
-      for (int w = 0; w < n_workers; ++w) {
-        const int nr = sm->slot[w].n_ready;
-        if (nr > 0 && !fenced) { queue_fill_fence(); fenced = true; }
-        for (int i = 0; i < nr; ++i) {
-          const ReadyItem it = sm->slot[w].ready[i];
-          queue_fill(ctx, it.cls, it.base, sm->slot[w].fin.inst, it.node, it.res_units, lane, it.n_tiles, 32);
-        }
-      }
-      __syncwarp();
-      if (serving) {
-        for (int i = 0; i < slot->n_ready; ++i) queue_commit(ctx, slot->ready[i].cls, slot->ready[i].n_tiles);
-        slot->n_ready = 0;
-      }
-      __syncwarp();
-    } else {
+    if (!__any_sync(0xffffffffu, ended || started)) {
       if (sm->quit) break;
       bell_wait(&sm->bell_retire, bell_parity, RETIRE_SLEEP_NS);
+      continue;
+    }
+    // ---- starts.  The last tile of a node has been taken by a worker: tiles of a class are handed out in queue order, so
+    // all of them have.  Where that was the last predecessor of a successor, and the GPU has idle SMs for it, the successor
+    // is queued now: its tiles are taken, fetch their weights and wait for the release, instead of going through the queues
+    // after it (hand-over 3 us instead of 9).  No cycle can arise: a waiting tile waits only for tiles taken before it, and
+    // it holds shared memory while it waits only on an SM where nothing taken before it still needs some (see the worker's
+    // allocation).
+    if (__any_sync(0xffffffffu, started)) {
+      uint32_t inst = 0;
+      int succ0 = 0, n_succ = 0;
+      if (started) {
+        inst = slot->start_inst;
+        const int4 d = __ldg(reinterpret_cast<const int4*>(ctx.nodes + slot->start_node) + 1);     // succ_begin, succ_count, phase, step
+        succ0 = d.x; n_succ = d.y;
+      }
+      __syncwarp();
+      if (started && sub == 0) { __threadfence_block(); slot->start_state = 0; }
+#pragma unroll 1
+      for (int i = sub; __any_sync(0xffffffffu, i < n_succ); i += RETIRE_LANES) {
+        SuccInfo si = {0, 0, 0, 0};
+        bool early = false;
+        if (i < n_succ) {
+          si = load_succ(ctx, succ0 + i);
+          const size_t at = (size_t)inst * ctx.n_nodes + si.node;
+          if (atomicSub(ctx.start_count + at, 1) == 1) {
+            ctx.start_count[at] = (int)((uint32_t)si.cls_res >> 20);
+            early = sm->outstanding + si.n_tiles <= EARLY_MAX_TILES;
+            // marked before this SM reports the tile finished, so whoever releases the node sees the mark
+            if (early) atomicOr(ctx.dep_word + at, 1ull << 63);
+          }
+        }
+        push_nodes(ctx, early, inst, si, RES_EARLY, lane);
+      }
+    }
+    // ---- ends.  Every successor's word (which counts its predecessors' tiles) goes down by one; one reaching zero is
+    // re-armed with its release count one up, which is what early-taken tiles of that node wait for; if the node was not
+    // queued early, it is now.
+    if (__any_sync(0xffffffffu, ended)) {
+      uint32_t inst = 0;
+      int succ0 = 0, n_succ = 0;
+      if (ended) {
+        const WorkerTile& f = slot->done;
+        inst = f.inst; succ0 = f.succ_begin; n_succ = f.succ_count;
+        if (sub == 0) {
+          sm->ema_ns[f.cls] = (3 * sm->ema_ns[f.cls] + (int)(f.t1 - f.t0)) >> 2;
+          write_trace(ctx, f.inst, f.node, f.tile, w, f.cls, f.frame, f.t0, f.t1);
+        }
+      }
+      __threadfence();        // the tile's writes, seen through the mailbox, go ahead of the counters below
+#pragma unroll 1
+      for (int i = sub; __any_sync(0xffffffffu, i < n_succ); i += RETIRE_LANES) {
+        SuccInfo si = {0, 0, 0, 0};
+        bool release = false;
+        if (i < n_succ) {
+          si = load_succ(ctx, succ0 + i);
+          unsigned long long* word = ctx.dep_word + (size_t)inst * ctx.n_nodes + si.node;
+          const unsigned long long old = atomicAdd(word, ~0ull);
+          if ((uint32_t)old == 1u) {
+            st_release_u64(word, ((((old >> 32) + 1ull) & 0x7FFFFFFFull) << 32) | (unsigned)si.n_pred);
+            release = (old >> 63) == 0ull;
+          }
+        }
+        push_nodes(ctx, release, inst, si, 0u, lane);
+      }
+      if (ended && sub == 0) {
+        atomicAdd(&ctx.queues[slot->done.cls].done, 1ull);
+        if (slot->done.op == OP_EMIT) atomicSub(&ctx.control->ctrl, 1u);
+        __threadfence_block();
+        slot->done_state = 0;
+      }
+      __syncwarp();
     }
   }
 }
@@ -381,34 +421,8 @@ __device__ inline void claim_loop(const DeviceCtx& ctx, SmState* sm, int n_worke
   const bool serving = lane < n_workers;
   Control* ctl = ctx.control;
   WorkerSlot* slot = sm->slot + (serving ? lane : 0);
-  // Per-class constants live in registers: the arrays below are only ever read at loop-constant positions, and the
-  // shared/tensor-memory needs are packed one byte per class.  (This loop runs on every tile hand-over of the SM;
-  // arrays in local memory and global loads here cost 5 % of the whole step's throughput.)
-  int tau[N_CLASSES * 3], res_units[N_CLASSES];
-  unsigned group_mask[N_CLASSES];
-  unsigned long long su_pack = 0ull, tu_pack = 0ull;
-  {
-    int group[N_CLASSES];
-#pragma unroll
-    for (int c = 0; c < N_CLASSES; ++c) {
-#pragma unroll
-      for (int x = 0; x < 3; ++x) tau[c * 3 + x] = ctx.classes[c].tau[x];
-      group[c] = ctx.classes[c].group;
-      const int su = ctx.classes[c].smem_units, tu = ctx.classes[c].tmem_units;
-      res_units[c] = su > 0 ? su : 1;                                                 // R_k of the -R score
-      su_pack |= (unsigned long long)(su & 0xFF) << (8 * c);
-      tu_pack |= (unsigned long long)(tu & 0xFF) << (8 * c);
-    }
-#pragma unroll
-    for (int c = 0; c < N_CLASSES; ++c) {
-      unsigned m = 0;
-#pragma unroll
-      for (int j = 0; j < N_CLASSES; ++j)
-        if (group[j] == group[c]) m |= 1u << j;
-      group_mask[c] = m;
-    }
-  }
-  const bool variant = ctx.policy == POLICY_TWO_PHASE_G || ctx.policy == POLICY_TWO_PHASE_R;
+  // (Class tables are read from shared memory, and the loops below stay rolled: this code runs on every hand-over of the SM,
+  // between tile bodies that need the instruction cache.)
   uint64_t idle_start = 0, last_progress = gtimer();
   unsigned iter = 0, nap = CLAIM_NAP_NS, lost = 0;
   uint32_t bell_parity = 0;
@@ -433,17 +447,26 @@ __device__ inline void claim_loop(const DeviceCtx& ctx, SmState* sm, int n_worke
     if (av > 0) { if (pending_since == 0) pending_since = gtimer(); } else pending_since = 0;
     const unsigned waiting = __ballot_sync(0xffffffffu, pending_since != 0 && gtimer() - pending_since >= HEAD_WAIT_NS) &
                              ((1u << N_CLASSES) - 1u);
-    int grid[N_CLASSES];                               // G_k of the -G score: the class's tiles still to place
-    if (variant) {
-      const int depth = (int)(av < 0 ? 0 : (av > (1 << 20) ? (1 << 20) : av));
+    int outstanding = lane < N_CLASSES ? (int)min(ld_volatile_u64(&ctx.queues[lane].tail) - ld_volatile_u64(&ctx.queues[lane].done), 1ull << 20) : 0;
 #pragma unroll
-      for (int c = 0; c < N_CLASSES; ++c) grid[c] = __shfl_sync(0xffffffffu, depth, c);
+    for (int o = 4; o > 0; o >>= 1) outstanding += __shfl_xor_sync(0xffffffffu, outstanding, o);
+    if (lane == 0) sm->outstanding = outstanding;
+    outstanding = __shfl_sync(0xffffffffu, outstanding, 0);
+    const int n_sms = (int)gridDim.x;
+    const int share = outstanding <= n_sms ? 1 : (outstanding <= 2 * n_sms ? 2 : MAX_WORKERS);
+    unsigned spread = 0xffffffffu;
+    int running = 0;
+    if (share < MAX_WORKERS) {
+      spread = __ballot_sync(0xffffffffu, pending_since != 0 && gtimer() - pending_since >= SPREAD_WAIT_NS) & ((1u << N_CLASSES) - 1u);
+      running = __popc(__ballot_sync(0xffffffffu, serving && (slot->busy != 0 || slot->held_tail != slot->held_head || slot->prio_tail != slot->prio_head)));
     }
+    if (lane < N_CLASSES) sm->grid[lane] = (int)(av < 0 ? 0 : (av > (1 << 20) ? (1 << 20) : av));   // G_k of the -G score: tiles still to place
     // ---- choose, lane by lane, which class each worker claims from
     int want = -1, promised_s = 0, promised_t = 0;
     bool to_prio = false;
     const unsigned avoid = lost;      // the class this lane just lost a race for: other SMs drained it
     lost = 0;
+#pragma unroll 1
     for (int w = 0; w < n_workers; ++w) {
       const unsigned queued = serving ? slot->held_tail - slot->held_head : 0u;
       const unsigned pq = serving ? slot->prio_tail - slot->prio_head : 0u;
@@ -459,12 +482,13 @@ __device__ inline void claim_loop(const DeviceCtx& ctx, SmState* sm, int n_worke
         unsigned cand;
         if (!busy) cand = head_pending ? (pending & act_mask) : pending;
         else if (pq == 0u && head_pending && (waiting & act_mask & ~avoid) != 0u && slot->busy != 0 &&
-                 (long long)(gtimer() - slot->t_busy) + PRIO_WINDOW_NS >= (long long)sm->ema_ns[sm->cur[w].cls]) {
+                 (long long)(gtimer() - slot->t_busy) + PRIO_WINDOW_NS >= (long long)sm->ema_ns[sm->cur_cls[w]]) {
           cand = waiting & act_mask; to_prio = true;
         }
         else if (queued < (unsigned)HELD_DEPTH) cand = deep & ((1u << N_KINDS) - 1u);
         else cand = 0u;
         cand &= ~avoid;
+        if (running >= share) cand &= spread;
         const unsigned long long smask = *reinterpret_cast<volatile unsigned long long*>(&sm->smem_mask);
         const unsigned tmask = *reinterpret_cast<volatile unsigned*>(&sm->tmem_mask);
         // room: a free run of units now, and enough units left after what was promised to tiles already handed
@@ -478,36 +502,30 @@ __device__ inline void claim_loop(const DeviceCtx& ctx, SmState* sm, int n_worke
         unsigned feasible = 0;
         if (busy) feasible = (1u << N_CLASSES) - 1u;   // a tile claimed ahead waits for room when its worker takes it
         else
+#pragma unroll 1
           for (unsigned m = cand; m != 0u; m &= m - 1u) {                // only the candidate classes are looked at
             const int c = __ffs((int)m) - 1;
-            const int su = (int)((su_pack >> (8 * c)) & 0xFFull), tu = (int)((tu_pack >> (8 * c)) & 0xFFull);
+            const int su = sm->smem_units[c], tu = sm->tmem_units[c];
             if (su <= smem_left && tu <= tmem_left && find_free(smask, su, sm->n_smem_units) >= 0 &&
                 find_free((unsigned long long)tmask, tu, sm->n_tmem_units) >= 0)
               feasible |= 1u << c;
           }
         if ((cand & feasible) != 0u) {
-          PickState ps;
-#pragma unroll
-          for (int c = 0; c < N_CLASSES; ++c) ps.cta_count[c] = *reinterpret_cast<volatile int*>(&sm->pick.cta_count[c]);
-#pragma unroll
-          for (int x = 0; x < 3; ++x) ps.u[x] = *reinterpret_cast<volatile int*>(&sm->pick.u[x]);
           int phase;
-          if (variant)
-            want = pick_choose(N_CLASSES, tau, group_mask, cand, feasible, ps, sm->pick.rr, ctx.policy, ctx.u_max, &phase, grid, res_units);
-          else
-            want = pick_choose(N_CLASSES, tau, group_mask, cand, feasible, ps, sm->pick.rr, ctx.policy, ctx.u_max, &phase);
+          want = pick_choose(N_CLASSES, sm->tau_tab, sm->group_mask, cand, feasible, sm->pick, sm->pick.rr, ctx.policy, ctx.u_max, &phase,
+                             sm->grid, sm->res);
         }
         if (want >= 0) {
           if (!busy) {                                   // promised until the worker has allocated (or the pop is lost)
-            promised_s = (int)((su_pack >> (8 * want)) & 0xFFull); promised_t = (int)((tu_pack >> (8 * want)) & 0xFFull);
+            promised_s = sm->smem_units[want]; promised_t = sm->tmem_units[want];
             atomicAdd(&sm->smem_promised, promised_s); atomicAdd(&sm->tmem_promised, promised_t);
           }
           atomicAdd(&sm->pick.cta_count[want], 1);     // counted from the claim on, so the next lane sees it
-          tau_add(&sm->pick.u[0], tau, want, 1);
+          for (int x = 0; x < 3; ++x) atomicAdd(&sm->pick.u[x], sm->tau_tab[want * 3 + x]);
           sm->pick.rr = (want + 1) % N_CLASSES;
         }
       }
-      __syncwarp();
+      if (__shfl_sync(0xffffffffu, want, w) >= 0) ++running;
     }
     // ---- the claims themselves run in parallel across lanes (global atomics)
     if (want >= 0) {
@@ -520,6 +538,7 @@ __device__ inline void claim_loop(const DeviceCtx& ctx, SmState* sm, int n_worke
         h.smem_units = (int)((e >> (QW_NODE_BITS + QW_INST_BITS + QW_TILE_BITS)) & ((1u << QW_SMEM_BITS) - 1u));
         h.tmem_units = (int)((e >> (QW_NODE_BITS + QW_INST_BITS + QW_TILE_BITS + QW_SMEM_BITS)) & ((1u << QW_TMEM_BITS) - 1u));
         h.cls = want;
+        h.early = (int)((e >> (64 - QW_GEN_BITS - 1)) & 1u);
         {   // the worker's first loads are from the node's description: bring its two lines into this SM's L1 now
           const char* ndp = reinterpret_cast<const char*>(ctx.nodes + h.node);
           asm volatile("prefetch.global.L1 [%0];" ::"l"(ndp));
@@ -533,7 +552,7 @@ __device__ inline void claim_loop(const DeviceCtx& ctx, SmState* sm, int n_worke
         progressed = true;
       } else {                                         // lost the race: undo the count
         atomicSub(&sm->pick.cta_count[want], 1);
-        tau_add(&sm->pick.u[0], tau, want, -1);
+        for (int x = 0; x < 3; ++x) atomicSub(&sm->pick.u[x], sm->tau_tab[want * 3 + x]);
         if (promised_s | promised_t) { atomicSub(&sm->smem_promised, promised_s); atomicSub(&sm->tmem_promised, promised_t); }
         lost = 1u << want;                             // look elsewhere in the next round, which follows at once
       }
@@ -586,6 +605,46 @@ __device__ inline void claim_loop(const DeviceCtx& ctx, SmState* sm, int n_worke
   }
 }
 
+// The worker's threads after a tile body.
+__device__ __forceinline__ void end_of_tile(const DeviceCtx& ctx, SmState* sm, WorkerSlot* slot) {
+  unsigned tid;
+  asm volatile("mov.u32 %0, %%tid.x;" : "=r"(tid));
+  const int worker = (int)tid / WORKER_THREADS, wt = (int)tid % WORKER_THREADS;
+  WorkerTile& cmd = sm->cur[worker][slot->turn];      // (looked up before the barrier: afterwards the leader moves on)
+  asm volatile("bar.sync %0, %1;" ::"r"(worker + 1), "r"(WORKER_THREADS) : "memory");
+  // Two lanes share the end of a tile: lane 0 frees the tile's memory and goes straight on to take the next
+  // tile, the first lane of warp 1 posts the finished one to the retire warp meanwhile (both meet again at the
+  // barrier that opens the next tile).
+  if (wt == 0) {
+    atomicAdd(&ctx.control->tiles_done, 1ull);
+    if (cmd.t0 == 1) {
+      if (cmd.smem_units) atomicAnd(&sm->smem_mask, ~(unit_bits(cmd.smem_units) << cmd.smem_unit0));
+      if (cmd.tmem_units) atomicAnd(&sm->tmem_mask, ~(unsigned)(unit_bits(cmd.tmem_units) << cmd.tmem_unit0));
+    }
+    slot->busy = 0;
+    if (slot->held_tail == slot->held_head && slot->prio_tail == slot->prio_head) bell_ring(&sm->bell_claim);   // out of work
+  } else if (wt == 32) {
+    const uint64_t t1 = gtimer();
+    WorkerTile d = cmd;
+    d.t0 = cmd.t1; d.t1 = t1;
+    unsigned naps = 0;
+    while (slot->done_state != 0) {
+      __nanosleep(40);
+      if ((++naps & 0xFFFFu) == 0 && gtimer() - t1 > 2 * ctx.wait_limit_ns) break;   // retire warp gone: give up posting
+    }
+    slot->done = d;
+    // The tile's writes (all threads, ordered by the barrier above) must be visible device-wide before any
+    // successor is released.  That fence is the retire warp's (first statement of complete_tile, after it has
+    // read this flag): fences are cumulative, and barrier -> block-scope fence -> flag -> device-scope fence
+    // keeps the writes ahead of the counter atomics without a device-scope round trip on the worker's path.
+    __threadfence_block();
+    slot->done_state = 1;
+    bell_ring(&sm->bell_retire);
+    atomicSub(&sm->pick.cta_count[d.cls], 1);    // the pick's view of this SM, after the completion is on its way
+    for (int x = 0; x < 3; ++x) atomicSub(&sm->pick.u[x], sm->tau_tab[d.cls * 3 + x]);
+  }
+}
+
 // ------------------------------------------------------------------ the persistent co-scheduling kernel
 // One CTA per SM: `workers` worker groups of WORKER_THREADS threads run tiles; one more warp is the
 // dispatcher.  Every wait is bounded by ctx.wait_limit_ns.
@@ -596,8 +655,6 @@ __global__ void __launch_bounds__(MAX_WORKERS* WORKER_THREADS + DISPATCH_THREADS
   char* slab = smem_raw + SM_STATE_BYTES;
   const int n_workers = (blockDim.x - DISPATCH_THREADS) / WORKER_THREADS;
   const bool is_dispatcher = threadIdx.x >= n_workers * WORKER_THREADS;
-  const int worker = threadIdx.x / WORKER_THREADS;
-  const int wt = threadIdx.x % WORKER_THREADS;
   if (threadIdx.x == 0) {
     sm->smem_mask = 0;
     sm->tmem_mask = 0;
@@ -610,19 +667,25 @@ __global__ void __launch_bounds__(MAX_WORKERS* WORKER_THREADS + DISPATCH_THREADS
     sm->tmem_base = 0;
     sm->quit = 0;
     sm->smem_promised = 0; sm->tmem_promised = 0;
-    sm->room_wait = 0u;
+    sm->room_wait = 0u; sm->outstanding = 0;
     mbar_init(smem_u32(&sm->bell_claim), 1); mbar_init(smem_u32(&sm->bell_retire), 1);
     for (int w = 0; w < MAX_WORKERS; ++w) mbar_init(smem_u32(&sm->bell_worker[w]), 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     for (int c = 0; c < N_CLASSES; ++c) sm->ema_ns[c] = 30000;
     for (int c = 0; c < N_CLASSES; ++c)
+    {
       for (int x = 0; x < 3; ++x) sm->tau_tab[c * 3 + x] = ctx.classes[c].tau[x];
+      sm->smem_units[c] = ctx.classes[c].smem_units; sm->tmem_units[c] = ctx.classes[c].tmem_units; sm->grid[c] = 0;
+      sm->res[c] = sm->smem_units[c] > 0 ? sm->smem_units[c] : 1;
+      unsigned m = 0;
+      for (int j = 0; j < N_CLASSES; ++j) m |= (ctx.classes[j].group == ctx.classes[c].group ? 1u : 0u) << j;
+      sm->group_mask[c] = m;
+    }
     for (int w = 0; w < MAX_WORKERS; ++w) {
       sm->slot[w].held_tail = 0; sm->slot[w].held_head = 0; sm->slot[w].leave = 0; sm->slot[w].done_state = 0;
-      sm->slot[w].prio_tail = 0; sm->slot[w].prio_head = 0; sm->slot[w].t_busy = 0;
-
+      sm->slot[w].prio_tail = 0; sm->slot[w].prio_head = 0; sm->slot[w].t_busy = 0; sm->slot[w].start_state = 0;
+      sm->slot[w].turn = 0; sm->slot[w].bell_parity = 0;
       sm->slot[w].busy = 0;
-      sm->slot[w].n_ready = 0;
     }
   }
   __syncthreads();
@@ -636,12 +699,16 @@ __global__ void __launch_bounds__(MAX_WORKERS* WORKER_THREADS + DISPATCH_THREADS
     if (threadIdx.x < n_workers * WORKER_THREADS + 32) claim_loop(ctx, sm, n_workers);
     else retire_loop(ctx, sm, n_workers);
   } else {
-    const int bar_id = worker + 1;
-    WorkerSlot* slot = sm->slot + worker;
-    unsigned long long tiles = 0;
-    uint32_t bell_parity = 0;
+    // Nothing is carried in registers through a tile body (it has use for all of them): a pass of this loop derives its
+    // place from the thread index again and keeps its few counters in the worker's slot.
     for (;;) {
+      unsigned tid;
+      asm volatile("mov.u32 %0, %%tid.x;" : "=r"(tid));
+      const int worker = (int)tid / WORKER_THREADS, wt = (int)tid % WORKER_THREADS, bar_id = worker + 1;
+      WorkerSlot* slot = sm->slot + worker;
       if (wt == 0) {
+        const int turn = slot->turn ^ 1;
+        uint32_t bell_parity = slot->bell_parity;
         // take the tile the claim warp holds for this worker, then give it its exact memory need
         int st;
         unsigned naps = 0;
@@ -653,10 +720,11 @@ __global__ void __launch_bounds__(MAX_WORKERS* WORKER_THREADS + DISPATCH_THREADS
           else bell_wait(&sm->bell_worker[worker], bell_parity, 2000u);
           ++naps;
         }
-        WorkerTile& cur = sm->cur[worker];
+        WorkerTile& cur = sm->cur[worker][turn];
         if (st == 1 || st == 3) {
           cur = st == 3 ? slot->prio : slot->held[slot->held_head % HELD_DEPTH];
           slot->t_busy = gtimer();
+          sm->cur_cls[worker] = cur.cls;
           slot->busy = 1;
           __threadfence_block();
           if (st == 3) slot->prio_head = slot->prio_head + 1;
@@ -664,14 +732,40 @@ __global__ void __launch_bounds__(MAX_WORKERS* WORKER_THREADS + DISPATCH_THREADS
           bell_ring(&sm->bell_claim);
           const uint64_t lim = gtimer() + ctx.wait_limit_ns;
           bool ok = false;
+          if (cur.early) {
+            // A tile taken before its node's release may hold memory while it waits only where no tile taken earlier can
+            // still need some, that is, where it is the only one this SM has taken.  Elsewhere it waits empty-handed.
+            int taken = 0;
+            for (int k = 0; k < N_CLASSES; ++k) taken += *reinterpret_cast<volatile int*>(&sm->pick.cta_count[k]);
+            if (taken != 1) {
+              TileCtx wc;
+              wc.wait_word = ctx.dep_word + (size_t)cur.inst * ctx.n_nodes + cur.node;
+              wc.wait_gen = release_count(ctx, cur.inst);
+              wc.t_start = &cur.t1;
+              wc.deadline = lim; wc.error = &ctl->error;
+              wait_release(wc);
+              cur.early = 0;
+            }
+          }
+          const int need_units = cur.smem_units;
+          int deep_units = 0;
+          if (sm->outstanding <= 2 * (int)gridDim.x) {
+            // Few tiles on the whole GPU: a GEMM tile takes the pipeline depth its K has use for, up to its share of the
+            // SM.  A k-block then costs its share of many loads in flight instead of half or a quarter of a round trip.
+            const int third = sm->n_smem_units / MAX_WORKERS;
+            const int share = sm->outstanding <= (int)gridDim.x / 2 ? sm->n_smem_units : (sm->outstanding <= (int)gridDim.x ? 2 * third : sm->n_smem_units / 2);
+            deep_units = min((__ldg(&ctx.nodes[cur.node].smem_deep) + SMEM_UNIT - 1) / SMEM_UNIT, share);
+          }
           for (unsigned spin = 0;; ++spin) {
+            cur.smem_units = need_units;
             const unsigned long long sm_old = *reinterpret_cast<volatile unsigned long long*>(&sm->smem_mask);
             // every worker has a home region (a third of the slab, a third of the columns): a tile that fits it goes
             // there whenever it is free, so tiles of the common shapes never fragment the slab; larger tiles and a
             // home occupied by one of them fall back to the first free run
             const int home_s = worker * (sm->n_smem_units / n_workers), home_t = worker * (sm->n_tmem_units / n_workers);
             int s0 = -1;
-            if (cur.smem_units <= sm->n_smem_units / n_workers && ((sm_old >> home_s) & unit_bits(cur.smem_units)) == 0ull) s0 = home_s;
+            if (deep_units > need_units && (s0 = find_free(sm_old, deep_units, sm->n_smem_units)) >= 0) cur.smem_units = deep_units;
+            else if (cur.smem_units <= sm->n_smem_units / n_workers && ((sm_old >> home_s) & unit_bits(cur.smem_units)) == 0ull) s0 = home_s;
             else s0 = find_free(sm_old, cur.smem_units, sm->n_smem_units);
             if (s0 >= 0) {
               const unsigned long long sbits = unit_bits(cur.smem_units) << s0;
@@ -691,7 +785,7 @@ __global__ void __launch_bounds__(MAX_WORKERS* WORKER_THREADS + DISPATCH_THREADS
             }
             if (spin == 0)        // waiting for room
               *reinterpret_cast<volatile unsigned*>(&sm->room_wait) =
-                  (unsigned)cur.smem_units | ((unsigned)cur.tmem_units << 8) | ((unsigned)(worker + 1) << 16);
+                  (unsigned)need_units | ((unsigned)cur.tmem_units << 8) | ((unsigned)(worker + 1) << 16);
             __nanosleep(100);
             if ((spin & 255u) == 255u && (gtimer() > lim || ld_volatile_u32(&ctl->error) != 0u)) break;
           }
@@ -701,79 +795,75 @@ __global__ void __launch_bounds__(MAX_WORKERS* WORKER_THREADS + DISPATCH_THREADS
             atomicSub(&sm->smem_promised, cur.succ_begin); atomicSub(&sm->tmem_promised, cur.succ_count);
           }
           if (!ok) set_error(ctx, DEV_ERR_IDLE_LIMIT, 0x2000u + (unsigned)blockIdx.x);
+          if (ok && (int)cur.tile + 1 == __ldg(&ctx.nodes[cur.node].n_tiles)) {   // the node's last tile: its successors may be queued
+            while (slot->start_state != 0 && gtimer() < lim) __nanosleep(20);
+            slot->start_inst = cur.inst; slot->start_node = cur.node;
+            __threadfence_block();
+            slot->start_state = 1;
+            bell_ring(&sm->bell_retire);
+          }
           cur.t0 = ok ? 1 : 2;              // 1 run, 2 skip (error), 0 leave
+          TileCtx& tc = sm->tc[worker];
+          tc.arena = ctx.arena;
+          tc.slot_base = __ldg(ctx.slot_base + cur.inst);
+          tc.smem = slab + (size_t)cur.smem_unit0 * SMEM_UNIT;
+          tc.smem_bytes = cur.smem_units * SMEM_UNIT;
+          tc.ctl = smem_raw + SM_STATE_BASE + worker * SM_CTL_BYTES;
+          tc.tmem = sm->tmem_base + (unsigned)cur.tmem_unit0 * TMEM_UNIT;
+          tc.bar_id = bar_id;
+          tc.error = &ctl->error;
+          tc.tmaps = ctx.tmaps;
+          tc.inputs = ctx.input_ptrs + (size_t)cur.inst * N_FRAME_INPUTS;
+          tc.amap_base = ctx.n_weight_tmaps + (int)cur.inst * ctx.n_act_tmaps;
+          tc.drop_loads = 0;
+          tc.deadline = gtimer() + ctx.wait_limit_ns;
+          tc.wait_word = nullptr;
+          if (cur.early) {
+            tc.wait_word = ctx.dep_word + (size_t)cur.inst * ctx.n_nodes + cur.node;
+            tc.wait_gen = release_count(ctx, cur.inst);
+            tc.t_start = &cur.t1;
+          }
         } else {
           cur.t0 = 0;
         }
+        slot->turn = turn;
+        slot->bell_parity = bell_parity;
+      }
+      if (wt < 32) {
+        __syncwarp();
+        const WorkerTile& cmd = sm->cur[worker][slot->turn];
+        if (cmd.t0 != 0 && wt < (int)(sizeof(NodeDesc) / 16))
+          reinterpret_cast<int4*>(sm->node + worker)[wt] = __ldg(reinterpret_cast<const int4*>(ctx.nodes + cmd.node) + wt);
       }
       asm volatile("bar.sync %0, %1;" ::"r"(bar_id), "r"(WORKER_THREADS) : "memory");
-      const WorkerTile cmd = sm->cur[worker];
+      WorkerTile& cmd = sm->cur[worker][slot->turn];
       if (cmd.t0 == 0) break;
-      const NodeDesc& n = ctx.nodes[cmd.node];
-      TileCtx tc;
-      tc.arena = ctx.arena;
-      tc.slot_base = ctx.slot_base[cmd.inst];
-      tc.smem = slab + (size_t)cmd.smem_unit0 * SMEM_UNIT;
-      tc.ctl = smem_raw + SM_STATE_BASE + worker * SM_CTL_BYTES;
-      tc.tmem = sm->tmem_base + (unsigned)cmd.tmem_unit0 * TMEM_UNIT;
-      tc.tid = wt;
-      tc.bar_id = bar_id;
-      tc.error = &ctl->error;
-      tc.tmaps = ctx.tmaps;
-      tc.inputs = ctx.input_ptrs + (size_t)cmd.inst * N_FRAME_INPUTS;
-      tc.amap_base = ctx.n_weight_tmaps + (int)cmd.inst * ctx.n_act_tmaps;
-      tc.drop_loads = 0;
-      const uint64_t t0 = gtimer();
-      tc.deadline = t0 + ctx.wait_limit_ns;
-      // the frame id is only needed by the emit tile and by the trace
-      const int n_op = __ldg(&n.op);
-      // the node's successor range travels with the finished tile; read it now, while the description is hot
-      const int n_succ_begin = __ldg(&n.succ_begin), n_succ_count = __ldg(&n.succ_count);
-      if (wt == 0) {     // the retire warp of this SM will read the successor records when the tile ends
-        const char* sp = reinterpret_cast<const char*>(ctx.succ + n_succ_begin);
-        asm volatile("prefetch.global.L1 [%0];" ::"l"(sp));
+      {
+        const NodeDesc& n = sm->node[worker];
+        const uint32_t inst = cmd.inst;
+        const TileCtx& tc = sm->tc[worker];
+        const int n_op = n.op;
+        if (cmd.early && n_op != OP_GEMM) {
+          if (wt == 0) wait_release(tc);
+          asm volatile("bar.sync %0, %1;" ::"r"(bar_id), "r"(WORKER_THREADS) : "memory");
+        }
+        // the frame id is only needed by the emit tile and by the trace
+        const uint64_t frame = (ctx.trace_capacity != 0 || n_op == OP_EMIT)
+                                   ? *reinterpret_cast<const volatile uint64_t*>(ctx.inst_frame + inst) : 0ull;
+        if (wt == 32) {     // what the retire warp of this SM will need when the tile ends; its successor records come into L1 now
+          cmd.op = n_op;
+          cmd.succ_begin = n.succ_begin; cmd.succ_count = n.succ_count;
+          cmd.frame = frame;
+          if (!cmd.early) cmd.t1 = gtimer();
+          asm volatile("prefetch.global.L1 [%0];" ::"l"(reinterpret_cast<const char*>(ctx.succ + cmd.succ_begin)));
+        }
+        if (cmd.t0 == 1) run_tile<false>(ctx, tc, n, (int)cmd.tile, (int)inst, frame);
       }
-      const uint64_t frame = (ctx.trace_capacity != 0 || n_op == OP_EMIT)
-                                 ? *reinterpret_cast<const volatile uint64_t*>(ctx.inst_frame + cmd.inst) : 0ull;
-      if (cmd.t0 == 1) run_tile(ctx, tc, n, (int)cmd.tile, (int)cmd.inst, frame);
       // Outputs written here by ordinary stores are read by TMA on other SMs.  The proxy fence that must lie between
       // the two in causality order is the consumer's (first statement of its TMA-issuing thread, after the
       // dependency was observed); a second one here cost 2 % of the throughput and is not needed.
-      asm volatile("bar.sync %0, %1;" ::"r"(bar_id), "r"(WORKER_THREADS) : "memory");
-      // Two lanes share the end of a tile: lane 0 frees the tile's memory and goes straight on to take the next
-      // tile, the first lane of warp 1 posts the finished one to the retire warp meanwhile (both meet again at the
-      // barrier that opens the next tile).
-      if (wt == 0) {
-        ++tiles;
-        if (cmd.t0 == 1) {
-          if (cmd.smem_units) atomicAnd(&sm->smem_mask, ~(unit_bits(cmd.smem_units) << cmd.smem_unit0));
-          if (cmd.tmem_units) atomicAnd(&sm->tmem_mask, ~(unsigned)(unit_bits(cmd.tmem_units) << cmd.tmem_unit0));
-        }
-        slot->busy = 0;
-        if (slot->held_tail == slot->held_head && slot->prio_tail == slot->prio_head) bell_ring(&sm->bell_claim);   // out of work
-      } else if (wt == 32) {
-        const uint64_t t1 = gtimer();
-        WorkerTile d = cmd;
-        d.t0 = t0; d.t1 = t1; d.frame = frame;
-        d.succ_begin = n_succ_begin; d.succ_count = n_succ_count; d.op = n_op;
-        unsigned naps = 0;
-        while (slot->done_state != 0) {
-          __nanosleep(40);
-          if ((++naps & 0xFFFFu) == 0 && gtimer() - t0 > 2 * ctx.wait_limit_ns) break;   // retire warp gone: give up posting
-        }
-        slot->done = d;
-        // The tile's writes (all threads, ordered by the barrier above) must be visible device-wide before any
-        // successor is released.  That fence is the retire warp's (first statement of complete_tile, after it has
-        // read this flag): fences are cumulative, and barrier -> block-scope fence -> flag -> device-scope fence
-        // keeps the writes ahead of the counter atomics without a device-scope round trip on the worker's path.
-        __threadfence_block();
-        slot->done_state = 1;
-        bell_ring(&sm->bell_retire);
-        atomicSub(&sm->pick.cta_count[cmd.cls], 1);    // the pick's view of this SM, after the completion is on its way
-        for (int x = 0; x < 3; ++x) atomicSub(&sm->pick.u[x], sm->tau_tab[cmd.cls * 3 + x]);
-      }
+      end_of_tile(ctx, sm, slot);
     }
-    if (wt == 0) atomicAdd(&ctl->tiles_done, tiles);
   }
   tc_fence_before();
   __syncthreads();
@@ -799,19 +889,20 @@ __global__ void __launch_bounds__(WORKER_THREADS) vla_node_kernel(DeviceCtx ctx,
   tc.arena = ctx.arena;
   tc.slot_base = inst >= 0 ? ctx.slot_base[inst] : 0;
   tc.smem = smem_raw;
+  tc.smem_bytes = n.smem_bytes;
   tc.ctl = ctl_block;
   tc.tmem = tmem_cols ? tmem_base_s : 0;
-  tc.tid = threadIdx.x;
   tc.bar_id = 1;
   tc.error = &ctx.control->error;
   tc.tmaps = ctx.tmaps;
   tc.inputs = ctx.input_ptrs + (size_t)(inst >= 0 ? inst : 0) * N_FRAME_INPUTS;
   tc.amap_base = ctx.n_weight_tmaps + (inst >= 0 ? inst : 0) * ctx.n_act_tmaps;
   tc.drop_loads = 0;
+  tc.wait_word = nullptr;
   const uint64_t t0 = gtimer();
   tc.deadline = t0 + ctx.wait_limit_ns;
   const uint64_t frame = inst >= 0 ? ctx.inst_frame[inst] : 0;
-  run_tile(ctx, tc, n, (int)blockIdx.x, inst, frame);
+  run_tile<true>(ctx, tc, n, (int)blockIdx.x, inst, frame);
   if (inst >= 0 && ctx.trace_capacity) {
     asm volatile("bar.sync 1, %0;" ::"r"(WORKER_THREADS) : "memory");
     if (threadIdx.x == 0) write_trace(ctx, (uint32_t)inst, (uint32_t)node_idx, blockIdx.x, 0, n.cls, frame, t0, gtimer());

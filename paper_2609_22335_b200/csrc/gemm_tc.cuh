@@ -2,19 +2,18 @@
 // 128-byte-swizzled shared memory, tcgen05.mma accumulating in tensor memory,
 // epilogue read back with tcgen05.ld.
 //
-// Tile: 128 output features (MMA M, one TMEM lane each) x bt tokens (MMA N,
-// one TMEM column each), K walked in 64-element stages.  The weight tile is
-// the MMA "A" operand and the activation tile the "B" operand, both K-major, so
-// small token counts (the action head's 9..51 rows) still fill the 128-row
-// datapath and stream each weight exactly once.  A gated MLP tile covers 64
-// output features: rows 0..63 of its weight tile are gate rows and rows 64..127
-// the matching up rows (two 64-row TMA boxes per stage), so it is one MMA stream
-// and one accumulator like any other tile; the epilogue multiplies act(gate) by up.
+// Tile: up to 128 tokens (MMA M, one TMEM lane each) x 128 weight rows (MMA N, one
+// TMEM column each), K walked in 64-element stages, both operands K-major.  Where a node
+// has few tokens (the action head's 9..51) the activation box is only as high as they
+// need; the MMA reads on into the weight tile behind it and leaves lanes nobody looks at.
+// A gated MLP tile covers 64 output features: gate and up rows alternate in its weight
+// matrix, so it is one MMA stream and one accumulator like any other tile; the epilogue
+// multiplies act(gate) by up.
 //
 // Roles inside the 128-thread worker: thread 0 of warp 0 issues TMA loads,
-// thread 0 of warp 1 issues MMAs, all four warps run the epilogue (warp w reads
-// TMEM lanes 32w..32w+31).  Every mbarrier wait is bounded; on expiry the worker
-// records an error and leaves the tile.
+// warp 1 issues MMAs, all four warps run the epilogue (warp w reads
+// TMEM lanes 32w..32w+31, a token per thread).  Every mbarrier wait is bounded; on expiry
+// the worker records an error and leaves the tile.
 #pragma once
 #include "tiles_common.cuh"
 
@@ -31,29 +30,28 @@ __device__ __forceinline__ void mbar_inval(uint32_t bar) {
 __device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
 }
-__device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
+// Suspended by the hardware until the phase completes or about `hint_ns` have passed: a waiting warp takes no issue slots
+// from the warps that share its scheduler.
+__device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity, uint32_t hint_ns) {
   uint32_t ok;
   asm volatile(
       "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
       "selp.b32 %0, 1, 0, p;\n\t}"
       : "=r"(ok)
-      : "r"(bar), "r"(parity)
+      : "r"(bar), "r"(parity), "r"(hint_ns)
       : "memory");
   return ok != 0;
 }
 // Bounded wait: false when the deadline passed or another worker already reported an error.
 __device__ __forceinline__ bool mbar_wait(const TileCtx& c, uint32_t bar, uint32_t parity) {
-  unsigned spins = 0;
-  while (!mbar_try_wait(bar, parity)) {
-    if ((++spins & 1023u) == 0) {
-      if (*reinterpret_cast<volatile unsigned*>(c.error) != 0u) return false;
-      uint64_t now;
-      asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
-      if (now > c.deadline) {
-        atomicCAS(c.error, 0u, (unsigned)DEV_ERR_WAIT_MBAR);
-        return false;
-      }
+  while (!mbar_try_wait(bar, parity, 20000u)) {
+    if (*reinterpret_cast<volatile unsigned*>(c.error) != 0u) return false;
+    uint64_t now;
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
+    if (now > c.deadline) {
+      atomicCAS(c.error, 0u, (unsigned)DEV_ERR_WAIT_MBAR);
+      return false;
     }
   }
   return true;
@@ -64,6 +62,10 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const void* tmap, uint
       "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
       ::"r"(dst), "l"(tmap), "r"(bar), "r"(x), "r"(y)
       : "memory");
+}
+
+__device__ __forceinline__ void tma_prefetch_2d(const void* tmap, int x, int y) {
+  asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global.tile [%0, {%1, %2}];" ::"l"(tmap), "r"(x), "r"(y) : "memory");
 }
 
 // Shared-memory matrix descriptor: K-major operand, 128-byte swizzle, rows of 128 bytes,
@@ -95,12 +97,6 @@ __device__ __forceinline__ void umma_commit(uint32_t bar) {
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
-// 16-byte asynchronous copy global -> shared through L2 (the source was written by other SMs)
-__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
-
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
   uint32_t r[16];
   asm volatile(
@@ -124,338 +120,342 @@ __device__ __forceinline__ void tmem_ld16_nowait(uint32_t taddr, uint32_t* r) {
 }
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
-// Epilogue phase 1 (thread = output feature, the TMEM lane it owns): read the accumulators 16 token columns at a
-// time, apply the row scale and the activation, and park the values in shared memory as [token][feature]; a
-// feature of the V^T part of a q|k|v projection is written from here, 16 consecutive tokens per store pair.
-struct Phase1Args {
-  float* St; const float* rs; unsigned short* outT_row;
-  float c_acc, c_x, bias; uint32_t lane_base; int bt, nt, tid, t0;
-  bool x_staged;            // the residual rows already sit in St: accumulate on top of them
-};
-template <int ACT>
-__device__ __forceinline__ void gemm_phase1(const Phase1Args& p) {
-  for (int c0 = 0; c0 < p.nt; c0 += 16) {
-    float a[16], v[16], sc[16];
-    tmem_ld16(p.lane_base + (uint32_t)c0, a);
-    if (p.rs) {                                        // 16 row scales in four broadcast 16-byte loads
+__device__ __forceinline__ void tmem_st16(uint32_t taddr, const float* v) {
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};"
+      ::"r"(taddr), "r"(__float_as_uint(v[0])), "r"(__float_as_uint(v[1])), "r"(__float_as_uint(v[2])),
+        "r"(__float_as_uint(v[3])), "r"(__float_as_uint(v[4])), "r"(__float_as_uint(v[5])), "r"(__float_as_uint(v[6])),
+        "r"(__float_as_uint(v[7])), "r"(__float_as_uint(v[8])), "r"(__float_as_uint(v[9])), "r"(__float_as_uint(v[10])),
+        "r"(__float_as_uint(v[11])), "r"(__float_as_uint(v[12])), "r"(__float_as_uint(v[13])), "r"(__float_as_uint(v[14])),
+        "r"(__float_as_uint(v[15]))
+      : "memory");
+}
+__device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+
+// One lane of a converged warp (warp-uniform control flow around the asynchronous instructions it guards lets their
+// descriptors live in uniform registers: 200 instead of 230 cycles per four-MMA k-block at N <= 64).
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.b32 %0, 1, 0, p;\n\t}" : "=r"(p));
+  return p != 0;
+}
+
+// ------------------------------------------------------------------ epilogue
+// Straight from tensor memory to global memory, sixteen columns at a time; nothing is staged.  A thread owns one token, so
+// its row scale, its sum of squares, gate and up values, rotary pairs and sixteen-byte stores all lie in its own registers.
+// A lone warp per scheduler pays for instructions (one every three or four cycles) and above all for branches (about 30
+// cycles each, taken or skipped over): the five common kinds of result have straight loops of their own, everything else
+// goes through one general loop.  (With every kind unrolled for every activation the kernel had 160 KB of epilogues and 30 %
+// of its instruction fetches missed the cache; with the general loop alone a chunk cost 600 cycles.)
+constexpr int EPI = 16;
+
+template <int ACT, int N>
+__device__ __forceinline__ void activate(float* v) {
 #pragma unroll
-      for (int j = 0; j < 16; j += 4) {
-        const float4 r4 = *reinterpret_cast<const float4*>(p.rs + c0 + j);
-        sc[j] = r4.x; sc[j + 1] = r4.y; sc[j + 2] = r4.z; sc[j + 3] = r4.w;
-      }
-    } else {
+  for (int j = 0; j < N; ++j) v[j] = apply_act_t<ACT>(v[j]);
+}
+__device__ __forceinline__ uint32_t pack_bf16(float x, float y) {
+  __nv_bfloat162 h = __floats2bfloat162_rn(x, y);
+  return *reinterpret_cast<uint32_t*>(&h);
+}
+__device__ __forceinline__ void put16(unsigned short* p, const float* v) {
 #pragma unroll
-      for (int j = 0; j < 16; ++j) sc[j] = 1.0f;
+  for (int j = 0; j < EPI; j += 8)
+    *reinterpret_cast<uint4*>(p + j) = make_uint4(pack_bf16(v[j], v[j + 1]), pack_bf16(v[j + 2], v[j + 3]), pack_bf16(v[j + 4], v[j + 5]), pack_bf16(v[j + 6], v[j + 7]));
+}
+// v[j] += scale * p[j], j < n (n = EPI: four 16-byte loads, else element by element)
+__device__ __forceinline__ void add_row(float* v, const float* p, int n, float scale) {
+  if (n == EPI) {
+#pragma unroll
+    for (int j = 0; j < EPI; j += 4) {
+      const float4 t = __ldcg(reinterpret_cast<const float4*>(p + j));
+      v[j] = fmaf(scale, t.x, v[j]); v[j + 1] = fmaf(scale, t.y, v[j + 1]);
+      v[j + 2] = fmaf(scale, t.z, v[j + 2]); v[j + 3] = fmaf(scale, t.w, v[j + 3]);
     }
+  } else {
 #pragma unroll
-    for (int j = 0; j < 16; ++j) {
-      v[j] = apply_act_t<ACT>(fmaf(a[j], sc[j], p.bias)) * p.c_acc;
-    }
-    if (p.outT_row) {
-      unsigned short* op = p.outT_row + p.t0 + c0;
-      uint32_t pk[8];
-#pragma unroll
-      for (int j = 0; j < 16; j += 2) {
-        __nv_bfloat162 h = __floats2bfloat162_rn(v[j], v[j + 1]);
-        pk[j >> 1] = *reinterpret_cast<uint32_t*>(&h);
-      }
-      if (p.nt - c0 >= 16) {
-        *reinterpret_cast<uint4*>(op) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
-        *reinterpret_cast<uint4*>(op + 8) = make_uint4(pk[4], pk[5], pk[6], pk[7]);
-      } else {
-#pragma unroll
-        for (int j = 0; j < 16; ++j)
-          if (j < p.nt - c0) op[j] = (unsigned short)((j & 1) ? (pk[j >> 1] >> 16) : (pk[j >> 1] & 0xFFFFu));
-      }
-    }
-    float* sp = p.St + (size_t)c0 * GEMM_BM + p.tid;
-    if (p.x_staged) {
-      float x[16];
-#pragma unroll
-      for (int j = 0; j < 16; ++j) x[j] = sp[j * GEMM_BM];
-#pragma unroll
-      for (int j = 0; j < 16; ++j) sp[j * GEMM_BM] = fmaf(p.c_x, x[j], v[j]);
-    } else {
-#pragma unroll
-      for (int j = 0; j < 16; ++j) sp[j * GEMM_BM] = v[j];
-    }
+    for (int j = 0; j < EPI; ++j)
+      if (j < n) v[j] = fmaf(scale, ld_act(p + j), v[j]);
   }
 }
 
-// Epilogue phase 2, rows of the staged tile (warp = token row, lane = four consecutive features).  A template
-// flag that is false removes that output or addend statically; one that is true is still checked per lane (a
-// lane beyond the last feature, or one whose columns went to V^T, has a null pointer).  Branches cost a lone warp
-// dearly, so the common shapes get straight-line code.
-struct Phase2Args {
-  const float* tab; const float* tab2; float* o32; unsigned short* o16; float* St;
-  float4 vecv;
-  size_t ldo32, ldo16, ldtab, ldtab2;
-  int nt, t0, warp, lane, gf;
-  bool fok, ss;
-};
-template <bool TAB, bool O32, bool O16, bool SS>
-__device__ __forceinline__ void gemm_phase2_row(const Phase2Args& p, int tok, float4 w) {
-  const int r = p.t0 + tok;
-  if (TAB) {
-    w.x += p.vecv.x; w.y += p.vecv.y; w.z += p.vecv.z; w.w += p.vecv.w;
-    if (p.tab) {
-      const float4 t = *reinterpret_cast<const float4*>(p.tab + (size_t)r * p.ldtab + p.gf);
-      w.x += t.x; w.y += t.y; w.z += t.z; w.w += t.w;
-    }
-    if (p.tab2) {
-      const float4 t = *reinterpret_cast<const float4*>(p.tab2 + (size_t)r * p.ldtab2 + p.gf);
-      w.x += t.x; w.y += t.y; w.z += t.z; w.w += t.w;
-    }
+// Calls body(c0, v) for the accumulator columns [lo, hi) of this thread's token, scaled by rs; the next chunk is on its way
+// from tensor memory meanwhile.
+template <typename F>
+__device__ __forceinline__ void epi_chunks(uint32_t tmem, int lo, int hi, float rs, F body) {
+  if (lo >= hi) return;
+  uint32_t nx[EPI];
+  tmem_ld16_nowait(tmem + (uint32_t)lo, nx);
+#pragma unroll 1
+  for (int c0 = lo; c0 < hi; c0 += EPI) {
+    float v[EPI];
+    tmem_ld_wait();
+#pragma unroll
+    for (int j = 0; j < EPI; ++j) v[j] = __uint_as_float(nx[j]) * rs;
+    tmem_ld16_nowait(tmem + (uint32_t)min(c0 + EPI, hi - EPI), nx);          // (the last chunk again after the last one)
+    body(c0, v);
   }
-  if (O32 && p.o32) *reinterpret_cast<float4*>(p.o32 + (size_t)r * p.ldo32 + p.gf) = w;
-  if (O16) {
-    __nv_bfloat162 lo = __floats2bfloat162_rn(w.x, w.y), hi = __floats2bfloat162_rn(w.z, w.w);
-    if (p.o16)
-      *reinterpret_cast<uint2*>(p.o16 + (size_t)r * p.ldo16 + p.gf) = make_uint2(*reinterpret_cast<uint32_t*>(&lo), *reinterpret_cast<uint32_t*>(&hi));
-  }
-  if (SS && p.ss) {
-    // the lane's share of the row's sum of squares, parked in the row's first 32 words at a position rotated by
-    // the row's slot so that the final per-row additions run without bank conflicts
-    const float sq = p.fok ? (w.x * w.x + w.y * w.y + w.z * w.z + w.w * w.w) : 0.f;
-    p.St[(size_t)tok * GEMM_BM + ((p.lane + (tok >> 2)) & 31)] = sq;
-  }
+  tmem_ld_wait();
 }
-template <bool TAB, bool O32, bool O16, bool SS>
-__device__ __forceinline__ void gemm_phase2_rows(const Phase2Args& p) {
-  constexpr int RP = 4;                              // token rows per pass
-  int tok0 = p.warp;
-  for (; tok0 + 4 * (RP - 1) < p.nt; tok0 += 4 * RP) {   // full passes: no per-row bound checks
-    float4 v[RP];
+template <int ACT>
+__device__ __forceinline__ void epi_gated(uint32_t tmem, int cols, float rs, float c_acc, unsigned short* out, bool live) {
+  epi_chunks(tmem, 0, cols, rs, [&](int c0, float* v) {      // columns 2i, 2i + 1: gate and up value of output feature i
+    float o[EPI / 2];
 #pragma unroll
-    for (int q = 0; q < RP; ++q) v[q] = *reinterpret_cast<const float4*>(p.St + (size_t)(tok0 + 4 * q) * GEMM_BM + 4 * p.lane);
-    if (SS) __syncwarp();                            // every lane has its part of the rows before partial sums overwrite them
+    for (int j = 0; j < EPI / 2; ++j) o[j] = v[2 * j];
+    activate<ACT, EPI / 2>(o);
 #pragma unroll
-    for (int q = 0; q < RP; ++q) gemm_phase2_row<TAB, O32, O16, SS>(p, tok0 + 4 * q, v[q]);
-  }
-  for (; tok0 < p.nt; tok0 += 4) {                   // ragged tail, one row at a time
-    const float4 v = *reinterpret_cast<const float4*>(p.St + (size_t)tok0 * GEMM_BM + 4 * p.lane);
-    if (SS) __syncwarp();
-    gemm_phase2_row<TAB, O32, O16, SS>(p, tok0, v);
-  }
+    for (int j = 0; j < EPI / 2; ++j) o[j] *= v[2 * j + 1] * c_acc;
+    if (live) *reinterpret_cast<uint4*>(out + (c0 >> 1)) = make_uint4(pack_bf16(o[0], o[1]), pack_bf16(o[2], o[3]), pack_bf16(o[4], o[5]), pack_bf16(o[6], o[7]));
+  });
 }
 
-// Rows of a gated tile: columns 0..63 of the staged row are gate values, 64..127 the up values of the same 64
-// features.  Sixteen lanes cover a row (four features each), so a warp does two rows per pass.
-template <int ACT>
-__device__ __forceinline__ void gemm_phase2_rows_gated(const Phase2Args& p, float c_acc, int f0, int N) {
-  const int sub = p.lane >> 4, l16 = p.lane & 15;
-  const int gf = f0 + 4 * l16;
-  const bool fok = gf < N;
-  for (int tok0 = p.warp; tok0 < p.nt; tok0 += 8) {
-    const int tok = tok0 + 4 * sub;
-    if (tok < p.nt && fok) {
-      const float4 gt = *reinterpret_cast<const float4*>(p.St + (size_t)tok * GEMM_BM + 4 * l16);
-      const float4 up = *reinterpret_cast<const float4*>(p.St + (size_t)tok * GEMM_BM + GEMM_BM / 2 + 4 * l16);
-      const float w0 = apply_act_t<ACT>(gt.x) * up.x * c_acc, w1 = apply_act_t<ACT>(gt.y) * up.y * c_acc;
-      const float w2 = apply_act_t<ACT>(gt.z) * up.z * c_acc, w3 = apply_act_t<ACT>(gt.w) * up.w * c_acc;
-      __nv_bfloat162 lo = __floats2bfloat162_rn(w0, w1), hi = __floats2bfloat162_rn(w2, w3);
-      *reinterpret_cast<uint2*>(p.o16 + (size_t)(p.t0 + tok) * p.ldo16 + gf) =
-          make_uint2(*reinterpret_cast<uint32_t*>(&lo), *reinterpret_cast<uint32_t*>(&hi));
+// One token's row of the tile.  `tok` is the token's index in the node (a lane past the last token repeats it, `live` false,
+// and stores nothing), `r0` the tile's first weight row, `rs` the token's row scale, `under` says that the accumulators
+// already hold X.
+__device__ __forceinline__ void gemm_epilogue(const TileCtx& c, const GemmArgs& g, uint32_t tmem, int tok, bool live, int r0, float rs, bool under,
+                                              int ft) {
+  const int act = g.act, N = g.N;
+  const float c_acc = g.c_acc;
+  const GemmPtrs ptrs = gemm_ptrs(c, g);
+  float* const ssq_out = resolve<float>(c, g.ss_out);
+  float* const out32 = ptrs.out32 ? ptrs.out32 + (size_t)tok * g.ldo32 + r0 : nullptr;
+  unsigned short* const out16 = ptrs.out16 ? ptrs.out16 + (size_t)tok * g.ldo16 + (g.dual ? r0 / 2 : r0) : nullptr;
+  const int cols = min(GEMM_BM, (g.dual ? 2 * N : N) - r0);
+  if (g.vec16) {
+    if (g.dual) {
+      if (act == ACT_SILU) epi_gated<ACT_SILU>(tmem, cols, rs, c_acc, out16, live);
+      else if (act == ACT_GELU) epi_gated<ACT_GELU>(tmem, cols, rs, c_acc, out16, live);
+      else epi_gated<ACT_NONE>(tmem, cols, rs, c_acc, out16, live);
+      return;
+    }
+    const bool plain = !ptrs.bias && !ptrs.vec && !ptrs.tab && !ptrs.tab2 && (!ptrs.X || under) && c_acc == 1.0f;
+    if (plain && !ssq_out && !ptrs.out32 && act != ACT_SILU) {            // bf16 only (q|k|v, MLP up, cross projections)
+      int split = cols;                                                     // columns from here on are V features
+      if (ptrs.outT) split = max(0, min(cols, g.t_col0 - r0));
+      if (act == ACT_GELU)
+        epi_chunks(tmem, 0, split, rs, [&](int c0, float* v) { activate<ACT_GELU, EPI>(v); if (live) put16(out16 + c0, v); });
+      else if (g.rope_cols > 0) {       // q and k columns: rotary pairs are neighbours; the table holds (cos, sin) per pair
+        const float* t0 = resolve<const float>(c, g.rope_tab) + (size_t)tok * g.rope_hd;
+        epi_chunks(tmem, 0, split, rs, [&](int c0, float* v) {
+          const float4* t = reinterpret_cast<const float4*>(t0 + (r0 + c0) % g.rope_hd);
+#pragma unroll
+          for (int j = 0; j < EPI; j += 4) {
+            const float4 cs = __ldg(t + (j >> 2));
+            const float x0 = v[j], x1 = v[j + 1], x2 = v[j + 2], x3 = v[j + 3];
+            v[j] = fmaf(x0, cs.x, -x1 * cs.y); v[j + 1] = fmaf(x1, cs.x, x0 * cs.y);
+            v[j + 2] = fmaf(x2, cs.z, -x3 * cs.w); v[j + 3] = fmaf(x3, cs.z, x2 * cs.w);
+          }
+          if (live) put16(out16 + c0, v);
+        });
+      } else
+        epi_chunks(tmem, 0, split, rs, [&](int c0, float* v) { if (live) put16(out16 + c0, v); });
+      if (split < cols) {               // rows of V^T, a warp's tokens side by side
+        unsigned short* const base = ptrs.outT + (ptrdiff_t)(r0 - g.t_col0) * g.ldoT + tok;
+        epi_chunks(tmem, split, cols, rs, [&](int c0, float* v) {
+          unsigned short* op = base + (ptrdiff_t)c0 * g.ldoT;
+          if (live) {
+#pragma unroll
+            for (int j = 0; j < EPI; ++j) { *op = f32_to_bf16_bits(v[j]); op += g.ldoT; }
+          }
+        });
+      }
+      return;
+    }
+    if (plain && act == ACT_NONE && out32 && out16 && ssq_out) {            // residual stream
+      float sq = 0.f;
+      epi_chunks(tmem, 0, cols, rs, [&](int c0, float* v) {
+#pragma unroll
+        for (int j = 0; j < EPI; ++j) sq = fmaf(v[j], v[j], sq);
+        if (live) {
+#pragma unroll
+          for (int j = 0; j < EPI; j += 4) *reinterpret_cast<float4*>(out32 + c0 + j) = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+          put16(out16 + c0, v);
+        }
+      });
+      if (live) ssq_out[(size_t)tok * g.ss_out_ld + ft] = sq;
+      return;
     }
   }
+  // ---- anything else: biases, tables, addends, solver coefficients, odd widths
+  float sq = 0.f;
+#pragma unroll 1
+  for (int c0 = 0; c0 < cols; c0 += EPI) {
+    const int f = r0 + c0, n = g.vec16 ? EPI : min(EPI, (g.dual ? 2 * N : N) - f);
+    float v[EPI];
+    tmem_ld16(tmem + (uint32_t)c0, v);
+#pragma unroll
+    for (int j = 0; j < EPI; ++j) v[j] *= rs;
+    if (g.dual) {
+#pragma unroll
+      for (int j = 0; j < EPI / 2; ++j)
+        if (live && 2 * j < n) out16[(c0 >> 1) + j] = f32_to_bf16_bits(apply_act(act, v[2 * j]) * v[2 * j + 1] * c_acc);
+      continue;
+    }
+    if (ptrs.bias) add_row(v, ptrs.bias + f, n, 1.0f);
+    if (act == ACT_GELU) activate<ACT_GELU, EPI>(v);
+    else if (act == ACT_SILU) activate<ACT_SILU, EPI>(v);
+#pragma unroll
+    for (int j = 0; j < EPI; ++j) v[j] *= c_acc;
+    if (ptrs.X && !under) add_row(v, ptrs.X + (size_t)tok * g.ldx + f, n, g.c_x);
+    if (ptrs.vec) add_row(v, ptrs.vec + f, n, 1.0f);
+    if (ptrs.tab) add_row(v, ptrs.tab + (size_t)tok * g.ldtab + f, n, 1.0f);
+    if (ptrs.tab2) add_row(v, ptrs.tab2 + (size_t)tok * g.ldtab2 + f, n, 1.0f);
+#pragma unroll
+    for (int j = 0; j < EPI; ++j)
+      if (j < n) sq = fmaf(v[j], v[j], sq);
+    if (!live) continue;
+    if (ptrs.outT && f >= g.t_col0) {
+      unsigned short* op = ptrs.outT + (size_t)(f - g.t_col0) * g.ldoT + tok;
+#pragma unroll
+      for (int j = 0; j < EPI; ++j) { *op = f32_to_bf16_bits(v[j]); op += g.ldoT; }
+    } else if (g.vec16) {
+      if (out32) {
+#pragma unroll
+        for (int j = 0; j < EPI; j += 4) *reinterpret_cast<float4*>(out32 + c0 + j) = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+      }
+      if (out16) put16(out16 + c0, v);
+    } else {
+#pragma unroll
+      for (int j = 0; j < EPI; ++j) {
+        if (j < n && out32) out32[c0 + j] = v[j];
+        if (j < n && out16) out16[c0 + j] = f32_to_bf16_bits(v[j]);
+      }
+    }
+  }
+  if (ssq_out && live) ssq_out[(size_t)tok * g.ss_out_ld + ft] = sq;
 }
 
 constexpr int GEMM_W_STAGE_BYTES = GEMM_BM * GEMM_BK * 2;
 
-__device__ void tile_gemm(const TileCtx& c, const GemmArgs& g, int tile) {
-  const int ft = tile / g.tiles_t, tt = tile % g.tiles_t;
-  const int f0 = ft * (g.dual ? GEMM_BM / 2 : GEMM_BM), t0 = tt * g.bt;    // a gated tile covers 64 output features
-  const int nt = min(g.bt, g.M - t0);
-  const int warp = c.tid >> 5, lane = c.tid & 31;
-  const int nkb = g.Kp / GEMM_BK;
-  const int S = g.stages;
-  const int a_bytes = g.bt * GEMM_BK * 2;
-  const bool dual = g.dual != 0;            // arguments used inside the loops, out of global memory once
+// What bounds it: with one tile per SM, the issuing lanes (per k-block one barrier test, two loads, four MMAs) and the
+// round trip of a stage; with three, instruction fetch and the L2-to-shared-memory path.  Stage and phase run along instead
+// of being divided out of the k-block index (a runtime division per role cost as much as the four MMAs).
+__device__ __forceinline__ void tile_gemm(const TileCtx& c, const GemmArgs& g, int tile) {
   const int bt = g.bt;
-  const int stage_bytes = GEMM_W_STAGE_BYTES + a_bytes;
+  const int ft = tile / g.tiles_t, t0 = tile % g.tiles_t * bt, r0 = ft * GEMM_BM;   // first token and first weight row of the tile
+  const int nt = min(bt, g.M - t0);
+  const int warp = worker_tid() >> 5, lane = worker_tid() & 31;
+  const int nkb = g.Kp / GEMM_BK;
+  const int S = gemm_stages_in(c.smem_bytes, bt, g.Kp, g.stages);
+  const uint32_t a_bytes = (uint32_t)(bt * GEMM_BK * 2), stage_bytes = a_bytes + GEMM_W_STAGE_BYTES;   // activations, then weights
 
-  uint64_t* bars = reinterpret_cast<uint64_t*>(c.ctl);           // full[S], empty[S], accum (the worker's control block)
-  const uint32_t bar0 = smem_u32(bars);
+  const uint32_t bar0 = smem_u32(c.ctl);               // full[S], empty[S], accum (the worker's control block)
   const uint32_t stage0 = smem_u32(c.smem);
-  auto full_bar = [&](int s) { return bar0 + 8u * s; };
-  auto empty_bar = [&](int s) { return bar0 + 8u * (S + s); };
-  const uint32_t accum_bar = bar0 + 8u * (2 * S);
+  const uint32_t accum_bar = bar0 + 16u * (uint32_t)S;
+  if (warp == 0) {
+    if (lane <= 2 * S) {                               // (2 S + 1 <= 25 barriers: one lane each)
+      mbar_init(bar0 + 8u * lane, 1);
+      asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    __syncwarp();
+  }
+  const char* tm = reinterpret_cast<const char*>(c.tmaps);
+  const void* wmap = tm + (size_t)g.wmap * 128;
+  const void* amap = tm + (size_t)(c.amap_base + g.amap) * 128;
+  auto load_w = [&](int kb, uint32_t bar, uint32_t dst) {
+    mbar_expect_tx(bar, stage_bytes);
+    tma_load_2d(dst + a_bytes, wmap, bar, kb * GEMM_BK, r0);
+  };
+  auto load_a = [&](int kb, uint32_t bar, uint32_t dst) { tma_load_2d(dst, amap, bar, kb * GEMM_BK, t0); };
+  if (warp == 0) {
+    if (lane == 0 && !c.drop_loads) {                  // the first stages are on their way before anything else happens
+      // The weights do not depend on anything: they fill the stages (and, where the tile was taken before its operands
+      // exist, the L2 beyond those) while the predecessors still run; the activations follow the release.
+#pragma unroll 1
+      for (int kb = 0; kb < S; ++kb) load_w(kb, bar0 + 8u * (uint32_t)kb, stage0 + (uint32_t)kb * stage_bytes);
+      if (c.wait_word) {
+#pragma unroll 1
+        for (int kb = S; kb < nkb; ++kb) tma_prefetch_2d(wmap, kb * GEMM_BK, r0);
+        asm volatile("prefetch.tensormap [%0];" ::"l"(amap) : "memory");
+        wait_release(c);
+      }
+      asm volatile("fence.proxy.async;" ::: "memory");   // operands were written by generic stores on other SMs
+#pragma unroll 1
+      for (int kb = 0; kb < S; ++kb) load_a(kb, bar0 + 8u * (uint32_t)kb, stage0 + (uint32_t)kb * stage_bytes);
+    }
+    __syncwarp();
+  }
+  if (c.wait_word) worker_sync(c);                     // nobody reads an operand before the release
 
-  if (c.tid == 0) {
-    for (int s = 0; s < S; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), 1); }
-    mbar_init(accum_bar, 1);
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  const int tok = t0 + min(worker_tid(), nt - 1);      // this thread's token (lanes past the last one repeat it)
+  const bool warp_live = warp * 32 < nt;
+  const uint32_t my_tmem = c.tmem + ((uint32_t)(warp * 32) << 16);
+  // Residual rows go into the accumulators before the first MMA: their round trip then lies beside that of the first
+  // operand stages, and the epilogue neither reads nor adds anything.
+  const bool under = g.X != 0 && g.vec16 && g.c_acc == 1.0f && g.c_x == 1.0f && g.rs_d == 0 && g.act == ACT_NONE;
+  if (under) {
+    if (warp_live) {
+      const float* x = resolve<const float>(c, g.X) + (size_t)tok * g.ldx + r0;
+      const int cols = min(GEMM_BM, g.N - r0);
+#pragma unroll 1
+      for (int c0 = 0; c0 < cols; c0 += 16) {
+        float v[16];
+#pragma unroll
+        for (int j = 0; j < 16; j += 4) *reinterpret_cast<float4*>(v + j) = __ldcg(reinterpret_cast<const float4*>(x + c0 + j));
+        tmem_st16(my_tmem + (uint32_t)c0, v);
+      }
+      tmem_st_wait();
+    }
+    tc_fence_before();
+  }
+  // Folded RMSNorm: the token's row scale from the stream's partial sums of squares, added in a fixed order.
+  float rs = 1.0f;
+  if (g.rs_d > 0 && warp_live) {
+    const float* sp = resolve<const float>(c, g.ss_in) + (size_t)tok * g.ss_nft;
+    float ssq = 0.f;
+#pragma unroll 4
+    for (int q = 0; q < g.ss_nft; ++q) ssq += ld_act(sp + q);
+    rs = 1.0f / sqrtf(ssq / (float)g.rs_d + 1e-6f);
   }
   worker_sync(c);
 
-  // epilogue pointers and shape facts are resolved now, so their loads overlap the main loop
-  const GemmPtrs ptrs = gemm_ptrs(c, g);
-  const bool vec4 = (g.N % 4 == 0) && (!ptrs.X || g.ldx % 4 == 0) && (!ptrs.tab || g.ldtab % 4 == 0) &&
-                    (!ptrs.tab2 || g.ldtab2 % 4 == 0) && (!ptrs.out32 || g.ldo32 % 4 == 0) && (!ptrs.out16 || g.ldo16 % 4 == 0);
-  const int gf = f0 + 4 * lane;            // epilogue phase 2: this lane's four consecutive features
-  const bool fok = gf < g.N;
-  const uint32_t tmem_d = c.tmem;                 // accumulator columns [0, bt)
-  float* rs_smem = reinterpret_cast<float*>(c.ctl + 256);        // [bt] row scales, in the control block
-  // Whole warps take a role: lanes 1..31 of the producer and MMA warps park at __syncwarp (they must not
-  // spin on a barrier, which would stall the issuing lane of the same warp).
   if (warp == 0) {
     if (lane == 0) {
-    // ---------------- TMA producer
-    asm volatile("fence.proxy.async;" ::: "memory");   // operands were written by generic stores on other SMs
-    const char* tm = reinterpret_cast<const char*>(c.tmaps);
-    const void* wmap = tm + (size_t)g.wmap * 128;
-    const void* w2map = tm + (size_t)g.w2map * 128;
-    const void* amap = tm + (size_t)(c.amap_base + g.amap) * 128;
-    for (int kb = 0; kb < nkb && !c.drop_loads; ++kb) {
-      const int s = kb % S;
-      const uint32_t ph = (uint32_t)(kb / S) & 1u;
-      if (!mbar_wait(c, empty_bar(s), ph ^ 1u)) break;
-      mbar_expect_tx(full_bar(s), (uint32_t)stage_bytes);
-      const uint32_t dst = stage0 + (uint32_t)(s * stage_bytes);
-      tma_load_2d(dst, wmap, full_bar(s), kb * GEMM_BK, f0);      // 128 rows, or the 64 gate rows of a gated tile
-      if (dual) tma_load_2d(dst + GEMM_W_STAGE_BYTES / 2, w2map, full_bar(s), kb * GEMM_BK, f0);   // its 64 up rows
-      tma_load_2d(dst + GEMM_W_STAGE_BYTES, amap, full_bar(s), kb * GEMM_BK, t0);
-    }
+      // ---------------- TMA producer
+      uint32_t bar = bar0, dst = stage0, ph = 0u;
+      int s = 0;
+#pragma unroll 1
+      for (int kb = S; kb < nkb && !c.drop_loads; ++kb) {
+        if (!mbar_wait(c, bar + 8u * (uint32_t)S, ph)) break;
+        load_w(kb, bar, dst);
+        load_a(kb, bar, dst);
+        bar += 8u; dst += stage_bytes;
+        if (++s == S) { s = 0; bar = bar0; dst = stage0; ph ^= 1u; }
+      }
     }
     __syncwarp();
   } else if (warp == 1) {
-    if (lane == 0) {
-    // ---------------- MMA issuer
-    const uint32_t idesc = umma_idesc_bf16(bt);
-    bool ok = true;
-    for (int kb = 0; kb < nkb && ok; ++kb) {
-      const int s = kb % S;
-      const uint32_t ph = (uint32_t)(kb / S) & 1u;
-      ok = mbar_wait(c, full_bar(s), ph);
-      if (!ok) break;
+    // ---------------- MMA issuer (the whole warp walks the loop, one elected lane issues)
+    const uint32_t idesc = umma_idesc_bf16(GEMM_BM);
+    const uint64_t desc0 = umma_desc_sw128(stage0);
+    uint32_t bar = bar0, ph = 0u, off = 0u;
+    int s = 0;
+#pragma unroll 1
+    for (int kb = 0; kb < nkb; ++kb) {
+      if (!mbar_wait(c, bar, ph)) break;
       tc_fence_after();
-      const uint32_t wsm = stage0 + (uint32_t)(s * stage_bytes);
-      const uint32_t asm_ = wsm + GEMM_W_STAGE_BYTES;
-      const uint64_t wd = umma_desc_sw128(wsm), ad = umma_desc_sw128(asm_);
+      const uint64_t ad = desc0 + off, wd = ad + (a_bytes >> 4);
+      if (elect_one()) {
 #pragma unroll
-      for (int k = 0; k < GEMM_BK / 16; ++k) {
-        const uint32_t accumulate = (kb | k) != 0 ? 1u : 0u;
-        umma_bf16(tmem_d, wd + 2u * k, ad + 2u * k, idesc, accumulate);          // 16 bf16 = 32 bytes per K step
+        for (int k = 0; k < GEMM_BK / 16; ++k)
+          umma_bf16(c.tmem, ad + 2u * k, wd + 2u * k, idesc, (kb | k) != 0 || under ? 1u : 0u);   // 16 bf16 = 32 bytes per K step
+        umma_commit(bar + 8u * (uint32_t)S);     // stage reusable once these MMAs have read it
+        if (kb == nkb - 1) umma_commit(accum_bar);   // accumulators complete
       }
-      umma_commit(empty_bar(s));        // stage reusable once these MMAs have read it
-    }
-    if (ok) umma_commit(accum_bar);     // accumulators complete
-    }
-    __syncwarp();
-  } else if (g.rs_d > 0) {
-    // ---------------- folded RMSNorm: row scales from the stream's per-row partial sums of squares, summed in a
-    // fixed order while the main loop runs (thread j: tokens j and j + 64)
-    const float* ssp = resolve<const float>(c, g.ss_in);
-    const int ss_nft = g.ss_nft;
-    const float inv_d = (float)g.rs_d;
-    for (int tkn = c.tid - 64; tkn < bt; tkn += 64) {
-      float ssq = 0.f;
-      if (tkn < nt)
-        for (int q = 0; q < ss_nft; ++q) ssq += ld_act(ssp + (size_t)(t0 + tkn) * ss_nft + q);
-      rs_smem[tkn] = 1.0f / sqrtf(ssq / inv_d + 1e-6f);
+      __syncwarp();
+      bar += 8u; off += stage_bytes >> 4;
+      if (++s == S) { s = 0; bar = bar0; off = 0u; ph ^= 1u; }
     }
   }
 
-  // ---------------- epilogue in two phases.
-  // Phase 1 (thread = output feature, the TMEM lane it owns): read the accumulators, apply the row scale and the
-  // activation, and park the values in shared memory (the pipeline stages are free now) as [token][feature];
-  // the V^T part of a q|k|v projection is written from here, 16 consecutive tokens per thread.
-  // Phase 2 (warp = token row, lane = 4 consecutive features): add the residual / vectors / tables and store
-  // whole 512-byte rows; the row's sum of squares over this tile's features goes to the stream's partials.
   const bool ready = mbar_wait(c, accum_bar, 0u);
   __syncwarp();
   tc_fence_after();
-  float* St = reinterpret_cast<float*>(c.smem);   // [bt][128] fp32
-  // The residual rows of this tile start their way into the staging area now (asynchronous 16-byte copies
-  // through L2, no registers held), so their latency overlaps the accumulator read-out.
-  const bool x_staged = vec4 && ptrs.X != nullptr;
-  if (x_staged) {
-    if (ready && fok)
-      for (int tok = warp; tok < nt; tok += 4)
-        cp_async16(smem_u32(St + (size_t)tok * GEMM_BM + 4 * lane), ptrs.X + (size_t)(t0 + tok) * g.ldx + gf);
-    cp_async_wait_all();
-  }
-  if (g.rs_d > 0 || x_staged) worker_sync(c);     // row scales written by warps 2 and 3; residual rows landed
-  if (ready) {
-    Phase1Args p1;
-    p1.St = St; p1.rs = g.rs_d > 0 ? rs_smem : nullptr; p1.c_acc = g.c_acc; p1.c_x = g.c_x; p1.x_staged = x_staged;
-    p1.lane_base = tmem_d + ((uint32_t)(warp * 32) << 16);
-    p1.bt = g.bt; p1.nt = nt; p1.tid = c.tid; p1.t0 = t0;
-    const int f = f0 + c.tid;
-    p1.bias = (ptrs.bias != nullptr && f < g.N) ? ptrs.bias[f] : 0.0f;      // this thread's output feature
-    p1.outT_row = (ptrs.outT != nullptr && f >= g.t_col0 && f < g.N) ? ptrs.outT + (size_t)(f - g.t_col0) * g.ldoT : nullptr;
-    if (dual) { p1.c_acc = 1.0f; gemm_phase1<ACT_NONE>(p1); }   // gate and up rows parked raw: phase 2 combines them
-    else if (g.act == ACT_GELU) gemm_phase1<ACT_GELU>(p1);
-    else if (g.act == ACT_SILU) gemm_phase1<ACT_SILU>(p1);
-    else gemm_phase1<ACT_NONE>(p1);
-  }
-  worker_sync(c);
-  if (ready) {
-    float* ssq_out = resolve<float>(c, g.ss_out);
-    if (vec4) {
-      // the node's arguments live in global memory, which the stores below might alias as far as the compiler
-      // knows: everything the row loop needs is taken into registers first
-      const size_t ldo32 = (size_t)g.ldo32, ldo16 = (size_t)g.ldo16, ldtab = (size_t)g.ldtab, ldtab2 = (size_t)g.ldtab2;
-      const size_t ss_ld = (size_t)g.ss_out_ld;
-      const float* const tab = fok ? ptrs.tab : nullptr;
-      const float* const tab2 = fok ? ptrs.tab2 : nullptr;
-      float* const o32 = fok ? ptrs.out32 : nullptr;
-      const bool skip16 = ptrs.outT != nullptr && gf >= g.t_col0;      // these columns went to V^T in phase 1
-      unsigned short* const o16 = (fok && !skip16) ? ptrs.out16 : nullptr;
-      Phase2Args p2;
-      p2.vecv = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (ptrs.vec && fok) p2.vecv = *reinterpret_cast<const float4*>(ptrs.vec + gf);
-      p2.tab = tab; p2.tab2 = tab2; p2.o32 = o32; p2.o16 = o16; p2.St = St;
-      p2.ldo32 = ldo32; p2.ldo16 = ldo16; p2.ldtab = ldtab; p2.ldtab2 = ldtab2;
-      p2.nt = nt; p2.t0 = t0; p2.warp = warp; p2.lane = lane; p2.gf = gf; p2.fok = fok; p2.ss = ssq_out != nullptr;
-      const bool has_tab = ptrs.tab || ptrs.tab2 || ptrs.vec;          // warp-uniform choices of the row code
-      if (dual) {
-        p2.o16 = ptrs.out16;
-        if (g.act == ACT_SILU) gemm_phase2_rows_gated<ACT_SILU>(p2, g.c_acc, f0, g.N);
-        else if (g.act == ACT_GELU) gemm_phase2_rows_gated<ACT_GELU>(p2, g.c_acc, f0, g.N);
-        else gemm_phase2_rows_gated<ACT_NONE>(p2, g.c_acc, f0, g.N);
-      } else if (!has_tab && !ptrs.out32 && !ssq_out) gemm_phase2_rows<false, false, true, false>(p2);      // bf16 only (q|k|v, MLP up)
-      else if (!has_tab) gemm_phase2_rows<false, true, true, true>(p2);                                // residual stream
-      else gemm_phase2_rows<true, true, true, true>(p2);
-      if (ssq_out) {
-        __syncwarp();
-        const int tok = warp + 4 * lane;                 // this lane's row: slot `lane` of this warp
-        if (tok < nt) {
-          float sq = 0.f;
-#pragma unroll 8
-          for (int i = 0; i < 32; ++i) sq += St[(size_t)tok * GEMM_BM + ((i + lane) & 31)];   // lane order 0..31
-          ssq_out[(size_t)(t0 + tok) * ss_ld + ft] = sq;
-        }
-      }
-    } else {
-      // odd widths (e.g. a 7-wide action output): one feature per lane and pass
-      for (int tok = warp; tok < nt; tok += 4) {
-        const int r = t0 + tok;
-        float sq = 0.f;
-        for (int q = lane; q < GEMM_BM; q += 32) {
-          const int of = f0 + q;
-          if (of >= g.N) continue;
-          float v = St[(size_t)tok * GEMM_BM + q];
-          if (ptrs.X) v = fmaf(g.c_x, ld_act(ptrs.X + (size_t)r * g.ldx + of), v);
-          if (ptrs.vec) v += ptrs.vec[of];
-          if (ptrs.tab) v += ptrs.tab[(size_t)r * g.ldtab + of];
-          if (ptrs.tab2) v += ptrs.tab2[(size_t)r * g.ldtab2 + of];
-          if (ptrs.out32) ptrs.out32[(size_t)r * g.ldo32 + of] = v;
-          if (ptrs.out16 && !(ptrs.outT && of >= g.t_col0)) ptrs.out16[(size_t)r * g.ldo16 + of] = f32_to_bf16_bits(v);
-          sq = fmaf(v, v, sq);
-        }
-        if (ssq_out) {
-          sq = warp_sum(sq);
-          if (lane == 0) ssq_out[(size_t)r * g.ss_out_ld + ft] = sq;
-        }
-      }
-    }
-  }
+  if (ready && warp_live) gemm_epilogue(c, g, my_tmem, tok, worker_tid() < nt, r0, rs, under, ft);
   tc_fence_before();
   worker_sync(c);
-  if (c.tid == 0) {
-    for (int s = 0; s < 2 * S + 1; ++s) mbar_inval(bar0 + 8u * s);
-  }
+  if (worker_tid() <= 2 * S) mbar_inval(bar0 + 8u * worker_tid());
 }
 
 }  // namespace vla

@@ -56,15 +56,22 @@ inline OpFault& op_fault() {
   return f;
 }
 
+}  // namespace vla
+
+#include "op_linear.cuh"
+
+namespace vla {
+
 __device__ __forceinline__ TileCtx op_tile_ctx(char* smem, char* ctl, uint32_t tmem, const void* maps, unsigned* err,
                                                OpFault fault) {
   TileCtx tc;
   tc.arena = nullptr;          // Refs of the stand-alone operators are absolute device addresses
   tc.slot_base = 0;
   tc.smem = smem;
+  tc.smem_bytes = 0;
+  tc.wait_word = nullptr;
   tc.ctl = ctl;
   tc.tmem = tmem;
-  tc.tid = threadIdx.x;
   tc.bar_id = 1;
   tc.error = err;
   tc.tmaps = maps;
@@ -91,22 +98,6 @@ __global__ void __launch_bounds__(WORKER_THREADS) vla_op_attention_kernel(AttnAr
   if (threadIdx.x < 32) tmem_dealloc(tmem_base_s, (uint32_t)tmem_cols);
 }
 
-__global__ void __launch_bounds__(WORKER_THREADS) vla_op_linear_kernel(GemmArgs g, const __grid_constant__ OpMaps maps,
-                                                                       int tmem_cols, unsigned* err, OpFault fault) {
-  extern __shared__ __align__(1024) char smem_raw[];
-  __shared__ uint32_t tmem_base_s;
-  __shared__ __align__(16) char ctl_block[1024];
-  if (threadIdx.x < 32) tmem_alloc(&tmem_base_s, (uint32_t)tmem_cols);
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  TileCtx tc = op_tile_ctx(smem_raw, ctl_block, tmem_base_s, &maps, err, fault);
-  tile_gemm(tc, g, (int)blockIdx.x);
-  tc_fence_before();
-  __syncthreads();
-  if (threadIdx.x < 32) tmem_dealloc(tmem_base_s, (uint32_t)tmem_cols);
-}
-
 // vt[c][t] = v[t][c] for a bf16 matrix v [rows, cols] (row pitch ldv), vt row pitch ldt.
 __global__ void vla_op_transpose_kernel(const unsigned short* v, unsigned short* vt, int rows, int cols, int ldv, int ldt) {
   __shared__ unsigned short tile[32][33];
@@ -124,31 +115,39 @@ __global__ void vla_op_transpose_kernel(const unsigned short* v, unsigned short*
 
 constexpr size_t OP_ATTN_HEADER = 256;   // error word + padding in front of V^T
 
-// Error word of vla_op_linear: one per device, in a fixed device array of the library, looked up on the first call
-// made with that device current.  Calls on one device share it (see the header: check vla_op_status before
-// launching another operator call that could overwrite it).
+// What vla_op_linear keeps per device, looked up on the first call made with that device current: SM count, the error word
+// (in a fixed device array of the library) and the number of the latest call.  A kernel whose wait runs out writes its
+// call's number there; nothing has to be cleared in front of a call.
 static __device__ __align__(256) unsigned g_op_linear_error[64];
-inline unsigned* op_linear_error_word() {
+struct OpDevice {
+  std::atomic<unsigned*> error{nullptr};
+  int sms = 0;
+  std::atomic<unsigned> calls{0};
+};
+inline OpDevice* op_device() {
   constexpr int kMax = 64;
-  static std::atomic<unsigned*> ptr[kMax];
+  static OpDevice devices[kMax];
   int dev = -1;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMax) return nullptr;
-  unsigned* p = ptr[dev].load(std::memory_order_acquire);
-  if (!p) {
+  OpDevice& d = devices[dev];
+  if (!d.error.load(std::memory_order_acquire)) {
     void* a = nullptr;
+    int sms = 0;
     if (cudaGetSymbolAddress(&a, g_op_linear_error) != cudaSuccess || !a) return nullptr;
-    p = static_cast<unsigned*>(a);
-    ptr[dev].store(p, std::memory_order_release);
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return nullptr;
+    if (cudaFuncSetAttribute(vla_op_linear_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, LIN_SMEM) != cudaSuccess) return nullptr;
+    d.sms = sms;
+    d.error.store(static_cast<unsigned*>(a), std::memory_order_release);
   }
-  return p;
+  return &d;
 }
 
 // Reads an operator's error word back after the stream has drained.
-inline int op_status_of(const unsigned* dev_word, cudaStream_t s) {
+inline int op_status_of(const unsigned* dev_word, cudaStream_t s, unsigned call = 0) {
   if (cudaStreamSynchronize(s) != cudaSuccess) return VLA_ERR_CUDA;
   unsigned v = 0;
   if (cudaMemcpy(&v, dev_word, sizeof v, cudaMemcpyDeviceToHost) != cudaSuccess) return VLA_ERR_CUDA;
-  return v == 0 ? VLA_OK : VLA_ERR_TIMEOUT;
+  return (call ? v != call : v == 0) ? VLA_OK : VLA_ERR_TIMEOUT;       // (call: the number that would mean a time-out)
 }
 
 inline int64_t op_pad(int64_t x, int64_t m) { return (x + m - 1) / m * m; }
@@ -191,7 +190,7 @@ inline int op_attention_run(const void* q, const void* k, const void* v, void* o
     return VLA_ERR_CUDA;
   const int smem = attn_smem_bytes(hd);
   int tmem_cols = 32;
-  while (tmem_cols < a.bn + hd) tmem_cols <<= 1;
+  while (tmem_cols < attn_tmem_cols(hd)) tmem_cols <<= 1;
   if (cudaFuncSetAttribute(vla_op_attention_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
     return VLA_ERR_CUDA;
   vla_op_attention_kernel<<<n_tiles, WORKER_THREADS, smem, s>>>(a, maps, tmem_cols, err, op_fault());
@@ -221,28 +220,19 @@ int vla_op_linear(const void* a, const void* w, float* out32, void* out16, int32
                   void* stream) {
   using namespace vla;
   if (!a || !w || (!out32 && !out16) || m < 1 || n < 1 || k < 8 || k % 8 || act < 0 || act > 2) return VLA_ERR_INVALID;
-  GemmArgs g;
-  memset(&g, 0, sizeof g);
-  g.M = m; g.N = n; g.Kp = (int)op_pad(k, GEMM_BK);
-  g.out32 = reinterpret_cast<Ref>(out32); g.ldo32 = n;
-  g.out16 = reinterpret_cast<Ref>(out16); g.ldo16 = n;
-  g.act = act; g.c_acc = 1.f; g.c_x = 1.f;
-  g.tiles_t = (m + GEMM_MAX_BT - 1) / GEMM_MAX_BT;
-  g.bt = (int)op_pad((m + g.tiles_t - 1) / g.tiles_t, 16);
-  g.stages = gemm_stages(g.bt, g.Kp);
-  g.wmap = 0; g.w2map = 0; g.amap = 1;
+  OpDevice* dev = op_device();
+  if (!dev) return VLA_ERR_CUDA;
+  LinearArgs g;
+  g.m = m; g.n = n; g.kp = (int)op_pad(k, GEMM_BK); g.act = act;
+  g.out32 = out32; g.out16 = static_cast<unsigned short*>(out16);
+  g.vec16 = n % 16 == 0 && ((reinterpret_cast<uintptr_t>(out32) | reinterpret_cast<uintptr_t>(out16)) & 15) == 0;
+  linear_plan(g, dev->sms);
+  g.err = dev->error.load(std::memory_order_relaxed);
+  g.call = dev->calls.fetch_add(1u, std::memory_order_relaxed) + 1u;
   OpMaps maps;
-  memset(&maps, 0, sizeof maps);
-  if (!op_encode(&maps.m[0], w, n, k, k, GEMM_BM) || !op_encode(&maps.m[1], a, m, k, k, g.bt)) return VLA_ERR_CUDA;
-  const int smem = gemm_smem_bytes(g.bt, g.stages);
-  int tmem_cols = 32;
-  while (tmem_cols < g.bt) tmem_cols <<= 1;
-  unsigned* err = op_linear_error_word();     // this device's word (a fixed device array: nothing is allocated)
-  if (!err) return VLA_ERR_CUDA;
-  cudaStream_t s = static_cast<cudaStream_t>(stream);
-  if (cudaMemsetAsync(err, 0, 4, s) != cudaSuccess) return VLA_ERR_CUDA;
-  if (cudaFuncSetAttribute(vla_op_linear_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return VLA_ERR_CUDA;
-  vla_op_linear_kernel<<<((n + GEMM_BM - 1) / GEMM_BM) * g.tiles_t, WORKER_THREADS, smem, s>>>(g, maps, tmem_cols, err, op_fault());
+  if (!op_encode(&maps.m[0], w, n, k, k, g.bn) || !op_encode(&maps.m[1], a, m, k, k, g.bm)) return VLA_ERR_CUDA;
+  const int grid = g.tiles < 2 * dev->sms ? g.tiles : 2 * dev->sms;
+  vla_op_linear_kernel<<<grid, LIN_THREADS, linear_smem(g), static_cast<cudaStream_t>(stream)>>>(g, maps, op_fault());
   return cudaGetLastError() == cudaSuccess ? VLA_OK : VLA_ERR_CUDA;
 }
 

@@ -78,8 +78,8 @@ VLA_HD inline void pick_group_masks(int n_cls, const int* group, unsigned* group
 
 // Returns the chosen class or -1; *phase = 1 or 2 (0 when nothing was chosen).
 // group_mask: see pick_group_masks.  grid[k] (G_k, for POLICY_TWO_PHASE_G) and res[k] (R_k, for POLICY_TWO_PHASE_R)
-// may be null for the other policies.  Every array is read at loop-constant positions only, so a caller that inlines
-// this with a constant n_cls keeps them in registers (the persistent kernel calls it on every tile hand-over).
+// may be null for the other policies.  The loops stay rolled and visit candidates only: the persistent kernel runs this on
+// every tile hand-over with its tables in shared memory, and unrolled it took a share of the instruction cache.
 VLA_HD inline int pick_choose(int n_cls, const int* tau /*[n_cls][3]*/, const unsigned* group_mask /*[n_cls]*/, unsigned pending,
                               unsigned feasible, const PickState& st, int rr_start, int policy, int u_max, int* phase,
                               const int* grid = nullptr, const int* res = nullptr) {
@@ -91,37 +91,33 @@ VLA_HD inline int pick_choose(int n_cls, const int* tau /*[n_cls][3]*/, const un
   if (policy == POLICY_ROUND_ROBIN) { *phase = 1; return pick_first_from(ok, rr_start, n_cls); }
   // Phase 1: classes whose group has no tile resident on this SM
   unsigned occupied = 0, unrep = 0;
-#pragma unroll
-  for (int k = 0; k < PICK_MAX_CLASSES; ++k)
-    if (k < n_cls && st.cta_count[k] > 0) occupied |= 1u << k;
-#pragma unroll
-  for (int k = 0; k < PICK_MAX_CLASSES; ++k)
-    if (k < n_cls && (group_mask[k] & occupied) == 0u) unrep |= 1u << k;
+#pragma unroll 1
+  for (int k = 0; k < n_cls; ++k)
+    if (st.cta_count[k] > 0) occupied |= 1u << k;
+#pragma unroll 1
+  for (unsigned m = ok; m != 0u; m &= m - 1u) {
+    const int k = pick_lowest_bit(m);
+    if ((group_mask[k] & occupied) == 0u) unrep |= 1u << k;
+  }
   if (ok & unrep) { *phase = 1; return pick_first_from(ok & unrep, rr_start, n_cls); }
   // Phase 2: headroom per pipeline, then the largest score, strict '>' (first seen wins ties)
   int head[3];
 #pragma unroll
   for (int x = 0; x < 3; ++x) head[x] = u_max - (st.u[x] > u_max ? u_max : st.u[x]);
-  int best = -1;
-  if (policy == POLICY_TWO_PHASE || (policy == POLICY_TWO_PHASE_G && !grid) || (policy == POLICY_TWO_PHASE_R && !res)) {
-    int best_score = -1;                                  // Algorithm 1 as printed: integer scores
-#pragma unroll
-    for (int k = 0; k < PICK_MAX_CLASSES; ++k) {
-      if (k >= n_cls || !(ok & (1u << k))) continue;
-      const int s = head[0] * tau[k * 3] + head[1] * tau[k * 3 + 1] + head[2] * tau[k * 3 + 2];
+  int best = -1, best_score = -1;                         // Algorithm 1 as printed: integer scores
+  long long best_num = -1, best_den = 1;                  // the variants: ratios num/den compared by cross-multiplication
+  const bool by_grid = policy == POLICY_TWO_PHASE_G && grid, by_res = policy == POLICY_TWO_PHASE_R && res;
+#pragma unroll 1
+  for (unsigned m = ok; m != 0u; m &= m - 1u) {
+    const int k = pick_lowest_bit(m);
+    const int s = head[0] * tau[k * 3] + head[1] * tau[k * 3 + 1] + head[2] * tau[k * 3 + 2];
+    if (!by_grid && !by_res) {
       if (s > best_score) { best_score = s; best = k; }
+      continue;
     }
-  } else {
-    long long best_num = -1, best_den = 1;                // the variants: ratios num/den compared by cross-multiplication
-#pragma unroll
-    for (int k = 0; k < PICK_MAX_CLASSES; ++k) {
-      if (k >= n_cls || !(ok & (1u << k))) continue;
-      const int s = head[0] * tau[k * 3] + head[1] * tau[k * 3 + 1] + head[2] * tau[k * 3 + 2];
-      long long num = s, den = 1;
-      if (policy == POLICY_TWO_PHASE_G) { num = (long long)s * grid[k]; den = st.cta_count[k] + 1; }
-      else den = (long long)st.cta_count[k] * res[k] + 1;
-      if (num * best_den > best_num * den) { best_num = num; best_den = den; best = k; }
-    }
+    const long long num = by_grid ? (long long)s * grid[k] : s;
+    const long long den = by_grid ? st.cta_count[k] + 1 : (long long)st.cta_count[k] * res[k] + 1;
+    if (num * best_den > best_num * den) { best_num = num; best_den = den; best = k; }
   }
   if (best >= 0) *phase = 2;
   return best;

@@ -117,6 +117,15 @@ class Builder {
     return d;
   }
   int matrix1(const std::string& name, int64_t rows, int64_t cols) { return matrix(name, {name}, {rows}, cols); }
+  // gate and up matrices of a gated MLP, row by row in one device matrix
+  int gated(const std::string& pre, int64_t rows, int64_t cols) {
+    int d = dev_tensor(pre + "wgu", 2 * rows, cols, true);
+    source(pre + "wg", rows, cols, d, 0);
+    p.sources.back().row_step = 2;
+    source(pre + "wu", rows, cols, d, 1);
+    p.sources.back().row_step = 2;
+    return d;
+  }
   // stacked per-head projections whose heads are padded from hd to hs rows (padding rows stay zero)
   int matrix_heads(const std::string& dev_name, const std::vector<std::string>& parts, const std::vector<int64_t>& part_heads,
                    int64_t hd, int64_t hs, int64_t cols) {
@@ -229,9 +238,9 @@ class Builder {
     View tabv;               // an fp32 [M, ld] addend that is one of the frame's buffers (read dependency tracked)
     int t_col0 = 0;
     int act = ACT_NONE;
-    int W2 = -1;
+    bool dual = false;       // gated: W holds gate and up rows alternating, N output features
     int bias = -1;           // >= 0: an fp32 [N] device tensor added to the accumulator before the activation
-    int64_t w_row0 = 0;
+    Ref rope_tab = 0; int rope_hd = 0, rope_cols = 0;   // rotary embedding of the q and k columns (see GemmArgs)
     int norm_gain = -1;      // >= 0: A is the raw residual stream; RMSNorm with this gain is folded into the GEMM
     int norm_d = 0;
   };
@@ -241,10 +250,7 @@ class Builder {
     std::memset(&n, 0, sizeof(n));
     n.op = OP_GEMM;
     GemmArgs& g = n.u.gemm;
-    g.A = ref(A); g.lda = (int)ld(A);
-    g.W = wref(W, o.w_row0);
-    g.W2 = o.W2 >= 0 ? wref(o.W2, o.w_row0) : 0;
-    g.dual = o.W2 >= 0;
+    g.dual = o.dual;
     g.M = (int)A.rows; g.N = (int)N; g.Kp = (int)wt.ld;
     g.X = ref(o.X); g.ldx = o.X.buf >= 0 ? (int)ld(o.X) : 0;
     g.c_x = o.c_x; g.c_acc = o.c_acc;
@@ -255,6 +261,7 @@ class Builder {
     g.out16 = ref(o.out16); g.ldo16 = o.out16.buf >= 0 ? (int)ld(o.out16) : 0;
     g.outT = ref(o.outT); g.ldoT = o.outT.buf >= 0 ? (int)ld(o.outT) : 0; g.t_col0 = o.t_col0;
     g.act = o.act;
+    g.rope_tab = o.rope_tab; g.rope_hd = o.rope_hd; g.rope_cols = o.rope_cols;
     g.rs_d = 0; g.ss_nft = 0; g.ss_out_ld = 0; g.ss_in = 0; g.ss_out = 0;
     const View ss_in = o.norm_gain >= 0 ? ss_view(A) : View();
     const View ss_out = ss_view(o.out16);
@@ -264,25 +271,31 @@ class Builder {
       if (ss_in.buf < 0) p.error = "internal: folded norm needs a stream mirror as operand (" + name + ")";
       g.rs_d = o.norm_d;
       p.folds.push_back({W, o.norm_gain});
-      if (o.W2 >= 0) p.folds.push_back({o.W2, o.norm_gain});
     }
     int tiles_t = (int)((g.M + GEMM_MAX_BT - 1) / GEMM_MAX_BT);
     int bt = (int)pad_to((g.M + tiles_t - 1) / tiles_t, 16);
     g.bt = bt; g.tiles_t = tiles_t;
     {
+      // sixteen columns at a time, each a whole 16-byte access at a 16-byte address: rows start at multiples of 256 bytes
+      // (buffers and weights), so pitches and column offsets decide
+      auto cols_ok = [&](const View& v, int64_t per) { return v.buf < 0 || (ld(v) % per == 0 && v.col0 % per == 0); };
+      g.vec16 = N % (g.dual ? 8 : 16) == 0 && cols_ok(o.X, 4) && cols_ok(o.tabv, 4) && cols_ok(o.out32, 4) && cols_ok(o.out16, 8) &&
+                (!o.tab || o.ldtab % 4 == 0) && (!o.tab2 || o.ldtab2 % 4 == 0) && (o.outT.buf < 0 || o.t_col0 % 16 == 0);
+      if (!g.vec16 && (o.outT.buf >= 0 || o.rope_cols > 0)) p.error = "internal: V^T and rotary columns come in chunks of 16 (" + name + ")";
+    }
+    {
       // pipeline depth from the stage size; tensor maps for the operands
-      // A gated tile covers 64 output features: rows 0..63 of its 128-row weight tile come from the gate matrix,
-      // rows 64..127 from the up matrix (two 64-row TMA boxes), so it is one accumulator and has the shared and
-      // tensor-memory shape of a plain tile.
+      // A gated tile covers 64 output features with 128 alternating gate and up rows: one accumulator, one weight box, the
+      // shared and tensor-memory shape of a plain tile.
       const int S = gemm_stages(bt, g.Kp);
       g.stages = S;
       n.smem_bytes = gemm_smem_bytes(bt, S);
-      n.tmem_cols = (int)pad_to((int64_t)bt, TMEM_UNIT);
-      g.wmap = weight_map(W, N, g.dual ? GEMM_BM / 2 : GEMM_BM);
-      g.w2map = o.W2 >= 0 ? weight_map(o.W2, N, GEMM_BM / 2) : 0;
+      n.smem_deep = gemm_smem_bytes(bt, std::min(GEMM_MAX_STAGES, g.Kp / GEMM_BK));
+      n.tmem_cols = GEMM_BM;
+      g.wmap = weight_map(W, g.dual ? 2 * N : N);
       if (g.dual && o.bias >= 0) p.error = "a gated GEMM takes no bias";
-      if (g.dual && (N % 4 != 0 || o.X.buf >= 0 || o.outT.buf >= 0 || o.out32.buf >= 0 || o.tab || o.tab2 || o.vec))
-        p.error = "internal: a gated GEMM writes bf16 only, width a multiple of 4 (" + name + ")";
+      if (g.dual && (o.X.buf >= 0 || o.outT.buf >= 0 || o.out32.buf >= 0 || o.tab || o.tab2 || o.vec))
+        p.error = "internal: a gated GEMM writes bf16 only (" + name + ")";
       g.amap = act_map(A, g.Kp, bt);
     }
     const int feat_per_tile = g.dual ? GEMM_BM / 2 : GEMM_BM;
@@ -339,7 +352,8 @@ class Builder {
     NormArgs& a = n.u.norm;
     a.x = ref(x); a.g = wref(g_dev); a.mod = mod; a.out = ref(out);
     a.M = (int)x.rows; a.d = (int)p.dev_tensors[g_dev].cols; a.ldx = (int)ld(x); a.ldo = (int)ld(out);
-    a.rows_per_tile = 16; a.shuffle = shuffle; a.grid = grid;
+    a.rows_per_tile = a.M <= 512 ? 4 : 16;      // few rows: one row per warp (latency); many: fewer, larger tiles
+    a.shuffle = shuffle; a.grid = grid;
     if (beta_dev >= 0) { a.ln = 1; a.beta = wref(beta_dev); }
     if (a.d % 4) p.error = "model widths must be multiples of 4";
     if (a.ln && a.d > 2048) p.error = "LayerNorm rows wider than 2048 are not supported";
@@ -378,7 +392,7 @@ class Builder {
     a.q_blocks = (tq + 127) / 128;
     a.scale_log2e = 1.4426950408889634f / std::sqrt((float)hd);
     n.smem_bytes = attn_smem_bytes(hs);
-    n.tmem_cols = (int)pad_to(a.bn + hs, TMEM_UNIT);
+    n.tmem_cols = (int)pad_to(attn_tmem_cols(hs), TMEM_UNIT);
     n.n_tiles = hq * a.q_blocks;
     a.hpt = attn_fold(tq, hq, hkv, &a.rph);
     if (a.hpt > 1) n.n_tiles = hkv * (((hq / hkv) + a.hpt - 1) / a.hpt);
@@ -402,32 +416,16 @@ class Builder {
     return id;
   }
 
-  // q|k|v projection of `A` into `dst`: one GEMM whose V columns are written transposed; with RoPE the
-  // GEMM writes fp32 and a rotary tile produces the bf16 q|k and V^T.
-  void qkv_project(const std::string& name, const View& A, int W, const QKV& dst, int hd, int scratch32, int pos0,
+  // q|k|v projection of `A` into `dst`: one GEMM whose V columns are written transposed.  With RoPE (rope_tab >= 0, first
+  // position pos0) its epilogue rotates the q and k columns; the load step placed the two members of a rotary pair side by
+  // side, in q and in k alike, which leaves every q.k product as it was.
+  void qkv_project(const std::string& name, const View& A, int W, const QKV& dst, int hd, int rope_tab, int pos0,
                    int norm_gain = -1, int norm_d = 0, int bias = -1) {
     const int64_t nqk = (int64_t)(dst.hq + dst.hkv) * dst.hs, nall = nqk + (int64_t)dst.hkv * dst.hs;
-    if (scratch32 >= 0) {
-      GemmOpt gq; gq.out32 = all(scratch32); gq.norm_gain = norm_gain; gq.norm_d = norm_d;
-      gemm(name + "qkv", A, W, nall, gq);
-      NodeDesc n;
-      std::memset(&n, 0, sizeof n);
-      n.op = OP_ROPE;
-      RopeArgs& r = n.u.rope;
-      r.in = ref(all(scratch32)); r.out = ref(all(dst.qk)); r.outT = ref(all(dst.vt));
-      r.M = dst.T; r.ld = (int)nall; r.ldo = (int)nqk; r.ldoT = (int)p.bufs[dst.vt].ld;
-      r.n_rot_heads = dst.hq + dst.hkv; r.n_heads = dst.hq + 2 * dst.hkv; r.hd = hd; r.pos0 = pos0;
-      r.rows_per_tile = 16;
-      n.n_tiles = (dst.T + 15) / 16;
-      int id = add(n, name + "rope", KIND_ELEM);
-      read(id, all(scratch32));
-      write(id, all(dst.qk));
-      write(id, all(dst.vt));
-    } else {
-      GemmOpt gq; gq.out16 = all(dst.qk); gq.outT = all(dst.vt); gq.t_col0 = (int)nqk; gq.bias = bias;
-      gq.norm_gain = norm_gain; gq.norm_d = norm_d;
-      gemm(name + "qkv", A, W, nall, gq);
-    }
+    GemmOpt gq; gq.out16 = all(dst.qk); gq.outT = all(dst.vt); gq.t_col0 = (int)nqk; gq.bias = bias;
+    gq.norm_gain = norm_gain; gq.norm_d = norm_d;
+    if (rope_tab >= 0) { gq.rope_tab = ref(rows(rope_tab, pos0, dst.T)); gq.rope_hd = hd; gq.rope_cols = (int)nqk; }
+    gemm(name + "qkv", A, W, nall, gq);
   }
 
   int elem_node(NodeDesc& n, const std::string& name) { return add(n, name, KIND_ELEM); }
@@ -539,7 +537,7 @@ bool build_program(const vla_model_desc& d, const vla_runtime_opts& o, Program& 
   const int hvd = d.vis_heads * d.vis_hd;
   const int vhs = (int)pad_to(std::max(d.vis_hd, 1), 16);          // vision head stride (72 -> 80)
   const int lhs = (int)pad_to(d.hd, 16);                            // LLM head stride
-  const int nq = d.hq * d.hd, nkv = d.hkv * d.hd, nqkv = (d.hq + 2 * d.hkv) * lhs;
+  const int nq = d.hq * d.hd, nkv = d.hkv * d.hd;
   if (lhs != d.hd) { set_err(p, "LLM head dimension must be a multiple of 16"); return false; }
   auto P64 = [](int64_t x) { return pad_to(x, GEMM_BK); };
   char nm[96];
@@ -576,17 +574,22 @@ bool build_program(const vla_model_desc& d, const vla_runtime_opts& o, Program& 
   int w_conn = d.connector ? b.matrix1("conn.w", D, (int64_t)d.shuffle * d.shuffle * dv) : -1;
   int w_emb = b.matrix1("txt.emb", d.vocab, D);
   int w_lpos = d.rope ? -1 : b.table("llm.pos", S, D);
-  struct LlmW { int n1, wqkv, wo, n2, w1, w2, wg, wu, wd; };
+  // the q and k sources just declared: rotary pairs become neighbours at load
+  auto pair_qk = [&]() {
+    if (!d.rope) return;
+    for (size_t i = p.sources.size() - 3; i < p.sources.size() - 1; ++i) p.sources[i].pair_hd = d.hd;
+  };
+  struct LlmW { int n1, wqkv, wo, n2, w1, w2, wgu, wd; };
   std::vector<LlmW> lw(d.llm_layers);
   for (int i = 0; i < d.llm_layers; ++i) {
     std::string pre = N_("llm.L%d.", i);
     lw[i].n1 = b.gain(pre + "n1", D);
     lw[i].wqkv = b.matrix(pre + "wqkv", {pre + "wq", pre + "wk", pre + "wv"}, {nq, nkv, nkv}, D);
+    pair_qk();
     lw[i].wo = b.matrix1(pre + "wo", D, nq);
     lw[i].n2 = b.gain(pre + "n2", D);
     if (gated) {
-      lw[i].wg = b.matrix1(pre + "wg", d.mlp, D);
-      lw[i].wu = b.matrix1(pre + "wu", d.mlp, D);
+      lw[i].wgu = b.gated(pre, d.mlp, D);
       lw[i].wd = b.matrix1(pre + "wd", D, d.mlp);
     } else {
       lw[i].w1 = b.matrix1(pre + "w1", d.mlp, D);
@@ -601,7 +604,7 @@ bool build_program(const vla_model_desc& d, const vla_runtime_opts& o, Program& 
   int w_apos = head_pos ? b.table("act.pos", Ta, da) : -1;
   int w_t1 = b.matrix1("act.t1", da, da);
   int w_t2 = b.matrix1("act.t2", da, da);
-  struct ActW { int n1, n2, n3, wqkv, wo, cq, ckv, co, ada1, ada2, w1, w2, wg, wu, wd; };
+  struct ActW { int n1, n2, n3, wqkv, wo, cq, ckv, co, ada1, ada2, w1, w2, wgu, wd; };
   std::vector<ActW> aw(d.act_layers);
   for (int i = 0; i < d.act_layers; ++i) {
     std::string pre = N_("act.L%d.", i);
@@ -609,6 +612,7 @@ bool build_program(const vla_model_desc& d, const vla_runtime_opts& o, Program& 
     a.n1 = b.gain(pre + "n1", da);
     if (d.head == VLA_HEAD_B) {
       a.wqkv = b.matrix(pre + "wqkv", {pre + "wq", pre + "wk", pre + "wv"}, {nq, nkv, nkv}, da);
+      pair_qk();
       a.wo = b.matrix1(pre + "wo", da, nq);
     } else if (d.head == VLA_HEAD_C && (i % 2 == 1)) {
       a.cq = b.matrix1(pre + "cq", da, da);
@@ -629,8 +633,7 @@ bool build_program(const vla_model_desc& d, const vla_runtime_opts& o, Program& 
       a.ada2 = b.matrix1(pre + "ada2", 2 * da, da);
     }
     if (agated) {
-      a.wg = b.matrix1(pre + "wg", d.act_mlp, da);
-      a.wu = b.matrix1(pre + "wu", d.act_mlp, da);
+      a.wgu = b.gated(pre, d.act_mlp, da);
       a.wd = b.matrix1(pre + "wd", da, d.act_mlp);
     } else {
       a.w1 = b.matrix1(pre + "w1", d.act_mlp, da);
@@ -669,6 +672,12 @@ bool build_program(const vla_model_desc& d, const vla_runtime_opts& o, Program& 
   int c_th = b.buf("const.th", ns, P64(da), 2, false);
   int c_ct = b.buf("const.ct", ns, da, 4, false);
   int c_sct = d.head == VLA_HEAD_C ? b.buf("const.sct", ns, P64(da), 2, false) : -1;
+  // rotary table of every position a token can have (prefix, then the action head's own tokens)
+  int c_rope = -1;
+  if (d.rope) {
+    p.rope_rows = S + Ta; p.rope_hd = d.hd;
+    c_rope = b.buf("const.rope", p.rope_rows, d.hd, 4, false);
+  }
   std::vector<int> c_mod1(d.act_layers, -1), c_mod2(d.act_layers, -1);
   if (d.head == VLA_HEAD_C)
     for (int i = 0; i < d.act_layers; ++i) {
@@ -717,7 +726,6 @@ bool build_program(const vla_model_desc& d, const vla_runtime_opts& o, Program& 
   // LLM
   int x = b.buf("llm.x", S, D, 4);
   int xb = b.stream_mirror("llm.xb", S, D);                // bf16 mirror of the residual stream (GEMM operand)
-  int qkv32 = d.rope ? b.buf("llm.qkv32", S, nqkv, 4) : -1;
   std::vector<Builder::QKV> lq(d.llm_layers);
   {
     bool have_shared = false;
@@ -747,8 +755,8 @@ bool build_program(const vla_model_desc& d, const vla_runtime_opts& o, Program& 
       PatchArgs& a = n.u.patch;
       a.img = Builder::in_ref(0, (uint64_t)c * 3 * d.img * d.img * 4);
       a.out = b.ref(b.all(patches));
-      a.img_side = d.img; a.patch = d.patch; a.grid = grid; a.ldo = (int)P64(patch_k); a.rows_per_tile = 16;
-      n.n_tiles = (T + 15) / 16;
+      a.img_side = d.img; a.patch = d.patch; a.grid = grid; a.ldo = (int)P64(patch_k); a.rows_per_tile = 4;
+      n.n_tiles = (T + 3) / 4;
       int id = b.add(n, N_("vis%d.patchify", c), KIND_ELEM);
       b.write(id, b.all(patches));
     }
@@ -825,29 +833,29 @@ bool build_program(const vla_model_desc& d, const vla_runtime_opts& o, Program& 
     a.table = b.wref(w_emb);
     a.pos = w_lpos >= 0 ? b.wref(w_lpos, n_img) : 0;
     a.out = b.ref(b.rows(x, n_img, d.n_text));
-    a.n = d.n_text; a.d = D; a.ldo = D; a.vocab = d.vocab; a.rows_per_tile = 16; a.ldt = (int)P64(D);
+    a.n = d.n_text; a.d = D; a.ldo = D; a.vocab = d.vocab; a.rows_per_tile = 4; a.ldt = (int)P64(D);
     a.out16 = b.ref(b.rows(xb, n_img, d.n_text)); a.ldo16 = (int)P64(D);
     {
       View sv = b.ss_view(b.rows(xb, n_img, d.n_text));
       a.ss_out = b.ref(sv); a.ss_ld = (int)b.ld(sv);
     }
-    n.n_tiles = (d.n_text + 15) / 16;
+    n.n_tiles = (d.n_text + 3) / 4;
     int id = b.add(n, "llm.embed", KIND_ELEM);
     b.write(id, b.rows(x, n_img, d.n_text));
     b.write(id, b.rows(xb, n_img, d.n_text));
     b.write(id, b.ss_view(b.rows(xb, n_img, d.n_text)));
   }
   for (int i = 0; i < d.llm_layers; ++i) {
-    b.qkv_project(N_("llm.L%d.", i), b.all(xb), lw[i].wqkv, lq[i], d.hd, qkv32, 0, lw[i].n1, D);
+    b.qkv_project(N_("llm.L%d.", i), b.all(xb), lw[i].wqkv, lq[i], d.hd, c_rope, 0, lw[i].n1, D);
     b.attention(N_("llm.L%d.attn", i), b.rows(lq[i].qk, 0, S, 0), S, lq[i], nullptr, b.all(att), d.hq, d.hkv, d.hd, lhs,
                 d.causal != 0);
     Builder::GemmOpt go; go.X = b.all(x); go.out32 = b.all(x); go.out16 = b.all(xb);
     b.gemm(N_("llm.L%d.wo", i), b.all(att), lw[i].wo, D, go);
     Builder::GemmOpt g1; g1.out16 = b.all(mid); g1.norm_gain = lw[i].n2; g1.norm_d = D;
     if (gated) {
-      g1.W2 = lw[i].wu;
+      g1.dual = true;
       g1.act = d.mlp_kind == VLA_MLP_SWIGLU ? ACT_SILU : ACT_GELU;
-      b.gemm(N_("llm.L%d.gu", i), b.all(xb), lw[i].wg, d.mlp, g1);
+      b.gemm(N_("llm.L%d.gu", i), b.all(xb), lw[i].wgu, d.mlp, g1);
     } else {
       g1.act = ACT_GELU;
       b.gemm(N_("llm.L%d.w1", i), b.all(xb), lw[i].w1, d.mlp, g1);
@@ -870,14 +878,13 @@ bool build_program(const vla_model_desc& d, const vla_runtime_opts& o, Program& 
   b.phase = PHASE_ACT;
   b.step = -1;
   const int a_hq = d.head == VLA_HEAD_B ? d.hq : d.act_heads, a_hkv = d.head == VLA_HEAD_B ? d.hkv : d.act_heads;
-  const int a_nq = a_hq * ahs, a_nqkv = (a_hq + 2 * a_hkv) * ahs;
+  const int a_nq = a_hq * ahs;
   int xs = b.buf("act.x", d.horizon, d.act_dim, 4);
   int xbf = b.buf("act.xbf", d.horizon, P64(d.act_dim), 2);
   int z = b.buf("act.z", Ta, da, 4);
   int zb = b.stream_mirror("act.zb", Ta, da);              // bf16 mirror of the head's residual stream (GEMM operand)
   int hz = d.head == VLA_HEAD_C ? b.buf("act.h", Ta, P64(da), 2) : -1;   // adaLN-modulated norms are separate tiles
   Builder::QKV aq = b.make_qkv("act.qkv", Ta, a_hq, a_hkv, ahs);
-  int aqkv32 = (d.head == VLA_HEAD_B && d.rope) ? b.buf("act.qkv32", Ta, a_nqkv, 4) : -1;
   int aatt = b.buf("act.att", Ta, P64(std::max(a_nq, nq)), 2);
   int aqc = (d.head == VLA_HEAD_A || d.head == VLA_HEAD_C) ? b.buf("act.qc", Ta, d.head == VLA_HEAD_A ? nq : da, 2) : -1;
   int amid = b.buf("act.mid", Ta, P64(d.act_mlp), 2);
@@ -944,7 +951,7 @@ bool build_program(const vla_model_desc& d, const vla_runtime_opts& o, Program& 
       bool cross_only = d.head == VLA_HEAD_C && (i % 2 == 1);
       auto resid = [&]() { Builder::GemmOpt go; go.X = b.all(z); go.out32 = b.all(z); go.out16 = b.all(zb); return go; };
       if (!cross_only) {
-        b.qkv_project(NN(""), nin, a.wqkv, aq, ahd, aqkv32, S, fold ? a.n1 : -1, da);
+        b.qkv_project(NN(""), nin, a.wqkv, aq, ahd, d.head == VLA_HEAD_B ? c_rope : -1, S, fold ? a.n1 : -1, da);
         View att_out = b.rows(aatt, 0, Ta);
         if (d.head == VLA_HEAD_B)
           b.attention(NN("attn"), b.rows(aq.qk, 0, Ta, 0), Ta, lq[i], &aq, att_out, d.hq, d.hkv, d.hd, lhs, false,
@@ -972,9 +979,9 @@ bool build_program(const vla_model_desc& d, const vla_runtime_opts& o, Program& 
       Builder::GemmOpt g1; g1.out16 = b.all(amid);
       if (fold) { g1.norm_gain = mlp_gain; g1.norm_d = da; }
       if (agated) {
-        g1.W2 = a.wu;
+        g1.dual = true;
         g1.act = d.act_mlp_kind == VLA_MLP_SWIGLU ? ACT_SILU : ACT_GELU;
-        b.gemm(NN("gu"), nin, a.wg, d.act_mlp, g1);
+        b.gemm(NN("gu"), nin, a.wgu, d.act_mlp, g1);
       } else {
         g1.act = ACT_GELU;
         b.gemm(NN("w1"), nin, a.w1, d.act_mlp, g1);
@@ -1034,6 +1041,8 @@ bool build_program(const vla_model_desc& d, const vla_runtime_opts& o, Program& 
     int pred_tiles = 0;                     // the counter a node waits on counts its predecessors' tiles
     for (int q : pr) pred_tiles += p.nodes[q].n_tiles;
     p.nodes[i].n_pred = pred_tiles;
+    p.pred_nodes.push_back((int)pr.size());
+    if (pr.size() >= (1u << 12)) { set_err(p, "a node has too many predecessors"); return false; }
     for (int q : pr) succ[q].push_back(i);
     if (pr.empty()) p.roots.push_back(i);
   }
@@ -1092,7 +1101,8 @@ bool build_program(const vla_model_desc& d, const vla_runtime_opts& o, Program& 
   p.admit_capacity = 1;
   while (p.admit_capacity < 2 * p.n_inst) p.admit_capacity <<= 1;
   p.off_admit = place(sizeof(AdmitRec) * p.admit_capacity);
-  p.off_dep = place(sizeof(int32_t) * (uint64_t)nn * p.n_inst);
+  p.off_dep = place(sizeof(uint64_t) * (uint64_t)nn * p.n_inst);
+  p.off_start = place(sizeof(int32_t) * (uint64_t)nn * p.n_inst);
   p.off_inst_frame = place(sizeof(uint64_t) * p.n_inst);
   p.off_slot_base = place(sizeof(uint64_t) * p.n_inst);
   p.off_input_ptrs = place(sizeof(uint64_t) * N_FRAME_INPUTS * p.n_inst);

@@ -18,6 +18,8 @@ struct SourceTensor {
   int64_t row_offset;       // first row inside the device tensor
   int64_t group_rows = 0;   // > 0: rows arrive in groups of group_rows (one head) placed group_stride rows apart
   int64_t group_stride = 0;
+  int64_t pair_hd = 0;      // > 0: heads of this width have their rotary pairs (i, i + hd/2) placed side by side (rows 2i, 2i + 1)
+  int64_t row_step = 1;     // 2: rows go to every second row (gate and up matrices share one device tensor)
   bool loaded = false;
 };
 
@@ -57,6 +59,7 @@ struct Program {
   std::vector<double> node_flops, node_wbytes;   // algorithmic FLOPs of a node and the weight bytes its tiles stream
   std::vector<int32_t> succ;
   std::vector<int32_t> roots;
+  std::vector<int32_t> pred_nodes;      // predecessor nodes of each node
   std::vector<int> init_nodes;          // nodes of the one-off constant precomputation (separate program)
   std::vector<NodeDesc> init_program;   // run serially once after the weights are loaded
   ClassInfo classes[N_CLASSES];
@@ -71,12 +74,14 @@ struct Program {
   std::vector<TmapSpec> wmaps;          // weight maps (shared by all frame slots)
   std::vector<TmapSpec> amaps;          // activation maps, instantiated once per frame slot
 
+  int rope_rows = 0, rope_hd = 0;       // rotary table const.rope [rope_rows, rope_hd] filled at init (0: none)
+
   // time arguments of the denoising steps and solver coefficients
   std::vector<float> step_args, step_c_x, step_c_acc;
 
   // arena layout (byte offsets)
   uint64_t off_weights = 0, off_consts = 0, off_nodes = 0, off_succ = 0, off_roots = 0, off_classes = 0,
-           off_control = 0, off_queues = 0, off_q_entries = 0, off_admit = 0, off_dep = 0,
+           off_control = 0, off_queues = 0, off_q_entries = 0, off_admit = 0, off_dep = 0, off_start = 0,
            off_inst_frame = 0, off_slot_base = 0, off_input_ptrs = 0, off_trace = 0, off_tmaps = 0,
            off_init_nodes = 0, off_slots = 0;
   uint64_t slot_bytes = 0, arena_bytes = 0, zero_bytes_begin = 0;

@@ -12,23 +12,31 @@
 
 namespace vla {
 
+// What a tile body needs to know beside its node's arguments.  The persistent kernel keeps one per worker in shared memory:
+// the bodies have use for every register, and values that are the same in all threads are read from there when needed.
 struct TileCtx {
   char* arena;
   uint64_t slot_base;   // arena offset of this frame slot's buffers
   char* smem;           // this tile's shared-memory slab (1024-byte aligned): operand stages, staging tiles
+  int smem_bytes;       // size of the slab handed over (at least the node's smem_bytes)
   char* ctl;            // this worker's 1 KB control block (mbarriers, row scales): outside the slab, so tile
                         // slabs are whole powers-of-two-friendly sizes (64 KB, 72 KB, 48 KB)
   uint32_t tmem;        // this worker's tensor-memory column base
-  int tid;              // 0 .. WORKER_THREADS-1
   int bar_id;           // named barrier of this worker
   uint64_t deadline;    // %globaltimer value after which bounded waits give up
   unsigned int* error;  // sticky device error word
   const uint64_t* inputs;  // this frame slot's input pointer table
   const void* tmaps;    // tensor-map table (128 bytes per entry)
   int amap_base;        // index of this frame slot's first activation map
+  const unsigned long long* wait_word;   // not null: the tile was taken early and waits for its node's release, the moment the
+  unsigned wait_gen;                     // release count of this word (bits 32..62) equals wait_gen; GEMM tiles fetch weights meanwhile
+  uint64_t* t_start;                     // where the time of that moment goes
   int drop_loads;       // test hook of the stand-alone operators: the TMA producer issues nothing, so the consumers'
                         // bounded waits run out (0 everywhere else)
 };
+
+// 0 .. WORKER_THREADS-1 (a kernel's workers are consecutive groups of WORKER_THREADS threads)
+__device__ __forceinline__ int worker_tid() { return (int)(threadIdx.x % WORKER_THREADS); }
 
 template <typename T>
 __device__ __forceinline__ T* resolve(const TileCtx& c, Ref r) {
@@ -42,6 +50,27 @@ __device__ __forceinline__ T* resolve(const TileCtx& c, Ref r) {
 
 __device__ __forceinline__ void worker_sync(const TileCtx& c) {
   asm volatile("bar.sync %0, %1;" ::"r"(c.bar_id), "r"(WORKER_THREADS) : "memory");
+}
+
+// One thread: waits (bounded) until the tile's node is released.  After a time-out the error is recorded and the tile runs
+// on whatever its operands hold, so that everything it has in flight ends in the ordinary way.
+__device__ __forceinline__ void wait_release(const TileCtx& c) {
+  unsigned spins = 0;
+  for (;;) {
+    unsigned long long w;
+    asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(w) : "l"(c.wait_word) : "memory");
+    uint64_t now;
+    if (((unsigned)(w >> 32) & 0x7FFFFFFFu) == c.wait_gen) {
+      asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
+      *c.t_start = now;
+      return;
+    }
+    if ((++spins & 63u) == 0) {
+      asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
+      if (now > c.deadline) atomicCAS(c.error, 0u, (unsigned)DEV_ERR_WAIT_DEP);
+      if (*reinterpret_cast<volatile unsigned*>(c.error) != 0u) { *c.t_start = now; return; }
+    }
+  }
 }
 
 // Activations are produced by other SMs during the same kernel: read them through L2.

@@ -6,6 +6,7 @@
 #include <algorithm>
 #include <atomic>
 #include <chrono>
+#include <cmath>
 #include <cstdarg>
 #include <cstdio>
 #include <cstdlib>
@@ -331,7 +332,7 @@ int vla_init(const vla_model_desc* desc, const vla_runtime_opts* opts, vla_ctx**
   CU(cudaDeviceGetAttribute(&c->sm_count, cudaDevAttrMultiProcessorCount, dev));
   int max_optin = 0;
   CU(cudaDeviceGetAttribute(&max_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-  c->dyn_smem = max_optin - 1024;   // leave the static/reserved part alone
+  c->dyn_smem = max_optin;          // (the kernel has no static shared memory)
   c->workers = opts->workers_per_sm > 0 ? (opts->workers_per_sm > MAX_WORKERS ? MAX_WORKERS : opts->workers_per_sm) : MAX_WORKERS;
   CU(cudaFuncSetAttribute(vla_cosched_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, c->dyn_smem));
   for (auto& n : p.nodes) c->max_node_smem = std::max(c->max_node_smem, n.smem_bytes);
@@ -359,22 +360,37 @@ int vla_init(const vla_model_desc* desc, const vla_runtime_opts* opts, vla_ctx**
     for (size_t i = 0; i < si.size(); ++i) {
       const NodeDesc& sn = p.nodes[p.succ[i]];
       const int res = ((sn.smem_bytes + SMEM_UNIT - 1) / SMEM_UNIT) | (((sn.tmem_cols + TMEM_UNIT - 1) / TMEM_UNIT) << QW_SMEM_BITS);
-      si[i] = SuccInfo{p.succ[i], sn.n_tiles, sn.cls | (res << 8), sn.n_pred};
+      si[i] = SuccInfo{p.succ[i], sn.n_tiles, (int)((uint32_t)(sn.cls | (res << 8)) | ((uint32_t)p.pred_nodes[p.succ[i]] << 20)), sn.n_pred};
     }
     CU(cudaMemcpy(at<char>(c, p.off_succ), si.data(), sizeof(SuccInfo) * si.size(), cudaMemcpyHostToDevice));
   }
   CU(cudaMemcpy(at<char>(c, p.off_roots), p.roots.data(), 4 * p.roots.size(), cudaMemcpyHostToDevice));
   CU(cudaMemcpy(at<char>(c, p.off_classes), p.classes, sizeof(ClassInfo) * N_CLASSES, cudaMemcpyHostToDevice));
   {
-    std::vector<int32_t> dep((size_t)p.n_inst * p.nodes.size());
+    std::vector<uint64_t> dep((size_t)p.n_inst * p.nodes.size());
+    std::vector<int32_t> start(dep.size());
     for (int i = 0; i < p.n_inst; ++i)
-      for (size_t k = 0; k < p.nodes.size(); ++k) dep[(size_t)i * p.nodes.size() + k] = p.nodes[k].n_pred;
-    CU(cudaMemcpy(at<char>(c, p.off_dep), dep.data(), 4 * dep.size(), cudaMemcpyHostToDevice));
+      for (size_t k = 0; k < p.nodes.size(); ++k) {
+        dep[(size_t)i * p.nodes.size() + k] = (uint64_t)p.nodes[k].n_pred;
+        start[(size_t)i * p.nodes.size() + k] = p.pred_nodes[k];
+      }
+    CU(cudaMemcpy(at<char>(c, p.off_dep), dep.data(), 8 * dep.size(), cudaMemcpyHostToDevice));
+    CU(cudaMemcpy(at<char>(c, p.off_start), start.data(), 4 * start.size(), cudaMemcpyHostToDevice));
     std::vector<uint64_t> sb(p.n_inst);
     for (int i = 0; i < p.n_inst; ++i) sb[i] = p.off_slots + (uint64_t)i * p.slot_bytes;
     CU(cudaMemcpy(at<char>(c, p.off_slot_base), sb.data(), 8 * sb.size(), cudaMemcpyHostToDevice));
     int args_buf = p.buf_index.at("const.args");
     CU(cudaMemcpy(c->arena + p.off_consts + p.bufs[args_buf].offset, p.step_args.data(), 4 * p.step_args.size(), cudaMemcpyHostToDevice));
+    if (p.rope_rows > 0) {      // rotary table: (cos, sin) of position * 10000^(-2i/hd)
+      std::vector<float> tab((size_t)p.rope_rows * p.rope_hd);
+      for (int r = 0; r < p.rope_rows; ++r)
+        for (int i = 0; i < p.rope_hd / 2; ++i) {
+          const double a = (double)r * std::pow(10000.0, -2.0 * i / p.rope_hd);
+          tab[(size_t)r * p.rope_hd + 2 * i] = (float)std::cos(a);
+          tab[(size_t)r * p.rope_hd + 2 * i + 1] = (float)std::sin(a);
+        }
+      CU(cudaMemcpy(c->arena + p.off_consts + p.bufs[p.buf_index.at("const.rope")].offset, tab.data(), 4 * tab.size(), cudaMemcpyHostToDevice));
+    }
   }
 
   // pinned host memory
@@ -404,7 +420,9 @@ int vla_init(const vla_model_desc* desc, const vla_runtime_opts* opts, vla_ctx**
   x.queues = at<TileQueue>(c, p.off_queues);
   x.q_entries = at<QueueEntry>(c, p.off_q_entries);
   x.admit_ring = at<AdmitRec>(c, p.off_admit);
-  x.dep_count = at<int32_t>(c, p.off_dep);
+  x.dep_word = at<unsigned long long>(c, p.off_dep);
+  x.start_count = at<int32_t>(c, p.off_start);
+  x.ring_depth = p.ring_depth;
   x.inst_frame = at<uint64_t>(c, p.off_inst_frame);
   x.slot_base = at<uint64_t>(c, p.off_slot_base);
   x.input_ptrs = at<uint64_t>(c, p.off_input_ptrs);
@@ -492,13 +510,20 @@ int vla_load_weights(vla_ctx* c, const vla_tensor* tensors, size_t n, int32_t fi
         return fail(c, VLA_ERR_INVALID, "tensor '%s': unknown dtype", t.name);
       }
       // padding columns [cols, ld) and padding rows between heads stay zero (the arena was cleared at init)
-      if (s.group_rows > 0) {
+      if (s.pair_hd > 0) {
+        // rotary pairs (i, i + hd/2) of a head become rows 2i and 2i + 1: each half of a head goes to every second row
+        const int64_t half = s.pair_hd / 2;
+        for (int64_t r = 0; r < s.rows; r += half)
+          CU(cudaMemcpy2D(dst + (size_t)(r / s.pair_hd * s.pair_hd + (r % s.pair_hd ? 1 : 0)) * dt.ld * 2, (size_t)dt.ld * 4,
+                          static_cast<const char*>(src) + (size_t)r * s.cols * 2, (size_t)s.cols * 2, (size_t)s.cols * 2, (size_t)half,
+                          cudaMemcpyHostToDevice));
+      } else if (s.group_rows > 0) {
         for (int64_t g0 = 0, gi = 0; g0 < s.rows; g0 += s.group_rows, ++gi)
           CU(cudaMemcpy2D(dst + (size_t)gi * s.group_stride * dt.ld * 2, (size_t)dt.ld * 2,
                           static_cast<const char*>(src) + (size_t)g0 * s.cols * 2, (size_t)s.cols * 2, (size_t)s.cols * 2,
                           (size_t)s.group_rows, cudaMemcpyHostToDevice));
       } else {
-        CU(cudaMemcpy2D(dst, (size_t)dt.ld * 2, src, (size_t)s.cols * 2, (size_t)s.cols * 2, (size_t)s.rows, cudaMemcpyHostToDevice));
+        CU(cudaMemcpy2D(dst, (size_t)dt.ld * 2 * s.row_step, src, (size_t)s.cols * 2, (size_t)s.cols * 2, (size_t)s.rows, cudaMemcpyHostToDevice));
       }
     }
     s.loaded = true;
@@ -777,7 +802,8 @@ int vla_debug_bump_dependency(vla_ctx* c, int32_t stream, int32_t slot, int32_t 
     return fail(c, VLA_ERR_INVALID, "bad stream, slot or node");
   if (c->pending_frames != 0) return fail(c, VLA_ERR_STATE, "frames are in flight");
   CU(cudaDeviceSynchronize());
-  int32_t* cnt = c->dctx.dep_count + (size_t)(stream * p.ring_depth + slot) * p.nodes.size() + node;
+  // (the count is the low half of the node's state word)
+  int32_t* cnt = reinterpret_cast<int32_t*>(c->dctx.dep_word + (size_t)(stream * p.ring_depth + slot) * p.nodes.size() + node);
   int32_t v = 0;
   CU(cudaMemcpy(&v, cnt, sizeof v, cudaMemcpyDeviceToHost));
   v += delta;
@@ -872,8 +898,8 @@ int vla_op_attention_static(const void* q, const void* k, const void* v, void* o
 int vla_op_status(int32_t op, const void* scratch, void* stream) {
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   if (op == VLA_OP_LINEAR) {
-    unsigned* w = vla::op_linear_error_word();
-    return w ? vla::op_status_of(w, s) : VLA_ERR_CUDA;
+    vla::OpDevice* d = vla::op_device();
+    return d ? vla::op_status_of(d->error.load(), s, d->calls.load()) : VLA_ERR_CUDA;
   }
   if (op == VLA_OP_ATTENTION) {
     if (!scratch) return VLA_ERR_INVALID;

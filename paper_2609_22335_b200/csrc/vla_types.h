@@ -11,7 +11,6 @@ enum Op : int32_t {
   OP_ATTN = 2,      // fused softmax(QK^T/sqrt(hd))V over up to two K/V segments
   OP_PATCHIFY = 3,  // image fp32 -> bf16 patch rows
   OP_EMBED = 4,     // text-embedding gather (+ position table) into the fp32 residual stream
-  OP_ROPE = 5,      // fp32 q|k|v rows -> bf16 with rotary embedding on the q and k heads
   OP_ADDROWS = 6,   // out fp32 [M,N] = in fp32 (+ vec) (+ table)
   OP_TIMEEMB = 7,   // sinusoidal timestep embedding rows -> bf16
   OP_EMIT = 8,      // copy the finished chunk to the host-visible ring and publish its frame id
@@ -35,10 +34,10 @@ constexpr Ref REF_SLOT = 1ull << 63;
 constexpr Ref REF_INPUT = 1ull << 62;
 constexpr int N_FRAME_INPUTS = 4;
 
-constexpr int GEMM_BM = 128;   // output features per GEMM tile (the MMA M dimension)
+constexpr int GEMM_BM = 128;   // weight rows per GEMM tile (the MMA N dimension; tokens are M)
 constexpr int GEMM_BK = 64;    // K elements per pipeline stage (one 128-byte swizzle row of bf16)
 constexpr int WORKER_THREADS = 128;
-constexpr int GEMM_MAX_BT = 128;     // most tokens per GEMM tile (MMA N)
+constexpr int GEMM_MAX_BT = 128;     // most tokens per GEMM tile (MMA M)
 constexpr int GEMM_SMEM_BUDGET = 64 * 1024;  // stage memory a token-rich GEMM tile aims for (at least two stages are always taken)
 constexpr int GEMM_SMEM_BUDGET_SMALL = 84 * 1024;  // token-poor tiles (<= 64 tokens) are bound by TMA latency and get deeper
                                                    // pipelines, but must fit the room one finished token-rich tile leaves
@@ -52,17 +51,26 @@ inline int gemm_stages(int bt, int Kp) {
   const int nkb = Kp / GEMM_BK;
   return S < nkb ? S : (nkb < 1 ? 1 : nkb);
 }
-inline int gemm_smem_bytes(int bt, int S) {      // the epilogue parks the tile in the stage memory as fp32
-  const int a = S * gemm_stage_bytes(bt), b = bt * GEMM_BM * 4;
-  return a > b ? a : b;
+constexpr int GEMM_MAX_STAGES = 12;
+// Stages of a tile that got `bytes` of shared memory: the node's own depth, or more where there is room and K has use for it.
+#ifdef __CUDACC__
+__host__ __device__
+#endif
+inline int gemm_stages_in(int bytes, int bt, int Kp, int stages) {
+  int S = bytes / (GEMM_BM * GEMM_BK * 2 + bt * GEMM_BK * 2);
+  S = S > GEMM_MAX_STAGES ? GEMM_MAX_STAGES : S;
+  S = S > Kp / GEMM_BK ? Kp / GEMM_BK : S;
+  return S > stages ? S : stages;
 }
+inline int gemm_smem_bytes(int bt, int S) { return S * gemm_stage_bytes(bt); }
 
-// Shared memory of one attention tile: Q (128 rows), one K block and one V^T block of 64 keys,
-// and the probability tile.  hs = head stride (head dim padded to a multiple of 16).
+// Shared memory of one attention tile: Q (128 rows), two K and two V^T blocks of 64 keys.  Tensor-memory columns: scores,
+// probabilities (bf16 pairs), output.  hs = head stride (head dim padded to a multiple of 16).
 inline int attn_smem_bytes(int hs) {
   const int nbox = (hs + 63) / 64;
-  return nbox * 128 * 128 + nbox * 64 * 128 + hs * 128 + 128 * 128;
+  return nbox * 128 * 128 + 2 * (nbox * 64 * 128 + hs * 128);
 }
+inline int attn_tmem_cols(int hs) { return 64 + 32 + hs; }
 
 // Query heads that share a KV head (grouped or multi-query attention) and have few queries are folded into the 128
 // rows of one attention tile: the tile streams K and V^T once for all of them.  Returns heads per tile, sets rows per head.
@@ -75,24 +83,28 @@ inline int attn_fold(int tq, int hq, int hkv, int* rph) {
 }
 
 struct GemmArgs {
-  Ref A, W, W2;        // A bf16 [M,lda]; W (and W2 when dual) bf16 [N,Kp]
+  // operands: A bf16 [M,K] and W bf16 [N,Kp] (dual: [2N,Kp], gate and up rows alternating), reached through their tensor maps
   Ref X;               // optional fp32 addend [M,ldx], scaled by c_x
   Ref vec;             // optional fp32 [N], broadcast over rows
   Ref tab, tab2;       // optional fp32 tables [M,ldtab] added row by row
   Ref out32, out16;    // fp32 and/or bf16 outputs [M,ld]
   Ref outT;            // optional transposed bf16 output: features >= t_col0 go to outT[f - t_col0][token]
-  int32_t lda, ldx, ldtab, ldtab2, ldo32, ldo16, ldoT, t_col0;
+  int32_t ldx, ldtab, ldtab2, ldo32, ldo16, ldoT, t_col0;
   int32_t M, N, Kp;    // tokens, output features, padded reduction length (multiple of GEMM_BK)
   int32_t bt, tiles_t; // tokens per tile, number of token tiles
-  int32_t act, dual;   // activation; dual (gated): out = act(A W^T) * (A W2^T), 64 output features per tile
+  int32_t vec16;       // every row and column offset of the epilogue's operands allows 16-byte accesses and N whole chunks
+  int32_t act, dual;   // activation; dual (gated): out = act(A Wgate^T) * (A Wup^T), 64 output features per tile
   float c_acc, c_x;    // out = c_x * X + c_acc * acc + vec + tab + tab2
-  int32_t wmap, w2map, amap;  // tensor-map indices: shared weight maps, activation map relative to the slot's first
+  int32_t wmap, amap;         // tensor-map indices: shared weight maps, activation map relative to the slot's first
   int32_t stages;             // TMA pipeline depth
   int32_t rs_d;               // > 0: A holds the raw residual stream (bf16) and RMSNorm is folded into the GEMM: every
                               // output row is scaled by 1/sqrt(sum_j ss_in[row][j] / rs_d + 1e-6)
-  int32_t ss_nft, ss_out_ld, pad_;
+  int32_t ss_nft, ss_out_ld;
+  int32_t rope_hd, rope_cols; // rope_cols > 0: output features [0, rope_cols) are q and k heads of width rope_hd and leave
+                              // rotated (rows of a pair are neighbours in the matrix)
   Ref ss_in;                  // fp32 [M, ss_nft]: per-row sums of squares of the stream, one partial per 128 columns
   Ref ss_out;                 // optional fp32 [M, ss_out_ld]: this tile writes the partial of its 128 output features
+  Ref rope_tab;               // fp32 [M, rope_hd]: (cos, sin) of the token's position per frequency
   Ref bias;                   // optional fp32 [N] added to the accumulator before the activation (not with dual)
 };
 
@@ -132,11 +144,6 @@ struct EmbedArgs {
   int32_t n, d, ldo, vocab, rows_per_tile, ldt;
 };
 
-struct RopeArgs {
-  Ref in, out, outT;   // in fp32 [M,ld]; out bf16 [M,ldo] (rotated q and k heads); outT bf16 [v features, ldoT] = V^T
-  int32_t M, ld, ldo, ldoT, n_rot_heads, n_heads, hd, pos0, rows_per_tile;
-};
-
 struct AddRowsArgs {
   Ref in, vec, tab, out, out16;  // fp32; out16 optional bf16 copy
   Ref ss_out;                    // optional fp32 [M, ss_ld] per-row sums of squares, one partial per 128 columns
@@ -154,19 +161,18 @@ struct EmitArgs {
   int32_t chunk_off;   // first element of this pass's chunk inside the frame's host-visible chunk block
 };
 
-struct NodeDesc {
+struct alignas(16) NodeDesc {
   int32_t op, cls, n_tiles, n_pred;
   int32_t succ_begin, succ_count;
   int32_t phase, step;
   int32_t smem_bytes, tmem_cols;
-  int32_t pad0, pad1;
+  int32_t smem_deep, pad1;   // shared memory of the deepest useful pipeline (GEMM; taken when the SM has nothing else to run)
   union {
     GemmArgs gemm;
     NormArgs norm;
     AttnArgs attn;
     PatchArgs patch;
     EmbedArgs embed;
-    RopeArgs rope;
     AddRowsArgs addrows;
     TimeEmbArgs timeemb;
     EmitArgs emit;
@@ -190,12 +196,12 @@ struct TileQueue {             // one 128-byte line per queue
   unsigned long long head;     // next ticket to hand out
   unsigned long long tail;     // next ticket to reserve for a push
   long long avail;             // committed minus claimed (may dip below zero transiently)
-  unsigned long long pad[13];
+  unsigned long long done;     // tiles of this class that have finished: tail - done are queued or running
+  unsigned long long pad[12];
 };
 
 // One queued tile is one 64-bit word, written and read atomically:
-//   bits 63..48 generation tag ((ticket / capacity + 1) & 0xFFFF; 0 = never written),
-//   bits 47..32 tile index inside the node, bits 31..0 inst << 20 | node.
+// generation tag | early flag | tensor- and shared-memory units | tile | frame slot | node (widths: QW_* in dispatch.cuh).
 typedef unsigned long long QueueEntry;
 
 struct AdmitRec {              // written by the host (copy stream), read by the dispatcher
@@ -235,12 +241,13 @@ struct Control {                 // polled words and hot counters live on separa
 
 enum DevError : uint32_t {
   DEV_OK = 0, DEV_ERR_WAIT_QUEUE = 1, DEV_ERR_QUEUE_FULL = 2, DEV_ERR_WAIT_MBAR = 3, DEV_ERR_IDLE_LIMIT = 4,
-  DEV_ERR_BAD_OP = 5
+  DEV_ERR_BAD_OP = 5, DEV_ERR_WAIT_DEP = 6
 };
 
 // Everything a kernel needs, passed by value.
 // One successor edge as the retire path reads it: everything needed to release the node in one 16-byte load.
-struct SuccInfo { int32_t node, n_tiles, cls_res, n_pred; };   // cls_res = class | resource units of one tile << 8
+// cls_res = class | resource units of one tile << 8 | predecessor nodes << 20
+struct SuccInfo { int32_t node, n_tiles, cls_res, n_pred; };
 
 struct DeviceCtx {
   char* arena;
@@ -251,7 +258,10 @@ struct DeviceCtx {
   TileQueue* queues;             // [N_CLASSES]
   QueueEntry* q_entries;         // [N_CLASSES][q_capacity]
   AdmitRec* admit_ring;
-  int32_t* dep_count;            // [n_inst][n_nodes]
+  // [n_inst][n_nodes] state of a node in a frame slot: bits 0..31 predecessor tiles still to finish, bits 32..62 how often the
+  // node has been released (once per frame of the slot), bit 63 its tiles were queued early, before the release
+  unsigned long long* dep_word;
+  int32_t* start_count;          // [n_inst][n_nodes] predecessor nodes whose last tile has not been taken yet
   uint64_t* inst_frame;          // [n_inst] frame id currently owning the slot
   const uint64_t* slot_base;     // [n_inst] arena offset of the instance's buffers
   const uint64_t* input_ptrs;    // [n_inst][N_FRAME_INPUTS] device addresses of the frame's input arrays
@@ -265,7 +275,7 @@ struct DeviceCtx {
   int32_t n_nodes, n_inst, n_roots;
   int32_t q_capacity, q_shift, admit_capacity;   // q_capacity = 1 << q_shift
   uint32_t trace_capacity;
-  int32_t policy, workers_per_sm;
+  int32_t policy, workers_per_sm, ring_depth;
   int32_t u_max, pad_u;     // saturation value of the utilisation counters in the pick's score
   uint64_t wait_limit_ns, idle_exit_ns;
   int32_t chunk_elems;
