@@ -10,7 +10,7 @@ constexpr unsigned CTRL_EXITING = 0x80000000u;
 constexpr uint32_t TRACE_ADMIT_NODE = 0xFFFFFFFFu;   // node id of the trace record that marks a frame's admission
 constexpr int MAX_WORKERS = 3;
 constexpr int SM_CTL_BYTES = 1024;       // per-worker control block (mbarriers, row scales) handed to the tile bodies
-constexpr int SM_STATE_BASE = 4096;      // dispatcher state of the SM
+constexpr int SM_STATE_BASE = 8192;      // dispatcher state of the SM
 constexpr int SM_STATE_BYTES = SM_STATE_BASE + MAX_WORKERS * SM_CTL_BYTES;   // then the tile slab, 1024-byte aligned
 
 __device__ __forceinline__ uint64_t gtimer() {
@@ -168,30 +168,6 @@ constexpr unsigned long long SPREAD_WAIT_NS = 1000;
 constexpr int EARLY_MAX_TILES = 148;
 constexpr unsigned long long HEAD_WAIT_NS = 1500;   // an action-head tile nobody took for this long may go to a running worker
 
-struct WorkerTile {
-  uint32_t inst, node, tile;
-  int cls;
-  int smem_unit0, smem_units, tmem_unit0, tmem_units;
-  int succ_begin, succ_count, op, early;    // of the tile's node, filled in by the worker for the retire warp; queued before the release
-  uint64_t t0, t1, frame;
-};
-
-// Mailboxes between one worker group and the SM's dispatcher warp (all in shared memory).
-struct WorkerSlot {
-  volatile unsigned held_tail;   // claimed tiles pushed by the claim warp (single producer)
-  volatile unsigned held_head;   // claimed tiles taken by the worker (single consumer)
-  volatile int leave;            // claim warp -> worker: go home
-  volatile int done_state;       // 0 empty, 1 finished tile posted for the retire warp
-  volatile int busy;             // the worker is running a tile (set and cleared by the worker)
-  int turn;                      // which half of SmState::cur holds the running tile
-  uint32_t bell_parity;
-  volatile int start_state;      // 1: the worker took the last tile of (start_inst, start_node): its successors may be queued early
-  uint32_t start_inst, start_node;
-  volatile unsigned prio_tail, prio_head;   // one-deep slot for an action-head tile that goes ahead of the held VLM tiles
-  volatile unsigned long long t_busy;       // when the running tile was taken (worker), for the claim warp's estimate of its end
-  WorkerTile done, held[HELD_DEPTH], prio;
-};
-
 static_assert(sizeof(NodeDesc) % 16 == 0 && sizeof(NodeDesc) <= 512, "a node's description is copied by one warp, 16 bytes a lane");
 struct __align__(16) SmState {
   unsigned long long smem_mask;    // bit i set = shared-memory unit i in use
@@ -212,11 +188,7 @@ struct __align__(16) SmState {
   unsigned long long bell_claim;   // rung by a worker that took a claimed tile or ran out of work
   unsigned long long bell_retire;  // rung by a worker that posted a finished tile
   unsigned long long bell_worker[MAX_WORKERS];   // rung by the claim warp when it hands worker w a tile or sends it home
-  WorkerTile cur[MAX_WORKERS][2];  // the tile each worker is running and the one before it (written by its leader in turn): what the
-                                   // end of a tile needs is read back from here instead of living in registers through the tile body
-  TileCtx tc[MAX_WORKERS];         // context of the running tile ...
-  NodeDesc node[MAX_WORKERS];      // ... and the description of its node, copied here: the tile body's arguments
-  volatile int cur_cls[MAX_WORKERS];   // class of the running tile, for the claim warp
+  TileCtx tc[MAX_WORKERS];         // context of each worker's running tile
   WorkerSlot slot[MAX_WORKERS];
 };
 static_assert(sizeof(SmState) <= SM_STATE_BASE, "SM state too large");
@@ -248,9 +220,8 @@ __device__ inline void write_trace(const DeviceCtx& ctx, uint32_t inst, uint32_t
   ctx.trace[idx] = r;
 }
 
-// Release count that a node of the frame now in slot `inst` reaches when it is released.
-__device__ __forceinline__ unsigned release_count(const DeviceCtx& ctx, uint32_t inst) {
-  const uint64_t frame = *reinterpret_cast<const volatile uint64_t*>(ctx.inst_frame + inst);
+// Release count that a node reaches when it is released for this frame of its slot.
+__device__ __forceinline__ unsigned release_count(const DeviceCtx& ctx, uint64_t frame) {
   return (unsigned)(frame / (unsigned)ctx.ring_depth + 1u) & 0x7FFFFFFFu;
 }
 
@@ -382,7 +353,7 @@ __device__ __forceinline__ void retire_loop(const DeviceCtx& ctx, SmState* sm, i
       uint32_t inst = 0;
       int succ0 = 0, n_succ = 0;
       if (ended) {
-        const WorkerTile& f = slot->done;
+        const DoneTile& f = slot->done;
         inst = f.inst; succ0 = f.succ_begin; n_succ = f.succ_count;
         if (sub == 0) {
           sm->ema_ns[f.cls] = (3 * sm->ema_ns[f.cls] + (int)(f.t1 - f.t0)) >> 2;
@@ -481,8 +452,8 @@ __device__ inline void claim_loop(const DeviceCtx& ctx, SmState* sm, int n_worke
         const bool head_pending = pick_is_two_phase(ctx.policy) && (pending & act_mask & ~avoid) != 0u;
         unsigned cand;
         if (!busy) cand = head_pending ? (pending & act_mask) : pending;
-        else if (pq == 0u && head_pending && (waiting & act_mask & ~avoid) != 0u && slot->busy != 0 &&
-                 (long long)(gtimer() - slot->t_busy) + PRIO_WINDOW_NS >= (long long)sm->ema_ns[sm->cur_cls[w]]) {
+        else if (pq == 0u && head_pending && (waiting & act_mask & ~avoid) != 0u && slot->busy != 0 && slot->primed == 0 &&
+                 (long long)(gtimer() - slot->t_busy) + PRIO_WINDOW_NS >= (long long)sm->ema_ns[slot->cls]) {
           cand = waiting & act_mask; to_prio = true;
         }
         else if (queued < (unsigned)HELD_DEPTH) cand = deep & ((1u << N_KINDS) - 1u);
@@ -527,35 +498,51 @@ __device__ inline void claim_loop(const DeviceCtx& ctx, SmState* sm, int n_worke
       }
       if (__shfl_sync(0xffffffffu, want, w) >= 0) ++running;
     }
-    // ---- the claims themselves run in parallel across lanes (global atomics)
+    // ---- the claims themselves run in parallel across lanes (global atomics); the warp then brings the claimed tiles' node
+    // descriptions into their jobs, so that a worker finds all it needs in shared memory
+    bool popped = false;
+    int ji = 0;
+    uint32_t node = 0;
     if (want >= 0) {
       QueueEntry e;
       if (queue_try_pop(ctx, want, e, gtimer() + ctx.wait_limit_ns)) {
-        WorkerTile& h = to_prio ? slot->prio : slot->held[slot->held_tail % HELD_DEPTH];
-        h.node = (uint32_t)e & ((1u << QW_NODE_BITS) - 1u);
-        h.inst = (uint32_t)(e >> QW_NODE_BITS) & ((1u << QW_INST_BITS) - 1u);
+        popped = true;
+        ji = to_prio ? 2 + (int)(slot->prio_tail & 1u) : (int)(slot->held_tail & 1u);
+        TileJob& h = slot->job[ji];
+        node = (uint32_t)e & ((1u << QW_NODE_BITS) - 1u);
+        h.node = node;
+        const uint32_t inst = (uint32_t)(e >> QW_NODE_BITS) & ((1u << QW_INST_BITS) - 1u);
+        h.inst = inst;
         h.tile = (uint32_t)(e >> (QW_NODE_BITS + QW_INST_BITS)) & ((1u << QW_TILE_BITS) - 1u);
         h.smem_units = (int)((e >> (QW_NODE_BITS + QW_INST_BITS + QW_TILE_BITS)) & ((1u << QW_SMEM_BITS) - 1u));
         h.tmem_units = (int)((e >> (QW_NODE_BITS + QW_INST_BITS + QW_TILE_BITS + QW_SMEM_BITS)) & ((1u << QW_TMEM_BITS) - 1u));
         h.cls = want;
         h.early = (int)((e >> (64 - QW_GEN_BITS - 1)) & 1u);
-        {   // the worker's first loads are from the node's description: bring its two lines into this SM's L1 now
-          const char* ndp = reinterpret_cast<const char*>(ctx.nodes + h.node);
-          asm volatile("prefetch.global.L1 [%0];" ::"l"(ndp));
-          asm volatile("prefetch.global.L1 [%0];" ::"l"(ndp + 128));
-        }
-        h.succ_begin = promised_s; h.succ_count = promised_t;   // (fields reused until the worker fills them in) units to un-promise
-        __threadfence_block();
-        if (to_prio) slot->prio_tail = slot->prio_tail + 1;
-        else slot->held_tail = slot->held_tail + 1;      // the worker takes it as soon as it is free
-        bell_ring(&sm->bell_worker[lane]);
-        progressed = true;
+        h.promised_s = promised_s; h.promised_t = promised_t;
+        h.slot_base = __ldg(ctx.slot_base + inst);
+        h.frame = ld_volatile_u64(reinterpret_cast<const unsigned long long*>(ctx.inst_frame + inst));
+        if (h.early) h.gen = release_count(ctx, h.frame);
       } else {                                         // lost the race: undo the count
         atomicSub(&sm->pick.cta_count[want], 1);
         for (int x = 0; x < 3; ++x) atomicSub(&sm->pick.u[x], sm->tau_tab[want * 3 + x]);
         if (promised_s | promised_t) { atomicSub(&sm->smem_promised, promised_s); atomicSub(&sm->tmem_promised, promised_t); }
         lost = 1u << want;                             // look elsewhere in the next round, which follows at once
       }
+    }
+#pragma unroll 1
+    for (unsigned m = __ballot_sync(0xffffffffu, popped); m != 0u; m &= m - 1u) {
+      const int w = __ffs((int)m) - 1;
+      const int4* src = reinterpret_cast<const int4*>(ctx.nodes + __shfl_sync(0xffffffffu, node, w));
+      int4* dst = reinterpret_cast<int4*>(&sm->slot[w].job[__shfl_sync(0xffffffffu, ji, w)].desc);
+      if (lane < (int)(sizeof(NodeDesc) / 16)) dst[lane] = __ldg(src + lane);
+    }
+    __syncwarp();
+    if (popped) {
+      __threadfence_block();
+      if (to_prio) slot->prio_tail = slot->prio_tail + 1;
+      else slot->held_tail = slot->held_tail + 1;      // the worker takes it as soon as it is free
+      bell_ring(&sm->bell_worker[lane]);
+      progressed = true;
     }
     // ---- admission, exit and watchdog (lane 0 decides, every few rounds)
     int verdict = 0;   // 1 = leave
@@ -610,32 +597,37 @@ __device__ __forceinline__ void end_of_tile(const DeviceCtx& ctx, SmState* sm, W
   unsigned tid;
   asm volatile("mov.u32 %0, %%tid.x;" : "=r"(tid));
   const int worker = (int)tid / WORKER_THREADS, wt = (int)tid % WORKER_THREADS;
-  WorkerTile& cmd = sm->cur[worker][slot->turn];      // (looked up before the barrier: afterwards the leader moves on)
+  DoneTile d;
+  if (wt == 32) {              // (read before the barrier: afterwards the leader moves on)
+    const TileJob& j = slot->job[slot->run];
+    d.inst = j.inst; d.node = j.node; d.tile = j.tile; d.cls = j.cls; d.frame = j.frame; d.t0 = slot->t_start;
+    d.succ_begin = j.desc.succ_begin; d.succ_count = j.desc.succ_count; d.op = j.desc.op;
+  }
   asm volatile("bar.sync %0, %1;" ::"r"(worker + 1), "r"(WORKER_THREADS) : "memory");
   // Two lanes share the end of a tile: lane 0 frees the tile's memory and goes straight on to take the next
   // tile, the first lane of warp 1 posts the finished one to the retire warp meanwhile (both meet again at the
   // barrier that opens the next tile).
   if (wt == 0) {
     atomicAdd(&ctx.control->tiles_done, 1ull);
-    if (cmd.t0 == 1) {
-      if (cmd.smem_units) atomicAnd(&sm->smem_mask, ~(unit_bits(cmd.smem_units) << cmd.smem_unit0));
-      if (cmd.tmem_units) atomicAnd(&sm->tmem_mask, ~(unsigned)(unit_bits(cmd.tmem_units) << cmd.tmem_unit0));
+    if (!slot->primed) {
+      if (slot->verdict == 1) {
+        if (slot->smem_units) atomicAnd(&sm->smem_mask, ~(unit_bits(slot->smem_units) << slot->smem_unit0));
+        if (slot->tmem_units) atomicAnd(&sm->tmem_mask, ~(unsigned)(unit_bits(slot->tmem_units) << slot->tmem_unit0));
+      }
+      slot->busy = 0;
+      if (slot->held_tail == slot->held_head && slot->prio_tail == slot->prio_head) bell_ring(&sm->bell_claim);   // out of work
     }
-    slot->busy = 0;
-    if (slot->held_tail == slot->held_head && slot->prio_tail == slot->prio_head) bell_ring(&sm->bell_claim);   // out of work
   } else if (wt == 32) {
-    const uint64_t t1 = gtimer();
-    WorkerTile d = cmd;
-    d.t0 = cmd.t1; d.t1 = t1;
+    d.t1 = gtimer();
     unsigned naps = 0;
     while (slot->done_state != 0) {
       __nanosleep(40);
-      if ((++naps & 0xFFFFu) == 0 && gtimer() - t1 > 2 * ctx.wait_limit_ns) break;   // retire warp gone: give up posting
+      if ((++naps & 0xFFFFu) == 0 && gtimer() - d.t1 > 2 * ctx.wait_limit_ns) break;   // retire warp gone: give up posting
     }
     slot->done = d;
     // The tile's writes (all threads, ordered by the barrier above) must be visible device-wide before any
-    // successor is released.  That fence is the retire warp's (first statement of complete_tile, after it has
-    // read this flag): fences are cumulative, and barrier -> block-scope fence -> flag -> device-scope fence
+    // successor is released.  That fence is the retire warp's (after it has read this flag): fences are cumulative, and
+    // barrier -> block-scope fence -> flag -> device-scope fence
     // keeps the writes ahead of the counter atomics without a device-scope round trip on the worker's path.
     __threadfence_block();
     slot->done_state = 1;
@@ -643,6 +635,127 @@ __device__ __forceinline__ void end_of_tile(const DeviceCtx& ctx, SmState* sm, W
     atomicSub(&sm->pick.cta_count[d.cls], 1);    // the pick's view of this SM, after the completion is on its way
     for (int x = 0; x < 3; ++x) atomicSub(&sm->pick.u[x], sm->tau_tab[d.cls * 3 + x]);
   }
+}
+
+// The worker's leader: waits for a tile the claim warp has put together, gives it its memory and fills in its context.
+__device__ __forceinline__ void take_tile(const DeviceCtx& ctx, SmState* sm, WorkerSlot* slot, char* slab, int worker, int n_workers) {
+  Control* ctl = ctx.control;
+  TileCtx& tc = sm->tc[worker];
+  bool prio = false;
+  unsigned naps = 0;
+  if (!slot->primed) {
+    uint32_t bell_parity = slot->bell_parity;
+    for (;;) {
+      if (slot->prio_tail != slot->prio_head) { prio = true; break; }
+      if (slot->held_tail != slot->held_head) break;
+      if (slot->leave) { slot->verdict = 0; return; }
+      if (naps < 8) __nanosleep(20);                               // a claimed tile is usually a moment away
+      else bell_wait(&sm->bell_worker[worker], bell_parity, 2000u);
+      ++naps;
+    }
+    slot->bell_parity = bell_parity;
+  }
+  __threadfence_block();
+  const int ji = prio ? 2 + (int)(slot->prio_head & 1u) : (int)(slot->held_head & 1u);
+  TileJob& job = slot->job[ji];
+  const uint64_t now = gtimer(), lim = now + ctx.wait_limit_ns;
+  slot->run = ji;
+  slot->t_busy = now;
+  slot->cls = job.cls;
+  slot->busy = 1;
+  __threadfence_block();
+  if (prio) slot->prio_head = slot->prio_head + 1;
+  else slot->held_head = slot->held_head + 1;   // the claim warp may fill the other job of the pair
+  bell_ring(&sm->bell_claim);
+  int early = job.early;
+  bool ok = true;
+  tc.cont = slot->primed;
+  if (slot->primed) slot->primed = 0;           // memory and operand ring stay with the worker
+  else {
+    ok = false;
+    if (early) {
+      // A tile taken before its node's release may hold memory while it waits only where no tile taken earlier can
+      // still need some, that is, where it is the only one this SM has taken.  Elsewhere it waits empty-handed.
+      int taken = 0;
+#pragma unroll 1
+      for (int k = 0; k < N_CLASSES; ++k) taken += *reinterpret_cast<volatile int*>(&sm->pick.cta_count[k]);
+      if (taken != 1) {
+        tc.wait_word = ctx.dep_word + (size_t)job.inst * ctx.n_nodes + job.node;
+        tc.wait_gen = job.gen;
+        tc.t_start = &slot->t_wait;
+        tc.deadline = lim;
+        wait_release(tc);
+        early = 0;
+      }
+    }
+    const int need_units = job.smem_units, tmem_units = job.tmem_units;
+    int deep_units = 0;
+    if (sm->outstanding <= 2 * (int)gridDim.x) {
+      // Few tiles on the whole GPU: a GEMM tile takes the pipeline depth its K has use for, up to its share of the
+      // SM.  A k-block then costs its share of many loads in flight instead of half or a quarter of a round trip.
+      const int third = sm->n_smem_units / MAX_WORKERS;
+      const int share = sm->outstanding <= (int)gridDim.x / 2 ? sm->n_smem_units : (sm->outstanding <= (int)gridDim.x ? 2 * third : sm->n_smem_units / 2);
+      deep_units = min((job.desc.smem_deep + SMEM_UNIT - 1) / SMEM_UNIT, share);
+    }
+    // every worker has a home region (a third of the slab, a third of the columns): a tile that fits it goes
+    // there whenever it is free, so tiles of the common shapes never fragment the slab; larger tiles and a
+    // home occupied by one of them fall back to the first free run
+    const int third_s = sm->n_smem_units / n_workers, third_t = sm->n_tmem_units / n_workers;
+#pragma unroll 1
+    for (unsigned spin = 0;; ++spin) {
+      const unsigned long long sm_old = *reinterpret_cast<volatile unsigned long long*>(&sm->smem_mask);
+      int units = need_units, s0 = -1;
+      if (deep_units > need_units && (s0 = find_free(sm_old, deep_units, sm->n_smem_units)) >= 0) units = deep_units;
+      else if (units <= third_s && ((sm_old >> (worker * third_s)) & unit_bits(units)) == 0ull) s0 = worker * third_s;
+      else s0 = find_free(sm_old, units, sm->n_smem_units);
+      if (s0 >= 0) {
+        const unsigned long long sbits = unit_bits(units) << s0;
+        if (units == 0 || atomicCAS(&sm->smem_mask, sm_old, sm_old | sbits) == sm_old) {
+          const unsigned tm_old = *reinterpret_cast<volatile unsigned*>(&sm->tmem_mask);
+          int t0 = -1;
+          if (tmem_units <= third_t && ((tm_old >> (worker * third_t)) & (unsigned)unit_bits(tmem_units)) == 0u) t0 = worker * third_t;
+          else t0 = find_free((unsigned long long)tm_old, tmem_units, sm->n_tmem_units);
+          const unsigned tbits = (unsigned)(unit_bits(tmem_units) << (t0 < 0 ? 0 : t0));
+          if (t0 >= 0 && (tmem_units == 0 || atomicCAS(&sm->tmem_mask, tm_old, tm_old | tbits) == tm_old)) {
+            slot->smem_unit0 = s0; slot->smem_units = units; slot->tmem_unit0 = t0; slot->tmem_units = tmem_units;
+            ok = true;
+            break;
+          }
+          if (units) atomicAnd(&sm->smem_mask, ~sbits);   // no tensor memory yet: give the shared memory back
+        }
+      }
+      if (spin == 0)        // waiting for room
+        *reinterpret_cast<volatile unsigned*>(&sm->room_wait) =
+            (unsigned)need_units | ((unsigned)tmem_units << 8) | ((unsigned)(worker + 1) << 16);
+      __nanosleep(100);
+      if ((spin & 255u) == 255u && (gtimer() > lim || ld_volatile_u32(&ctl->error) != 0u)) break;
+    }
+    if ((*reinterpret_cast<volatile unsigned*>(&sm->room_wait) >> 16) == (unsigned)(worker + 1))
+      *reinterpret_cast<volatile unsigned*>(&sm->room_wait) = 0u;
+    if (job.promised_s | job.promised_t) {     // the claim warp's promise of room is settled either way
+      atomicSub(&sm->smem_promised, job.promised_s); atomicSub(&sm->tmem_promised, job.promised_t);
+    }
+    if (!ok) set_error(ctx, DEV_ERR_IDLE_LIMIT, 0x2000u + (unsigned)blockIdx.x);
+    tc.smem = slab + (size_t)slot->smem_unit0 * SMEM_UNIT;
+    tc.smem_bytes = slot->smem_units * SMEM_UNIT;
+    tc.tmem = sm->tmem_base + (unsigned)slot->tmem_unit0 * TMEM_UNIT;
+  }
+  if (ok && (int)job.tile + 1 == job.desc.n_tiles) {   // the node's last tile: its successors may be queued
+    while (slot->start_state != 0 && gtimer() < lim) __nanosleep(20);
+    slot->start_inst = job.inst; slot->start_node = job.node;
+    __threadfence_block();
+    slot->start_state = 1;
+    bell_ring(&sm->bell_retire);
+  }
+  slot->verdict = ok ? 1 : 2;
+  job.early = early;
+  tc.slot_base = job.slot_base;
+  tc.inputs = ctx.input_ptrs + (size_t)job.inst * N_FRAME_INPUTS;
+  tc.amap_base = ctx.n_weight_tmaps + (int)job.inst * ctx.n_act_tmaps;
+  tc.deadline = lim;
+  tc.wait_word = early ? ctx.dep_word + (size_t)job.inst * ctx.n_nodes + job.node : nullptr;
+  tc.wait_gen = job.gen;
+  tc.t_start = &slot->t_start;
 }
 
 // ------------------------------------------------------------------ the persistent co-scheduling kernel
@@ -684,8 +797,11 @@ __global__ void __launch_bounds__(MAX_WORKERS* WORKER_THREADS + DISPATCH_THREADS
     for (int w = 0; w < MAX_WORKERS; ++w) {
       sm->slot[w].held_tail = 0; sm->slot[w].held_head = 0; sm->slot[w].leave = 0; sm->slot[w].done_state = 0;
       sm->slot[w].prio_tail = 0; sm->slot[w].prio_head = 0; sm->slot[w].t_busy = 0; sm->slot[w].start_state = 0;
-      sm->slot[w].turn = 0; sm->slot[w].bell_parity = 0;
-      sm->slot[w].busy = 0;
+      sm->slot[w].bell_parity = 0; sm->slot[w].busy = 0; sm->slot[w].primed = 0; sm->slot[w].room_wait = &sm->room_wait;
+      TileCtx& tc = sm->tc[w];                           // what never changes
+      tc.arena = ctx.arena; tc.ctl = smem_raw + SM_STATE_BASE + w * SM_CTL_BYTES; tc.bar_id = w + 1; tc.error = &ctx.control->error;
+      tc.tmaps = ctx.tmaps; tc.n_weight_tmaps = ctx.n_weight_tmaps; tc.n_act_tmaps = ctx.n_act_tmaps;
+      tc.slot = &sm->slot[w]; tc.drop_loads = 0;
     }
   }
   __syncthreads();
@@ -693,8 +809,6 @@ __global__ void __launch_bounds__(MAX_WORKERS* WORKER_THREADS + DISPATCH_THREADS
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  Control* ctl = ctx.control;
-
   if (is_dispatcher) {
     if (threadIdx.x < n_workers * WORKER_THREADS + 32) claim_loop(ctx, sm, n_workers);
     else retire_loop(ctx, sm, n_workers);
@@ -706,158 +820,21 @@ __global__ void __launch_bounds__(MAX_WORKERS* WORKER_THREADS + DISPATCH_THREADS
       asm volatile("mov.u32 %0, %%tid.x;" : "=r"(tid));
       const int worker = (int)tid / WORKER_THREADS, wt = (int)tid % WORKER_THREADS, bar_id = worker + 1;
       WorkerSlot* slot = sm->slot + worker;
-      if (wt == 0) {
-        const int turn = slot->turn ^ 1;
-        uint32_t bell_parity = slot->bell_parity;
-        // take the tile the claim warp holds for this worker, then give it its exact memory need
-        int st;
-        unsigned naps = 0;
-        for (;;) {
-          if (slot->prio_tail != slot->prio_head) { st = 3; break; }
-          if (slot->held_tail != slot->held_head) { st = 1; break; }
-          if (slot->leave) { st = 2; break; }
-          if (naps < 8) __nanosleep(20);                               // a claimed tile is usually a moment away
-          else bell_wait(&sm->bell_worker[worker], bell_parity, 2000u);
-          ++naps;
-        }
-        WorkerTile& cur = sm->cur[worker][turn];
-        if (st == 1 || st == 3) {
-          cur = st == 3 ? slot->prio : slot->held[slot->held_head % HELD_DEPTH];
-          slot->t_busy = gtimer();
-          sm->cur_cls[worker] = cur.cls;
-          slot->busy = 1;
-          __threadfence_block();
-          if (st == 3) slot->prio_head = slot->prio_head + 1;
-          else slot->held_head = slot->held_head + 1;   // the claim warp may refill the slot
-          bell_ring(&sm->bell_claim);
-          const uint64_t lim = gtimer() + ctx.wait_limit_ns;
-          bool ok = false;
-          if (cur.early) {
-            // A tile taken before its node's release may hold memory while it waits only where no tile taken earlier can
-            // still need some, that is, where it is the only one this SM has taken.  Elsewhere it waits empty-handed.
-            int taken = 0;
-            for (int k = 0; k < N_CLASSES; ++k) taken += *reinterpret_cast<volatile int*>(&sm->pick.cta_count[k]);
-            if (taken != 1) {
-              TileCtx wc;
-              wc.wait_word = ctx.dep_word + (size_t)cur.inst * ctx.n_nodes + cur.node;
-              wc.wait_gen = release_count(ctx, cur.inst);
-              wc.t_start = &cur.t1;
-              wc.deadline = lim; wc.error = &ctl->error;
-              wait_release(wc);
-              cur.early = 0;
-            }
-          }
-          const int need_units = cur.smem_units;
-          int deep_units = 0;
-          if (sm->outstanding <= 2 * (int)gridDim.x) {
-            // Few tiles on the whole GPU: a GEMM tile takes the pipeline depth its K has use for, up to its share of the
-            // SM.  A k-block then costs its share of many loads in flight instead of half or a quarter of a round trip.
-            const int third = sm->n_smem_units / MAX_WORKERS;
-            const int share = sm->outstanding <= (int)gridDim.x / 2 ? sm->n_smem_units : (sm->outstanding <= (int)gridDim.x ? 2 * third : sm->n_smem_units / 2);
-            deep_units = min((__ldg(&ctx.nodes[cur.node].smem_deep) + SMEM_UNIT - 1) / SMEM_UNIT, share);
-          }
-          for (unsigned spin = 0;; ++spin) {
-            cur.smem_units = need_units;
-            const unsigned long long sm_old = *reinterpret_cast<volatile unsigned long long*>(&sm->smem_mask);
-            // every worker has a home region (a third of the slab, a third of the columns): a tile that fits it goes
-            // there whenever it is free, so tiles of the common shapes never fragment the slab; larger tiles and a
-            // home occupied by one of them fall back to the first free run
-            const int home_s = worker * (sm->n_smem_units / n_workers), home_t = worker * (sm->n_tmem_units / n_workers);
-            int s0 = -1;
-            if (deep_units > need_units && (s0 = find_free(sm_old, deep_units, sm->n_smem_units)) >= 0) cur.smem_units = deep_units;
-            else if (cur.smem_units <= sm->n_smem_units / n_workers && ((sm_old >> home_s) & unit_bits(cur.smem_units)) == 0ull) s0 = home_s;
-            else s0 = find_free(sm_old, cur.smem_units, sm->n_smem_units);
-            if (s0 >= 0) {
-              const unsigned long long sbits = unit_bits(cur.smem_units) << s0;
-              if (cur.smem_units == 0 || atomicCAS(&sm->smem_mask, sm_old, sm_old | sbits) == sm_old) {
-                const unsigned tm_old = *reinterpret_cast<volatile unsigned*>(&sm->tmem_mask);
-                int t0 = -1;
-                if (cur.tmem_units <= sm->n_tmem_units / n_workers && ((tm_old >> home_t) & (unsigned)unit_bits(cur.tmem_units)) == 0u) t0 = home_t;
-                else t0 = find_free((unsigned long long)tm_old, cur.tmem_units, sm->n_tmem_units);
-                const unsigned tbits = (unsigned)(unit_bits(cur.tmem_units) << (t0 < 0 ? 0 : t0));
-                if (t0 >= 0 && (cur.tmem_units == 0 || atomicCAS(&sm->tmem_mask, tm_old, tm_old | tbits) == tm_old)) {
-                  cur.smem_unit0 = s0; cur.tmem_unit0 = t0;
-                  ok = true;
-                  break;
-                }
-                if (cur.smem_units) atomicAnd(&sm->smem_mask, ~sbits);   // no tensor memory yet: give the shared memory back
-              }
-            }
-            if (spin == 0)        // waiting for room
-              *reinterpret_cast<volatile unsigned*>(&sm->room_wait) =
-                  (unsigned)need_units | ((unsigned)cur.tmem_units << 8) | ((unsigned)(worker + 1) << 16);
-            __nanosleep(100);
-            if ((spin & 255u) == 255u && (gtimer() > lim || ld_volatile_u32(&ctl->error) != 0u)) break;
-          }
-          if ((*reinterpret_cast<volatile unsigned*>(&sm->room_wait) >> 16) == (unsigned)(worker + 1))
-            *reinterpret_cast<volatile unsigned*>(&sm->room_wait) = 0u;
-          if (cur.succ_begin | cur.succ_count) {     // the claim warp's promise of room is settled either way
-            atomicSub(&sm->smem_promised, cur.succ_begin); atomicSub(&sm->tmem_promised, cur.succ_count);
-          }
-          if (!ok) set_error(ctx, DEV_ERR_IDLE_LIMIT, 0x2000u + (unsigned)blockIdx.x);
-          if (ok && (int)cur.tile + 1 == __ldg(&ctx.nodes[cur.node].n_tiles)) {   // the node's last tile: its successors may be queued
-            while (slot->start_state != 0 && gtimer() < lim) __nanosleep(20);
-            slot->start_inst = cur.inst; slot->start_node = cur.node;
-            __threadfence_block();
-            slot->start_state = 1;
-            bell_ring(&sm->bell_retire);
-          }
-          cur.t0 = ok ? 1 : 2;              // 1 run, 2 skip (error), 0 leave
-          TileCtx& tc = sm->tc[worker];
-          tc.arena = ctx.arena;
-          tc.slot_base = __ldg(ctx.slot_base + cur.inst);
-          tc.smem = slab + (size_t)cur.smem_unit0 * SMEM_UNIT;
-          tc.smem_bytes = cur.smem_units * SMEM_UNIT;
-          tc.ctl = smem_raw + SM_STATE_BASE + worker * SM_CTL_BYTES;
-          tc.tmem = sm->tmem_base + (unsigned)cur.tmem_unit0 * TMEM_UNIT;
-          tc.bar_id = bar_id;
-          tc.error = &ctl->error;
-          tc.tmaps = ctx.tmaps;
-          tc.inputs = ctx.input_ptrs + (size_t)cur.inst * N_FRAME_INPUTS;
-          tc.amap_base = ctx.n_weight_tmaps + (int)cur.inst * ctx.n_act_tmaps;
-          tc.drop_loads = 0;
-          tc.deadline = gtimer() + ctx.wait_limit_ns;
-          tc.wait_word = nullptr;
-          if (cur.early) {
-            tc.wait_word = ctx.dep_word + (size_t)cur.inst * ctx.n_nodes + cur.node;
-            tc.wait_gen = release_count(ctx, cur.inst);
-            tc.t_start = &cur.t1;
-          }
-        } else {
-          cur.t0 = 0;
-        }
-        slot->turn = turn;
-        slot->bell_parity = bell_parity;
-      }
-      if (wt < 32) {
-        __syncwarp();
-        const WorkerTile& cmd = sm->cur[worker][slot->turn];
-        if (cmd.t0 != 0 && wt < (int)(sizeof(NodeDesc) / 16))
-          reinterpret_cast<int4*>(sm->node + worker)[wt] = __ldg(reinterpret_cast<const int4*>(ctx.nodes + cmd.node) + wt);
-      }
+      if (wt == 0) take_tile(ctx, sm, slot, slab, worker, n_workers);
       asm volatile("bar.sync %0, %1;" ::"r"(bar_id), "r"(WORKER_THREADS) : "memory");
-      WorkerTile& cmd = sm->cur[worker][slot->turn];
-      if (cmd.t0 == 0) break;
+      if (slot->verdict == 0) break;
       {
-        const NodeDesc& n = sm->node[worker];
-        const uint32_t inst = cmd.inst;
+        const TileJob& job = slot->job[slot->run];
         const TileCtx& tc = sm->tc[worker];
-        const int n_op = n.op;
-        if (cmd.early && n_op != OP_GEMM) {
+        if (job.early && job.desc.op != OP_GEMM) {
           if (wt == 0) wait_release(tc);
           asm volatile("bar.sync %0, %1;" ::"r"(bar_id), "r"(WORKER_THREADS) : "memory");
         }
-        // the frame id is only needed by the emit tile and by the trace
-        const uint64_t frame = (ctx.trace_capacity != 0 || n_op == OP_EMIT)
-                                   ? *reinterpret_cast<const volatile uint64_t*>(ctx.inst_frame + inst) : 0ull;
-        if (wt == 32) {     // what the retire warp of this SM will need when the tile ends; its successor records come into L1 now
-          cmd.op = n_op;
-          cmd.succ_begin = n.succ_begin; cmd.succ_count = n.succ_count;
-          cmd.frame = frame;
-          if (!cmd.early) cmd.t1 = gtimer();
-          asm volatile("prefetch.global.L1 [%0];" ::"l"(reinterpret_cast<const char*>(ctx.succ + cmd.succ_begin)));
+        if (wt == 32) {     // the retire warp will need the tile's successor records when it ends: into L1 now
+          if (!job.early) slot->t_start = gtimer();
+          asm volatile("prefetch.global.L1 [%0];" ::"l"(reinterpret_cast<const char*>(ctx.succ + job.desc.succ_begin)));
         }
-        if (cmd.t0 == 1) run_tile<false>(ctx, tc, n, (int)cmd.tile, (int)inst, frame);
+        if (slot->verdict == 1) run_tile<false>(ctx, tc, job.desc, (int)job.tile, (int)job.inst, job.frame);
       }
       // Outputs written here by ordinary stores are read by TMA on other SMs.  The proxy fence that must lie between
       // the two in causality order is the consumer's (first statement of its TMA-issuing thread, after the
@@ -865,6 +842,9 @@ __global__ void __launch_bounds__(MAX_WORKERS* WORKER_THREADS + DISPATCH_THREADS
       end_of_tile(ctx, sm, slot);
     }
   }
+  // After a wait that ran out, copies may still be in flight: they land before the block's memory goes.
+  if (ld_volatile_u32(&ctx.control->error) != 0u)
+    for (int i = 0; i < 200; ++i) __nanosleep(1000);
   tc_fence_before();
   __syncthreads();
   if (threadIdx.x < 32) tmem_dealloc(sm->tmem_base, 512);
@@ -899,6 +879,8 @@ __global__ void __launch_bounds__(WORKER_THREADS) vla_node_kernel(DeviceCtx ctx,
   tc.amap_base = ctx.n_weight_tmaps + (inst >= 0 ? inst : 0) * ctx.n_act_tmaps;
   tc.drop_loads = 0;
   tc.wait_word = nullptr;
+  tc.slot = nullptr;
+  tc.cont = 0;
   const uint64_t t0 = gtimer();
   tc.deadline = t0 + ctx.wait_limit_ns;
   const uint64_t frame = inst >= 0 ? ctx.inst_frame[inst] : 0;

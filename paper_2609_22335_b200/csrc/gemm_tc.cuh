@@ -328,6 +328,35 @@ __device__ __forceinline__ void gemm_epilogue(const TileCtx& c, const GemmArgs& 
 
 constexpr int GEMM_W_STAGE_BYTES = GEMM_BM * GEMM_BK * 2;
 
+// The producer lane's look at the worker's next tile (see tile_gemm).  Not while another worker of the SM waits for room (this
+// one would keep its own), and not past a waiting action-head tile, which goes first and needs the memory.
+__device__ __forceinline__ void prime_next(const TileCtx& c, int bt, int S, int s, uint32_t ph, uint32_t acc_ph, uint32_t bar0, uint32_t stage0,
+                                           uint32_t a_bytes, uint32_t stage_bytes) {
+  WorkerSlot* const w = c.slot;
+  if (w->held_tail == w->held_head || w->prio_tail != w->prio_head || *w->room_wait != 0u) return;
+  __threadfence_block();
+  const TileJob& j = w->job[w->held_head & 1u];
+  const GemmArgs& g = j.desc.u.gemm;
+  if (j.desc.op != OP_GEMM || j.early || g.bt != bt || j.smem_units > w->smem_units) return;
+  const int nkb = g.Kp / GEMM_BK, n = min(S, nkb);
+  w->ring_stages = S; w->ring_s = s; w->ring_ph = ph; w->ring_acc = acc_ph ^ 1u; w->ring_n = n;
+  w->primed = 1;
+  const char* tm = reinterpret_cast<const char*>(c.tmaps);
+  const void* wmap = tm + (size_t)g.wmap * 128;
+  const void* amap = tm + (size_t)(c.n_weight_tmaps + (int)j.inst * c.n_act_tmaps + g.amap) * 128;
+  const int r0 = (int)j.tile / g.tiles_t * GEMM_BM, t0 = (int)j.tile % g.tiles_t * bt;
+  asm volatile("fence.proxy.async;" ::: "memory");
+#pragma unroll 1
+  for (int kb = 0; kb < n; ++kb) {
+    const uint32_t bar = bar0 + 8u * (uint32_t)s, dst = stage0 + (uint32_t)s * stage_bytes;
+    mbar_wait(c, bar + 8u * (uint32_t)S, ph ^ 1u);     // (after a wait that ran out the tile only has to end)
+    mbar_expect_tx(bar, stage_bytes);
+    tma_load_2d(dst + a_bytes, wmap, bar, kb * GEMM_BK, r0);
+    tma_load_2d(dst, amap, bar, kb * GEMM_BK, t0);
+    if (++s == S) { s = 0; ph ^= 1u; }
+  }
+}
+
 // What bounds it: with one tile per SM, the issuing lanes (per k-block one barrier test, two loads, four MMAs) and the
 // round trip of a stage; with three, instruction fetch and the L2-to-shared-memory path.  Stage and phase run along instead
 // of being divided out of the k-block index (a runtime division per role cost as much as the four MMAs).
@@ -337,13 +366,19 @@ __device__ __forceinline__ void tile_gemm(const TileCtx& c, const GemmArgs& g, i
   const int nt = min(bt, g.M - t0);
   const int warp = worker_tid() >> 5, lane = worker_tid() & 31;
   const int nkb = g.Kp / GEMM_BK;
-  const int S = gemm_stages_in(c.smem_bytes, bt, g.Kp, g.stages);
   const uint32_t a_bytes = (uint32_t)(bt * GEMM_BK * 2), stage_bytes = a_bytes + GEMM_W_STAGE_BYTES;   // activations, then weights
+  // The operand ring starts afresh, or goes on where the tile before left it (its producer has requested this tile's first
+  // k-blocks already).  s0, ph0: stage and full-barrier parity of the first k-block; pre: k-blocks on their way.
+  int S, s0 = 0, pre;
+  uint32_t ph0 = 0u, acc_ph = 0u;
+  const bool cont = c.cont != 0;
+  if (cont) { S = c.slot->ring_stages; s0 = c.slot->ring_s; ph0 = c.slot->ring_ph; acc_ph = c.slot->ring_acc; pre = c.slot->ring_n; }
+  else { S = gemm_stages_in(c.smem_bytes, bt, g.Kp, g.stages); pre = S; }
 
   const uint32_t bar0 = smem_u32(c.ctl);               // full[S], empty[S], accum (the worker's control block)
   const uint32_t stage0 = smem_u32(c.smem);
   const uint32_t accum_bar = bar0 + 16u * (uint32_t)S;
-  if (warp == 0) {
+  if (warp == 0 && !cont) {
     if (lane <= 2 * S) {                               // (2 S + 1 <= 25 barriers: one lane each)
       mbar_init(bar0 + 8u * lane, 1);
       asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -359,7 +394,7 @@ __device__ __forceinline__ void tile_gemm(const TileCtx& c, const GemmArgs& g, i
   };
   auto load_a = [&](int kb, uint32_t bar, uint32_t dst) { tma_load_2d(dst, amap, bar, kb * GEMM_BK, t0); };
   if (warp == 0) {
-    if (lane == 0 && !c.drop_loads) {                  // the first stages are on their way before anything else happens
+    if (lane == 0 && !c.drop_loads && !cont) {         // the first stages are on their way before anything else happens
       // The weights do not depend on anything: they fill the stages (and, where the tile was taken before its operands
       // exist, the L2 beyond those) while the predecessors still run; the activations follow the release.
 #pragma unroll 1
@@ -413,29 +448,37 @@ __device__ __forceinline__ void tile_gemm(const TileCtx& c, const GemmArgs& g, i
   if (warp == 0) {
     if (lane == 0) {
       // ---------------- TMA producer
-      uint32_t bar = bar0, dst = stage0, ph = 0u;
-      int s = 0;
+      uint32_t ph = ph0;
+      int s = s0 + pre;
+      if (s >= S) { s -= S; ph ^= 1u; }
+      bool go = !c.drop_loads;
 #pragma unroll 1
-      for (int kb = S; kb < nkb && !c.drop_loads; ++kb) {
-        if (!mbar_wait(c, bar + 8u * (uint32_t)S, ph)) break;
+      for (int kb = pre; kb < nkb && go; ++kb) {
+        const uint32_t bar = bar0 + 8u * (uint32_t)s, dst = stage0 + (uint32_t)s * stage_bytes;
+        if (!(go = mbar_wait(c, bar + 8u * (uint32_t)S, ph ^ 1u))) break;
         load_w(kb, bar, dst);
         load_a(kb, bar, dst);
-        bar += 8u; dst += stage_bytes;
-        if (++s == S) { s = 0; bar = bar0; dst = stage0; ph ^= 1u; }
+        if (++s == S) { s = 0; ph ^= 1u; }
       }
+      // While this tile's last MMAs and its epilogue run, the stages would stand empty: if the tile this worker runs next is
+      // already here and has the same shape, its first k-blocks go into them now.  It then keeps this tile's memory and
+      // barriers.  (Operand loads cover about half a worker's time otherwise, and the L2-to-shared-memory path is what
+      // three workers share.)
+      if (go && c.slot) prime_next(c, bt, S, s, ph, acc_ph, bar0, stage0, a_bytes, stage_bytes);
     }
     __syncwarp();
   } else if (warp == 1) {
     // ---------------- MMA issuer (the whole warp walks the loop, one elected lane issues)
     const uint32_t idesc = umma_idesc_bf16(GEMM_BM);
     const uint64_t desc0 = umma_desc_sw128(stage0);
-    uint32_t bar = bar0, ph = 0u, off = 0u;
-    int s = 0;
+    uint32_t ph = ph0;
+    int s = s0;
 #pragma unroll 1
     for (int kb = 0; kb < nkb; ++kb) {
+      const uint32_t bar = bar0 + 8u * (uint32_t)s;
       if (!mbar_wait(c, bar, ph)) break;
       tc_fence_after();
-      const uint64_t ad = desc0 + off, wd = ad + (a_bytes >> 4);
+      const uint64_t ad = desc0 + (uint32_t)s * (stage_bytes >> 4), wd = ad + (a_bytes >> 4);
       if (elect_one()) {
 #pragma unroll
         for (int k = 0; k < GEMM_BK / 16; ++k)
@@ -444,18 +487,17 @@ __device__ __forceinline__ void tile_gemm(const TileCtx& c, const GemmArgs& g, i
         if (kb == nkb - 1) umma_commit(accum_bar);   // accumulators complete
       }
       __syncwarp();
-      bar += 8u; off += stage_bytes >> 4;
-      if (++s == S) { s = 0; bar = bar0; off = 0u; ph ^= 1u; }
+      if (++s == S) { s = 0; ph ^= 1u; }
     }
   }
 
-  const bool ready = mbar_wait(c, accum_bar, 0u);
+  const bool ready = mbar_wait(c, accum_bar, acc_ph);
   __syncwarp();
   tc_fence_after();
   if (ready && warp_live) gemm_epilogue(c, g, my_tmem, tok, worker_tid() < nt, r0, rs, under, ft);
   tc_fence_before();
   worker_sync(c);
-  if (worker_tid() <= 2 * S) mbar_inval(bar0 + 8u * worker_tid());
+  if (!(c.slot && c.slot->primed) && worker_tid() <= 2 * S) mbar_inval(bar0 + 8u * worker_tid());
 }
 
 }  // namespace vla

@@ -70,6 +70,8 @@ __device__ __forceinline__ TileCtx op_tile_ctx(char* smem, char* ctl, uint32_t t
   tc.smem = smem;
   tc.smem_bytes = 0;
   tc.wait_word = nullptr;
+  tc.slot = nullptr;
+  tc.cont = 0;
   tc.ctl = ctl;
   tc.tmem = tmem;
   tc.bar_id = 1;

@@ -12,6 +12,53 @@
 
 namespace vla {
 
+// A claimed tile with everything its worker needs to start it, put together by the claim warp while the worker still runs
+// the tile before.
+struct TileJob {
+  uint32_t inst, node, tile;
+  int cls, smem_units, tmem_units;
+  int early;                     // queued before its node's release ...
+  unsigned gen;                  // ... which brings the node's release count to this
+  int promised_s, promised_t;    // room promised to the tile when it was claimed
+  uint64_t frame, slot_base;
+  alignas(16) NodeDesc desc;
+};
+constexpr int N_JOBS = 4;        // held tiles use jobs 0 and 1 in turn, priority tiles 2 and 3: one running, one waiting
+
+// A finished tile on its way to the retire warp.
+struct DoneTile {
+  uint32_t inst, node, tile;
+  int cls, succ_begin, succ_count, op;
+  uint64_t t0, t1, frame;
+};
+
+// Mailboxes between one worker group and the SM's service warps, and what the worker keeps from one tile to the next (all in
+// shared memory).
+struct WorkerSlot {
+  volatile unsigned held_tail;   // claimed tiles pushed by the claim warp (single producer)
+  volatile unsigned held_head;   // claimed tiles taken by the worker (single consumer)
+  volatile unsigned prio_tail, prio_head;   // one-deep slot for an action-head tile that goes ahead of the held VLM tiles
+  volatile int leave;            // claim warp -> worker: go home
+  volatile int done_state;       // 0 empty, 1 finished tile posted for the retire warp
+  volatile int busy;             // the worker is running a tile (set and cleared by the worker)
+  volatile int cls;              // class of the running tile
+  volatile unsigned long long t_busy;       // when the running tile was taken (worker), for the claim warp's estimate of its end
+  volatile int start_state;      // 1: the worker took the last tile of (start_inst, start_node): its successors may be queued early
+  uint32_t start_inst, start_node;
+  uint32_t bell_parity;
+  int run;                       // job of the running tile
+  int verdict;                   // 1 run, 2 skip (error), 0 leave
+  int smem_unit0, smem_units, tmem_unit0, tmem_units;      // what the running tile occupies
+  uint64_t t_start, t_wait;                                // (t_wait: end of a wait for the release without memory, not kept)
+  // GEMM operand ring carried over to the next tile: it is the held one, its first loads are in flight (see tile_gemm)
+  volatile int primed;
+  int ring_stages, ring_s, ring_n;          // stages; the next tile's first stage; its k-blocks already requested
+  uint32_t ring_ph, ring_acc;               // parity of that stage's full barrier; of the accumulator barrier
+  const volatile unsigned* room_wait;       // the SM's note of a worker waiting for room
+  DoneTile done;
+  TileJob job[N_JOBS];
+};
+
 // What a tile body needs to know beside its node's arguments.  The persistent kernel keeps one per worker in shared memory:
 // the bodies have use for every register, and values that are the same in all threads are read from there when needed.
 struct TileCtx {
@@ -28,9 +75,12 @@ struct TileCtx {
   const uint64_t* inputs;  // this frame slot's input pointer table
   const void* tmaps;    // tensor-map table (128 bytes per entry)
   int amap_base;        // index of this frame slot's first activation map
+  int n_weight_tmaps, n_act_tmaps;      // weight maps; activation maps per frame slot
   const unsigned long long* wait_word;   // not null: the tile was taken early and waits for its node's release, the moment the
   unsigned wait_gen;                     // release count of this word (bits 32..62) equals wait_gen; GEMM tiles fetch weights meanwhile
   uint64_t* t_start;                     // where the time of that moment goes
+  WorkerSlot* slot;     // the persistent kernel's worker, null elsewhere
+  int cont;             // this tile's operand ring was primed by the tile before
   int drop_loads;       // test hook of the stand-alone operators: the TMA producer issues nothing, so the consumers'
                         // bounded waits run out (0 everywhere else)
 };
