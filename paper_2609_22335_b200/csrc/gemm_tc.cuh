@@ -141,12 +141,14 @@ __device__ __forceinline__ bool elect_one() {
 }
 
 // ------------------------------------------------------------------ epilogue
-// Straight from tensor memory to global memory, sixteen columns at a time; nothing is staged.  A thread owns one token, so
-// its row scale, its sum of squares, gate and up values, rotary pairs and sixteen-byte stores all lie in its own registers.
-// A lone warp per scheduler pays for instructions (one every three or four cycles) and above all for branches (about 30
-// cycles each, taken or skipped over): the five common kinds of result have straight loops of their own, everything else
-// goes through one general loop.  (With every kind unrolled for every activation the kernel had 160 KB of epilogues and 30 %
-// of its instruction fetches missed the cache; with the general loop alone a chunk cost 600 cycles.)
+// Straight from tensor memory to global memory; nothing is staged.  The accumulators are read in the 16x256b fragment layout
+// (a quad of lanes per token, two columns of every eight per lane), and the weight rows were reordered at load so that a
+// lane's eight columns of a 32-column group are eight consecutive features: a quad writes a whole 128-byte line of fp32 (or
+// 64 bytes of bf16), eight lines per instruction.  With a token per lane -- 32 lines per instruction -- the load/store unit
+// was what three workers of an SM waited for (28 cycles a store; epilogues and residual rows cost 31 % of a full-load step).
+// Gate and up values, rotary pairs and a token's partial sum of squares still meet in one lane or quad.
+// A lone warp per scheduler pays for every branch (about 30 cycles), so the common kinds of result have straight loops of
+// their own and everything else goes through one general loop; more variants than that and the instruction cache pays.
 constexpr int EPI = 16;
 
 template <int ACT, int N>
@@ -163,24 +165,24 @@ __device__ __forceinline__ void put16(unsigned short* p, const float* v) {
   for (int j = 0; j < EPI; j += 8)
     *reinterpret_cast<uint4*>(p + j) = make_uint4(pack_bf16(v[j], v[j + 1]), pack_bf16(v[j + 2], v[j + 3]), pack_bf16(v[j + 4], v[j + 5]), pack_bf16(v[j + 6], v[j + 7]));
 }
-// v[j] += scale * p[j], j < n (n = EPI: four 16-byte loads, else element by element)
-__device__ __forceinline__ void add_row(float* v, const float* p, int n, float scale) {
-  if (n == EPI) {
-#pragma unroll
-    for (int j = 0; j < EPI; j += 4) {
-      const float4 t = __ldcg(reinterpret_cast<const float4*>(p + j));
-      v[j] = fmaf(scale, t.x, v[j]); v[j + 1] = fmaf(scale, t.y, v[j + 1]);
-      v[j + 2] = fmaf(scale, t.z, v[j + 2]); v[j + 3] = fmaf(scale, t.w, v[j + 3]);
-    }
-  } else {
-#pragma unroll
-    for (int j = 0; j < EPI; ++j)
-      if (j < n) v[j] = fmaf(scale, ld_act(p + j), v[j]);
-  }
+// One 16-lane half of a warp's tensor memory x 32 columns: v[4 b + 2 r + e] = token (lane / 4) + 8 r, column 8 b + 2 (lane % 4) + e.
+__device__ __forceinline__ void tmem_ld_frag(uint32_t taddr, uint32_t* r) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.16x256b.x4.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr)
+      : "memory");
 }
-
-// Calls body(c0, v) for the accumulator columns [lo, hi) of this thread's token, scaled by rs; the next chunk is on its way
-// from tensor memory meanwhile.
+__device__ __forceinline__ void tmem_st_frag(uint32_t taddr, const float* v) {
+  asm volatile(
+      "tcgen05.st.sync.aligned.16x256b.x4.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};"
+      ::"r"(taddr), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7]), "f"(v[8]), "f"(v[9]),
+        "f"(v[10]), "f"(v[11]), "f"(v[12]), "f"(v[13]), "f"(v[14]), "f"(v[15])
+      : "memory");
+}
+// Calls body(c0, v) for the accumulator columns [lo, hi) of this thread's token (one TMEM lane), scaled by rs; the next
+// chunk is on its way from tensor memory meanwhile.
 template <typename F>
 __device__ __forceinline__ void epi_chunks(uint32_t tmem, int lo, int hi, float rs, F body) {
   if (lo >= hi) return;
@@ -197,133 +199,252 @@ __device__ __forceinline__ void epi_chunks(uint32_t tmem, int lo, int hi, float 
   }
   tmem_ld_wait();
 }
+// Calls body(c0, v) for 32-column groups [0, cols) of one half, v in the order of tmem_ld_frag, the two tokens scaled.
+template <typename F>
+__device__ __forceinline__ void epi_frags(uint32_t tmem, int cols, float ra, float rb, F body) {
+  uint32_t nx[EPI];
+  tmem_ld_frag(tmem, nx);
+#pragma unroll 1
+  for (int c0 = 0; c0 < cols; c0 += 32) {
+    float v[EPI];
+    tmem_ld_wait();
+#pragma unroll
+    for (int j = 0; j < EPI; ++j) v[j] = __uint_as_float(nx[j]) * ((j & 2) ? rb : ra);
+    tmem_ld_frag(tmem + (uint32_t)(c0 + 32 < cols ? c0 + 32 : c0), nx);
+    body(c0, v);
+  }
+  tmem_ld_wait();
+}
+__device__ __forceinline__ void st_row8(float* p, const float* v) {     // v: one token's values of a fragment, at 0, 1, 4, 5, 8, 9, 12, 13
+  asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
+               ::"l"(p), "f"(v[0]), "f"(v[1]), "f"(v[4]), "f"(v[5]), "f"(v[8]), "f"(v[9]), "f"(v[12]), "f"(v[13]) : "memory");
+}
+__device__ __forceinline__ void st_row8(unsigned short* p, const float* v) {
+  *reinterpret_cast<uint4*>(p) = make_uint4(pack_bf16(v[0], v[1]), pack_bf16(v[4], v[5]), pack_bf16(v[8], v[9]), pack_bf16(v[12], v[13]));
+}
+// (cos, sin) per pair: the lane's four pairs of one token
+__device__ __forceinline__ void rotate8(float* v, const float* tab) {
+  const float4 lo = __ldg(reinterpret_cast<const float4*>(tab)), hi = __ldg(reinterpret_cast<const float4*>(tab) + 1);
+  const float cs[4] = {lo.x, lo.z, hi.x, hi.z}, sn[4] = {lo.y, lo.w, hi.y, hi.w};
+#pragma unroll
+  for (int b = 0; b < 4; ++b) {
+    const float x = v[4 * b], y = v[4 * b + 1];
+    v[4 * b] = fmaf(x, cs[b], -y * sn[b]); v[4 * b + 1] = fmaf(y, cs[b], x * sn[b]);
+  }
+}
+
+// What a straight epilogue needs beside the tile's place: `live` tokens of this warp exist, `tok` is the warp's first token.
+struct EpiPlace { uint32_t tmem; int tok, live, lane, r0, cols; float rs; };
+
+// Walks the two halves of the warp: fn(row, tmem, ra, rb) with this lane's tokens `row` and `row` + 8 of the warp.
+template <typename F>
+__device__ __forceinline__ void epi_halves(const EpiPlace& e, F fn) {
+#pragma unroll 1
+  for (int h = 0; h < 2 && 16 * h < e.live; ++h) {
+    const int row = 16 * h + (e.lane >> 2);
+    fn(row, e.tmem + ((uint32_t)(16 * h) << 16), __shfl_sync(0xffffffffu, e.rs, row), __shfl_sync(0xffffffffu, e.rs, row + 8));
+  }
+}
 template <int ACT>
-__device__ __forceinline__ void epi_gated(uint32_t tmem, int cols, float rs, float c_acc, unsigned short* out, bool live) {
-  epi_chunks(tmem, 0, cols, rs, [&](int c0, float* v) {      // columns 2i, 2i + 1: gate and up value of output feature i
-    float o[EPI / 2];
+__device__ __forceinline__ void epi_gated(const EpiPlace& e, const GemmArgs& g, unsigned short* out16) {
+  const int q = e.lane & 3;
+  const float c_acc = g.c_acc;
+  epi_halves(e, [&](int row, uint32_t tmem, float ra, float rb) {
+    unsigned short* pa = out16 + (size_t)(e.tok + row) * g.ldo16 + e.r0 / 2 + 4 * q;
+    unsigned short* pb = pa + (size_t)8 * g.ldo16;
+    epi_frags(tmem, e.cols, ra, rb, [&](int c0, float* v) {       // a lane's columns 2 i, 2 i + 1: gate and up value of one feature
+      float o[8];
 #pragma unroll
-    for (int j = 0; j < EPI / 2; ++j) o[j] = v[2 * j];
-    activate<ACT, EPI / 2>(o);
+      for (int b = 0; b < 4; ++b) { o[b] = v[4 * b]; o[4 + b] = v[4 * b + 2]; }
+      activate<ACT, 8>(o);
 #pragma unroll
-    for (int j = 0; j < EPI / 2; ++j) o[j] *= v[2 * j + 1] * c_acc;
-    if (live) *reinterpret_cast<uint4*>(out + (c0 >> 1)) = make_uint4(pack_bf16(o[0], o[1]), pack_bf16(o[2], o[3]), pack_bf16(o[4], o[5]), pack_bf16(o[6], o[7]));
+      for (int b = 0; b < 4; ++b) { o[b] *= v[4 * b + 1] * c_acc; o[4 + b] *= v[4 * b + 3] * c_acc; }
+      const bool fok = c0 + 8 * q < e.cols;
+      if (fok && row < e.live) *reinterpret_cast<uint2*>(pa + c0 / 2) = make_uint2(pack_bf16(o[0], o[1]), pack_bf16(o[2], o[3]));
+      if (fok && row + 8 < e.live) *reinterpret_cast<uint2*>(pb + c0 / 2) = make_uint2(pack_bf16(o[4], o[5]), pack_bf16(o[6], o[7]));
+    });
+  });
+}
+template <int ACT, bool ROPE>
+__device__ __forceinline__ void epi_bf16(const EpiPlace& e, const GemmArgs& g, unsigned short* out16, const float* rope) {
+  const int q = e.lane & 3;
+  epi_halves(e, [&](int row, uint32_t tmem, float ra, float rb) {
+    unsigned short* pa = out16 + (size_t)(e.tok + row) * g.ldo16 + e.r0 + 8 * q;
+    unsigned short* pb = pa + (size_t)8 * g.ldo16;
+    const int last = e.live - 1;
+    const float* ta = ROPE ? rope + (size_t)(e.tok + min(row, last)) * g.rope_hd : nullptr;
+    const float* tb = ROPE ? rope + (size_t)(e.tok + min(row + 8, last)) * g.rope_hd : nullptr;
+    epi_frags(tmem, e.cols, ra, rb, [&](int c0, float* v) {
+      activate<ACT, EPI>(v);
+      if (ROPE) {
+        const int i = (e.r0 + c0 + 8 * q) % g.rope_hd;
+        rotate8(v, ta + i);
+        rotate8(v + 2, tb + i);
+      }
+      const bool fok = c0 + 8 * q < e.cols;
+      if (fok && row < e.live) st_row8(pa + c0, v);
+      if (fok && row + 8 < e.live) st_row8(pb + c0, v + 2);
+    });
+  });
+}
+// fp32 rows with, optionally, their bf16 mirror and the tile's share of each token's sum of squares (residual streams).
+template <bool MIRROR>
+__device__ __forceinline__ void epi_stream(const EpiPlace& e, const GemmArgs& g, float* out32, unsigned short* out16, float* ssq, int ft) {
+  const int q = e.lane & 3;
+  epi_halves(e, [&](int row, uint32_t tmem, float ra, float rb) {
+    float* pa = out32 + (size_t)(e.tok + row) * g.ldo32 + e.r0 + 8 * q;
+    float* pb = pa + (size_t)8 * g.ldo32;
+    unsigned short* ha = MIRROR ? out16 + (size_t)(e.tok + row) * g.ldo16 + e.r0 + 8 * q : nullptr;
+    unsigned short* hb = MIRROR ? ha + (size_t)8 * g.ldo16 : nullptr;
+    float sa = 0.f, sb = 0.f;
+    epi_frags(tmem, e.cols, ra, rb, [&](int c0, float* v) {
+      const bool fok = c0 + 8 * q < e.cols;
+      if (MIRROR && fok) {
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+          sa = fmaf(v[4 * b], v[4 * b], sa); sa = fmaf(v[4 * b + 1], v[4 * b + 1], sa);
+          sb = fmaf(v[4 * b + 2], v[4 * b + 2], sb); sb = fmaf(v[4 * b + 3], v[4 * b + 3], sb);
+        }
+      }
+      if (fok && row < e.live) { st_row8(pa + c0, v); if (MIRROR) st_row8(ha + c0, v); }
+      if (fok && row + 8 < e.live) { st_row8(pb + c0, v + 2); if (MIRROR) st_row8(hb + c0, v + 2); }
+    });
+    if (MIRROR && ssq) {
+      sa += __shfl_xor_sync(0xffffffffu, sa, 1); sb += __shfl_xor_sync(0xffffffffu, sb, 1);
+      sa += __shfl_xor_sync(0xffffffffu, sa, 2); sb += __shfl_xor_sync(0xffffffffu, sb, 2);
+      float* sp = ssq + (size_t)(e.tok + row) * g.ss_out_ld + ft;
+      if (q == 0 && row < e.live) sp[0] = sa;
+      if (q == 0 && row + 8 < e.live) sp[(size_t)8 * g.ss_out_ld] = sb;
+    }
+  });
+}
+// Rows of V^T: a token per lane, so that a warp writes 32 consecutive tokens of a feature.
+__device__ __forceinline__ void epi_vt(const EpiPlace& e, const GemmArgs& g, unsigned short* outT, int split) {
+  unsigned short* const base = outT + e.tok + e.lane;
+  const size_t ld = (size_t)g.ldoT;
+  epi_chunks(e.tmem, split, e.cols, e.rs, [&](int c0, float* v) {
+    unsigned short* op = base + (size_t)(e.r0 + (c0 & ~31) + ((c0 & 16) >> 2) - g.t_col0) * ld;
+    if (e.lane < e.live) {
+#pragma unroll
+      for (int j = 0; j < EPI; ++j) op[(size_t)perm_feature(j) * ld] = f32_to_bf16_bits(v[j]);
+    }
   });
 }
 
-// One token's row of the tile.  `tok` is the token's index in the node (a lane past the last token repeats it, `live` false,
-// and stores nothing), `r0` the tile's first weight row, `rs` the token's row scale, `under` says that the accumulators
-// already hold X.
-__device__ __forceinline__ void gemm_epilogue(const TileCtx& c, const GemmArgs& g, uint32_t tmem, int tok, bool live, int r0, float rs, bool under,
-                                              int ft) {
-  const int act = g.act, N = g.N;
-  const float c_acc = g.c_acc;
+// Anything else -- solver coefficients, norms with addends, odd widths and offsets: a token per lane, element by element.
+__device__ __forceinline__ void epi_general(const TileCtx& c, const GemmArgs& g, const EpiPlace& e, int ft) {
   const GemmPtrs ptrs = gemm_ptrs(c, g);
-  float* const ssq_out = resolve<float>(c, g.ss_out);
-  float* const out32 = ptrs.out32 ? ptrs.out32 + (size_t)tok * g.ldo32 + r0 : nullptr;
-  unsigned short* const out16 = ptrs.out16 ? ptrs.out16 + (size_t)tok * g.ldo16 + (g.dual ? r0 / 2 : r0) : nullptr;
-  const int cols = min(GEMM_BM, (g.dual ? 2 * N : N) - r0);
-  if (g.vec16) {
-    if (g.dual) {
-      if (act == ACT_SILU) epi_gated<ACT_SILU>(tmem, cols, rs, c_acc, out16, live);
-      else if (act == ACT_GELU) epi_gated<ACT_GELU>(tmem, cols, rs, c_acc, out16, live);
-      else epi_gated<ACT_NONE>(tmem, cols, rs, c_acc, out16, live);
-      return;
-    }
-    const bool plain = !ptrs.bias && !ptrs.vec && !ptrs.tab && !ptrs.tab2 && (!ptrs.X || under) && c_acc == 1.0f;
-    if (plain && !ssq_out && !ptrs.out32 && act != ACT_SILU) {            // bf16 only (q|k|v, MLP up, cross projections)
-      int split = cols;                                                     // columns from here on are V features
-      if (ptrs.outT) split = max(0, min(cols, g.t_col0 - r0));
-      if (act == ACT_GELU)
-        epi_chunks(tmem, 0, split, rs, [&](int c0, float* v) { activate<ACT_GELU, EPI>(v); if (live) put16(out16 + c0, v); });
-      else if (g.rope_cols > 0) {       // q and k columns: rotary pairs are neighbours; the table holds (cos, sin) per pair
-        const float* t0 = resolve<const float>(c, g.rope_tab) + (size_t)tok * g.rope_hd;
-        epi_chunks(tmem, 0, split, rs, [&](int c0, float* v) {
-          const float4* t = reinterpret_cast<const float4*>(t0 + (r0 + c0) % g.rope_hd);
-#pragma unroll
-          for (int j = 0; j < EPI; j += 4) {
-            const float4 cs = __ldg(t + (j >> 2));
-            const float x0 = v[j], x1 = v[j + 1], x2 = v[j + 2], x3 = v[j + 3];
-            v[j] = fmaf(x0, cs.x, -x1 * cs.y); v[j + 1] = fmaf(x1, cs.x, x0 * cs.y);
-            v[j + 2] = fmaf(x2, cs.z, -x3 * cs.w); v[j + 3] = fmaf(x3, cs.z, x2 * cs.w);
-          }
-          if (live) put16(out16 + c0, v);
-        });
-      } else
-        epi_chunks(tmem, 0, split, rs, [&](int c0, float* v) { if (live) put16(out16 + c0, v); });
-      if (split < cols) {               // rows of V^T, a warp's tokens side by side
-        unsigned short* const base = ptrs.outT + (ptrdiff_t)(r0 - g.t_col0) * g.ldoT + tok;
-        epi_chunks(tmem, split, cols, rs, [&](int c0, float* v) {
-          unsigned short* op = base + (ptrdiff_t)c0 * g.ldoT;
-          if (live) {
-#pragma unroll
-            for (int j = 0; j < EPI; ++j) { *op = f32_to_bf16_bits(v[j]); op += g.ldoT; }
-          }
-        });
-      }
-      return;
-    }
-    if (plain && act == ACT_NONE && out32 && out16 && ssq_out) {            // residual stream
-      float sq = 0.f;
-      epi_chunks(tmem, 0, cols, rs, [&](int c0, float* v) {
-#pragma unroll
-        for (int j = 0; j < EPI; ++j) sq = fmaf(v[j], v[j], sq);
-        if (live) {
-#pragma unroll
-          for (int j = 0; j < EPI; j += 4) *reinterpret_cast<float4*>(out32 + c0 + j) = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
-          put16(out16 + c0, v);
-        }
-      });
-      if (live) ssq_out[(size_t)tok * g.ss_out_ld + ft] = sq;
-      return;
-    }
-  }
-  // ---- anything else: biases, tables, addends, solver coefficients, odd widths
+  const int N = g.dual ? 2 * g.N : g.N, act = g.act;
+  const int cols = g.perm ? (e.cols + 31) & ~31 : (e.cols + 1) & ~1;     // a reordered last group spreads over all its columns
+  const bool live = e.lane < e.live;
+  const size_t tok = (size_t)(e.tok + min(e.lane, e.live - 1));
+  float* const ssq = resolve<float>(c, g.ss_out);
   float sq = 0.f;
 #pragma unroll 1
-  for (int c0 = 0; c0 < cols; c0 += EPI) {
-    const int f = r0 + c0, n = g.vec16 ? EPI : min(EPI, (g.dual ? 2 * N : N) - f);
-    float v[EPI];
-    tmem_ld16(tmem + (uint32_t)c0, v);
-#pragma unroll
-    for (int j = 0; j < EPI; ++j) v[j] *= rs;
+  for (int c0 = 0; c0 < cols; c0 += 2) {                 // (rolled: few nodes come here, and the code would crowd the others out)
+    const int f = e.r0 + (g.perm ? (c0 & ~31) + perm_feature(c0 & 31) : c0);         // a pair of features
+    uint32_t acc[2];
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x2.b32 {%0, %1}, [%2];" : "=r"(acc[0]), "=r"(acc[1]) : "r"(e.tmem + (uint32_t)c0) : "memory");
+    tmem_ld_wait();
+    float x0 = __uint_as_float(acc[0]) * e.rs, x1 = __uint_as_float(acc[1]) * e.rs;
     if (g.dual) {
-#pragma unroll
-      for (int j = 0; j < EPI / 2; ++j)
-        if (live && 2 * j < n) out16[(c0 >> 1) + j] = f32_to_bf16_bits(apply_act(act, v[2 * j]) * v[2 * j + 1] * c_acc);
+      if (live && f < N) ptrs.out16[tok * g.ldo16 + f / 2] = f32_to_bf16_bits(apply_act(act, x0) * x1 * g.c_acc);
       continue;
     }
-    if (ptrs.bias) add_row(v, ptrs.bias + f, n, 1.0f);
-    if (act == ACT_GELU) activate<ACT_GELU, EPI>(v);
-    else if (act == ACT_SILU) activate<ACT_SILU, EPI>(v);
-#pragma unroll
-    for (int j = 0; j < EPI; ++j) v[j] *= c_acc;
-    if (ptrs.X && !under) add_row(v, ptrs.X + (size_t)tok * g.ldx + f, n, g.c_x);
-    if (ptrs.vec) add_row(v, ptrs.vec + f, n, 1.0f);
-    if (ptrs.tab) add_row(v, ptrs.tab + (size_t)tok * g.ldtab + f, n, 1.0f);
-    if (ptrs.tab2) add_row(v, ptrs.tab2 + (size_t)tok * g.ldtab2 + f, n, 1.0f);
-#pragma unroll
-    for (int j = 0; j < EPI; ++j)
-      if (j < n) sq = fmaf(v[j], v[j], sq);
-    if (!live) continue;
-    if (ptrs.outT && f >= g.t_col0) {
-      unsigned short* op = ptrs.outT + (size_t)(f - g.t_col0) * g.ldoT + tok;
-#pragma unroll
-      for (int j = 0; j < EPI; ++j) { *op = f32_to_bf16_bits(v[j]); op += g.ldoT; }
-    } else if (g.vec16) {
-      if (out32) {
-#pragma unroll
-        for (int j = 0; j < EPI; j += 4) *reinterpret_cast<float4*>(out32 + c0 + j) = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
-      }
-      if (out16) put16(out16 + c0, v);
-    } else {
-#pragma unroll
-      for (int j = 0; j < EPI; ++j) {
-        if (j < n && out32) out32[c0 + j] = v[j];
-        if (j < n && out16) out16[c0 + j] = f32_to_bf16_bits(v[j]);
+    if (f < g.rope_cols) {
+      const float2 cs = __ldg(reinterpret_cast<const float2*>(resolve<const float>(c, g.rope_tab) + tok * g.rope_hd + f % g.rope_hd));
+      const float r = fmaf(x0, cs.x, -x1 * cs.y);
+      x1 = fmaf(x1, cs.x, x0 * cs.y);
+      x0 = r;
+    }
+#pragma unroll 1
+    for (int fk = f; fk < min(f + 2, N); ++fk) {
+      float x = x0;
+      x0 = x1;
+      if (ptrs.bias) x += __ldg(ptrs.bias + fk);
+      x = apply_act(act, x) * g.c_acc;
+      if (ptrs.X) x = fmaf(g.c_x, ld_act(ptrs.X + tok * g.ldx + fk), x);
+      if (ptrs.vec) x += ld_act(ptrs.vec + fk);
+      if (ptrs.tab) x += ld_act(ptrs.tab + tok * g.ldtab + fk);
+      if (ptrs.tab2) x += ld_act(ptrs.tab2 + tok * g.ldtab2 + fk);
+      sq = fmaf(x, x, sq);
+      if (!live) continue;
+      if (ptrs.outT && fk >= g.t_col0) ptrs.outT[(size_t)(fk - g.t_col0) * g.ldoT + tok] = f32_to_bf16_bits(x);
+      else {
+        if (ptrs.out32) ptrs.out32[tok * g.ldo32 + fk] = x;
+        if (ptrs.out16) ptrs.out16[tok * g.ldo16 + fk] = f32_to_bf16_bits(x);
       }
     }
   }
-  if (ssq_out && live) ssq_out[(size_t)tok * g.ss_out_ld + ft] = sq;
+  if (ssq && live) ssq[tok * g.ss_out_ld + ft] = sq;
+}
+
+// This warp's tokens of the tile.  t0: the tile's first token, nt: its tokens, r0: its first weight row, rs: row scale of the
+// token in this lane.
+__device__ __forceinline__ void gemm_epilogue(const TileCtx& c, const GemmArgs& g, uint32_t tmem, int t0, int nt, int warp, int lane, int r0, float rs,
+                                              int ft) {
+  EpiPlace e;
+  e.tmem = tmem; e.tok = t0 + 32 * warp; e.live = nt - 32 * warp; e.lane = lane; e.r0 = r0; e.rs = rs;
+  e.cols = min(GEMM_BM, (g.dual ? 2 * g.N : g.N) - r0);
+  if (!g.fast) { epi_general(c, g, e, ft); return; }
+  unsigned short* const out16 = resolve<unsigned short>(c, g.out16);
+  if (g.dual) {
+    if (g.act == ACT_SILU) epi_gated<ACT_SILU>(e, g, out16);
+    else if (g.act == ACT_GELU) epi_gated<ACT_GELU>(e, g, out16);
+    else epi_gated<ACT_NONE>(e, g, out16);
+  } else if (g.out32 != 0) {
+    if (out16) epi_stream<true>(e, g, resolve<float>(c, g.out32), out16, resolve<float>(c, g.ss_out), ft);
+    else epi_stream<false>(e, g, resolve<float>(c, g.out32), nullptr, nullptr, ft);
+  } else {
+    const int all = e.cols;
+    if (g.outT != 0) e.cols = max(0, min(all, g.t_col0 - r0));              // columns from here on are V features
+    if (e.cols > 0) {
+      if (g.act == ACT_GELU) epi_bf16<ACT_GELU, false>(e, g, out16, nullptr);
+      else if (g.rope_cols > 0) epi_bf16<ACT_NONE, true>(e, g, out16, resolve<const float>(c, g.rope_tab));
+      else epi_bf16<ACT_NONE, false>(e, g, out16, nullptr);
+    }
+    if (e.cols < all) {
+      const int split = e.cols;
+      e.cols = all;
+      epi_vt(e, g, resolve<unsigned short>(c, g.outT), split);
+    }
+  }
+}
+
+// Addends of the tile's tokens into the accumulators (fragment layout; columns past the last feature get zero).
+__device__ __forceinline__ void preload_rows(const TileCtx& c, const GemmArgs& g, uint32_t tmem, int t0, int nt, int warp, int lane, int r0) {
+  const GemmPtrs ptrs = gemm_ptrs(c, g);
+  const int q = lane & 3, cols = min(GEMM_BM, g.N - r0);
+  auto add8 = [](float* v, const float* p) {
+    const float4 a = __ldcg(reinterpret_cast<const float4*>(p)), b = __ldcg(reinterpret_cast<const float4*>(p) + 1);
+    v[0] += a.x; v[1] += a.y; v[4] += a.z; v[5] += a.w; v[8] += b.x; v[9] += b.y; v[12] += b.z; v[13] += b.w;
+  };
+#pragma unroll 1
+  for (int c0 = 0; c0 < cols; c0 += 32) {
+    float v[2][EPI];
+    const int f = r0 + c0 + 8 * q;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+#pragma unroll
+      for (int j = 0; j < EPI; ++j) v[h][j] = 0.f;
+      if (c0 + 8 * q >= cols) continue;
+#pragma unroll
+      for (int r = 0; r < 2; ++r) {
+        const size_t tok = (size_t)(t0 + min(32 * warp + 16 * h + 8 * r + (lane >> 2), nt - 1));
+        float* p = v[h] + 2 * r;
+        if (g.under & 4) add8(p, ptrs.X + tok * g.ldx + f);
+        if (g.under & 27) {
+          if (g.under & 1) add8(p, ptrs.bias + f);
+          if (g.under & 2) add8(p, ptrs.vec + f);
+          if (g.under & 8) add8(p, ptrs.tab + tok * g.ldtab + f);
+          if (g.under & 16) add8(p, ptrs.tab2 + tok * g.ldtab2 + f);
+        }
+      }
+    }
+    tmem_st_frag(tmem + (uint32_t)c0, v[0]);
+    tmem_st_frag(tmem + (16u << 16) + (uint32_t)c0, v[1]);
+  }
+  tmem_st_wait();
 }
 
 constexpr int GEMM_W_STAGE_BYTES = GEMM_BM * GEMM_BK * 2;
@@ -413,31 +534,19 @@ __device__ __forceinline__ void tile_gemm(const TileCtx& c, const GemmArgs& g, i
   }
   if (c.wait_word) worker_sync(c);                     // nobody reads an operand before the release
 
-  const int tok = t0 + min(worker_tid(), nt - 1);      // this thread's token (lanes past the last one repeat it)
   const bool warp_live = warp * 32 < nt;
   const uint32_t my_tmem = c.tmem + ((uint32_t)(warp * 32) << 16);
-  // Residual rows go into the accumulators before the first MMA: their round trip then lies beside that of the first
-  // operand stages, and the epilogue neither reads nor adds anything.
-  const bool under = g.X != 0 && g.vec16 && g.c_acc == 1.0f && g.c_x == 1.0f && g.rs_d == 0 && g.act == ACT_NONE;
+  // What is added to the product goes into the accumulators before the first MMA: its round trip then lies beside that of
+  // the first operand stages, and the epilogue neither reads nor adds anything.
+  const bool under = g.under != 0;
   if (under) {
-    if (warp_live) {
-      const float* x = resolve<const float>(c, g.X) + (size_t)tok * g.ldx + r0;
-      const int cols = min(GEMM_BM, g.N - r0);
-#pragma unroll 1
-      for (int c0 = 0; c0 < cols; c0 += 16) {
-        float v[16];
-#pragma unroll
-        for (int j = 0; j < 16; j += 4) *reinterpret_cast<float4*>(v + j) = __ldcg(reinterpret_cast<const float4*>(x + c0 + j));
-        tmem_st16(my_tmem + (uint32_t)c0, v);
-      }
-      tmem_st_wait();
-    }
+    if (warp_live) preload_rows(c, g, my_tmem, t0, nt, warp, lane, r0);
     tc_fence_before();
   }
   // Folded RMSNorm: the token's row scale from the stream's partial sums of squares, added in a fixed order.
   float rs = 1.0f;
   if (g.rs_d > 0 && warp_live) {
-    const float* sp = resolve<const float>(c, g.ss_in) + (size_t)tok * g.ss_nft;
+    const float* sp = resolve<const float>(c, g.ss_in) + (size_t)(t0 + min(worker_tid(), nt - 1)) * g.ss_nft;
     float ssq = 0.f;
 #pragma unroll 4
     for (int q = 0; q < g.ss_nft; ++q) ssq += ld_act(sp + q);
@@ -494,7 +603,7 @@ __device__ __forceinline__ void tile_gemm(const TileCtx& c, const GemmArgs& g, i
   const bool ready = mbar_wait(c, accum_bar, acc_ph);
   __syncwarp();
   tc_fence_after();
-  if (ready && warp_live) gemm_epilogue(c, g, my_tmem, tok, worker_tid() < nt, r0, rs, under, ft);
+  if (ready && warp_live) gemm_epilogue(c, g, my_tmem, t0, nt, warp, lane, r0, rs, ft);
   tc_fence_before();
   worker_sync(c);
   if (!(c.slot && c.slot->primed) && worker_tid() <= 2 * S) mbar_inval(bar0 + 8u * worker_tid());

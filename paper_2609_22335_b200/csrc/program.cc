@@ -92,7 +92,7 @@ class Builder {
     t.ld = is_bf16 ? pad_to(cols, GEMM_BK) : cols;
     weight_cursor = align_up(weight_cursor, 256);
     t.offset = weight_cursor;
-    weight_cursor += (uint64_t)rows * t.ld * (is_bf16 ? 2 : 4);
+    weight_cursor += (uint64_t)(is_bf16 ? pad_to(rows, 32) : rows) * t.ld * (is_bf16 ? 2 : 4);    // (padding rows stay zero)
     p.dev_tensors.push_back(t);
     p.dev_index[name] = (int)p.dev_tensors.size() - 1;
     return (int)p.dev_tensors.size() - 1;
@@ -276,12 +276,26 @@ class Builder {
     int bt = (int)pad_to((g.M + tiles_t - 1) / tiles_t, 16);
     g.bt = bt; g.tiles_t = tiles_t;
     {
-      // sixteen columns at a time, each a whole 16-byte access at a 16-byte address: rows start at multiples of 256 bytes
-      // (buffers and weights), so pitches and column offsets decide
+      // Straight epilogue: eight features per access (four outputs where gated), 16-byte or larger, rows starting at
+      // multiples of 256 bytes (buffers and weights), so pitches, column offsets and widths decide.
       auto cols_ok = [&](const View& v, int64_t per) { return v.buf < 0 || (ld(v) % per == 0 && v.col0 % per == 0); };
-      g.vec16 = N % (g.dual ? 8 : 16) == 0 && cols_ok(o.X, 4) && cols_ok(o.tabv, 4) && cols_ok(o.out32, 4) && cols_ok(o.out16, 8) &&
-                (!o.tab || o.ldtab % 4 == 0) && (!o.tab2 || o.ldtab2 % 4 == 0) && (o.outT.buf < 0 || o.t_col0 % 16 == 0);
-      if (!g.vec16 && (o.outT.buf >= 0 || o.rope_cols > 0)) p.error = "internal: V^T and rotary columns come in chunks of 16 (" + name + ")";
+      const bool aligned = N % (g.dual ? 4 : 8) == 0 && cols_ok(o.X, 4) && cols_ok(o.tabv, 4) && cols_ok(o.out32, 8) && cols_ok(o.out16, g.dual ? 4 : 8) &&
+                           (!o.tab || o.ldtab % 4 == 0) && (!o.tab2 || o.ldtab2 % 4 == 0) && (o.outT.buf < 0 || (N % 32 == 0 && o.t_col0 % 32 == 0)) &&
+                           o.rope_cols % 32 == 0 && (o.rope_cols == 0 || o.rope_hd % 8 == 0);
+      // A matrix is reordered if its first GEMM allows it; all GEMMs of a matrix have its width.
+      DevTensor& wd = p.dev_tensors[W];
+      if (wd.uses++ == 0) wd.perm = aligned;
+      g.perm = wd.perm;
+
+      const bool adds = g.X || g.vec || g.tab || g.tab2, scaled = g.c_acc != 1.0f || g.c_x != 1.0f;
+      const bool plain_add = o.norm_gain < 0 && !scaled && g.act == ACT_NONE;           // sums may start from the addends
+      if (aligned && !g.dual && (!adds || plain_add) && (!g.bias || o.norm_gain < 0))
+        g.under = (g.bias ? 1 : 0) | (g.vec ? 2 : 0) | (g.X ? 4 : 0) | (g.tab ? 8 : 0) | (g.tab2 ? 16 : 0);
+      const bool all_under = (g.bias ? 1 : 0) + (g.vec ? 2 : 0) + (g.X ? 4 : 0) + (g.tab ? 8 : 0) + (g.tab2 ? 16 : 0) == g.under;
+      g.fast = aligned && g.perm && all_under && !(scaled && !g.dual) &&
+               (g.dual || g.act == ACT_NONE || (g.act == ACT_GELU && !g.out32 && !g.outT && o.rope_cols == 0));
+      if (!g.fast) g.under = 0;
+
     }
     {
       // pipeline depth from the stage size; tensor maps for the operands
@@ -292,7 +306,7 @@ class Builder {
       n.smem_bytes = gemm_smem_bytes(bt, S);
       n.smem_deep = gemm_smem_bytes(bt, std::min(GEMM_MAX_STAGES, g.Kp / GEMM_BK));
       n.tmem_cols = GEMM_BM;
-      g.wmap = weight_map(W, g.dual ? 2 * N : N);
+      g.wmap = weight_map(W, pad_to(g.dual ? 2 * N : N, 32));
       if (g.dual && o.bias >= 0) p.error = "a gated GEMM takes no bias";
       if (g.dual && (o.X.buf >= 0 || o.outT.buf >= 0 || o.out32.buf >= 0 || o.tab || o.tab2 || o.vec))
         p.error = "internal: a gated GEMM writes bf16 only (" + name + ")";

@@ -26,6 +26,8 @@ struct SourceTensor {
 struct DevTensor {
   std::string name;
   int64_t rows, cols, ld;   // ld = padded row length in elements
+  int uses = 0;             // GEMMs of the program that read it
+  bool perm = false;        // rows reordered in groups of 32 once everything is loaded (GEMM weights, see perm_feature)
   bool is_bf16;             // matrices bf16, gains/position tables fp32
   uint64_t offset;          // arena byte offset
   int tmap = -1;            // tensor-map index for GEMM weights

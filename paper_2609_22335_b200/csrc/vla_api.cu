@@ -194,6 +194,18 @@ __global__ void vla_fold_gain_kernel(unsigned short* w, int64_t rows, int cols, 
   }
 }
 
+// Reorders the rows of a GEMM weight matrix in groups of 32 (see perm_feature): a thread owns eight columns of a group.
+__global__ void vla_permute_rows_kernel(uint4* w, int64_t groups, int64_t ld8) {
+  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < groups * ld8; e += (int64_t)gridDim.x * blockDim.x) {
+    uint4* p = w + e / ld8 * 32 * ld8 + e % ld8;
+    uint4 r[32];
+#pragma unroll
+    for (int i = 0; i < 32; ++i) r[i] = p[i * ld8];
+#pragma unroll
+    for (int i = 0; i < 32; ++i) p[i * ld8] = r[perm_feature(i)];
+  }
+}
+
 // (Re)launch the persistent kernel if it is not running and frames are waiting.
 int ensure_persistent(vla_ctx* c) {
   if (c->pending_frames == 0 || c->hold_launches) return VLA_OK;
@@ -544,6 +556,11 @@ int vla_load_weights(vla_ctx* c, const vla_tensor* tensors, size_t n, int32_t fi
                                                    reinterpret_cast<const float*>(c->arena + p.off_weights + gt.offset));
       CU(cudaGetLastError());
     }
+  }
+  for (const DevTensor& t : p.dev_tensors) {
+    if (!t.perm) continue;
+    vla_permute_rows_kernel<<<592, 128, 0, c->sa>>>(reinterpret_cast<uint4*>(c->arena + p.off_weights + t.offset), (t.rows + 31) / 32, t.ld / 8);
+    CU(cudaGetLastError());
   }
   // one-off constants (time-embedding MLP, adaLN modulation) on the GPU, serially
   const NodeDesc* init_dev = at<NodeDesc>(c, p.off_init_nodes);

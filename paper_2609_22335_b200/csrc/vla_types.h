@@ -38,6 +38,13 @@ constexpr int GEMM_BM = 128;   // weight rows per GEMM tile (the MMA N dimension
 constexpr int GEMM_BK = 64;    // K elements per pipeline stage (one 128-byte swizzle row of bf16)
 constexpr int WORKER_THREADS = 128;
 constexpr int GEMM_MAX_BT = 128;     // most tokens per GEMM tile (MMA M)
+// Weight rows (output features) are stored so that a thread that reads the accumulators in the 16x256b fragment layout --
+// columns 8b + 2q + e for b = 0..3, e = 0, 1 in lane q of a quad -- holds eight consecutive features: row p of every 32
+// holds feature perm_feature(p).
+#ifdef __CUDACC__
+__host__ __device__
+#endif
+inline int perm_feature(int p) { return 8 * ((p >> 1) & 3) + 2 * (p >> 3) + (p & 1); }
 constexpr int GEMM_SMEM_BUDGET = 64 * 1024;  // stage memory a token-rich GEMM tile aims for (at least two stages are always taken)
 constexpr int GEMM_SMEM_BUDGET_SMALL = 84 * 1024;  // token-poor tiles (<= 64 tokens) are bound by TMA latency and get deeper
                                                    // pipelines, but must fit the room one finished token-rich tile leaves
@@ -92,7 +99,10 @@ struct GemmArgs {
   int32_t ldx, ldtab, ldtab2, ldo32, ldo16, ldoT, t_col0;
   int32_t M, N, Kp;    // tokens, output features, padded reduction length (multiple of GEMM_BK)
   int32_t bt, tiles_t; // tokens per tile, number of token tiles
-  int32_t vec16;       // every row and column offset of the epilogue's operands allows 16-byte accesses and N whole chunks
+  int32_t fast;        // straight epilogue: addresses allow whole vectors, nothing but row scale, activation, rotation, gating
+  int32_t perm;        // the weight rows stand in the accumulator's register order (see perm_feature)
+  int32_t under;       // addends lie in the accumulators before the first MMA: 1 bias, 2 vec, 4 X, 8 tab, 16 tab2
+  int32_t pad_;
   int32_t act, dual;   // activation; dual (gated): out = act(A Wgate^T) * (A Wup^T), 64 output features per tile
   float c_acc, c_x;    // out = c_x * X + c_acc * acc + vec + tab + tab2
   int32_t wmap, amap;         // tensor-map indices: shared weight maps, activation map relative to the slot's first
