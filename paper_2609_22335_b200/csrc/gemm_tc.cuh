@@ -288,8 +288,9 @@ __device__ __forceinline__ void epi_bf16(const EpiPlace& e, const GemmArgs& g, u
   });
 }
 // fp32 rows with, optionally, their bf16 mirror and the tile's share of each token's sum of squares (residual streams).
-template <bool MIRROR>
-__device__ __forceinline__ void epi_stream(const EpiPlace& e, const GemmArgs& g, float* out32, unsigned short* out16, float* ssq, int ft) {
+// POST: the solver update, out = c_acc * v + c_x * X + tab, whose addends cannot lie under a product that gets scaled.
+template <bool MIRROR, bool POST>
+__device__ __forceinline__ void epi_stream(const TileCtx& c, const EpiPlace& e, const GemmArgs& g, float* out32, unsigned short* out16, float* ssq, int ft) {
   const int q = e.lane & 3;
   epi_halves(e, [&](int row, uint32_t tmem, float ra, float rb) {
     float* pa = out32 + (size_t)(e.tok + row) * g.ldo32 + e.r0 + 8 * q;
@@ -299,6 +300,27 @@ __device__ __forceinline__ void epi_stream(const EpiPlace& e, const GemmArgs& g,
     float sa = 0.f, sb = 0.f;
     epi_frags(tmem, e.cols, ra, rb, [&](int c0, float* v) {
       const bool fok = c0 + 8 * q < e.cols;
+      if (POST && fok) {
+#pragma unroll
+        for (int j = 0; j < EPI; ++j) v[j] *= g.c_acc;
+        auto add = [&](Ref ref, int ld, float scale) {
+          const float* p = resolve<const float>(c, ref) + e.r0 + c0 + 8 * q;
+          float4 t[2][2];
+#pragma unroll
+          for (int k = 0; k < 2; ++k) {
+            const float4* x = reinterpret_cast<const float4*>(p + (size_t)(e.tok + min(row + 8 * k, e.live - 1)) * ld);
+            t[k][0] = __ldcg(x); t[k][1] = __ldcg(x + 1);
+          }
+#pragma unroll
+          for (int k = 0; k < 2; ++k) {
+            float* u = v + 2 * k;
+            u[0] = fmaf(scale, t[k][0].x, u[0]); u[1] = fmaf(scale, t[k][0].y, u[1]); u[4] = fmaf(scale, t[k][0].z, u[4]); u[5] = fmaf(scale, t[k][0].w, u[5]);
+            u[8] = fmaf(scale, t[k][1].x, u[8]); u[9] = fmaf(scale, t[k][1].y, u[9]); u[12] = fmaf(scale, t[k][1].z, u[12]); u[13] = fmaf(scale, t[k][1].w, u[13]);
+          }
+        };
+        if (g.X) add(g.X, g.ldx, g.c_x);
+        if (g.tab) add(g.tab, g.ldtab, 1.0f);
+      }
       if (MIRROR && fok) {
 #pragma unroll
         for (int b = 0; b < 4; ++b) {
@@ -357,24 +379,29 @@ __device__ __forceinline__ void epi_general(const TileCtx& c, const GemmArgs& g,
       x1 = fmaf(x1, cs.x, x0 * cs.y);
       x0 = r;
     }
-#pragma unroll 1
-    for (int fk = f; fk < min(f + 2, N); ++fk) {
-      float x = x0;
-      x0 = x1;
-      if (ptrs.bias) x += __ldg(ptrs.bias + fk);
-      x = apply_act(act, x) * g.c_acc;
-      if (ptrs.X) x = fmaf(g.c_x, ld_act(ptrs.X + tok * g.ldx + fk), x);
-      if (ptrs.vec) x += ld_act(ptrs.vec + fk);
-      if (ptrs.tab) x += ld_act(ptrs.tab + tok * g.ldtab + fk);
-      if (ptrs.tab2) x += ld_act(ptrs.tab2 + tok * g.ldtab2 + fk);
-      sq = fmaf(x, x, sq);
-      if (!live) continue;
-      if (ptrs.outT && fk >= g.t_col0) ptrs.outT[(size_t)(fk - g.t_col0) * g.ldoT + tok] = f32_to_bf16_bits(x);
-      else {
-        if (ptrs.out32) ptrs.out32[tok * g.ldo32 + fk] = x;
-        if (ptrs.out16) ptrs.out16[tok * g.ldo16 + fk] = f32_to_bf16_bits(x);
-      }
-    }
+    if (f >= N) continue;
+    const int f1 = min(f + 1, N - 1);                     // (the pair's loads go out together)
+    const bool two = f + 1 < N;
+    if (ptrs.bias) { x0 += __ldg(ptrs.bias + f); x1 += __ldg(ptrs.bias + f1); }
+    x0 = apply_act(act, x0) * g.c_acc; x1 = apply_act(act, x1) * g.c_acc;
+    auto add = [&](const float* p, size_t ld, float scale) {
+      const float a0 = ld_act(p + tok * ld + f), a1 = ld_act(p + tok * ld + f1);
+      x0 = fmaf(scale, a0, x0); x1 = fmaf(scale, a1, x1);
+    };
+    if (ptrs.X) add(ptrs.X, g.ldx, g.c_x);
+    if (ptrs.vec) add(ptrs.vec, 0, 1.0f);
+    if (ptrs.tab) add(ptrs.tab, g.ldtab, 1.0f);
+    if (ptrs.tab2) add(ptrs.tab2, g.ldtab2, 1.0f);
+    sq = fmaf(x0, x0, sq);
+    if (two) sq = fmaf(x1, x1, sq);
+    if (!live) continue;
+    const bool t0_ = ptrs.outT && f >= g.t_col0, t1_ = ptrs.outT && f1 >= g.t_col0;
+    if (t0_) ptrs.outT[(size_t)(f - g.t_col0) * g.ldoT + tok] = f32_to_bf16_bits(x0);
+    if (two && t1_) ptrs.outT[(size_t)(f1 - g.t_col0) * g.ldoT + tok] = f32_to_bf16_bits(x1);
+    if (ptrs.out32 && !t0_) ptrs.out32[tok * g.ldo32 + f] = x0;
+    if (ptrs.out32 && !t1_ && two) ptrs.out32[tok * g.ldo32 + f1] = x1;
+    if (ptrs.out16 && !t0_) ptrs.out16[tok * g.ldo16 + f] = f32_to_bf16_bits(x0);
+    if (ptrs.out16 && !t1_ && two) ptrs.out16[tok * g.ldo16 + f1] = f32_to_bf16_bits(x1);
   }
   if (ssq && live) ssq[tok * g.ss_out_ld + ft] = sq;
 }
@@ -393,8 +420,12 @@ __device__ __forceinline__ void gemm_epilogue(const TileCtx& c, const GemmArgs& 
     else if (g.act == ACT_GELU) epi_gated<ACT_GELU>(e, g, out16);
     else epi_gated<ACT_NONE>(e, g, out16);
   } else if (g.out32 != 0) {
-    if (out16) epi_stream<true>(e, g, resolve<float>(c, g.out32), out16, resolve<float>(c, g.ss_out), ft);
-    else epi_stream<false>(e, g, resolve<float>(c, g.out32), nullptr, nullptr, ft);
+    float* const out32 = resolve<float>(c, g.out32);
+    if (g.fast == 2) {
+      if (out16) epi_stream<true, true>(c, e, g, out32, out16, nullptr, ft);
+      else epi_stream<false, true>(c, e, g, out32, nullptr, nullptr, ft);
+    } else if (out16) epi_stream<true, false>(c, e, g, out32, out16, resolve<float>(c, g.ss_out), ft);
+    else epi_stream<false, false>(c, e, g, out32, nullptr, nullptr, ft);
   } else {
     const int all = e.cols;
     if (g.outT != 0) e.cols = max(0, min(all, g.t_col0 - r0));              // columns from here on are V features
@@ -411,38 +442,52 @@ __device__ __forceinline__ void gemm_epilogue(const TileCtx& c, const GemmArgs& 
   }
 }
 
-// Addends of the tile's tokens into the accumulators (fragment layout; columns past the last feature get zero).
+// Addends of the tile's tokens into the accumulators (fragment layout; columns past the last feature get zero).  All loads of
+// an addend and a 32-column group go out before the first of them is used.
 __device__ __forceinline__ void preload_rows(const TileCtx& c, const GemmArgs& g, uint32_t tmem, int t0, int nt, int warp, int lane, int r0) {
-  const GemmPtrs ptrs = gemm_ptrs(c, g);
-  const int q = lane & 3, cols = min(GEMM_BM, g.N - r0);
-  auto add8 = [](float* v, const float* p) {
-    const float4 a = __ldcg(reinterpret_cast<const float4*>(p)), b = __ldcg(reinterpret_cast<const float4*>(p) + 1);
-    v[0] += a.x; v[1] += a.y; v[4] += a.z; v[5] += a.w; v[8] += b.x; v[9] += b.y; v[12] += b.z; v[13] += b.w;
-  };
+  const int q = lane & 3, cols = min(GEMM_BM, g.N - r0), under = g.under;
+  int row[4];                                          // (lanes past the last token read that one)
+#pragma unroll
+  for (int k = 0; k < 4; ++k) row[k] = t0 + min(32 * warp + 8 * k + (lane >> 2), nt - 1);
 #pragma unroll 1
   for (int c0 = 0; c0 < cols; c0 += 32) {
-    float v[2][EPI];
+    float v[4][8];
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+#pragma unroll
+      for (int j = 0; j < 8; ++j) v[k][j] = 0.f;
     const int f = r0 + c0 + 8 * q;
+    if (c0 + 8 * q < cols) {
+      auto add = [&](Ref ref, int ld) {                // ld 0: the same row for every token
+        const float* p = resolve<const float>(c, ref) + f;
+        float4 t[4][2];
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
+        for (int k = 0; k < 4; ++k) {
+          const float4* x = reinterpret_cast<const float4*>(p + (size_t)row[k] * ld);
+          t[k][0] = __ldcg(x); t[k][1] = __ldcg(x + 1);
+        }
 #pragma unroll
-      for (int j = 0; j < EPI; ++j) v[h][j] = 0.f;
-      if (c0 + 8 * q >= cols) continue;
-#pragma unroll
-      for (int r = 0; r < 2; ++r) {
-        const size_t tok = (size_t)(t0 + min(32 * warp + 16 * h + 8 * r + (lane >> 2), nt - 1));
-        float* p = v[h] + 2 * r;
-        if (g.under & 4) add8(p, ptrs.X + tok * g.ldx + f);
-        if (g.under & 27) {
-          if (g.under & 1) add8(p, ptrs.bias + f);
-          if (g.under & 2) add8(p, ptrs.vec + f);
-          if (g.under & 8) add8(p, ptrs.tab + tok * g.ldtab + f);
-          if (g.under & 16) add8(p, ptrs.tab2 + tok * g.ldtab2 + f);
+        for (int k = 0; k < 4; ++k) {
+          v[k][0] += t[k][0].x; v[k][1] += t[k][0].y; v[k][2] += t[k][0].z; v[k][3] += t[k][0].w;
+          v[k][4] += t[k][1].x; v[k][5] += t[k][1].y; v[k][6] += t[k][1].z; v[k][7] += t[k][1].w;
+        }
+      };
+      if (under & 4) add(g.X, g.ldx);
+      if (under & 27) {
+#pragma unroll 1
+        for (int m = under & 27; m != 0; m &= m - 1) {
+          const int which = m & -m;
+          add(which == 1 ? g.bias : (which == 2 ? g.vec : (which == 8 ? g.tab : g.tab2)), which == 8 ? g.ldtab : (which == 16 ? g.ldtab2 : 0));
         }
       }
     }
-    tmem_st_frag(tmem + (uint32_t)c0, v[0]);
-    tmem_st_frag(tmem + (16u << 16) + (uint32_t)c0, v[1]);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const float* a = v[2 * h];
+      const float* b = v[2 * h + 1];
+      const float w[EPI] = {a[0], a[1], b[0], b[1], a[2], a[3], b[2], b[3], a[4], a[5], b[4], b[5], a[6], a[7], b[6], b[7]};
+      tmem_st_frag(tmem + ((uint32_t)(16 * h) << 16) + (uint32_t)c0, w);
+    }
   }
   tmem_st_wait();
 }
@@ -543,14 +588,19 @@ __device__ __forceinline__ void tile_gemm(const TileCtx& c, const GemmArgs& g, i
     if (warp_live) preload_rows(c, g, my_tmem, t0, nt, warp, lane, r0);
     tc_fence_before();
   }
-  // Folded RMSNorm: the token's row scale from the stream's partial sums of squares, added in a fixed order.
-  float rs = 1.0f;
-  if (g.rs_d > 0 && warp_live) {
+  // Folded RMSNorm: the partial sums of squares of this lane's token are requested now and added after the main loop, in a
+  // fixed order (streams wider than 1024: the rest at once).
+  float part[8], ssq = 0.f;
+  const bool scaled = g.rs_d > 0 && warp_live;
+#pragma unroll
+  for (int j = 0; j < 8; ++j) part[j] = 0.f;
+  if (scaled) {
     const float* sp = resolve<const float>(c, g.ss_in) + (size_t)(t0 + min(worker_tid(), nt - 1)) * g.ss_nft;
-    float ssq = 0.f;
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+      if (j < g.ss_nft) part[j] = ld_act(sp + j);
 #pragma unroll 4
-    for (int q = 0; q < g.ss_nft; ++q) ssq += ld_act(sp + q);
-    rs = 1.0f / sqrtf(ssq / (float)g.rs_d + 1e-6f);
+    for (int j = 8; j < g.ss_nft; ++j) ssq += ld_act(sp + j);
   }
   worker_sync(c);
 
@@ -603,6 +653,12 @@ __device__ __forceinline__ void tile_gemm(const TileCtx& c, const GemmArgs& g, i
   const bool ready = mbar_wait(c, accum_bar, acc_ph);
   __syncwarp();
   tc_fence_after();
+  float rs = 1.0f;
+  if (scaled) {
+#pragma unroll
+    for (int j = 0; j < 8; ++j) ssq += part[j];
+    rs = 1.0f / sqrtf(ssq / (float)g.rs_d + 1e-6f);
+  }
   if (ready && warp_live) gemm_epilogue(c, g, my_tmem, t0, nt, warp, lane, r0, rs, ft);
   tc_fence_before();
   worker_sync(c);

@@ -295,6 +295,10 @@ class Builder {
       g.fast = aligned && g.perm && all_under && !(scaled && !g.dual) &&
                (g.dual || g.act == ACT_NONE || (g.act == ACT_GELU && !g.out32 && !g.outT && o.rope_cols == 0));
       if (!g.fast) g.under = 0;
+      // the solver update: scaled product, addends behind it
+      if (!g.fast && aligned && g.perm && !g.dual && g.act == ACT_NONE && !g.bias && !g.vec && !g.tab2 && g.out32 && !g.outT && g.rope_cols == 0 &&
+          ss_view(o.out16).buf < 0)
+        g.fast = 2;
 
     }
     {

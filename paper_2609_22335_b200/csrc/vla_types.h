@@ -99,7 +99,8 @@ struct GemmArgs {
   int32_t ldx, ldtab, ldtab2, ldo32, ldo16, ldoT, t_col0;
   int32_t M, N, Kp;    // tokens, output features, padded reduction length (multiple of GEMM_BK)
   int32_t bt, tiles_t; // tokens per tile, number of token tiles
-  int32_t fast;        // straight epilogue: addresses allow whole vectors, nothing but row scale, activation, rotation, gating
+  int32_t fast;        // straight epilogue: addresses allow whole vectors, nothing but row scale, activation, rotation, gating (2: and
+                       // the solver's scaled update)
   int32_t perm;        // the weight rows stand in the accumulator's register order (see perm_feature)
   int32_t under;       // addends lie in the accumulators before the first MMA: 1 bias, 2 vec, 4 X, 8 tab, 16 tab2
   int32_t pad_;
