@@ -127,27 +127,17 @@ __device__ inline void queue_push(const DeviceCtx& ctx, int cls, uint32_t inst, 
   queue_commit(ctx, cls, n);
 }
 
-// Claim one tile if any is committed.  Bounded wait for the claimed ticket's entry to land.
-__device__ inline bool queue_try_pop(const DeviceCtx& ctx, int cls, QueueEntry& e, uint64_t deadline) {
-  TileQueue* q = ctx.queues + cls;
-  long long old = (long long)atomicAdd(reinterpret_cast<unsigned long long*>(&q->avail), (unsigned long long)(-1LL));
-  if (old <= 0) {
-    atomicAdd(reinterpret_cast<unsigned long long*>(&q->avail), 1ull);
-    return false;
-  }
-  const unsigned long long t = atomicAdd(&q->head, 1ull);
-  const unsigned long long mask = (unsigned long long)ctx.q_capacity - 1;
+// The entry of a claimed ticket.  Bounded wait for it to land.
+__device__ __forceinline__ bool queue_entry(const DeviceCtx& ctx, int cls, unsigned long long t, QueueEntry& e, uint64_t deadline) {
   const unsigned long long want = queue_gen(ctx, t);
-  const unsigned long long* slot = ctx.q_entries + (size_t)cls * ctx.q_capacity + (t & mask);
+  const unsigned long long* slot = ctx.q_entries + (size_t)cls * ctx.q_capacity + (t & ((unsigned long long)ctx.q_capacity - 1));
   unsigned spins = 0;
-  unsigned long long w;
-  while (((w = ld_acquire_u64(slot)) >> (64 - QW_GEN_BITS)) != want) {
+  while (((e = ld_acquire_u64(slot)) >> (64 - QW_GEN_BITS)) != want) {
     if ((++spins & 63u) == 0 && gtimer() > deadline) {
       set_error(ctx, DEV_ERR_WAIT_QUEUE, cls);
       return false;
     }
   }
-  e = w;
   return true;
 }
 
@@ -400,10 +390,20 @@ __device__ inline void claim_loop(const DeviceCtx& ctx, SmState* sm, int n_worke
   uint64_t pending_since = 0;     // lane c: since when class c has had committed tiles without a break (0: it has none)
   bool leaving = false;
 
+  // What this warp polls is one 16-byte word per lane, so that a round costs one trip to L2: lanes 0..7 a class's claimable
+  // tiles, lanes 8..15 its tail and done, lane 16 the control words, lane 17 the admission ring.
+  const void* poll_at = ctx.queues;
+  if (lane < N_CLASSES) poll_at = &ctx.queues[lane].avail;
+  else if (lane < 2 * N_CLASSES) poll_at = &ctx.queues[lane - N_CLASSES].tail;
+  else if (lane == 16) poll_at = &ctl->ctrl;
+  else if (lane == 17) poll_at = &ctl->admit_head;
   for (;;) {
     ++iter;
     bool progressed = false;
-    long long av = lane < N_CLASSES ? ld_volatile_s64(&ctx.queues[lane].avail) : 0;
+    unsigned long long px, py;
+    asm volatile("ld.volatile.global.v2.u64 {%0, %1}, [%2];" : "=l"(px), "=l"(py) : "l"(poll_at) : "memory");
+    const uint64_t now = gtimer();
+    const long long av = lane < N_CLASSES ? (long long)px : 0;
     const unsigned pending = __ballot_sync(0xffffffffu, av > 0) & ((1u << N_CLASSES) - 1u);
     // Tiles are claimed ahead of need only while the VLM backlog as a whole exceeds what the GPU's workers can hold
     // (a held tile is a tile no idle worker elsewhere can take), and then from every VLM queue that is not nearly empty.
@@ -415,20 +415,20 @@ __device__ inline void claim_loop(const DeviceCtx& ctx, SmState* sm, int n_worke
                           ((1u << N_CLASSES) - 1u);
     // classes whose tiles free workers elsewhere did not drain within head_wait_ns (by the clock, not by polling
     // rounds: how fast this loop spins must not change what it decides)
-    if (av > 0) { if (pending_since == 0) pending_since = gtimer(); } else pending_since = 0;
-    const unsigned waiting = __ballot_sync(0xffffffffu, pending_since != 0 && gtimer() - pending_since >= HEAD_WAIT_NS) &
+    if (av > 0) { if (pending_since == 0) pending_since = now; } else pending_since = 0;
+    const unsigned waiting = __ballot_sync(0xffffffffu, pending_since != 0 && now - pending_since >= HEAD_WAIT_NS) &
                              ((1u << N_CLASSES) - 1u);
-    int outstanding = lane < N_CLASSES ? (int)min(ld_volatile_u64(&ctx.queues[lane].tail) - ld_volatile_u64(&ctx.queues[lane].done), 1ull << 20) : 0;
+    int outstanding = lane >= N_CLASSES && lane < 2 * N_CLASSES ? (int)min(px - py, 1ull << 20) : 0;
 #pragma unroll
     for (int o = 4; o > 0; o >>= 1) outstanding += __shfl_xor_sync(0xffffffffu, outstanding, o);
+    outstanding = __shfl_sync(0xffffffffu, outstanding, N_CLASSES);
     if (lane == 0) sm->outstanding = outstanding;
-    outstanding = __shfl_sync(0xffffffffu, outstanding, 0);
     const int n_sms = (int)gridDim.x;
     const int share = outstanding <= n_sms ? 1 : (outstanding <= 2 * n_sms ? 2 : MAX_WORKERS);
     unsigned spread = 0xffffffffu;
     int running = 0;
     if (share < MAX_WORKERS) {
-      spread = __ballot_sync(0xffffffffu, pending_since != 0 && gtimer() - pending_since >= SPREAD_WAIT_NS) & ((1u << N_CLASSES) - 1u);
+      spread = __ballot_sync(0xffffffffu, pending_since != 0 && now - pending_since >= SPREAD_WAIT_NS) & ((1u << N_CLASSES) - 1u);
       running = __popc(__ballot_sync(0xffffffffu, serving && (slot->busy != 0 || slot->held_tail != slot->held_head || slot->prio_tail != slot->prio_head)));
     }
     if (lane < N_CLASSES) sm->grid[lane] = (int)(av < 0 ? 0 : (av > (1 << 20) ? (1 << 20) : av));   // G_k of the -G score: tiles still to place
@@ -453,7 +453,7 @@ __device__ inline void claim_loop(const DeviceCtx& ctx, SmState* sm, int n_worke
         unsigned cand;
         if (!busy) cand = head_pending ? (pending & act_mask) : pending;
         else if (pq == 0u && head_pending && (waiting & act_mask & ~avoid) != 0u && slot->busy != 0 && slot->primed == 0 &&
-                 (long long)(gtimer() - slot->t_busy) + PRIO_WINDOW_NS >= (long long)sm->ema_ns[slot->cls]) {
+                 (long long)(now - slot->t_busy) + PRIO_WINDOW_NS >= (long long)sm->ema_ns[slot->cls]) {
           cand = waiting & act_mask; to_prio = true;
         }
         else if (queued < (unsigned)HELD_DEPTH) cand = deep & ((1u << N_KINDS) - 1u);
@@ -503,9 +503,24 @@ __device__ inline void claim_loop(const DeviceCtx& ctx, SmState* sm, int n_worke
     bool popped = false;
     int ji = 0;
     uint32_t node = 0;
+    const unsigned same = __match_any_sync(0xffffffffu, want);      // lanes that want the same class claim together
+    const int rank = __popc(same & ((1u << lane) - 1u)), first = __ffs((int)same) - 1;
+    int got = 0;
+    unsigned long long ticket = 0;
+    if (want >= 0 && rank == 0) {
+      // (a compare-and-swap on the head alone, one trip instead of two, collapses when many SMs want the same few tiles)
+      const int n = __popc(same);
+      TileQueue* q = ctx.queues + want;
+      const long long old = (long long)atomicAdd(reinterpret_cast<unsigned long long*>(&q->avail), (unsigned long long)(-(long long)n));
+      got = old <= 0 ? 0 : (int)min(old, (long long)n);
+      if (got < n) atomicAdd(reinterpret_cast<unsigned long long*>(&q->avail), (unsigned long long)(n - got));
+      if (got > 0) ticket = atomicAdd(&q->head, (unsigned long long)got);
+    }
+    got = __shfl_sync(0xffffffffu, got, first);
+    ticket = __shfl_sync(0xffffffffu, ticket, first) + (unsigned long long)rank;
     if (want >= 0) {
       QueueEntry e;
-      if (queue_try_pop(ctx, want, e, gtimer() + ctx.wait_limit_ns)) {
+      if (rank < got && queue_entry(ctx, want, ticket, e, now + ctx.wait_limit_ns)) {
         popped = true;
         ji = to_prio ? 2 + (int)(slot->prio_tail & 1u) : (int)(slot->held_tail & 1u);
         TileJob& h = slot->job[ji];
@@ -544,28 +559,24 @@ __device__ inline void claim_loop(const DeviceCtx& ctx, SmState* sm, int n_worke
       bell_ring(&sm->bell_worker[lane]);
       progressed = true;
     }
-    // ---- admission, exit and watchdog (lane 0 decides, every few rounds)
+    // ---- admission, exit and watchdog (lane 0 decides)
     int verdict = 0;   // 1 = leave
-    if (lane == 0 && (iter & 3u) == 0) {              // several dependent round trips: not on every poll
-      if (ld_volatile_u32(&ctl->error) != 0u || ld_volatile_u32(&ctl->stop) != 0u) verdict = 1;
-      const unsigned cw = ld_volatile_u32(&ctl->ctrl);
-      if (cw & CTRL_EXITING) verdict = 1;
-      if (!verdict) {
-        try_admit(ctx);
-        const uint64_t now = gtimer();
-        const bool none = cw == 0u && ld_volatile_u64(&ctl->admit_head) >= ld_volatile_u64(&ctl->admit_tail);
-        if (none) {
-          if (idle_start == 0) idle_start = now;
-          else if (now - idle_start > ctx.idle_exit_ns) atomicCAS(&ctl->ctrl, 0u, CTRL_EXITING);
-        } else {
-          idle_start = 0;
-        }
+    const unsigned cw = (unsigned)__shfl_sync(0xffffffffu, px, 16), err = (unsigned)(__shfl_sync(0xffffffffu, px, 16) >> 32);
+    const unsigned stop = (unsigned)(__shfl_sync(0xffffffffu, py, 16) >> 32);
+    const bool admissions = __shfl_sync(0xffffffffu, px, 17) < __shfl_sync(0xffffffffu, py, 17);
+    if (err != 0u || stop != 0u || (cw & CTRL_EXITING)) verdict = 1;
+    else if (lane == 0) {
+      if (admissions) try_admit(ctx);
+      if (cw == 0u && !admissions) {
+        if (idle_start == 0) idle_start = now;
+        else if (now - idle_start > ctx.idle_exit_ns) atomicCAS(&ctl->ctrl, 0u, CTRL_EXITING);
+      } else {
+        idle_start = 0;
       }
     }
     const bool any_progress = __any_sync(0xffffffffu, progressed || (serving && slot->busy != 0));
-    if (any_progress) last_progress = gtimer();
-    else if (lane == 0 && !verdict && (iter & 63u) == 0 && gtimer() - last_progress > ctx.wait_limit_ns &&
-             ld_volatile_u32(&ctl->ctrl) != 0u) {
+    if (any_progress) last_progress = now;
+    else if (lane == 0 && !verdict && (iter & 63u) == 0 && now - last_progress > ctx.wait_limit_ns && cw != 0u) {
       set_error(ctx, DEV_ERR_IDLE_LIMIT, (unsigned)blockIdx.x);   // frames in flight, nothing moved for too long
       verdict = 1;
     }

@@ -1105,8 +1105,8 @@ bool build_program(const vla_model_desc& d, const vla_runtime_opts& o, Program& 
   p.off_succ = place(sizeof(SuccInfo) * std::max<size_t>(p.succ.size(), 1));
   p.off_roots = place(sizeof(int32_t) * std::max<size_t>(p.roots.size(), 1));
   p.off_classes = place(sizeof(ClassInfo) * N_CLASSES);
-  p.off_control = place(sizeof(Control));
-  p.off_queues = place(sizeof(TileQueue) * N_CLASSES);
+  p.off_control = place(sizeof(Control), 128);
+  p.off_queues = place(sizeof(TileQueue) * N_CLASSES, 128);
   // queue capacity: every tile of every in-flight frame could be queued at once in the worst case
   uint64_t tiles_per_frame = 0;
   for (const NodeDesc& n : p.nodes) tiles_per_frame += n.n_tiles;

@@ -203,11 +203,11 @@ constexpr int SMEM_UNIT = 4096;
 constexpr int TMEM_UNIT = 32;
 
 // A multi-producer multi-consumer ring of tile tickets (one per class).
-struct TileQueue {             // one 128-byte line per queue
-  unsigned long long head;     // next ticket to hand out
-  unsigned long long tail;     // next ticket to reserve for a push
+struct alignas(128) TileQueue {   // one 128-byte line per queue; each pair is read by one 16-byte load
   long long avail;             // committed minus claimed (may dip below zero transiently)
-  unsigned long long done;     // tiles of this class that have finished: tail - done are queued or running
+  unsigned long long head;     // next ticket to hand out
+  unsigned long long tail;     // next ticket to reserve for a push ...
+  unsigned long long done;     // ... and tiles of this class that have finished: tail - done are queued or running
   unsigned long long pad[12];
 };
 
@@ -235,14 +235,14 @@ struct DoneRec {
 };
 
 // Device-resident control block.
-struct Control {                 // polled words and hot counters live on separate 128-byte lines
+struct alignas(128) Control {    // polled words and hot counters live on separate 128-byte lines
   unsigned int ctrl;             // bit 31 = exiting; low bits = frames in flight
   unsigned int error;            // sticky error code (0 = none)
   unsigned int error_info;
-  unsigned int stop;             // host request to exit
+  unsigned int stop;             // host request to exit (these four are read by one 16-byte load)
   unsigned int pad0[28];
   unsigned long long admit_head; // admission records consumed
-  unsigned long long admit_tail; // admission records published (written by host copies)
+  unsigned long long admit_tail; // admission records published (written by host copies; read with admit_head by one load)
   unsigned long long pad1[14];
   unsigned long long doorbell;   // bumped whenever tiles are committed to any queue
   unsigned long long pad2[15];
