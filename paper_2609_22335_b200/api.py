@@ -280,7 +280,7 @@ class Engine:
         nxt = [0] * R
         got = [[None] * len(frames[r]) for r in range(R)]
         remaining = sum(len(f) for f in frames)
-        t0 = time.time()
+        t0 = last = time.time()
         while remaining:
             progressed = False
             for r in range(R):
@@ -298,9 +298,12 @@ class Engine:
                     got[r][fid - base[r]] = chunk
                     remaining -= 1
                     progressed = True
-            if not progressed:
-                if time.time() - t0 > timeout_s:
-                    raise TimeoutError("no progress")
+            now = time.time()
+            if progressed:
+                last = now
+            elif now - t0 > timeout_s:
+                raise TimeoutError("no progress")
+            elif now - last > 0.1:        # a chunk is usually milliseconds away: a sleep would add its 60 us and more
                 time.sleep(0.0002)
         return got
 

@@ -210,11 +210,6 @@ __device__ inline void write_trace(const DeviceCtx& ctx, uint32_t inst, uint32_t
   ctx.trace[idx] = r;
 }
 
-// Release count that a node reaches when it is released for this frame of its slot.
-__device__ __forceinline__ unsigned release_count(const DeviceCtx& ctx, uint64_t frame) {
-  return (unsigned)(frame / (unsigned)ctx.ring_depth + 1u) & 0x7FFFFFFFu;
-}
-
 // A frame became ready (its inputs are in HBM): take its admission record and queue its root tiles.
 __device__ inline void try_admit(const DeviceCtx& ctx) {
   Control* ctl = ctx.control;
@@ -238,6 +233,7 @@ __device__ inline void try_admit(const DeviceCtx& ctx) {
   const uint32_t inst = rec->inst;
   const uint64_t frame = rec->frame;
   *reinterpret_cast<volatile uint64_t*>(ctx.inst_frame + inst) = frame;
+  *reinterpret_cast<volatile uint32_t*>(ctx.inst_gen + inst) = rec->gen;
   {   // the frame's admission is a trace record of its own (node = TRACE_ADMIT_NODE): no tile of the frame may start earlier
     const uint64_t now = gtimer();
     write_trace(ctx, inst, TRACE_ADMIT_NODE, 0, 0, 0xFF, frame, now, now);
@@ -336,15 +332,15 @@ __device__ __forceinline__ void retire_loop(const DeviceCtx& ctx, SmState* sm, i
         push_nodes(ctx, early, inst, si, RES_EARLY, lane);
       }
     }
-    // ---- ends.  Every successor's word (which counts its predecessors' tiles) goes down by one; one reaching zero is
-    // re-armed with its release count one up, which is what early-taken tiles of that node wait for; if the node was not
-    // queued early, it is now.
+    // ---- ends.  Every successor's word counts one more finished predecessor tile; reaching the frame's total is the release,
+    // which early-taken tiles of that node wait for; if the node was not queued early, it is now.
     if (__any_sync(0xffffffffu, ended)) {
       uint32_t inst = 0;
       int succ0 = 0, n_succ = 0;
+      unsigned gen = 0;
       if (ended) {
         const DoneTile& f = slot->done;
-        inst = f.inst; succ0 = f.succ_begin; n_succ = f.succ_count;
+        inst = f.inst; gen = f.gen; succ0 = f.succ_begin; n_succ = f.succ_count;
         if (sub == 0) {
           sm->ema_ns[f.cls] = (3 * sm->ema_ns[f.cls] + (int)(f.t1 - f.t0)) >> 2;
           write_trace(ctx, f.inst, f.node, f.tile, w, f.cls, f.frame, f.t0, f.t1);
@@ -358,10 +354,10 @@ __device__ __forceinline__ void retire_loop(const DeviceCtx& ctx, SmState* sm, i
         if (i < n_succ) {
           si = load_succ(ctx, succ0 + i);
           unsigned long long* word = ctx.dep_word + (size_t)inst * ctx.n_nodes + si.node;
-          const unsigned long long old = atomicAdd(word, ~0ull);
-          if ((uint32_t)old == 1u) {
-            st_release_u64(word, ((((old >> 32) + 1ull) & 0x7FFFFFFFull) << 32) | (unsigned)si.n_pred);
-            release = (old >> 63) == 0ull;
+          const unsigned long long old = atomicAdd(word, 1ull);
+          if ((old & ((1ull << 62) - 1ull)) + 1ull == DEP_BIAS + (unsigned long long)(unsigned)si.n_pred * gen) {
+            if (old >> 63) atomicAnd(word, ~(1ull << 63));
+            else release = true;
           }
         }
         push_nodes(ctx, release, inst, si, 0u, lane);
@@ -536,7 +532,7 @@ __device__ inline void claim_loop(const DeviceCtx& ctx, SmState* sm, int n_worke
         h.promised_s = promised_s; h.promised_t = promised_t;
         h.slot_base = __ldg(ctx.slot_base + inst);
         h.frame = ld_volatile_u64(reinterpret_cast<const unsigned long long*>(ctx.inst_frame + inst));
-        if (h.early) h.gen = release_count(ctx, h.frame);
+        h.gen = ld_volatile_u32(ctx.inst_gen + inst);
       } else {                                         // lost the race: undo the count
         atomicSub(&sm->pick.cta_count[want], 1);
         for (int x = 0; x < 3; ++x) atomicSub(&sm->pick.u[x], sm->tau_tab[want * 3 + x]);
@@ -611,7 +607,7 @@ __device__ __forceinline__ void end_of_tile(const DeviceCtx& ctx, SmState* sm, W
   DoneTile d;
   if (wt == 32) {              // (read before the barrier: afterwards the leader moves on)
     const TileJob& j = slot->job[slot->run];
-    d.inst = j.inst; d.node = j.node; d.tile = j.tile; d.cls = j.cls; d.frame = j.frame; d.t0 = slot->t_start;
+    d.inst = j.inst; d.node = j.node; d.tile = j.tile; d.cls = j.cls; d.gen = j.gen; d.frame = j.frame; d.t0 = slot->t_start;
     d.succ_begin = j.desc.succ_begin; d.succ_count = j.desc.succ_count; d.op = j.desc.op;
   }
   asm volatile("bar.sync %0, %1;" ::"r"(worker + 1), "r"(WORKER_THREADS) : "memory");
@@ -692,7 +688,7 @@ __device__ __forceinline__ void take_tile(const DeviceCtx& ctx, SmState* sm, Wor
       for (int k = 0; k < N_CLASSES; ++k) taken += *reinterpret_cast<volatile int*>(&sm->pick.cta_count[k]);
       if (taken != 1) {
         tc.wait_word = ctx.dep_word + (size_t)job.inst * ctx.n_nodes + job.node;
-        tc.wait_gen = job.gen;
+        tc.wait_count = DEP_BIAS + (unsigned long long)(unsigned)job.desc.n_pred * job.gen;
         tc.t_start = &slot->t_wait;
         tc.deadline = lim;
         wait_release(tc);
@@ -765,7 +761,7 @@ __device__ __forceinline__ void take_tile(const DeviceCtx& ctx, SmState* sm, Wor
   tc.amap_base = ctx.n_weight_tmaps + (int)job.inst * ctx.n_act_tmaps;
   tc.deadline = lim;
   tc.wait_word = early ? ctx.dep_word + (size_t)job.inst * ctx.n_nodes + job.node : nullptr;
-  tc.wait_gen = job.gen;
+  tc.wait_count = DEP_BIAS + (unsigned long long)(unsigned)job.desc.n_pred * job.gen;
   tc.t_start = &slot->t_start;
 }
 

@@ -1122,6 +1122,7 @@ bool build_program(const vla_model_desc& d, const vla_runtime_opts& o, Program& 
   p.off_dep = place(sizeof(uint64_t) * (uint64_t)nn * p.n_inst);
   p.off_start = place(sizeof(int32_t) * (uint64_t)nn * p.n_inst);
   p.off_inst_frame = place(sizeof(uint64_t) * p.n_inst);
+  p.off_inst_gen = place(sizeof(uint32_t) * p.n_inst);
   p.off_slot_base = place(sizeof(uint64_t) * p.n_inst);
   p.off_input_ptrs = place(sizeof(uint64_t) * N_FRAME_INPUTS * p.n_inst);
   p.trace_capacity = o.trace_capacity;

@@ -17,8 +17,8 @@ namespace vla {
 struct TileJob {
   uint32_t inst, node, tile;
   int cls, smem_units, tmem_units;
-  int early;                     // queued before its node's release ...
-  unsigned gen;                  // ... which brings the node's release count to this
+  int early;                     // queued before its node's release
+  unsigned gen;                  // the frame's number in its slot
   int promised_s, promised_t;    // room promised to the tile when it was claimed
   uint64_t frame, slot_base;
   alignas(16) NodeDesc desc;
@@ -29,6 +29,7 @@ constexpr int N_JOBS = 4;        // held tiles use jobs 0 and 1 in turn, priorit
 struct DoneTile {
   uint32_t inst, node, tile;
   int cls, succ_begin, succ_count, op;
+  unsigned gen;
   uint64_t t0, t1, frame;
 };
 
@@ -76,8 +77,8 @@ struct TileCtx {
   const void* tmaps;    // tensor-map table (128 bytes per entry)
   int amap_base;        // index of this frame slot's first activation map
   int n_weight_tmaps, n_act_tmaps;      // weight maps; activation maps per frame slot
-  const unsigned long long* wait_word;   // not null: the tile was taken early and waits for its node's release, the moment the
-  unsigned wait_gen;                     // release count of this word (bits 32..62) equals wait_gen; GEMM tiles fetch weights meanwhile
+  const unsigned long long* wait_word;   // not null: the tile was taken early and waits for its node's release, the moment this
+  unsigned long long wait_count;         // word counts so many finished predecessor tiles; GEMM tiles fetch weights meanwhile
   uint64_t* t_start;                     // where the time of that moment goes
   WorkerSlot* slot;     // the persistent kernel's worker, null elsewhere
   int cont;             // this tile's operand ring was primed by the tile before
@@ -110,7 +111,7 @@ __device__ __forceinline__ void wait_release(const TileCtx& c) {
     unsigned long long w;
     asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(w) : "l"(c.wait_word) : "memory");
     uint64_t now;
-    if (((unsigned)(w >> 32) & 0x7FFFFFFFu) == c.wait_gen) {
+    if ((w & ((1ull << 62) - 1ull)) >= c.wait_count) {
       asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
       *c.t_start = now;
       return;

@@ -280,7 +280,7 @@ int submit_common(vla_ctx* c, int32_t stream, const float* image, const int32_t*
   const unsigned long long t = c->n_admitted++;
   const size_t ri = (size_t)(t % (unsigned long long)p.admit_capacity);
   c->admit_pinned[ri].inst = (uint32_t)inst;
-  c->admit_pinned[ri].pad = 0;
+  c->admit_pinned[ri].gen = (uint32_t)(f / (uint64_t)p.ring_depth) + 1u;
   c->admit_pinned[ri].frame = f;
   c->tail_pinned[ri] = t + 1;
 
@@ -379,13 +379,10 @@ int vla_init(const vla_model_desc* desc, const vla_runtime_opts* opts, vla_ctx**
   CU(cudaMemcpy(at<char>(c, p.off_roots), p.roots.data(), 4 * p.roots.size(), cudaMemcpyHostToDevice));
   CU(cudaMemcpy(at<char>(c, p.off_classes), p.classes, sizeof(ClassInfo) * N_CLASSES, cudaMemcpyHostToDevice));
   {
-    std::vector<uint64_t> dep((size_t)p.n_inst * p.nodes.size());
-    std::vector<int32_t> start(dep.size());
+    std::vector<int32_t> start((size_t)p.n_inst * p.nodes.size());
     for (int i = 0; i < p.n_inst; ++i)
-      for (size_t k = 0; k < p.nodes.size(); ++k) {
-        dep[(size_t)i * p.nodes.size() + k] = (uint64_t)p.nodes[k].n_pred;
-        start[(size_t)i * p.nodes.size() + k] = p.pred_nodes[k];
-      }
+      for (size_t k = 0; k < p.nodes.size(); ++k) start[(size_t)i * p.nodes.size() + k] = p.pred_nodes[k];
+    std::vector<uint64_t> dep(start.size(), DEP_BIAS);
     CU(cudaMemcpy(at<char>(c, p.off_dep), dep.data(), 8 * dep.size(), cudaMemcpyHostToDevice));
     CU(cudaMemcpy(at<char>(c, p.off_start), start.data(), 4 * start.size(), cudaMemcpyHostToDevice));
     std::vector<uint64_t> sb(p.n_inst);
@@ -434,7 +431,7 @@ int vla_init(const vla_model_desc* desc, const vla_runtime_opts* opts, vla_ctx**
   x.admit_ring = at<AdmitRec>(c, p.off_admit);
   x.dep_word = at<unsigned long long>(c, p.off_dep);
   x.start_count = at<int32_t>(c, p.off_start);
-  x.ring_depth = p.ring_depth;
+  x.inst_gen = at<uint32_t>(c, p.off_inst_gen);
   x.inst_frame = at<uint64_t>(c, p.off_inst_frame);
   x.slot_base = at<uint64_t>(c, p.off_slot_base);
   x.input_ptrs = at<uint64_t>(c, p.off_input_ptrs);
@@ -819,11 +816,11 @@ int vla_debug_bump_dependency(vla_ctx* c, int32_t stream, int32_t slot, int32_t 
     return fail(c, VLA_ERR_INVALID, "bad stream, slot or node");
   if (c->pending_frames != 0) return fail(c, VLA_ERR_STATE, "frames are in flight");
   CU(cudaDeviceSynchronize());
-  // (the count is the low half of the node's state word)
-  int32_t* cnt = reinterpret_cast<int32_t*>(c->dctx.dep_word + (size_t)(stream * p.ring_depth + slot) * p.nodes.size() + node);
-  int32_t v = 0;
+  // (the word counts finished predecessor tiles: a tile too many to wait for is one finished too few)
+  unsigned long long* cnt = c->dctx.dep_word + (size_t)(stream * p.ring_depth + slot) * p.nodes.size() + node;
+  unsigned long long v = 0;
   CU(cudaMemcpy(&v, cnt, sizeof v, cudaMemcpyDeviceToHost));
-  v += delta;
+  v -= (unsigned long long)(long long)delta;
   CU(cudaMemcpy(cnt, &v, sizeof v, cudaMemcpyHostToDevice));
   return VLA_OK;
 }

@@ -33,6 +33,7 @@ constexpr Ref REF_SLOT = 1ull << 63;
 // reached through the per-slot input pointer table so resident inputs are read in place.
 constexpr Ref REF_INPUT = 1ull << 62;
 constexpr int N_FRAME_INPUTS = 4;
+constexpr unsigned long long DEP_BIAS = 1ull << 40;   // dependency words start here (a test hook may take some away)
 
 constexpr int GEMM_BM = 128;   // weight rows per GEMM tile (the MMA N dimension; tokens are M)
 constexpr int GEMM_BK = 64;    // K elements per pipeline stage (one 128-byte swizzle row of bf16)
@@ -217,7 +218,7 @@ typedef unsigned long long QueueEntry;
 
 struct AdmitRec {              // written by the host (copy stream), read by the dispatcher
   uint32_t inst;
-  uint32_t pad;
+  uint32_t gen;                // how many frames the slot has had with this one
   uint64_t frame;
 };
 
@@ -269,11 +270,12 @@ struct DeviceCtx {
   TileQueue* queues;             // [N_CLASSES]
   QueueEntry* q_entries;         // [N_CLASSES][q_capacity]
   AdmitRec* admit_ring;
-  // [n_inst][n_nodes] state of a node in a frame slot: bits 0..31 predecessor tiles still to finish, bits 32..62 how often the
-  // node has been released (once per frame of the slot), bit 63 its tiles were queued early, before the release
+  // [n_inst][n_nodes] DEP_BIAS + predecessor tiles of a node that have finished, counted over all frames of the slot (the
+  // node is released when those reach n_pred x the frame's number in the slot); bit 63: its tiles were queued before that
   unsigned long long* dep_word;
   int32_t* start_count;          // [n_inst][n_nodes] predecessor nodes whose last tile has not been taken yet
   uint64_t* inst_frame;          // [n_inst] frame id currently owning the slot
+  uint32_t* inst_gen;            // [n_inst] its number among the slot's frames, from 1
   const uint64_t* slot_base;     // [n_inst] arena offset of the instance's buffers
   const uint64_t* input_ptrs;    // [n_inst][N_FRAME_INPUTS] device addresses of the frame's input arrays
   const int32_t* roots;          // nodes without predecessors
@@ -286,7 +288,7 @@ struct DeviceCtx {
   int32_t n_nodes, n_inst, n_roots;
   int32_t q_capacity, q_shift, admit_capacity;   // q_capacity = 1 << q_shift
   uint32_t trace_capacity;
-  int32_t policy, workers_per_sm, ring_depth;
+  int32_t policy, workers_per_sm;
   int32_t u_max, pad_u;     // saturation value of the utilisation counters in the pick's score
   uint64_t wait_limit_ns, idle_exit_ns;
   int32_t chunk_elems;
