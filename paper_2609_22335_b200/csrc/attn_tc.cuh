@@ -13,7 +13,8 @@
 //
 // What bounds it: one tile alone is a chain of barrier tests, MMA issue and tensor-memory round trips around 800 cycles of
 // softmax per block.  So S of block b+1 is issued as soon as the scores of block b are in registers (warp 0), P V of block b
-// by warp 1, and the loads run two blocks (K) and one block (V) ahead on warps 2 and 3: 3560 -> MEASURED cycles per block.
+// by warp 1, and the loads run two blocks (K) and one block (V) ahead on warps 2 and 3: 3560 -> 3010 cycles per block of a
+// tile alone on its SM, 52 -> 40 us for a 16-block tile among three.
 #pragma once
 #include "gemm_tc.cuh"
 
@@ -71,6 +72,54 @@ __device__ __forceinline__ float max3(float x, float y, float z) {
   float r;
   asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(x), "f"(y), "f"(z));
   return r;
+}
+
+// Scores of the keys a row must not see, [lim, 64), become -inf.
+__device__ __forceinline__ void attn_mask(uint32_t* sr, int lim) {
+  if (!__any_sync(0xffffffffu, lim < ATTN_BN)) return;
+#pragma unroll
+  for (int j = 0; j < ATTN_BN; ++j)
+    if (j >= lim) sr[j] = 0xFF800000u;
+}
+// One block of a row's online softmax: 64 scores in, 32 bf16 probability pairs out (front half of the registers).
+__device__ __forceinline__ void attn_softmax_block(uint32_t* sr, float sl2, float& m_run, float& l_run, float& alpha) {
+  float m4[4] = {m_run, __uint_as_float(sr[0]), __uint_as_float(sr[1]), __uint_as_float(sr[2])};
+#pragma unroll
+  for (int j = 3; j < ATTN_BN - 1; j += 2) m4[(j >> 1) & 3] = max3(m4[(j >> 1) & 3], __uint_as_float(sr[j]), __uint_as_float(sr[j + 1]));
+  float mx = fmaxf(max3(m4[0], m4[1], m4[2]), fmaxf(m4[3], __uint_as_float(sr[ATTN_BN - 1])));
+  // The running maximum only has to keep the exponentials in range, not to be exact: softmax does not depend on
+  // the shift, and l and O are accumulated with the same one.  It follows the true maximum only when that has
+  // moved by more than 8 in the exponent (p then stays below 2^8), so O is rescaled on few blocks instead of
+  // on nearly every one (with 32 rows per warp some row's maximum moves in almost every block).
+  if (m_run == -INFINITY) alpha = 0.f;
+  else if ((mx - m_run) * sl2 <= ATTN_RESCALE_LOG2) { mx = m_run; alpha = 1.0f; }
+  else alpha = exp2_fast((m_run - mx) * sl2);
+  const float mb = mx == -INFINITY ? 0.f : -mx * sl2;
+  const uint64_t sl2_2 = pack2(sl2, sl2), mb_2 = pack2(mb, mb);
+  uint64_t s2[2] = {0ull, 0ull};
+#pragma unroll
+  for (int j = 0; j < ATTN_BN; j += 2) {
+    const uint64_t e2 = fma2(pack2(__uint_as_float(sr[j]), __uint_as_float(sr[j + 1])), sl2_2, mb_2);
+    float p0, p1;
+    unpack2(e2, p0, p1);
+    p0 = exp2_fast(p0); p1 = exp2_fast(p1);
+    s2[(j >> 1) & 1] = add2(s2[(j >> 1) & 1], pack2(p0, p1));
+    sr[j >> 1] = pack_bf16(p0, p1);
+  }
+  float x0, x1;
+  unpack2(add2(s2[0], s2[1]), x0, x1);
+  l_run = l_run * alpha + (x0 + x1);
+  m_run = mx;
+}
+__device__ __forceinline__ void attn_rescale(uint32_t tmem, int hs, float alpha) {
+#pragma unroll 1
+  for (int c0 = 0; c0 < hs; c0 += 16) {
+    float o[16];
+    tmem_ld16(tmem + (uint32_t)c0, o);
+#pragma unroll
+    for (int j = 0; j < 16; ++j) o[j] *= alpha;
+    tmem_st16(tmem + (uint32_t)c0, o);
+  }
 }
 
 // Key blocks of a tile: segment 0 (cached prefix) then segment 1 (the head's own keys), 64 keys each,
@@ -229,59 +278,16 @@ __device__ __forceinline__ void tile_attention(const TileCtx& c, const AttnArgs&
         ragged = true;
         if (row < a.sfx) lim = min(lim, a.sfx - kv0);
       }
-      if (ragged && __any_sync(0xffffffffu, lim < ATTN_BN)) {
-#pragma unroll
-        for (int j = 0; j < ATTN_BN; ++j)
-          if (j >= lim) sr[j] = 0xFF800000u;
-      }
+      if (ragged) attn_mask(sr, lim);
     }
-    float m4[4] = {m_run, __uint_as_float(sr[0]), __uint_as_float(sr[1]), __uint_as_float(sr[2])};
-#pragma unroll
-    for (int j = 3; j < ATTN_BN - 1; j += 2) m4[(j >> 1) & 3] = max3(m4[(j >> 1) & 3], __uint_as_float(sr[j]), __uint_as_float(sr[j + 1]));
-    float mx = fmaxf(max3(m4[0], m4[1], m4[2]), fmaxf(m4[3], __uint_as_float(sr[ATTN_BN - 1])));
-    // The running maximum only has to keep the exponentials in range, not to be exact: softmax does not depend on
-    // the shift, and l and O are accumulated with the same one.  It follows the true maximum only when that has
-    // moved by more than 8 in the exponent (p then stays below 2^8), so O is rescaled on few blocks instead of
-    // on nearly every one (with 32 rows per warp some row's maximum moves in almost every block).
-    const float sl2 = a.scale_log2e;
     float alpha;
-    if (m_run == -INFINITY) alpha = 0.f;
-    else if ((mx - m_run) * sl2 <= ATTN_RESCALE_LOG2) { mx = m_run; alpha = 1.0f; }
-    else alpha = exp2_fast((m_run - mx) * sl2);
-    const float mb = mx == -INFINITY ? 0.f : -mx * sl2;
-    const uint64_t sl2_2 = pack2(sl2, sl2), mb_2 = pack2(mb, mb);
-    uint64_t s2[2] = {0ull, 0ull};
-#pragma unroll
-    for (int j = 0; j < ATTN_BN; j += 2) {              // probabilities as bf16 pairs, into the front half of the registers
-      const uint64_t e2 = fma2(pack2(__uint_as_float(sr[j]), __uint_as_float(sr[j + 1])), sl2_2, mb_2);
-      float p0, p1;
-      unpack2(e2, p0, p1);
-      p0 = exp2_fast(p0); p1 = exp2_fast(p1);
-      s2[(j >> 1) & 1] = add2(s2[(j >> 1) & 1], pack2(p0, p1));
-      __nv_bfloat162 h2 = __floats2bfloat162_rn(p0, p1);
-      sr[j >> 1] = *reinterpret_cast<uint32_t*>(&h2);
-    }
-    {
-      float x0, x1;
-      unpack2(add2(s2[0], s2[1]), x0, x1);
-      l_run = l_run * alpha + (x0 + x1);
-    }
-    m_run = mx;
+    attn_softmax_block(sr, a.scale_log2e, m_run, l_run, alpha);
     if (blk > 0) {
       mbar_wait(c, bar_o, ph ^ 1u);                     // P V (blk-1) complete: P, O and its V^T buffer are free
       __syncwarp();
       tc_fence_after();
       // rescale O where a row maximum moved (warp-uniform decision: the TMEM accesses are warp-wide)
-      if (__any_sync(0xffffffffu, alpha != 1.0f)) {
-#pragma unroll 1
-        for (int c0 = 0; c0 < a.hs; c0 += 16) {
-          float o[16];
-          tmem_ld16(tmem_o + lane_off + (uint32_t)c0, o);
-#pragma unroll
-          for (int j = 0; j < 16; ++j) o[j] *= alpha;
-          tmem_st16(tmem_o + lane_off + (uint32_t)c0, o);
-        }
-      }
+      if (__any_sync(0xffffffffu, alpha != 1.0f)) attn_rescale(tmem_o + lane_off, a.hs, alpha);
     }
     if (warp == 3 && lane == 0 && more && loads_on) attn_load_v(c, a, kv, g, blk + 1);
     __syncwarp();

@@ -58,62 +58,10 @@ inline OpFault& op_fault() {
 
 }  // namespace vla
 
+#include "op_attention.cuh"
 #include "op_linear.cuh"
 
 namespace vla {
-
-__device__ __forceinline__ TileCtx op_tile_ctx(char* smem, char* ctl, uint32_t tmem, const void* maps, unsigned* err,
-                                               OpFault fault) {
-  TileCtx tc;
-  tc.arena = nullptr;          // Refs of the stand-alone operators are absolute device addresses
-  tc.slot_base = 0;
-  tc.smem = smem;
-  tc.smem_bytes = 0;
-  tc.wait_word = nullptr;
-  tc.slot = nullptr;
-  tc.cont = 0;
-  tc.ctl = ctl;
-  tc.tmem = tmem;
-  tc.bar_id = 1;
-  tc.error = err;
-  tc.tmaps = maps;
-  tc.inputs = nullptr;
-  tc.amap_base = 0;
-  tc.drop_loads = fault.drop_loads;
-  tc.deadline = gtimer() + fault.wait_limit_ns;
-  return tc;
-}
-
-__global__ void __launch_bounds__(WORKER_THREADS) vla_op_attention_kernel(AttnArgs a, const __grid_constant__ OpMaps maps,
-                                                                          int tmem_cols, unsigned* err, OpFault fault) {
-  extern __shared__ __align__(1024) char smem_raw[];
-  __shared__ uint32_t tmem_base_s;
-  __shared__ __align__(16) char ctl_block[1024];
-  if (threadIdx.x < 32) tmem_alloc(&tmem_base_s, (uint32_t)tmem_cols);
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  TileCtx tc = op_tile_ctx(smem_raw, ctl_block, tmem_base_s, &maps, err, fault);
-  tile_attention(tc, a, (int)blockIdx.x);
-  tc_fence_before();
-  __syncthreads();
-  if (threadIdx.x < 32) tmem_dealloc(tmem_base_s, (uint32_t)tmem_cols);
-}
-
-// vt[c][t] = v[t][c] for a bf16 matrix v [rows, cols] (row pitch ldv), vt row pitch ldt.
-__global__ void vla_op_transpose_kernel(const unsigned short* v, unsigned short* vt, int rows, int cols, int ldv, int ldt) {
-  __shared__ unsigned short tile[32][33];
-  const int c0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
-  for (int i = threadIdx.y; i < 32; i += blockDim.y) {
-    int r = r0 + i, c = c0 + threadIdx.x;
-    tile[i][threadIdx.x] = (r < rows && c < cols) ? v[(size_t)r * ldv + c] : (unsigned short)0;
-  }
-  __syncthreads();
-  for (int i = threadIdx.y; i < 32; i += blockDim.y) {
-    int c = c0 + i, r = r0 + threadIdx.x;
-    if (c < cols && r < rows) vt[(size_t)c * ldt + r] = tile[threadIdx.x][i];
-  }
-}
 
 constexpr size_t OP_ATTN_HEADER = 256;   // error word + padding in front of V^T
 
@@ -138,6 +86,7 @@ inline OpDevice* op_device() {
     if (cudaGetSymbolAddress(&a, g_op_linear_error) != cudaSuccess || !a) return nullptr;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return nullptr;
     if (cudaFuncSetAttribute(vla_op_linear_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, LIN_SMEM) != cudaSuccess) return nullptr;
+    if (cudaFuncSetAttribute(vla_op_attention_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 224 * 1024) != cudaSuccess) return nullptr;
     d.sms = sms;
     d.error.store(static_cast<unsigned*>(a), std::memory_order_release);
   }
@@ -162,16 +111,11 @@ inline size_t op_attention_scratch_bytes(int tkv, int hkv, int hd) {
   return OP_ATTN_HEADER + (size_t)hkv * hd * (size_t)op_pad(tkv, 64) * 2;
 }
 
-// Shared implementation of the two attention entry points: `scratch` holds an error word and V^T.
+// Shared implementation of the two attention entry points: the first word of `scratch` is the call's error word.
 inline int op_attention_run(const void* q, const void* k, const void* v, void* out, int tq, int tkv, int hq, int hkv, int hd,
                             int causal, void* scratch, cudaStream_t s) {
-  const int64_t tpad = op_pad(tkv, 64);
-  unsigned* err = static_cast<unsigned*>(scratch);
-  unsigned short* vt = reinterpret_cast<unsigned short*>(static_cast<char*>(scratch) + OP_ATTN_HEADER);
-  if (cudaMemsetAsync(scratch, 0, OP_ATTN_HEADER, s) != cudaSuccess) return VLA_ERR_CUDA;
-  dim3 tb(32, 8), tg((unsigned)((hkv * hd + 31) / 32), (unsigned)((tkv + 31) / 32));
-  vla_op_transpose_kernel<<<tg, tb, 0, s>>>(static_cast<const unsigned short*>(v), vt, tkv, hkv * hd, hkv * hd, (int)tpad);
-
+  OpDevice* dev = op_device();
+  if (!dev) return VLA_ERR_CUDA;
   AttnArgs a;
   memset(&a, 0, sizeof a);
   a.out = reinterpret_cast<Ref>(out);
@@ -183,20 +127,24 @@ inline int op_attention_run(const void* q, const void* k, const void* v, void* o
   a.hpt = attn_fold(tq, hq, hkv, &a.rph);
   const int n_tiles = a.hpt > 1 ? hkv * (((hq / hkv) + a.hpt - 1) / a.hpt) : hq * a.q_blocks;
   a.scale_log2e = 1.4426950408889634f / sqrtf((float)hd);
-  a.qmap = 0; a.k0map = 1; a.v0map = 2; a.k1map = 1; a.v1map = 2;
   OpMaps maps;
-  memset(&maps, 0, sizeof maps);
   if (!op_encode(&maps.m[0], q, tq, (int64_t)hq * hd, (int64_t)hq * hd, a.hpt > 1 ? a.rph : 128) ||
       !op_encode(&maps.m[1], k, tkv, (int64_t)hkv * hd, (int64_t)hkv * hd, a.bn) ||
-      !op_encode(&maps.m[2], vt, (int64_t)hkv * hd, tkv, tpad, hd))
+      !op_encode(&maps.m[2], v, tkv, (int64_t)hkv * hd, (int64_t)hkv * hd, a.bn))
     return VLA_ERR_CUDA;
-  const int smem = attn_smem_bytes(hd);
-  int tmem_cols = 32;
-  while (tmem_cols < attn_tmem_cols(hd)) tmem_cols <<= 1;
-  if (cudaFuncSetAttribute(vla_op_attention_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
-    return VLA_ERR_CUDA;
-  vla_op_attention_kernel<<<n_tiles, WORKER_THREADS, smem, s>>>(a, maps, tmem_cols, err, op_fault());
-  return cudaGetLastError() == cudaSuccess ? VLA_OK : VLA_ERR_CUDA;
+  const OpAttnLaunch p = opa_plan(n_tiles, tkv, hd, dev->sms);
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute at[1];
+  cfg.gridDim = dim3((unsigned)(n_tiles * p.split));
+  cfg.blockDim = dim3(OPA_THREADS);
+  cfg.dynamicSmemBytes = (size_t)p.smem;
+  cfg.stream = s;
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = (unsigned)p.split; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, vla_op_attention_kernel, (const AttnArgs)a, (const OpMaps)maps, (const OpAttnLaunch)p, static_cast<unsigned*>(scratch), op_fault()) == cudaSuccess
+             ? VLA_OK : VLA_ERR_CUDA;
 }
 
 }  // namespace vla
