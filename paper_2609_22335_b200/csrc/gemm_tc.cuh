@@ -492,6 +492,9 @@ __device__ __forceinline__ void preload_rows(const TileCtx& c, const GemmArgs& g
   tmem_st_wait();
 }
 
+// The producer of a node's first token tile asks the L2 for weights this many k-blocks ahead: they come from HBM once per
+// frame, and two to four stages do not cover that latency.
+constexpr int GEMM_AHEAD = 6;
 constexpr int GEMM_W_STAGE_BYTES = GEMM_BM * GEMM_BK * 2;
 
 // The producer lane's look at the worker's next tile (see tile_gemm).  Not while another worker of the SM waits for room (this
@@ -617,6 +620,7 @@ __device__ __forceinline__ void tile_gemm(const TileCtx& c, const GemmArgs& g, i
         if (!(go = mbar_wait(c, bar + 8u * (uint32_t)S, ph ^ 1u))) break;
         load_w(kb, bar, dst);
         load_a(kb, bar, dst);
+        if (t0 == 0 && !c.wait_word && kb + GEMM_AHEAD < nkb) tma_prefetch_2d(wmap, (kb + GEMM_AHEAD) * GEMM_BK, r0);
         if (++s == S) { s = 0; ph ^= 1u; }
       }
       // While this tile's last MMAs and its epilogue run, the stages would stand empty: if the tile this worker runs next is

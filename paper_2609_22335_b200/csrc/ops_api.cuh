@@ -101,6 +101,22 @@ inline int op_status_of(const unsigned* dev_word, cudaStream_t s, unsigned call 
   return (call ? v != call : v == 0) ? VLA_OK : VLA_ERR_TIMEOUT;       // (call: the number that would mean a time-out)
 }
 
+// Launches a kernel in clusters of `cluster` blocks (1: none).
+template <typename... P, typename... A>
+inline int op_launch(void (*kernel)(P...), int grid, int threads, int smem, int cluster, cudaStream_t s, const A&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute at[1];
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = (size_t)smem;
+  cfg.stream = s;
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = (unsigned)cluster; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = cluster > 1 ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...) == cudaSuccess ? VLA_OK : VLA_ERR_CUDA;
+}
+
 inline int64_t op_pad(int64_t x, int64_t m) { return (x + m - 1) / m * m; }
 
 inline bool op_attention_shape_ok(int tq, int tkv, int hq, int hkv, int hd) {
@@ -133,18 +149,7 @@ inline int op_attention_run(const void* q, const void* k, const void* v, void* o
       !op_encode(&maps.m[2], v, tkv, (int64_t)hkv * hd, (int64_t)hkv * hd, a.bn))
     return VLA_ERR_CUDA;
   const OpAttnLaunch p = opa_plan(n_tiles, tkv, hd, dev->sms);
-  cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute at[1];
-  cfg.gridDim = dim3((unsigned)(n_tiles * p.split));
-  cfg.blockDim = dim3(OPA_THREADS);
-  cfg.dynamicSmemBytes = (size_t)p.smem;
-  cfg.stream = s;
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = (unsigned)p.split; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, vla_op_attention_kernel, (const AttnArgs)a, (const OpMaps)maps, (const OpAttnLaunch)p, static_cast<unsigned*>(scratch), op_fault()) == cudaSuccess
-             ? VLA_OK : VLA_ERR_CUDA;
+  return op_launch(vla_op_attention_kernel, n_tiles * p.split, OPA_THREADS, p.smem, p.split, s, a, maps, p, static_cast<unsigned*>(scratch), op_fault());
 }
 
 }  // namespace vla
@@ -175,15 +180,15 @@ int vla_op_linear(const void* a, const void* w, float* out32, void* out16, int32
   LinearArgs g;
   g.m = m; g.n = n; g.kp = (int)op_pad(k, GEMM_BK); g.act = act;
   g.out32 = out32; g.out16 = static_cast<unsigned short*>(out16);
-  g.vec16 = n % 16 == 0 && ((reinterpret_cast<uintptr_t>(out32) | reinterpret_cast<uintptr_t>(out16)) & 15) == 0;
+  g.vec8 = n % 8 == 0 && ((reinterpret_cast<uintptr_t>(out32) | reinterpret_cast<uintptr_t>(out16)) & 15) == 0;
   linear_plan(g, dev->sms);
   g.err = dev->error.load(std::memory_order_relaxed);
   g.call = dev->calls.fetch_add(1u, std::memory_order_relaxed) + 1u;
   OpMaps maps;
   if (!op_encode(&maps.m[0], w, n, k, k, g.bn) || !op_encode(&maps.m[1], a, m, k, k, g.bm)) return VLA_ERR_CUDA;
-  const int grid = g.tiles < 2 * dev->sms ? g.tiles : 2 * dev->sms;
-  vla_op_linear_kernel<<<grid, LIN_THREADS, linear_smem(g), static_cast<cudaStream_t>(stream)>>>(g, maps, op_fault());
-  return cudaGetLastError() == cudaSuccess ? VLA_OK : VLA_ERR_CUDA;
+  const int grid = g.ks > 1 ? g.tiles * g.ks : (g.tiles < 2 * dev->sms ? g.tiles : 2 * dev->sms);
+  const int rc = op_launch(vla_op_linear_kernel, grid, LIN_THREADS, linear_smem(g), g.ks, static_cast<cudaStream_t>(stream), g, maps, op_fault());
+  return rc;
 }
 
 int vla_debug_op_fault(int32_t drop_operand_loads, uint64_t wait_limit_ns) {

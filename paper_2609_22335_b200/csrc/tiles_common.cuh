@@ -148,9 +148,9 @@ __device__ __forceinline__ float tanh_fast(float x) {
   asm("tanh.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
-__device__ __forceinline__ float gelu_tanh_f(float x) {
-  const float c = 0.7978845608028654f;
-  return 0.5f * x * (1.0f + tanh_fast(c * (x + 0.044715f * x * x * x)));
+__device__ __forceinline__ float gelu_tanh_f(float x) {     // 0.5 x (1 + tanh(c x + c 0.044715 x^3))
+  const float c = 0.7978845608028654f, h = 0.5f * x;
+  return fmaf(h, tanh_fast(x * fmaf(x * x, c * 0.044715f, c)), h);
 }
 __device__ __forceinline__ float silu_f(float x) { return __fdividef(x, 1.0f + __expf(-x)); }
 template <int ACT>
