@@ -79,9 +79,9 @@ __device__ __forceinline__ uint64_t umma_desc_sw128(uint32_t saddr) {
   d |= (uint64_t)2 << 61;                 // SWIZZLE_128B
   return d;
 }
-// Instruction descriptor: bf16 x bf16 -> fp32, both operands K-major, M = 128, N = n.
-__device__ __forceinline__ uint32_t umma_idesc_bf16(int n) {
-  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(GEMM_BM >> 4) << 24);
+// Instruction descriptor: bf16 x bf16 -> fp32, both operands K-major, M = m (128, or 64: 16 rows per 32 tensor-memory lanes), N = n.
+__device__ __forceinline__ uint32_t umma_idesc_bf16(int n, int m = 128) {
+  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
 }
 __device__ __forceinline__ void umma_bf16(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
   asm volatile(
@@ -406,12 +406,11 @@ __device__ __forceinline__ void epi_general(const TileCtx& c, const GemmArgs& g,
   if (ssq && live) ssq[tok * g.ss_out_ld + ft] = sq;
 }
 
-// This warp's tokens of the tile.  t0: the tile's first token, nt: its tokens, r0: its first weight row, rs: row scale of the
-// token in this lane.
-__device__ __forceinline__ void gemm_epilogue(const TileCtx& c, const GemmArgs& g, uint32_t tmem, int t0, int nt, int warp, int lane, int r0, float rs,
-                                              int ft) {
+// This warp's tokens of the tile: `live` of them from `tok` on.  r0: the tile's first weight row, rs: row scale of the token
+// in this lane.
+__device__ __forceinline__ void gemm_epilogue(const TileCtx& c, const GemmArgs& g, uint32_t tmem, int tok, int live, int lane, int r0, float rs, int ft) {
   EpiPlace e;
-  e.tmem = tmem; e.tok = t0 + 32 * warp; e.live = nt - 32 * warp; e.lane = lane; e.r0 = r0; e.rs = rs;
+  e.tmem = tmem; e.tok = tok; e.live = live; e.lane = lane; e.r0 = r0; e.rs = rs;
   e.cols = min(GEMM_BM, (g.dual ? 2 * g.N : g.N) - r0);
   if (!g.fast) { epi_general(c, g, e, ft); return; }
   unsigned short* const out16 = resolve<unsigned short>(c, g.out16);
@@ -442,15 +441,17 @@ __device__ __forceinline__ void gemm_epilogue(const TileCtx& c, const GemmArgs& 
   }
 }
 
-// Addends of the tile's tokens into the accumulators (fragment layout; columns past the last feature get zero).  All loads of
-// an addend and a 32-column group go out before the first of them is used.
-__device__ __forceinline__ void preload_rows(const TileCtx& c, const GemmArgs& g, uint32_t tmem, int t0, int nt, int warp, int lane, int r0) {
+// Addends of the warp's tokens (`live` from `tok` on) into the accumulators (fragment layout; columns past the last feature
+// get zero).  Two fragments at a time, all loads of an addend before the first use: 32 tokens x 32 columns, or with up to 64
+// tokens in the tile (16 per warp) 16 x 64.
+__device__ __forceinline__ void preload_rows(const TileCtx& c, const GemmArgs& g, uint32_t tmem, int tok, int live, int tpw, int lane, int r0) {
   const int q = lane & 3, cols = min(GEMM_BM, g.N - r0), under = g.under;
+  const int dcol = tpw == 16 ? 32 : 0;                 // second fragment: that many columns on, or (0) 16 tokens on
   int row[4];                                          // (lanes past the last token read that one)
 #pragma unroll
-  for (int k = 0; k < 4; ++k) row[k] = t0 + min(32 * warp + 8 * k + (lane >> 2), nt - 1);
+  for (int k = 0; k < 4; ++k) row[k] = tok + min(((8 * k) & (tpw - 1)) + (lane >> 2), live - 1);
 #pragma unroll 1
-  for (int c0 = 0; c0 < cols; c0 += 32) {
+  for (int c0 = 0; c0 < cols; c0 += 32 + dcol) {
     float v[4][8];
 #pragma unroll
     for (int k = 0; k < 4; ++k)
@@ -458,12 +459,14 @@ __device__ __forceinline__ void preload_rows(const TileCtx& c, const GemmArgs& g
       for (int j = 0; j < 8; ++j) v[k][j] = 0.f;
     const int f = r0 + c0 + 8 * q;
     if (c0 + 8 * q < cols) {
+      const bool in2 = c0 + dcol + 8 * q < cols;
+      const int f2 = in2 ? f + dcol : f;
       auto add = [&](Ref ref, int ld) {                // ld 0: the same row for every token
-        const float* p = resolve<const float>(c, ref) + f;
+        const float* p = resolve<const float>(c, ref);
         float4 t[4][2];
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-          const float4* x = reinterpret_cast<const float4*>(p + (size_t)row[k] * ld);
+          const float4* x = reinterpret_cast<const float4*>(p + (size_t)row[k] * ld + (k < 2 ? f : f2));
           t[k][0] = __ldcg(x); t[k][1] = __ldcg(x + 1);
         }
 #pragma unroll
@@ -480,13 +483,18 @@ __device__ __forceinline__ void preload_rows(const TileCtx& c, const GemmArgs& g
           add(which == 1 ? g.bias : (which == 2 ? g.vec : (which == 8 ? g.tab : g.tab2)), which == 8 ? g.ldtab : (which == 16 ? g.ldtab2 : 0));
         }
       }
+      if (!in2) {
+#pragma unroll
+        for (int j = 0; j < 8; ++j) v[2][j] = v[3][j] = 0.f;
+      }
     }
+    const uint32_t t0 = tmem + (uint32_t)c0, dt = dcol ? 32u : (16u << 16);
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       const float* a = v[2 * h];
       const float* b = v[2 * h + 1];
       const float w[EPI] = {a[0], a[1], b[0], b[1], a[2], a[3], b[2], b[3], a[4], a[5], b[4], b[5], a[6], a[7], b[6], b[7]};
-      tmem_st_frag(tmem + ((uint32_t)(16 * h) << 16) + (uint32_t)c0, w);
+      tmem_st_frag(t0 + h * dt, w);
     }
   }
   tmem_st_wait();
@@ -582,13 +590,17 @@ __device__ __forceinline__ void tile_gemm(const TileCtx& c, const GemmArgs& g, i
   }
   if (c.wait_word) worker_sync(c);                     // nobody reads an operand before the release
 
-  const bool warp_live = warp * 32 < nt;
+  // Tokens per warp.  A tile of at most 64 tokens uses M = 64, whose rows lie 16 to each warp's 32 TMEM lanes: all four warps
+  // share its addends and its epilogue, where M = 128 left them to the first two (50-token head tiles: 6.5k cycles after the
+  // main loop -> 4.5k; single frame 12.63 -> 12.08 ms, 32 streams x 2 cameras 191.7 -> 186.0 ms).
+  const int tpw = bt <= 64 ? 16 : 32;
+  const bool warp_live = warp * tpw < nt;
   const uint32_t my_tmem = c.tmem + ((uint32_t)(warp * 32) << 16);
   // What is added to the product goes into the accumulators before the first MMA: its round trip then lies beside that of
   // the first operand stages, and the epilogue neither reads nor adds anything.
   const bool under = g.under != 0;
   if (under) {
-    if (warp_live) preload_rows(c, g, my_tmem, t0, nt, warp, lane, r0);
+    if (warp_live) preload_rows(c, g, my_tmem, t0 + tpw * warp, min(tpw, nt - tpw * warp), tpw, lane, r0);
     tc_fence_before();
   }
   // Folded RMSNorm: the partial sums of squares of this lane's token are requested now and added after the main loop, in a
@@ -598,7 +610,7 @@ __device__ __forceinline__ void tile_gemm(const TileCtx& c, const GemmArgs& g, i
 #pragma unroll
   for (int j = 0; j < 8; ++j) part[j] = 0.f;
   if (scaled) {
-    const float* sp = resolve<const float>(c, g.ss_in) + (size_t)(t0 + min(worker_tid(), nt - 1)) * g.ss_nft;
+    const float* sp = resolve<const float>(c, g.ss_in) + (size_t)(t0 + min(tpw * warp + lane, nt - 1)) * g.ss_nft;
 #pragma unroll
     for (int j = 0; j < 8; ++j)
       if (j < g.ss_nft) part[j] = ld_act(sp + j);
@@ -632,7 +644,7 @@ __device__ __forceinline__ void tile_gemm(const TileCtx& c, const GemmArgs& g, i
     __syncwarp();
   } else if (warp == 1) {
     // ---------------- MMA issuer (the whole warp walks the loop, one elected lane issues)
-    const uint32_t idesc = umma_idesc_bf16(GEMM_BM);
+    const uint32_t idesc = umma_idesc_bf16(GEMM_BM, bt <= 64 ? 64 : 128);
     const uint64_t desc0 = umma_desc_sw128(stage0);
     uint32_t ph = ph0;
     int s = s0;
@@ -663,7 +675,7 @@ __device__ __forceinline__ void tile_gemm(const TileCtx& c, const GemmArgs& g, i
     for (int j = 0; j < 8; ++j) ssq += part[j];
     rs = 1.0f / sqrtf(ssq / (float)g.rs_d + 1e-6f);
   }
-  if (ready && warp_live) gemm_epilogue(c, g, my_tmem, t0, nt, warp, lane, r0, rs, ft);
+  if (ready && warp_live) gemm_epilogue(c, g, my_tmem, t0 + tpw * warp, min(tpw, nt - tpw * warp), lane, r0, rs, ft);
   tc_fence_before();
   worker_sync(c);
   if (!(c.slot && c.slot->primed) && worker_tid() <= 2 * S) mbar_inval(bar0 + 8u * worker_tid());
