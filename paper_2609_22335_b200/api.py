@@ -435,12 +435,17 @@ def op_attention(q, k, v, hq, hkv, hd, causal=False, scratch=None, stream=None):
 
 def op_linear(a, w, act=0, out_bf16=False, stream=None):
     """a [m,k], w [n,k]: CUDA bf16 torch tensors.  Returns act(a w^T) as fp32 (or bf16) [m,n]."""
-    import torch
+    import torch                               # (the call's host time is what a small layer costs: nothing is looked up twice)
     m, k = a.shape
     n = w.shape[0]
-    out = torch.empty((m, n), dtype=torch.bfloat16 if out_bf16 else torch.float32, device=a.device)
-    rc = load_library().vla_op_linear(a.data_ptr(), w.data_ptr(), None if out_bf16 else out.data_ptr(),
-                                      out.data_ptr() if out_bf16 else None, m, n, k, act, _stream_ptr(stream))
+    if out_bf16:
+        out = a.new_empty((m, n), dtype=torch.bfloat16)
+        p32, p16 = None, out.data_ptr()
+    else:
+        out = a.new_empty((m, n), dtype=torch.float32)
+        p32, p16 = out.data_ptr(), None
+    rc = (_lib or load_library()).vla_op_linear(a.data_ptr(), w.data_ptr(), p32, p16, m, n, k, act,
+                                                None if stream is None else stream.cuda_stream)
     if rc != VLA_OK:
         raise VlaError(rc, "vla_op_linear failed")
     return out
