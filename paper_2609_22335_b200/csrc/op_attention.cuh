@@ -94,15 +94,18 @@ __global__ void __launch_bounds__(OPA_THREADS) vla_op_attention_kernel(const __g
       mbar_init(bar0 + 8u * lane, is_p ? 4 : 1);
       asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (lane == 0) { failed_s = 0; if (blockIdx.x == 0) *err = 0u; }
+    if (lane == 0) failed_s = 0;
   } else if (warp == 5) {
     tmem_alloc(&tmem_base_s, (uint32_t)p.tmem_cols);
   }
+  op_wait_previous(maps, 3);
+  if (threadIdx.x == 0 && blockIdx.x == 0) *err = 0u;
   TileCtx c;                                    // (what the bounded waits look at)
   c.error = &failed_s;
   c.deadline = gtimer() + fault.wait_limit_ns;
   tc_fence_before();
   __syncthreads();
+  op_let_next_start();
   tc_fence_after();
   const uint32_t tmem = tmem_base_s, tmem_o = tmem + 2u * ATTN_BN;     // two score buffers, then O
 

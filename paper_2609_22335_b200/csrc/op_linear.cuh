@@ -167,11 +167,13 @@ __global__ void __launch_bounds__(LIN_THREADS, 2) vla_op_linear_kernel(const __g
   } else if (warp == 1) {
     tmem_alloc(&tmem_base_s, LIN_TMEM_COLS);
   }
+  op_wait_previous(maps, 2);
   TileCtx c;                                   // (what the bounded waits look at)
   c.error = &failed_s;
   c.deadline = gtimer() + fault.wait_limit_ns;
   tc_fence_before();
   __syncthreads();
+  op_let_next_start();
   tc_fence_after();
   const uint32_t tmem = tmem_base_s;
   bool ok = true;

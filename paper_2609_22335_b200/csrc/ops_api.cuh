@@ -56,6 +56,19 @@ inline OpFault& op_fault() {
   return f;
 }
 
+// Start of an operator kernel.  A call's kernel is launched while the previous one on the stream is still running (programmatic
+// stream serialisation, op_launch): barriers, tensor memory and descriptors are set up behind that one's last tiles, and
+// nothing of global memory is touched before op_wait_previous has returned, that is before all earlier work on the stream is
+// complete and visible.  op_let_next_start lets the next call's kernel do the same.  It takes effect once every block of this
+// grid has come to it, and stands behind the block's tensor-memory allocation: a block that waits for this grid can then
+// neither keep one of its blocks out nor hold columns that one of them still needs.  Back to back: linear 50x2048x720
+// 8.2 -> 6.1 us, 288x11008x4096 45.9 -> 43.9, attention 1024x1024 (12 heads of 64) 16.4 -> 14.5.
+__device__ __forceinline__ void op_wait_previous(const OpMaps& maps, int n) {
+  if ((int)threadIdx.x < n) asm volatile("prefetch.tensormap [%0];" ::"l"(&maps.m[threadIdx.x]) : "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+__device__ __forceinline__ void op_let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 }  // namespace vla
 
 #include "op_attention.cuh"
@@ -101,19 +114,22 @@ inline int op_status_of(const unsigned* dev_word, cudaStream_t s, unsigned call 
   return (call ? v != call : v == 0) ? VLA_OK : VLA_ERR_TIMEOUT;       // (call: the number that would mean a time-out)
 }
 
-// Launches a kernel in clusters of `cluster` blocks (1: none).
+// Launches a kernel in clusters of `cluster` blocks (1: none), overlapping the end of the kernel in front of it
+// (op_wait_previous).
 template <typename... P, typename... A>
 inline int op_launch(void (*kernel)(P...), int grid, int threads, int smem, int cluster, cudaStream_t s, const A&... args) {
   cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute at[1];
+  cudaLaunchAttribute at[2];
   cfg.gridDim = dim3((unsigned)grid);
   cfg.blockDim = dim3((unsigned)threads);
   cfg.dynamicSmemBytes = (size_t)smem;
   cfg.stream = s;
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = (unsigned)cluster; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  at[1].id = cudaLaunchAttributeClusterDimension;
+  at[1].val.clusterDim.x = (unsigned)cluster; at[1].val.clusterDim.y = 1; at[1].val.clusterDim.z = 1;
   cfg.attrs = at;
-  cfg.numAttrs = cluster > 1 ? 1 : 0;
+  cfg.numAttrs = cluster > 1 ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...) == cudaSuccess ? VLA_OK : VLA_ERR_CUDA;
 }
 
