@@ -12,9 +12,11 @@
 // a multiple of 16 (72 -> 80) costs only its padding.  All waits are bounded.
 //
 // What bounds it: one tile alone is a chain of barrier tests, MMA issue and tensor-memory round trips around 800 cycles of
-// softmax per block.  So S of block b+1 is issued as soon as the scores of block b are in registers (warp 0), P V of block b
-// by warp 1, and the loads run two blocks (K) and one block (V) ahead on warps 2 and 3: 3560 -> 3010 cycles per block of a
-// tile alone on its SM, 52 -> 40 us for a 16-block tile among three.
+// softmax per block.  So S of block b+1 is issued as soon as the scores of block b are in registers (warp 0), and the loads run
+// two blocks (K) and one block (V) ahead on warps 2 and 3: 3560 -> 3010 cycles per block of a tile alone on its SM, 52 -> 40 us
+// for a 16-block tile among three.  Warp 1 issues P V of block b-1 behind its reading of S, where it no longer delays S of the
+// next block, and warps 2 and 3, which issue nothing, wait for K and V on the issuers' behalf (a test of a barrier that is
+// ready costs 160-190 cycles): single frame 12.07 -> 11.98 ms, 4 x 2 pi0 streams 77.9 -> 77.3.
 #pragma once
 #include "gemm_tc.cuh"
 
@@ -222,23 +224,42 @@ __device__ __forceinline__ void tile_attention(const TileCtx& c, const AttnArgs&
   const uint32_t tmem_s = c.tmem;                            // S: columns [0, 64)
   const uint32_t tmem_p = c.tmem + (uint32_t)ATTN_BN;        // P: 32 columns of bf16 pairs
   const uint32_t tmem_o = tmem_p + (uint32_t)ATTN_BN / 2;    // O: hs columns
+  // Low words of the descriptors a warp issues from, worked out once: warp 0 Q and K, warp 1 V^T.
+  const uint64_t desc_hi = umma_desc_sw128(0u);
+  uint32_t lo_k, lo_q, step;
+  {
+    const AttnSmem m = attn_smem(c, a);
+    lo_q = m.q >> 4; lo_k = (warp == 1 ? m.v : m.k) >> 4; step = (warp == 1 ? m.v_bytes : m.k_bytes) >> 4;
+  }
+  const int hs16 = a.hs / 16;
   auto issue_s = [&](uint32_t buf) {                         // warp 0, converged: S of the K block in `buf`
     tc_fence_after();
-    const AttnSmem m = attn_smem(c, a);
     const uint32_t idesc_s = umma_idesc_bf16(ATTN_BN);
-    const int hs = a.hs;
-    uint64_t qd = umma_desc_sw128(m.q), kd = umma_desc_sw128(m.k + buf * m.k_bytes);
+    uint64_t qd = desc_hi + lo_q, kd = desc_hi + (lo_k + buf * step);
     if (elect_one()) {
       int kc = 0;
 #pragma unroll 1
-      for (; kc + 4 <= hs / 16; kc += 4) {                   // one 64-column box
+      for (; kc + 4 <= hs16; kc += 4) {                      // one 64-column box
 #pragma unroll
         for (int k = 0; k < 4; ++k) umma_bf16(tmem_s, qd + 2u * k, kd + 2u * k, idesc_s, (kc | k) != 0 ? 1u : 0u);
         qd += (ATTN_BQ * 128) >> 4; kd += (ATTN_BN * 128) >> 4;
       }
 #pragma unroll 1
-      for (int k = 0; kc < hs / 16; ++kc, ++k) umma_bf16(tmem_s, qd + 2u * k, kd + 2u * k, idesc_s, kc != 0 ? 1u : 0u);
+      for (int k = 0; kc < hs16; ++kc, ++k) umma_bf16(tmem_s, qd + 2u * k, kd + 2u * k, idesc_s, kc != 0 ? 1u : 0u);
       umma_commit(bar_s);
+    }
+    __syncwarp();
+  };
+  auto issue_pv = [&](int blk) {                             // warp 1: O += P V of block blk, once every warp has its rows of P (and O) in place
+    const uint32_t ph = (uint32_t)blk & 1u;
+    if (!mbar_wait(c, met_p, ph)) return;
+    tc_fence_after();
+    const uint32_t idesc_o = umma_idesc_bf16(16) + ((uint32_t)(hs16 - 1) << 18);         // N = hs
+    const uint64_t vd = desc_hi + (lo_k + ph * step);
+    if (elect_one()) {
+#pragma unroll
+      for (int k = 0; k < ATTN_BN / 16; ++k) umma_bf16_ta(tmem_o, tmem_p + 8u * k, vd + 2u * k, idesc_o, (blk | k) != 0 ? 1u : 0u);
+      umma_commit(bar_o);
     }
     __syncwarp();
   };
@@ -260,12 +281,14 @@ __device__ __forceinline__ void tile_attention(const TileCtx& c, const AttnArgs&
     tmem_ld16_nowait(tmem_s + lane_off + 16u, sr + 16);
     tmem_ld16_nowait(tmem_s + lane_off + 32u, sr + 32);
     tmem_ld16_nowait(tmem_s + lane_off + 48u, sr + 48);
+    if (warp == 2 && more) mbar_wait(c, bar_k + 8u * (ph ^ 1u), ((uint32_t)(blk + 1) >> 1) & 1u);   // (its arrival tells warp 0)
     tmem_ld_wait();
     if (more) {                                         // the scores are in registers: the next block's go on their way
       tc_fence_before();
       arrive_warp(met_s, lane);
-      if (warp == 0 && mbar_wait(c, met_s, ph) && mbar_wait(c, bar_k + 8u * (ph ^ 1u), ((uint32_t)(blk + 1) >> 1) & 1u)) issue_s(ph ^ 1u);
+      if (warp == 0 && mbar_wait(c, met_s, ph)) issue_s(ph ^ 1u);
     }
+    if (warp == 1 && blk > 0) issue_pv(blk - 1);        // (only now: it runs under this softmax, and no other warp waited for warp 1)
     // ---- softmax of this block: one thread per query row.  Keys a row must not see get a score of -inf first (ragged,
     // diagonal and suffix blocks only), then every block runs the same straight code: three-input maxima, two-wide
     // multiply-adds and sums (660 -> 300 instructions per warp and block), which leaves the 64 exponentials as the bulk
@@ -289,27 +312,18 @@ __device__ __forceinline__ void tile_attention(const TileCtx& c, const AttnArgs&
       // rescale O where a row maximum moved (warp-uniform decision: the TMEM accesses are warp-wide)
       if (__any_sync(0xffffffffu, alpha != 1.0f)) attn_rescale(tmem_o + lane_off, a.hs, alpha);
     }
-    if (warp == 3 && lane == 0 && more && loads_on) attn_load_v(c, a, kv, g, blk + 1);
-    __syncwarp();
     tmem_st16u(tmem_p + lane_off, sr);
     tmem_st16u(tmem_p + lane_off + 16u, sr + 16);
+    if (warp == 3) {
+      if (lane == 0 && more && loads_on) attn_load_v(c, a, kv, g, blk + 1);
+      __syncwarp();
+      mbar_wait(c, bar_v + 8u * ph, ((uint32_t)blk >> 1) & 1u);                                      // (its arrival tells warp 1)
+    }
     tmem_st_wait();
     tc_fence_before();
-    // ---- O += P V, issued by warp 1 once every warp has its rows of P (and O) in place
     arrive_warp(met_p, lane);
-    if (warp == 1 && mbar_wait(c, met_p, ph) && mbar_wait(c, bar_v + 8u * ph, ((uint32_t)blk >> 1) & 1u)) {
-      tc_fence_after();
-      const AttnSmem m = attn_smem(c, a);
-      const uint32_t idesc_o = umma_idesc_bf16(a.hs);
-      const uint64_t vd = umma_desc_sw128(m.v + ph * m.v_bytes);
-      if (elect_one()) {
-#pragma unroll
-        for (int k = 0; k < ATTN_BN / 16; ++k) umma_bf16_ta(tmem_o, tmem_p + 8u * k, vd + 2u * k, idesc_o, (blk | k) != 0 ? 1u : 0u);
-        umma_commit(bar_o);
-      }
-      __syncwarp();
-    }
     if (!more) {
+      if (warp == 1) issue_pv(blk);
       mbar_wait(c, bar_o, ph);
       break;
     }
