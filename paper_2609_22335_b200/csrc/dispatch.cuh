@@ -142,7 +142,13 @@ __device__ __forceinline__ bool queue_entry(const DeviceCtx& ctx, int cls, unsig
 }
 
 // ------------------------------------------------------------------ per-SM state of the persistent kernel
-constexpr int DISPATCH_THREADS = 64;     // two service warps per SM (claim, retire), after the worker groups
+constexpr int DISPATCH_THREADS = 128;    // a warpgroup with the two service warps of the SM (claim, retire), after the worker groups
+// Registers a thread, after the split: the launch gives every thread 128 (four warps on each scheduler), and a tile body wants
+// more: what it spilled came back from L2, since the slab leaves L1 next to nothing.  The service warpgroup hands back what it
+// does not use: n * 144 + 80 <= (n + 1) * 128 for one, two and three workers.  120 -> 16 bytes of spills; single frame
+// 11.97 -> 11.58 ms, 32 streams x 4 184.2 -> 181.4.
+constexpr int WORKER_REGS = 144, DISPATCH_REGS = 80;
+static_assert(MAX_WORKERS * WORKER_REGS + DISPATCH_REGS <= (MAX_WORKERS + 1) * 128, "the split must not exceed what the block was launched with");
 constexpr long long PRIO_WINDOW_NS = 8000;   // an action-head tile may be claimed for a worker this close to the end of its tile
 constexpr int PREFETCH_MIN_TOTAL = 600;   // tiles are claimed ahead of need only while this many VLM tiles are queued in all
 constexpr int PREFETCH_MIN_AVAIL = 8;     // ... and only from queues at least this deep
@@ -766,8 +772,8 @@ __device__ __forceinline__ void take_tile(const DeviceCtx& ctx, SmState* sm, Wor
 }
 
 // ------------------------------------------------------------------ the persistent co-scheduling kernel
-// One CTA per SM: `workers` worker groups of WORKER_THREADS threads run tiles; one more warp is the
-// dispatcher.  Every wait is bounded by ctx.wait_limit_ns.
+// One CTA per SM: `workers` worker groups of WORKER_THREADS threads run tiles; of one more warpgroup two warps are the
+// dispatcher (claim, retire), two only bring their registers.  Every wait is bounded by ctx.wait_limit_ns.
 __global__ void __launch_bounds__(MAX_WORKERS* WORKER_THREADS + DISPATCH_THREADS, 1)
     vla_cosched_kernel(DeviceCtx ctx, int dyn_smem_bytes) {
   extern __shared__ __align__(1024) char smem_raw[];
@@ -817,9 +823,12 @@ __global__ void __launch_bounds__(MAX_WORKERS* WORKER_THREADS + DISPATCH_THREADS
   __syncthreads();
   tc_fence_after();
   if (is_dispatcher) {
-    if (threadIdx.x < n_workers * WORKER_THREADS + 32) claim_loop(ctx, sm, n_workers);
-    else retire_loop(ctx, sm, n_workers);
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(DISPATCH_REGS));
+    const int warp = (int)(threadIdx.x - n_workers * WORKER_THREADS) >> 5;
+    if (warp == 0) claim_loop(ctx, sm, n_workers);
+    else if (warp == 1) retire_loop(ctx, sm, n_workers);
   } else {
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(WORKER_REGS));
     // Nothing is carried in registers through a tile body (it has use for all of them): a pass of this loop derives its
     // place from the thread index again and keeps its few counters in the worker's slot.
     for (;;) {
