@@ -250,8 +250,9 @@ int vla_debug_guards(vla_ctx* ctx, int32_t fill, size_t* n_bad);
  * decoder layers and of the action head (Section 2.1, Figure 1).  q [tq, hq*hd], k and v [tkv, hkv*hd],
  * out [tq, hq*hd]: bf16, row-major, DEVICE, 16-byte aligned.  hd a multiple of 16, at most 256; hq a
  * multiple of hkv; causal (key j visible to query i iff j <= i) needs tq == tkv.
- * scratch: DEVICE, 256-byte aligned, at least vla_op_attention_scratch_bytes(); the call writes an error
- * word and the transposed copy of v there, so calls sharing a scratch buffer must not overlap on the GPU. */
+ * scratch: DEVICE, 256-byte aligned, at least vla_op_attention_scratch_bytes() (room for a transposed v, which
+ * today's kernel does not need); the call writes its error word there, so calls sharing a scratch buffer must not
+ * overlap on the GPU. */
 int vla_op_attention_scratch_bytes(int32_t tkv, int32_t hkv, int32_t hd, size_t* out_bytes);
 int vla_op_attention(const void* q, const void* k, const void* v, void* out, int32_t tq, int32_t tkv, int32_t hq,
                      int32_t hkv, int32_t hd, int32_t causal, void* scratch, size_t scratch_bytes, void* stream);
@@ -260,7 +261,7 @@ int vla_op_attention(const void* q, const void* k, const void* v, void* out, int
  * deployment convenience).  Some callers of this library are not allowed to call cudaMalloc or to hand over
  * a scratch buffer: code that runs inside a real-time control loop with a fixed memory budget, a plugin whose
  * host owns every allocation, or a process that must not touch the allocator after start-up.  For them the
- * scratch of vla_op_attention (an error word plus the transposed copy of v) lives in a fixed array in device
+ * scratch of vla_op_attention (an error word, and room for a transposed v) lives in a fixed array in device
  * memory that every GPU loading this library holds until the process exits.  The call allocates nothing:
  * no cudaMalloc, no cudaFree, no allocating library routine; the caller passes only inputs and outputs.
  * Limit: vla_op_attention_scratch_bytes(tkv, hkv, hd) must not exceed vla_op_attention_static_capacity()

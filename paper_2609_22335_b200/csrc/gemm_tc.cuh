@@ -5,15 +5,16 @@
 // Tile: up to 128 tokens (MMA M, one TMEM lane each) x 128 weight rows (MMA N, one
 // TMEM column each), K walked in 64-element stages, both operands K-major.  Where a node
 // has few tokens (the action head's 9..51) the activation box is only as high as they
-// need; the MMA reads on into the weight tile behind it and leaves lanes nobody looks at.
+// need; the MMA (M = 64 there) reads on into the weight tile behind it and leaves lanes
+// nobody looks at.
 // A gated MLP tile covers 64 output features: gate and up rows alternate in its weight
 // matrix, so it is one MMA stream and one accumulator like any other tile; the epilogue
 // multiplies act(gate) by up.
 //
 // Roles inside the 128-thread worker: thread 0 of warp 0 issues TMA loads,
-// warp 1 issues MMAs, all four warps run the epilogue (warp w reads
-// TMEM lanes 32w..32w+31, a token per thread).  Every mbarrier wait is bounded; on expiry
-// the worker records an error and leaves the tile.
+// warp 1 issues MMAs, all four warps run the epilogue (warp w reads TMEM lanes
+// 32w..32w+31 in 16x256b fragments: a quad of lanes holds 32 features of a token).  Every
+// mbarrier wait is bounded; on expiry the worker records an error and leaves the tile.
 #pragma once
 #include "tiles_common.cuh"
 

@@ -76,7 +76,7 @@ __device__ __forceinline__ void op_let_next_start() { asm volatile("griddepcontr
 
 namespace vla {
 
-constexpr size_t OP_ATTN_HEADER = 256;   // error word + padding in front of V^T
+constexpr size_t OP_ATTN_HEADER = 256;   // error word + padding (behind it: room a transposed V would take, which the sizes of the interface count)
 
 // What vla_op_linear keeps per device, looked up on the first call made with that device current: SM count, the error word
 // (in a fixed device array of the library) and the number of the latest call.  A kernel whose wait runs out writes its

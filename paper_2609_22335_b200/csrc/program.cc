@@ -446,7 +446,6 @@ class Builder {
     gemm(name + "qkv", A, W, nall, gq);
   }
 
-  int elem_node(NodeDesc& n, const std::string& name) { return add(n, name, KIND_ELEM); }
 
   int addrows(const std::string& name, const View& in, Ref in_raw, int ldi, int M, int N, Ref vec, Ref tab, int ldt,
               const View& out, const View& out16) {

@@ -165,12 +165,6 @@ int capture_graph(vla_ctx* c, int inst, int phase_sel, cudaStream_t s, cudaGraph
   return VLA_OK;
 }
 
-uint64_t count_phase_nodes(const Program& p, int phase_sel) {
-  uint64_t n = 0;
-  for (auto& nd : p.nodes) if (phase_sel < 0 || nd.phase == phase_sel) ++n;
-  return n;
-}
-
 int launch_persistent(vla_ctx* c) {
   // reset the control word in stream order, then launch one CTA per SM
   CU(cudaMemcpyAsync(&c->dctx.control->ctrl, c->zero_pinned, sizeof(unsigned), cudaMemcpyHostToDevice, c->sa));
@@ -863,7 +857,7 @@ int vla_destroy(vla_ctx* c) {
 #include "ops_api.cuh"
 
 // ------------------------------------------------------------------------------------------------
-// Attention without any allocation: the scratch of vla_op_attention (error word + transposed V)
+// Attention without any allocation: the scratch of vla_op_attention (error word + room for a transposed V)
 // lives in a fixed array in device memory that every GPU loading this library holds until exit.
 // In host code the array's name is only a handle; the device address is looked up once per device
 // with cudaGetSymbolAddress and that pointer is what the kernels receive.
@@ -905,7 +899,7 @@ int vla_op_attention_static(const void* q, const void* k, const void* v, void* o
   void* scratch = nullptr;
   int rc = static_scratch_for_current_device(&scratch);
   if (rc != VLA_OK) return rc;
-  // op_attention_run clears the error word itself; V^T is fully rewritten for the rows and tokens it reads
+  // (the kernel clears the error word itself)
   return vla::op_attention_run(q, k, v, out, tq, tkv, hq, hkv, hd, causal, scratch, static_cast<cudaStream_t>(stream));
 }
 

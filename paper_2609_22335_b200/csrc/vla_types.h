@@ -245,8 +245,6 @@ struct alignas(128) Control {    // polled words and hot counters live on separa
   unsigned long long admit_head; // admission records consumed
   unsigned long long admit_tail; // admission records published (written by host copies; read with admit_head by one load)
   unsigned long long pad1[14];
-  unsigned long long doorbell;   // bumped whenever tiles are committed to any queue
-  unsigned long long pad2[15];
   unsigned long long tiles_done;
   unsigned long long trace_count;
 };
