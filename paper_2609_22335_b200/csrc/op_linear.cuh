@@ -43,7 +43,10 @@ inline void linear_plan(LinearArgs& g, int sms) {
   g.bm = (int)(((g.m + g.tiles_m - 1) / g.tiles_m + 15) / 16 * 16);
   const int nkb = g.kp / GEMM_BK;
   double best = 1e300;
-  for (int bn = 256; bn >= 16; bn >>= 1)
+  // Widths: powers of two; with more tiles than the chip holds at once also the multiples of 16 above 128, which fill the last
+  // round better (4225 x 2304 x 768 28 -> 21 us, 9000 x 3000 x 264 45 -> 37, 8192 x 3072 x 768 48.2 -> 47.4).
+  const bool fine = (long long)g.tiles_m * ((g.n + 255) / 256) > 2 * sms;
+  for (int bn = 256; bn >= 16; bn = fine && bn > 128 ? bn - 16 : bn >> 1)
     for (int ks = 1; ks <= 8 && (ks == 1 || (bn >= 32 * ks && nkb >= 2 * ks)); ks <<= 1) {
       if (ks > 1 && 128 * (bn / ks) * (ks - 1) * 4 > linear_stages(g.bm, bn) * (g.bm + bn) * GEMM_BK * 2) continue;
       const long long tiles = (long long)g.tiles_m * ((g.n + bn - 1) / bn), ctas = tiles * ks;

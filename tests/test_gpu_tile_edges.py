@@ -24,7 +24,8 @@ def _rand(rng, shape, scale=1.0):
 @pytest.mark.parametrize("m,n,k", [
     (16, 16, 8), (17, 33, 8), (63, 31, 64), (64, 32, 72), (65, 40, 128),      # one k-block; heights around 64; widths around 32
     (50, 720, 2048), (50, 721, 2048), (1, 16, 4096), (128, 128, 8192),        # few tiles, long K: a cluster shares it
-    (129, 257, 1024), (300, 1000, 264), (2500, 1032, 136), (9000, 520, 64)])  # remainders; several tiles to a block
+    (129, 257, 1024), (300, 1000, 264), (2500, 1032, 136), (9000, 520, 64),            # remainders; several tiles to a block
+    (4100, 2500, 136), (7000, 1801, 72)])                                     # widths between 128 and 256
 @pytest.mark.parametrize("act,bf16", [(0, False), (1, True), (2, False)])
 def test_linear_at_tile_edges(m, n, k, act, bf16):
     import torch
