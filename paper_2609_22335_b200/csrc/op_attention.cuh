@@ -211,12 +211,15 @@ __global__ void __launch_bounds__(OPA_THREADS) vla_op_attention_kernel(const __g
       }
       float alpha;
       attn_softmax_block(sr, sl2, m_run, l_run, alpha);
-      // O follows a moved maximum (rarely); everything before has been added by then
-      if (i > 0 && __any_sync(0xffffffffu, alpha != 1.0f)) {
+      // O follows a moved maximum (rarely); everything before has been added by then.  The last block waits for P V of the one
+      // before it in any case: the wait behind the loop tells phases apart by parity, and this warp may be a whole block ahead
+      // of another one, whose part of that P V is still to come.  (P V of this block cannot start before this warp arrives.)
+      const bool moved = __any_sync(0xffffffffu, alpha != 1.0f);
+      if (i > 0 && (moved || i == n - 1)) {
         mbar_wait(c, bar_o, (uint32_t)(i - 1) & 1u);
         __syncwarp();
         tc_fence_after();
-        attn_rescale(tmem_o + my_lanes, hs, alpha);
+        if (moved) attn_rescale(tmem_o + my_lanes, hs, alpha);
       }
       tmem_st16u(buf, sr);
       tmem_st16u(buf + 16u, sr + 16);

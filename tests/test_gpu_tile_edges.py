@@ -65,6 +65,18 @@ def test_attention_at_block_edges(tq, tkv, hq, hkv, hd, causal):
     assert np.linalg.norm(err) / np.linalg.norm(ref) < 1e-2
 
 
+@pytest.mark.parametrize("t,hq,hd", [(1500, 20, 64), (640, 2, 128)])
+def test_attention_repeats_itself(t, hq, hd):
+    """Causal masks put a tile's warps a block apart; the last P V must be waited for all the same."""
+    import torch
+    from paper_2609_22335_b200 import api
+    rng = np.random.default_rng(t)
+    q, k, v = (_dev(_rand(rng, (t, hq * hd), 1.5)) for _ in range(3))
+    first = api.op_attention(q, k, v, hq, hq, hd, causal=True)
+    for _ in range(200):
+        assert torch.equal(api.op_attention(q, k, v, hq, hq, hd, causal=True), first)
+
+
 @pytest.mark.parametrize("m,n", [(1, 64), (50, 256), (300, 1024)])
 def test_calls_that_follow_one_another_see_each_others_results(m, n):
     """A call's kernel sets up while the previous one still runs; what it reads must be that one's finished output."""
