@@ -150,15 +150,18 @@ constexpr int DISPATCH_THREADS = 128;    // a warpgroup with the two service war
 constexpr int WORKER_REGS = 144, DISPATCH_REGS = 80;
 static_assert(MAX_WORKERS * WORKER_REGS + DISPATCH_REGS <= (MAX_WORKERS + 1) * 128, "the split must not exceed what the block was launched with");
 constexpr long long PRIO_WINDOW_NS = 8000;   // an action-head tile may be claimed for a worker this close to the end of its tile
-constexpr int PREFETCH_MIN_TOTAL = 600;   // tiles are claimed ahead of need only while this many VLM tiles are queued in all
+constexpr int PREFETCH_MIN_TOTAL = 300;   // tiles are claimed ahead of need only while this many VLM tiles are queued in all
+                                          // (32 streams x 4: 181.5 ms at 600, 178.9 at 300, no better at 150)
 constexpr int PREFETCH_MIN_AVAIL = 8;     // ... and only from queues at least this deep
 constexpr int HELD_DEPTH = 1;            // claimed tiles a worker may have waiting
 constexpr unsigned CLAIM_NAP_NS = 60, CLAIM_NAP_MAX_NS = 240;   // claim warp, while a worker of its SM has nothing to run
 constexpr unsigned CLAIM_SLEEP_NS = 2000;    // claim warp, every worker busy: longest sleep without a ring
 constexpr unsigned RETIRE_SLEEP_NS = 4000;   // retire warp: longest sleep without a ring
 // With no more tiles queued or running than the GPU has SMs, tiles are spread one per SM (two per SM up to twice as many) and
-// take the pipeline depth that leaves room for; an SM that has its share leaves the queue to the others for a moment.
-constexpr unsigned long long SPREAD_WAIT_NS = 1000;
+// take the pipeline depth that leaves room for; an SM that has its share leaves the queue to the others for about a tile's
+// length: the SM where the next tile ends is the better place, a second tile beside a first makes both of them late.  1, 4, 8,
+// 16 us: 4 streams x 3 43.4, 41.7, 40.3, 39.5 ms; 8 x 3 GR00T 40.1, 38.6, 37.1, 36.3; 64 us brings nothing more.
+constexpr unsigned long long SPREAD_WAIT_NS = 16000;
 // A node whose predecessors' tiles have all been taken may be queued before they finish (its workers wait holding their
 // weights) as long as everything queued or running still fits one tile per SM.
 constexpr int EARLY_MAX_TILES = 148;
