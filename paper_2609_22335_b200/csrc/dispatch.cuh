@@ -308,11 +308,12 @@ __device__ __forceinline__ void retire_loop(const DeviceCtx& ctx, SmState* sm, i
       bell_wait(&sm->bell_retire, bell_parity, RETIRE_SLEEP_NS);
       continue;
     }
-    // ---- starts.  The last tile of a node has been taken by a worker: tiles of a class are handed out in queue order, so
-    // all of them have.  Where that was the last predecessor of a successor, and the GPU has idle SMs for it, the successor
+    // ---- starts.  The last tile of a node has been taken by a worker: tiles of a class are claimed in queue order, so all of
+    // them have been claimed.  Where that was the last predecessor of a successor, and the GPU has idle SMs for it, the successor
     // is queued now: its tiles are taken, fetch their weights and wait for the release, instead of going through the queues
-    // after it (hand-over 3 us instead of 9).  No cycle can arise: a waiting tile waits only for tiles taken before it, and
-    // it holds shared memory while it waits only on an SM where nothing taken before it still needs some (see the worker's
+    // after it (hand-over 3 us instead of 9).  No cycle can arise: a waiting tile waits only for tiles claimed before it, a
+    // worker takes tiles that may have to wait in the order of their claims (see priority_goes_first), and such a tile holds
+    // shared memory while it waits only on an SM where nothing claimed before it still needs some (see the worker's
     // allocation).
     if (__any_sync(0xffffffffu, started)) {
       uint32_t inst = 0;
@@ -539,6 +540,7 @@ __device__ inline void claim_loop(const DeviceCtx& ctx, SmState* sm, int n_worke
         h.cls = want;
         h.early = (int)((e >> (64 - QW_GEN_BITS - 1)) & 1u);
         h.promised_s = promised_s; h.promised_t = promised_t;
+        h.held_at_claim = slot->held_tail;
         h.slot_base = __ldg(ctx.slot_base + inst);
         h.frame = ld_volatile_u64(reinterpret_cast<const unsigned long long*>(ctx.inst_frame + inst));
         h.gen = ld_volatile_u32(ctx.inst_gen + inst);
@@ -653,6 +655,14 @@ __device__ __forceinline__ void end_of_tile(const DeviceCtx& ctx, SmState* sm, W
   }
 }
 
+// What an early tile of `job` waits for: its node's dependency word and the count that releases it in this frame.
+__device__ __forceinline__ const unsigned long long* release_word(const DeviceCtx& ctx, const TileJob& job) {
+  return ctx.dep_word + (size_t)job.inst * ctx.n_nodes + job.node;
+}
+__device__ __forceinline__ unsigned long long release_count(const TileJob& job) {
+  return DEP_BIAS + (unsigned long long)(unsigned)job.desc.n_pred * job.gen;
+}
+
 // The worker's leader: waits for a tile the claim warp has put together, gives it its memory and fills in its context.
 __device__ __forceinline__ void take_tile(const DeviceCtx& ctx, SmState* sm, WorkerSlot* slot, char* slab, int worker, int n_workers) {
   Control* ctl = ctx.control;
@@ -662,7 +672,11 @@ __device__ __forceinline__ void take_tile(const DeviceCtx& ctx, SmState* sm, Wor
   if (!slot->primed) {
     uint32_t bell_parity = slot->bell_parity;
     for (;;) {
-      if (slot->prio_tail != slot->prio_head) { prio = true; break; }
+      if (slot->prio_tail != slot->prio_head) {
+        __threadfence_block();
+        const TileJob& j = slot->job[2 + (int)(slot->prio_head & 1u)];
+        if (priority_goes_first(j.early != 0, slot->held_head, j.held_at_claim) || released(release_word(ctx, j), release_count(j))) { prio = true; break; }
+      }
       if (slot->held_tail != slot->held_head) break;
       if (slot->leave) { slot->verdict = 0; return; }
       if (naps < 8) __nanosleep(20);                               // a claimed tile is usually a moment away
@@ -696,8 +710,8 @@ __device__ __forceinline__ void take_tile(const DeviceCtx& ctx, SmState* sm, Wor
 #pragma unroll 1
       for (int k = 0; k < N_CLASSES; ++k) taken += *reinterpret_cast<volatile int*>(&sm->pick.cta_count[k]);
       if (taken != 1) {
-        tc.wait_word = ctx.dep_word + (size_t)job.inst * ctx.n_nodes + job.node;
-        tc.wait_count = DEP_BIAS + (unsigned long long)(unsigned)job.desc.n_pred * job.gen;
+        tc.wait_word = release_word(ctx, job);
+        tc.wait_count = release_count(job);
         tc.t_start = &slot->t_wait;
         tc.deadline = lim;
         wait_release(tc);
@@ -769,8 +783,8 @@ __device__ __forceinline__ void take_tile(const DeviceCtx& ctx, SmState* sm, Wor
   tc.inputs = ctx.input_ptrs + (size_t)job.inst * N_FRAME_INPUTS;
   tc.amap_base = ctx.n_weight_tmaps + (int)job.inst * ctx.n_act_tmaps;
   tc.deadline = lim;
-  tc.wait_word = early ? ctx.dep_word + (size_t)job.inst * ctx.n_nodes + job.node : nullptr;
-  tc.wait_count = DEP_BIAS + (unsigned long long)(unsigned)job.desc.n_pred * job.gen;
+  tc.wait_word = early ? release_word(ctx, job) : nullptr;
+  tc.wait_count = release_count(job);
   tc.t_start = &slot->t_start;
 }
 

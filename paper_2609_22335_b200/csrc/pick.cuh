@@ -133,4 +133,12 @@ VLA_HD inline void pick_release(PickState& st, int k, const int* tau) {
   for (int x = 0; x < 3; ++x) st.u[x] -= tau[k * 3 + x];
 }
 
+// Whether the tile in a worker's priority slot goes ahead of the tiles claimed for it earlier and still held.  A tile that was
+// queued before its node's release (`early`) may have to wait for any tile claimed before it, those held by its own worker
+// among them: it goes in the order of the claims, that is once everything held when it was claimed has been taken.  Tiles then
+// wait only for tiles claimed before them, and no cycle can arise.  A tile that need not wait goes first at once.
+VLA_HD inline bool priority_goes_first(bool early, unsigned held_head, unsigned held_at_claim) {
+  return !early || (int)(held_head - held_at_claim) >= 0;
+}
+
 }  // namespace vla

@@ -20,6 +20,7 @@ struct TileJob {
   int early;                     // queued before its node's release
   unsigned gen;                  // the frame's number in its slot
   int promised_s, promised_t;    // room promised to the tile when it was claimed
+  unsigned held_at_claim;        // held_tail when it was claimed: tiles its worker had been given before it
   uint64_t frame, slot_base;
   alignas(16) NodeDesc desc;
 };
@@ -103,15 +104,18 @@ __device__ __forceinline__ void worker_sync(const TileCtx& c) {
   asm volatile("bar.sync %0, %1;" ::"r"(c.bar_id), "r"(WORKER_THREADS) : "memory");
 }
 
+__device__ __forceinline__ bool released(const unsigned long long* word, unsigned long long count) {
+  unsigned long long w;
+  asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(w) : "l"(word) : "memory");
+  return (w & ((1ull << 62) - 1ull)) >= count;
+}
 // One thread: waits (bounded) until the tile's node is released.  After a time-out the error is recorded and the tile runs
 // on whatever its operands hold, so that everything it has in flight ends in the ordinary way.
 __device__ __forceinline__ void wait_release(const TileCtx& c) {
   unsigned spins = 0;
   for (;;) {
-    unsigned long long w;
-    asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(w) : "l"(c.wait_word) : "memory");
     uint64_t now;
-    if ((w & ((1ull << 62) - 1ull)) >= c.wait_count) {
+    if (released(c.wait_word, c.wait_count)) {
       asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
       *c.t_start = now;
       return;

@@ -16,3 +16,7 @@ extern "C" int pick_host(int n_cls, const int* tau, const int* group, unsigned p
   for (int x = 0; x < 3; ++x) u[x] = st.u[x];
   return k;
 }
+
+extern "C" int priority_goes_first_host(int early, unsigned held_head, unsigned held_at_claim) {
+  return vla::priority_goes_first(early != 0, held_head, held_at_claim) ? 1 : 0;
+}
