@@ -45,6 +45,12 @@ __device__ __forceinline__ void set_error(const DeviceCtx& ctx, unsigned code, u
   }
 }
 
+// Shows the host the error word, whichever wait has set it.
+__device__ __forceinline__ void mirror_error(const DeviceCtx& ctx) {
+  *reinterpret_cast<volatile unsigned*>(ctx.error_host) = ld_volatile_u32(&ctx.control->error);
+  __threadfence_system();
+}
+
 // ------------------------------------------------------------------ doorbells inside an SM
 // The service warps and idle workers must not spin: every instruction they issue is taken from the worker warps that
 // share their scheduler (a claim loop polling flat out cost the tile bodies 10-40 % of their speed).  They wait on
@@ -875,9 +881,12 @@ __global__ void __launch_bounds__(MAX_WORKERS* WORKER_THREADS + DISPATCH_THREADS
       end_of_tile(ctx, sm, slot);
     }
   }
-  // After a wait that ran out, copies may still be in flight: they land before the block's memory goes.
-  if (ld_volatile_u32(&ctx.control->error) != 0u)
+  // After a wait that ran out, copies may still be in flight: they land before the block's memory goes.  The host reads the
+  // mirror of the error word; the waits inside tile bodies set the word only (registers are short there).
+  if (ld_volatile_u32(&ctx.control->error) != 0u) {
+    if (threadIdx.x == 0) mirror_error(ctx);
     for (int i = 0; i < 200; ++i) __nanosleep(1000);
+  }
   tc_fence_before();
   __syncthreads();
   if (threadIdx.x < 32) tmem_dealloc(sm->tmem_base, 512);
@@ -918,6 +927,7 @@ __global__ void __launch_bounds__(WORKER_THREADS) vla_node_kernel(DeviceCtx ctx,
   tc.deadline = t0 + ctx.wait_limit_ns;
   const uint64_t frame = inst >= 0 ? ctx.inst_frame[inst] : 0;
   run_tile<true>(ctx, tc, n, (int)blockIdx.x, inst, frame);
+  if (threadIdx.x == 0 && gtimer() > tc.deadline && ld_volatile_u32(&ctx.control->error) != 0u) mirror_error(ctx);   // a wait ran out
   if (inst >= 0 && ctx.trace_capacity) {
     asm volatile("bar.sync 1, %0;" ::"r"(WORKER_THREADS) : "memory");
     if (threadIdx.x == 0) write_trace(ctx, (uint32_t)inst, (uint32_t)node_idx, blockIdx.x, 0, n.cls, frame, t0, gtimer());

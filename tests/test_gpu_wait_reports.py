@@ -1,0 +1,35 @@
+"""A device-side wait that runs out inside a tile reaches the host as VLA_ERR_TIMEOUT.  The failure is made on the host (a
+dependency count raised while nothing is in flight); the wait is bounded, the kernel returns and the context can be closed."""
+import time
+
+import pytest
+
+from vla_synth.configs import CFG1
+from vla_synth.gen import make_weights, frame_inputs
+
+pytestmark = pytest.mark.gpu
+
+
+def test_tile_that_waits_for_its_release_in_vain_is_reported_while_other_streams_run():
+    """The stalled node's tile was queued before its release and waits on its worker.  Frames of the other stream keep every
+    SM busy now and then, so that the idle watchdog has nothing to say: the tile's own wait has to tell the host."""
+    from paper_2609_22335_b200 import Engine, api
+    eng = Engine(CFG1, mode="cosched", n_streams=2, wait_limit_ns=100_000_000)            # 0.1 s
+    try:
+        eng.load_weights(make_weights(CFG1, seed=0))
+        victim = next(i for i, n in enumerate(eng.program_info()) if n["phase"] == 1 and n["n_pred"] > 0 and n["name"].endswith("L1.w2"))
+        eng.bump_dependency(0, 0, victim, 1)
+        frame = frame_inputs(CFG1, 0, 0, seed=0)
+        assert eng.submit(0, frame) == api.VLA_OK
+        code, t0, served = None, time.time(), 0
+        while code is None and time.time() - t0 < 5.0:
+            try:
+                eng.submit(1, frame)                         # (VLA_ERR_BUSY: the ring is full)
+                served += eng.poll(1) is not None
+                assert eng.poll(0) is None
+            except api.VlaError as e:
+                code = e.code
+        assert code == api.VLA_ERR_TIMEOUT and "wait ran out" in eng.last_error()
+        assert served > 20                                   # the other stream was served until then
+    finally:
+        eng.close()
