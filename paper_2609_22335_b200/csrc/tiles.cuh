@@ -208,7 +208,9 @@ __device__ void tile_timeemb(const TileCtx& c, const TimeEmbArgs& a, int) {
   }
 }
 
-// Copies the chunk to the host-visible ring, then publishes the frame id (system-scope fence between).
+// Copies the chunk to the host-visible ring, then publishes the frame id (system-scope fence between).  After a wait that
+// ran out nothing is published any more: a tile of this very frame may have gone on with operands that were not there (it set
+// the error word before its end released anything, so it shows here).
 __device__ void tile_emit(const TileCtx& c, const EmitArgs& a, float* chunk_host, DoneRec* done, uint64_t frame, bool last) {
   const float* x = resolve<const float>(c, a.x);
   chunk_host += a.chunk_off;
@@ -219,7 +221,7 @@ __device__ void tile_emit(const TileCtx& c, const EmitArgs& a, float* chunk_host
   }
   __threadfence_system();
   worker_sync(c);
-  if (worker_tid() == 0 && last) {
+  if (worker_tid() == 0 && last && *reinterpret_cast<volatile unsigned*>(c.error) == 0u) {
     done->frame_plus1 = frame + 1;
     __threadfence_system();
   }

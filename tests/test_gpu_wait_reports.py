@@ -10,14 +10,24 @@ from vla_synth.gen import make_weights, frame_inputs
 pytestmark = pytest.mark.gpu
 
 
-def test_tile_that_waits_for_its_release_in_vain_is_reported_while_other_streams_run():
+def _head_gemm(node):
+    return node["phase"] == 1 and node["n_pred"] > 0 and node["name"].endswith("L1.w2")
+
+
+def _emit(node):
+    return node["op"] == 8
+
+
+@pytest.mark.parametrize("which", [_head_gemm, _emit])
+def test_tile_that_waits_for_its_release_in_vain_is_reported_while_other_streams_run(which):
     """The stalled node's tile was queued before its release and waits on its worker.  Frames of the other stream keep every
-    SM busy now and then, so that the idle watchdog has nothing to say: the tile's own wait has to tell the host."""
+    SM busy now and then, so that the idle watchdog has nothing to say: the tile's own wait has to tell the host, and the frame
+    it belongs to is never handed out, not even when that tile is the one that publishes it."""
     from paper_2609_22335_b200 import Engine, api
     eng = Engine(CFG1, mode="cosched", n_streams=2, wait_limit_ns=100_000_000)            # 0.1 s
     try:
         eng.load_weights(make_weights(CFG1, seed=0))
-        victim = next(i for i, n in enumerate(eng.program_info()) if n["phase"] == 1 and n["n_pred"] > 0 and n["name"].endswith("L1.w2"))
+        victim = next(i for i, n in enumerate(eng.program_info()) if which(n))
         eng.bump_dependency(0, 0, victim, 1)
         frame = frame_inputs(CFG1, 0, 0, seed=0)
         assert eng.submit(0, frame) == api.VLA_OK
