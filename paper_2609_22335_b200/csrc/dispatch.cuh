@@ -37,14 +37,6 @@ __device__ __forceinline__ unsigned long long ld_volatile_u64(const unsigned lon
 }
 __device__ __forceinline__ long long ld_volatile_s64(const long long* p) { return *reinterpret_cast<const volatile long long*>(p); }
 
-__device__ __forceinline__ void set_error(const DeviceCtx& ctx, unsigned code, unsigned info) {
-  if (atomicCAS(&ctx.control->error, 0u, code) == 0u) {
-    ctx.control->error_info = info;
-    *ctx.error_host = code;
-    __threadfence_system();
-  }
-}
-
 // Shows the host the error word, whichever wait has set it.
 __device__ __forceinline__ void mirror_error(const DeviceCtx& ctx) {
   *reinterpret_cast<volatile unsigned*>(ctx.error_host) = ld_volatile_u32(&ctx.control->error);

@@ -128,6 +128,14 @@ __device__ __forceinline__ void wait_release(const TileCtx& c) {
   }
 }
 
+__device__ __forceinline__ void set_error(const DeviceCtx& ctx, unsigned code, unsigned info) {
+  if (atomicCAS(&ctx.control->error, 0u, code) == 0u) {
+    ctx.control->error_info = info;
+    *ctx.error_host = code;
+    __threadfence_system();
+  }
+}
+
 // Activations are produced by other SMs during the same kernel: read them through L2.
 __device__ __forceinline__ float ld_act(const float* p) { return __ldcg(p); }
 __device__ __forceinline__ uint4 ld_act(const uint4* p) { return __ldcg(p); }
