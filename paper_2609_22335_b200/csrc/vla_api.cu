@@ -351,7 +351,11 @@ int vla_init(const vla_model_desc* desc, const vla_runtime_opts* opts, vla_ctx**
     if (n.n_tiles > (1 << QW_TILE_BITS) || (n.smem_bytes + SMEM_UNIT - 1) / SMEM_UNIT >= (1 << QW_SMEM_BITS) ||
         (n.tmem_cols + TMEM_UNIT - 1) / TMEM_UNIT >= (1 << QW_TMEM_BITS))
       return fail(c, VLA_ERR_INVALID, "a node has more tiles or needs more memory than a queue entry can describe");
-  CU(cudaFuncSetAttribute(vla_node_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, std::max(c->max_node_smem, 1024)));
+  {   // the limit belongs to the kernel, not to this context: always all there is, so that contexts do not undo one another
+    cudaFuncAttributes fa;
+    CU(cudaFuncGetAttributes(&fa, vla_node_kernel));
+    CU(cudaFuncSetAttribute(vla_node_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, max_optin - (int)fa.sharedSizeBytes));
+  }
   CU(cudaStreamCreateWithFlags(&c->scopy, cudaStreamNonBlocking));
   CU(cudaEventCreateWithFlags(&c->ev_kernel, cudaEventDisableTiming));
 
