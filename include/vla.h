@@ -243,7 +243,7 @@ int vla_debug_bump_dependency(vla_ctx* ctx, int32_t stream, int32_t slot, int32_
  * first one is named in vla_last_error).  An out-of-bounds store of a tile body shows up here. */
 int vla_debug_guards(vla_ctx* ctx, int32_t fill, size_t* n_bad);
 
-/* ---- stand-alone operators: the engine's tile bodies on caller-owned DEVICE tensors ------------------------
+/* ---- stand-alone operators on caller-owned DEVICE tensors --------------------------------------------------
  * Both run asynchronously on `stream` (a cudaStream_t; NULL = default stream). */
 
 /* Fused attention, softmax(Q K^T / sqrt(hd)) V per head with grouped KV heads -- the attention of the VLM
@@ -293,6 +293,22 @@ int vla_op_status(int32_t op, const void* scratch, void* stream);
  * wait for operands that never come and the bounded waits (wait_limit_ns; 0 = the default 2 s) run out.  Process-wide;
  * call with (0, 0) to restore normal operation. */
 int vla_debug_op_fault(int32_t drop_operand_loads, uint64_t wait_limit_ns);
+
+/* Test hooks: the engine's own GEMM and attention tile bodies (the operators above are kernels of their own) on
+ * caller-owned DEVICE tensors, one node run as the stream modes run it.  Blocking; they allocate and free; no context
+ * is needed.  VLA_ERR_TIMEOUT when a device-side wait ran out; vla_debug_op_fault applies.
+ * GEMM: a [m,k] bf16, w [n,k] bf16; gated: w holds 2n rows, gate and up rows alternating, out = act(gate) * up, out16
+ * only.  x (optional, fp32 [m,n]) is added to the product.  fast = 0 takes the general epilogue; fast = 1 the straight
+ * one, for which n is a multiple of 8 (gated: 4), the rows of w are padded to a multiple of 32 and reordered within each
+ * 32 as the engine's are (row p holds feature 8 * ((p >> 1) & 3) + 2 * (p >> 3) + (p & 1)), x comes with out32 and
+ * without act, and act = 1 with out16 alone.
+ * Attention: q [tq, hq*hd] and k0 [t0, hkv*hd] bf16, vt0 [hkv*hd, t0 rounded up to 64] bf16, V transposed; an optional
+ * second segment of t1 keys, of which the queries below sfx see only the first sfx; out [tq, hq*hd] bf16. */
+int vla_debug_tile_linear(const void* a, const void* w, const float* x, float* out32, void* out16, int32_t m, int32_t n,
+                          int32_t k, int32_t act, int32_t gated, int32_t fast);
+int vla_debug_tile_attention(const void* q, const void* k0, const void* vt0, const void* k1, const void* vt1, void* out,
+                             int32_t tq, int32_t t0, int32_t t1, int32_t hq, int32_t hkv, int32_t hd, int32_t causal,
+                             int32_t sfx);
 
 const char* vla_last_error(vla_ctx* ctx);
 int vla_destroy(vla_ctx* ctx);

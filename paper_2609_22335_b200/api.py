@@ -26,7 +26,7 @@ _SOLVER = {"euler": 0, "ddim": 1}
 EXPORTS = ["vla_required_arena_bytes", "vla_init", "vla_load_weights", "vla_submit_frame", "vla_submit_frame_device",
            "vla_poll_actions", "vla_hold_launches", "vla_wait_idle", "vla_get_trace", "vla_reset_trace", "vla_program_info", "vla_debug_fetch",
            "vla_get_counters", "vla_set_class_tags", "vla_get_class_tags", "vla_policy_probe", "vla_policy_probe_ex", "vla_debug_bump_dependency", "vla_debug_guards", "vla_last_error",
-           "vla_destroy", "vla_op_status", "vla_debug_op_fault",
+           "vla_destroy", "vla_op_status", "vla_debug_op_fault", "vla_debug_tile_linear", "vla_debug_tile_attention",
            "vla_op_attention_scratch_bytes", "vla_op_attention", "vla_op_linear",
            "vla_op_attention_static_capacity", "vla_op_attention_static"]
 
@@ -101,6 +101,8 @@ def load_library() -> C.CDLL:
     lib.vla_debug_bump_dependency.argtypes = [C.c_void_p] + [C.c_int32] * 4
     lib.vla_op_status.argtypes = [C.c_int32, C.c_void_p, C.c_void_p]
     lib.vla_debug_op_fault.argtypes = [C.c_int32, C.c_uint64]
+    lib.vla_debug_tile_linear.argtypes = [C.c_void_p] * 5 + [C.c_int32] * 6
+    lib.vla_debug_tile_attention.argtypes = [C.c_void_p] * 6 + [C.c_int32] * 8
     lib.vla_op_attention_scratch_bytes.argtypes = [C.c_int32, C.c_int32, C.c_int32, P(C.c_size_t)]
     lib.vla_op_attention.argtypes = [C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p] + [C.c_int32] * 6 + [C.c_void_p, C.c_size_t, C.c_void_p]
     lib.vla_op_linear.argtypes = [C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p] + [C.c_int32] * 4 + [C.c_void_p]
@@ -477,3 +479,34 @@ def debug_op_fault(drop_operand_loads, wait_limit_ns=0):
     rc = load_library().vla_debug_op_fault(int(bool(drop_operand_loads)), int(wait_limit_ns))
     if rc != VLA_OK:
         raise VlaError(rc, "vla_debug_op_fault failed")
+
+
+def debug_tile_linear(a, w, n, x=None, act=0, gated=False, fast=False, out32=True, out16=False):
+    """Test hook: the engine's GEMM tile body (see vla_debug_tile_linear).  Returns (fp32 [m,n] or None, bf16 [m,n] or None)."""
+    import torch
+    m, k = a.shape
+    o32 = a.new_empty((m, n), dtype=torch.float32) if out32 else None
+    o16 = a.new_empty((m, n), dtype=torch.bfloat16) if out16 else None
+    ptr = lambda t: None if t is None else t.data_ptr()
+    rc = load_library().vla_debug_tile_linear(a.data_ptr(), w.data_ptr(), ptr(x), ptr(o32), ptr(o16), m, n, k, act, int(gated), int(fast))
+    if rc != VLA_OK:
+        raise VlaError(rc, "vla_debug_tile_linear failed")
+    return o32, o16
+
+
+def debug_tile_attention(q, k0, v0, hq, hkv, hd, k1=None, v1=None, causal=False, sfx=0):
+    """Test hook: the engine's attention tile body (see vla_debug_tile_attention); v0, v1 [t, hkv*hd] as they lie."""
+    import torch
+
+    def transposed(v):
+        t = v.new_zeros((v.shape[1], (v.shape[0] + 63) // 64 * 64))
+        t[:, :v.shape[0]] = v.T
+        return t
+    vt0, vt1 = transposed(v0), None if v1 is None else transposed(v1)
+    out = torch.empty_like(q)
+    rc = load_library().vla_debug_tile_attention(q.data_ptr(), k0.data_ptr(), vt0.data_ptr(), None if k1 is None else k1.data_ptr(),
+                                                 None if vt1 is None else vt1.data_ptr(), out.data_ptr(), q.shape[0], k0.shape[0],
+                                                 0 if k1 is None else k1.shape[0], hq, hkv, hd, int(causal), sfx)
+    if rc != VLA_OK:
+        raise VlaError(rc, "vla_debug_tile_attention failed")
+    return out

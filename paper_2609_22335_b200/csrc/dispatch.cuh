@@ -911,7 +911,7 @@ __global__ void __launch_bounds__(WORKER_THREADS) vla_node_kernel(DeviceCtx ctx,
   tc.tmaps = ctx.tmaps;
   tc.inputs = ctx.input_ptrs + (size_t)(inst >= 0 ? inst : 0) * N_FRAME_INPUTS;
   tc.amap_base = ctx.n_weight_tmaps + (inst >= 0 ? inst : 0) * ctx.n_act_tmaps;
-  tc.drop_loads = 0;
+  tc.drop_loads = ctx.drop_loads;
   tc.wait_word = nullptr;
   tc.slot = nullptr;
   tc.cont = 0;

@@ -1,7 +1,6 @@
-// Stand-alone operator entry points: the GEMM and fused-attention tile bodies of the
-// engine, launched as ordinary kernels on caller-owned device tensors.  They exist so the
-// tile bodies can be checked operator by operator against the CPU oracle, and for callers
-// that want the kernels without the frame pipeline.
+// Stand-alone operator entry points: a linear layer and fused attention on caller-owned device tensors, for callers that
+// want the kernels without the frame pipeline.  They are kernels of their own (op_linear.cuh, op_attention.cuh); the engine's
+// tile bodies are reached one by one through tile_hooks.cuh.
 #pragma once
 #include <cuda.h>
 #include <cuda_runtime.h>

@@ -83,8 +83,8 @@ struct TileCtx {
   uint64_t* t_start;                     // where the time of that moment goes
   WorkerSlot* slot;     // the persistent kernel's worker, null elsewhere
   int cont;             // this tile's operand ring was primed by the tile before
-  int drop_loads;       // test hook of the stand-alone operators: the TMA producer issues nothing, so the consumers'
-                        // bounded waits run out (0 everywhere else)
+  int drop_loads;       // test hook (tile_hooks.cuh): the TMA producer issues nothing, so the consumers' bounded waits run out
+                        // (0 in the persistent kernel)
 };
 
 // 0 .. WORKER_THREADS-1 (a kernel's workers are consecutive groups of WORKER_THREADS threads)

@@ -859,6 +859,7 @@ int vla_destroy(vla_ctx* c) {
 }  // extern "C"
 
 #include "ops_api.cuh"
+#include "tile_hooks.cuh"
 
 // ------------------------------------------------------------------------------------------------
 // Attention without any allocation: the scratch of vla_op_attention (error word + room for a transposed V)

@@ -290,6 +290,7 @@ struct DeviceCtx {
   int32_t u_max, pad_u;     // saturation value of the utilisation counters in the pick's score
   uint64_t wait_limit_ns, idle_exit_ns;
   int32_t chunk_elems;
+  int32_t drop_loads;       // test hook of the node kernel (see TileCtx)
 };
 
 }  // namespace vla
