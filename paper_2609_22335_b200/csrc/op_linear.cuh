@@ -25,8 +25,7 @@ struct LinearArgs {
   int vec8;                                   // rows of the results allow 16-byte stores of eight bf16 or 8-byte pairs of fp32
   float* out32;
   unsigned short* out16;
-  unsigned* err;                              // gets `call` when a wait runs out
-  unsigned call;
+  unsigned* err;                              // 0, or why a wait ran out
 };
 
 inline int linear_stages(int bm, int bn) {
@@ -171,6 +170,7 @@ __global__ void __launch_bounds__(LIN_THREADS, 2) vla_op_linear_kernel(const __g
     tmem_alloc(&tmem_base_s, LIN_TMEM_COLS);
   }
   op_wait_previous(maps, 2);
+  if (threadIdx.x == 0 && blockIdx.x == 0) *g.err = 0u;
   TileCtx c;                                   // (what the bounded waits look at)
   c.error = &failed_s;
   c.deadline = gtimer() + fault.wait_limit_ns;
@@ -291,7 +291,7 @@ __global__ void __launch_bounds__(LIN_THREADS, 2) vla_op_linear_kernel(const __g
   tc_fence_before();
   __syncthreads();
   if (warp == 1) tmem_dealloc(tmem, LIN_TMEM_COLS);
-  if (threadIdx.x == 0 && *reinterpret_cast<volatile unsigned*>(&failed_s) != 0u) *g.err = g.call;
+  if (threadIdx.x == 0 && *reinterpret_cast<volatile unsigned*>(&failed_s) != 0u) *g.err = (unsigned)DEV_ERR_WAIT_MBAR;
 }
 
 }  // namespace vla

@@ -77,14 +77,13 @@ namespace vla {
 
 constexpr size_t OP_ATTN_HEADER = 256;   // error word + padding (behind it: room a transposed V would take, which the sizes of the interface count)
 
-// What vla_op_linear keeps per device, looked up on the first call made with that device current: SM count, the error word
-// (in a fixed device array of the library) and the number of the latest call.  A kernel whose wait runs out writes its
-// call's number there; nothing has to be cleared in front of a call.
+// What vla_op_linear keeps per device, looked up on the first call made with that device current: SM count and the error word
+// (in a fixed device array of the library).  The kernel clears the word itself before it waits for anything, so that a call
+// that was captured into a graph reports on its latest replay like any other.
 static __device__ __align__(256) unsigned g_op_linear_error[64];
 struct OpDevice {
   std::atomic<unsigned*> error{nullptr};
   int sms = 0;
-  std::atomic<unsigned> calls{0};
 };
 inline OpDevice* op_device() {
   constexpr int kMax = 64;
@@ -106,11 +105,11 @@ inline OpDevice* op_device() {
 }
 
 // Reads an operator's error word back after the stream has drained.
-inline int op_status_of(const unsigned* dev_word, cudaStream_t s, unsigned call = 0) {
+inline int op_status_of(const unsigned* dev_word, cudaStream_t s) {
   if (cudaStreamSynchronize(s) != cudaSuccess) return VLA_ERR_CUDA;
   unsigned v = 0;
   if (cudaMemcpy(&v, dev_word, sizeof v, cudaMemcpyDeviceToHost) != cudaSuccess) return VLA_ERR_CUDA;
-  return (call ? v != call : v == 0) ? VLA_OK : VLA_ERR_TIMEOUT;       // (call: the number that would mean a time-out)
+  return v == 0 ? VLA_OK : VLA_ERR_TIMEOUT;
 }
 
 // Launches a kernel in clusters of `cluster` blocks (1: none), overlapping the end of the kernel in front of it
@@ -198,7 +197,6 @@ int vla_op_linear(const void* a, const void* w, float* out32, void* out16, int32
   g.vec8 = n % 8 == 0 && ((reinterpret_cast<uintptr_t>(out32) | reinterpret_cast<uintptr_t>(out16)) & 15) == 0;
   linear_plan(g, dev->sms);
   g.err = dev->error.load(std::memory_order_relaxed);
-  g.call = dev->calls.fetch_add(1u, std::memory_order_relaxed) + 1u;
   OpMaps maps;
   if (!op_encode(&maps.m[0], w, n, k, k, g.bn) || !op_encode(&maps.m[1], a, m, k, k, g.bm)) return VLA_ERR_CUDA;
   const int grid = g.ks > 1 ? g.tiles * g.ks : (g.tiles < 2 * dev->sms ? g.tiles : 2 * dev->sms);

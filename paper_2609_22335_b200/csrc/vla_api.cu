@@ -912,7 +912,7 @@ int vla_op_status(int32_t op, const void* scratch, void* stream) {
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   if (op == VLA_OP_LINEAR) {
     vla::OpDevice* d = vla::op_device();
-    return d ? vla::op_status_of(d->error.load(), s, d->calls.load()) : VLA_ERR_CUDA;
+    return d ? vla::op_status_of(d->error.load(), s) : VLA_ERR_CUDA;
   }
   if (op == VLA_OP_ATTENTION) {
     if (!scratch) return VLA_ERR_INVALID;
