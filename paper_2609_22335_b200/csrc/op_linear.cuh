@@ -22,7 +22,6 @@ constexpr int LIN_TMEM_COLS = 256;            // half an SM: two accumulators of
 
 struct LinearArgs {
   int m, n, n_end, kp, bm, bn, ks, tiles_m, tiles, stages, act;
-  int vec8;                                   // rows of the results allow 16-byte stores of eight bf16 or 8-byte pairs of fp32
   float* out32;
   unsigned short* out16;
   unsigned* err;                              // 0, or why a wait ran out
@@ -61,6 +60,15 @@ inline void linear_plan(LinearArgs& g, int sms) {
   g.tiles = g.tiles_m * ((g.n + g.bn - 1) / g.bn);
   g.stages = linear_stages(g.bm, g.bn);
 }
+// Features a store may cover: what every row's start and the width allow.  Eight go out as 16 bytes of bf16 or four pairs of
+// fp32, two as a pair, and an odd width (or address) leaves single elements.  8192 tokens, K = 768, GELU, bf16: 3072 features 40 us,
+// 3076 in pairs 47 (96 in single elements), 3073 105; K = 64 without GELU 13.7, 24 (71), 87.  A kernel for each: chosen at run time
+// inside one, the branches cost the wide rows 3 %.
+inline int linear_vec(int n, const float* out32, const void* out16) {
+  const uintptr_t a32 = reinterpret_cast<uintptr_t>(out32), a16 = reinterpret_cast<uintptr_t>(out16);
+  if (n % 8 == 0 && ((a32 | a16) & 15) == 0) return 8;
+  return n % 2 == 0 && (a32 & 7) == 0 && (a16 & 3) == 0 ? 2 : 1;
+}
 inline int linear_smem(const LinearArgs& g) {
   const int stage = (g.bm + g.bn) * GEMM_BK * 2;
   return g.stages * stage + (stage < 16384 ? 16384 - stage : 0);
@@ -81,12 +89,14 @@ __device__ __forceinline__ void quad_transpose(uint32_t* w, int q) {
   }
 }
 // One fragment (see tmem_ld_frag) of finished values: rows `row` and `row` + 8 of the output, 32 features from `f`.
+// VEC: features a store may cover (linear_vec).
+template <int VEC>
 __device__ __forceinline__ void linear_store(const LinearArgs& g, float* v, int row, int f, int q) {
 #pragma unroll
   for (int r = 0; r < 2; ++r) {
     const bool live = row + 8 * r < g.m;
     const size_t at = (size_t)(row + 8 * r) * g.n + f;
-    if (g.vec8) {
+    if (VEC == 8) {
       if (g.out32) {
 #pragma unroll
         for (int b = 0; b < 4; ++b)
@@ -98,6 +108,14 @@ __device__ __forceinline__ void linear_store(const LinearArgs& g, float* v, int 
         for (int b = 0; b < 4; ++b) w[b] = pack_bf16(v[4 * b + 2 * r], v[4 * b + 2 * r + 1]);
         quad_transpose(w, q);
         if (live && f + 8 * q < g.n_end) *reinterpret_cast<uint4*>(g.out16 + at + 8 * q) = make_uint4(w[0], w[1], w[2], w[3]);
+      }
+    } else if (VEC == 2) {
+#pragma unroll
+      for (int b = 0; b < 4; ++b) {
+        const int c = 8 * b + 2 * q;
+        if (!live || f + c >= g.n_end) continue;
+        if (g.out32) *reinterpret_cast<float2*>(g.out32 + at + c) = make_float2(v[4 * b + 2 * r], v[4 * b + 2 * r + 1]);
+        if (g.out16) *reinterpret_cast<uint32_t*>(g.out16 + at + c) = pack_bf16(v[4 * b + 2 * r], v[4 * b + 2 * r + 1]);
       }
     } else {
 #pragma unroll
@@ -114,7 +132,7 @@ __device__ __forceinline__ void linear_store(const LinearArgs& g, float* v, int 
 }
 // This warp's share of a tile's columns: groups of 32, [lo, hi), for its 32 lanes.  `part` (split K): the other CTAs'
 // fragments of the same group, written by the threads that hold the same place.
-template <int ACT>
+template <int ACT, int VEC>
 __device__ __forceinline__ void linear_rows(const LinearArgs& g, uint32_t tmem, int lane, int row0, int rows, int n0, int lo, int hi, const float4* part,
                                             int n_part, int part_stride) {
   const int q = lane & 3;
@@ -141,12 +159,13 @@ __device__ __forceinline__ void linear_rows(const LinearArgs& g, uint32_t tmem, 
         }
       }
       activate<ACT, EPI>(v);
-      linear_store(g, v, row0 + 16 * h + (lane >> 2), n0 + 32 * c, q);
+      linear_store<VEC>(g, v, row0 + 16 * h + (lane >> 2), n0 + 32 * c, q);
     }
     tmem_ld_wait();
   }
 }
 
+template <int VEC>
 __global__ void __launch_bounds__(LIN_THREADS, 2) vla_op_linear_kernel(const __grid_constant__ LinearArgs g, const __grid_constant__ OpMaps maps,
                                                                        OpFault fault) {
   extern __shared__ __align__(1024) char smem_raw[];
@@ -232,9 +251,9 @@ __global__ void __launch_bounds__(LIN_THREADS, 2) vla_op_linear_kernel(const __g
     LinearArgs gg = g;
     gg.m = row0 + max(rows, 0);                                       // (this tile's rows and features only)
     gg.n_end = min(g.n, n0 + g.bn);
-    if (g.act == ACT_GELU) linear_rows<ACT_GELU>(gg, acc + lanes, lane, row0, rows, n0, lo, hi, part, n_part, part_stride);
-    else if (g.act == ACT_SILU) linear_rows<ACT_SILU>(gg, acc + lanes, lane, row0, rows, n0, lo, hi, part, n_part, part_stride);
-    else linear_rows<ACT_NONE>(gg, acc + lanes, lane, row0, rows, n0, lo, hi, part, n_part, part_stride);
+    if (g.act == ACT_GELU) linear_rows<ACT_GELU, VEC>(gg, acc + lanes, lane, row0, rows, n0, lo, hi, part, n_part, part_stride);
+    else if (g.act == ACT_SILU) linear_rows<ACT_SILU, VEC>(gg, acc + lanes, lane, row0, rows, n0, lo, hi, part, n_part, part_stride);
+    else linear_rows<ACT_NONE, VEC>(gg, acc + lanes, lane, row0, rows, n0, lo, hi, part, n_part, part_stride);
   };
   if (g.ks == 1) {
     if (warp >= 2) {

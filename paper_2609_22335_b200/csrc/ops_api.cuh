@@ -96,7 +96,8 @@ inline OpDevice* op_device() {
     int sms = 0;
     if (cudaGetSymbolAddress(&a, g_op_linear_error) != cudaSuccess || !a) return nullptr;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return nullptr;
-    if (cudaFuncSetAttribute(vla_op_linear_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, LIN_SMEM) != cudaSuccess) return nullptr;
+    for (auto* kernel : {vla_op_linear_kernel<1>, vla_op_linear_kernel<2>, vla_op_linear_kernel<8>})
+      if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, LIN_SMEM) != cudaSuccess) return nullptr;
     if (cudaFuncSetAttribute(vla_op_attention_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 224 * 1024) != cudaSuccess) return nullptr;
     d.sms = sms;
     d.error.store(static_cast<unsigned*>(a), std::memory_order_release);
@@ -194,14 +195,14 @@ int vla_op_linear(const void* a, const void* w, float* out32, void* out16, int32
   LinearArgs g;
   g.m = m; g.n = n; g.kp = (int)op_pad(k, GEMM_BK); g.act = act;
   g.out32 = out32; g.out16 = static_cast<unsigned short*>(out16);
-  g.vec8 = n % 8 == 0 && ((reinterpret_cast<uintptr_t>(out32) | reinterpret_cast<uintptr_t>(out16)) & 15) == 0;
   linear_plan(g, dev->sms);
   g.err = dev->error.load(std::memory_order_relaxed);
   OpMaps maps;
   if (!op_encode(&maps.m[0], w, n, k, k, g.bn) || !op_encode(&maps.m[1], a, m, k, k, g.bm)) return VLA_ERR_CUDA;
   const int grid = g.ks > 1 ? g.tiles * g.ks : (g.tiles < 2 * dev->sms ? g.tiles : 2 * dev->sms);
-  const int rc = op_launch(vla_op_linear_kernel, grid, LIN_THREADS, linear_smem(g), g.ks, static_cast<cudaStream_t>(stream), g, maps, op_fault());
-  return rc;
+  const int vec = linear_vec(n, out32, out16);
+  const auto kernel = vec == 8 ? vla_op_linear_kernel<8> : (vec == 2 ? vla_op_linear_kernel<2> : vla_op_linear_kernel<1>);
+  return op_launch(kernel, grid, LIN_THREADS, linear_smem(g), g.ks, static_cast<cudaStream_t>(stream), g, maps, op_fault());
 }
 
 int vla_debug_op_fault(int32_t drop_operand_loads, uint64_t wait_limit_ns) {
