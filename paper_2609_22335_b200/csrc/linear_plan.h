@@ -1,0 +1,77 @@
+// Tile shape of a stand-alone linear layer (op_linear.cuh): plain arithmetic, compiled for the host in the CPU tests too.
+#pragma once
+#include "vla_types.h"
+
+namespace vla {
+
+constexpr int LIN_MAX_STAGES = 12;
+constexpr int LIN_SMEM = 110 * 1024;          // half an SM
+
+struct LinearPlan { int bm, bn, ks, tiles_m, tiles, stages; };   // tokens and features of a tile, CTAs that share its K, tiles, pipeline depth
+
+inline int linear_stages(int bm, int bn) {
+  const int stage = (bm + bn) * GEMM_BK * 2, tail = stage < 16384 ? 16384 - stage : 0;        // the MMA always reads 128 rows
+  const int s = (LIN_SMEM - tail) / stage;
+  return s > LIN_MAX_STAGES ? LIN_MAX_STAGES : s;
+}
+// Whether a cluster of `ks` CTAs can share the K range of a tile of `bn` features: each finishes a whole number of 32-column
+// groups, and the others' partial sums of those have to fit its stages.
+inline bool linear_split_fits(int bm, int bn, int ks, int nkb) {
+  return ks == 1 || ((bn & (bn - 1)) == 0 && bn >= 32 * ks && nkb >= 2 * ks &&
+                     128 * (bn / ks) * (ks - 1) * 4 <= linear_stages(bm, bn) * (bm + bn) * GEMM_BK * 2);
+}
+// Split of a call with fp32 results, and the width that goes with it.  A split shortens the tensor core's sums (K = 4096: rel-L2
+// 2.4e-6 for 5.1e-6), which shows in fp32 and vanishes in bf16; so here it is not traded for the time that a width without one
+// gains.  An estimate over powers of two: per k-block max(operand bytes over 47 B/clk, MMA issue) cycles for a CTA alone on its
+// SM, max(2 x bytes over 90 B/clk, 2 x MMA) beside another one, a round trip and an epilogue per tile, an exchange per split.
+inline void linear_split_f32(LinearPlan& g, int n, int nkb, int sms) {
+  double best = 1e300;
+  for (int bn = 256; bn >= 16; bn >>= 1)
+    for (int ks = 1; ks <= 8; ks <<= 1) {
+      const long long ctas = (long long)g.tiles_m * ((n - 1) / bn + 1) * ks, rounds = (ctas + 2 * sms - 1) / (2 * sms);
+      if (!linear_split_fits(g.bm, bn, ks, nkb) || (ks > 1 && ctas > 2 * sms)) continue;         // (a split tile is a cluster of its own)
+      const double bytes = (double)(g.bm + bn) * GEMM_BK * 2, mma = bn <= 64 ? 200 : 2.0 * bn;
+      const double kb = ctas > sms ? (2 * bytes / 90 > 2 * mma ? 2 * bytes / 90 : 2 * mma) : (bytes / 47 > mma ? bytes / 47 : mma);
+      const double t = (double)(rounds * ((nkb + ks - 1) / ks)) * kb + (bn <= 128 ? 1 : rounds) * (1500 + 16.0 * bn / ks) + (ks > 1 ? 2500 + 8.0 * bn : 0);
+      if (t < best) { best = t; g.bn = bn; g.ks = ks; }
+    }
+}
+// Tile width and K split of a call: the pair with the least estimated time.  A k-block of a tile costs a CTA that has its SM to
+// itself max(400, 4 x width, 2600 / stages) cycles -- issue, MMA with its operands, a load's round trip -- and two on an SM
+// twice the first two, or the time of their operands at 58 B/clk (42 where K is no multiple of 64: rows then straddle 128-byte
+// lines).  A tile adds its epilogue (behind the next tile's main loop where there are two accumulators), a split its exchange.
+// Fitted to 280 shapes of 1..8192 x 7..16384 x 64..12288 with every width and split timed: the pair chosen is 1.8 % behind the
+// best one on average, more than 10 % behind on 20, 24 % at most.  (By the estimate above, with powers of two alone up to the
+// chip's two CTAs per SM: 8 %, 87 shapes, 83 %; 3455 x 1392 x 8448 100 us at width 256 and 71 at 144, 653 x 7782 x 2248 with GELU
+// 96 and 60, 91 x 9152 x 1344 with its K split four ways 1.8 times the 64-wide tiles that need no split.)
+inline LinearPlan linear_plan(int m, int n, int k, bool f32, int sms) {
+  LinearPlan g;
+  g.tiles_m = (m - 1) / 128 + 1;
+  g.bm = ((m - 1) / g.tiles_m / 16 + 1) * 16;
+  g.bn = 16; g.ks = 1;
+  const int nkb = (k - 1) / GEMM_BK + 1;
+  if (f32) linear_split_f32(g, n, nkb, sms);
+  if (g.ks == 1) {
+    const double operand_rate = k % GEMM_BK == 0 ? 2.0 / 58 : 2.0 / 42;      // cycles a byte of two CTAs' operands takes
+    double best = 1e300;
+    for (int ks = 1; ks <= (f32 ? 1 : 8); ks <<= 1)
+      for (int bn = ks == 1 ? 16 : 32 * ks; bn <= 256 && (ks > 1 || bn < n + 16); bn += ks == 1 ? 16 : bn) {       // (of equals the narrowest)
+        const long long ctas = (long long)g.tiles_m * ((n - 1) / bn + 1) * ks;
+        if (!linear_split_fits(g.bm, bn, ks, nkb) || (ks > 1 && ctas > 2 * sms)) continue;
+        const long long rounds = ctas <= 2 * sms ? 1 : (ctas - 1) / (2 * sms) + 1;
+        const double own = bn > 100 ? 4.0 * bn : 400.0, operands = (g.bm + bn) * GEMM_BK * 2 * operand_rate;
+        double kb = 2 * own > operands ? 2 * own : operands;
+        if (ctas <= sms) {
+          const double trip = 2600.0 / linear_stages(g.bm, bn);
+          kb = own > trip ? own : (trip < kb ? trip : kb);
+        }
+        const double t = (double)(rounds * ((nkb + ks - 1) / ks)) * kb + (bn <= 128 ? 1 : rounds) * 2400.0 + (ks > 1 ? 50.0 * bn : 0);
+        if (t < best) { best = t; g.bn = bn; g.ks = ks; }
+      }
+  }
+  g.tiles = g.tiles_m * ((n - 1) / g.bn + 1);
+  g.stages = linear_stages(g.bm, g.bn);
+  return g;
+}
+
+}  // namespace vla

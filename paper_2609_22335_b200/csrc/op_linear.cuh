@@ -10,13 +10,12 @@
 // distributed shared memory, each CTA its share of the columns.
 #pragma once
 #include "dispatch.cuh"
+#include "linear_plan.h"
 
 namespace vla {
 
 constexpr int LIN_EPI_WARPS = 8;
 constexpr int LIN_THREADS = 64 + 32 * LIN_EPI_WARPS;
-constexpr int LIN_MAX_STAGES = 12;
-constexpr int LIN_SMEM = 110 * 1024;          // half an SM
 constexpr int LIN_AHEAD = 8;                  // k-blocks
 constexpr int LIN_TMEM_COLS = 256;            // half an SM: two accumulators of up to 128 columns, or one of 256
 
@@ -27,39 +26,6 @@ struct LinearArgs {
   unsigned* err;                              // 0, or why a wait ran out
 };
 
-inline int linear_stages(int bm, int bn) {
-  const int stage = (bm + bn) * GEMM_BK * 2, tail = stage < 16384 ? 16384 - stage : 0;        // the MMA always reads 128 rows
-  const int s = (LIN_SMEM - tail) / stage;
-  return s > LIN_MAX_STAGES ? LIN_MAX_STAGES : s;
-}
-// Tile width and K split of a call: the pair with the least estimated time.  Per k-block a CTA needs max(operand bytes over
-// 47 B/clk, MMA issue) cycles alone on its SM and max(2 x bytes over 90 B/clk, 2 x MMA) beside another one; a tile adds its
-// operand round trip and epilogue (behind the next tile's main loop where there are two accumulators), a split its
-// exchange.  Cycles, from sweeps over six shapes: the pair chosen is within 6 % of the best one there.
-inline void linear_plan(LinearArgs& g, int sms) {
-  g.tiles_m = (g.m + 127) / 128;
-  g.bm = (int)(((g.m + g.tiles_m - 1) / g.tiles_m + 15) / 16 * 16);
-  const int nkb = g.kp / GEMM_BK;
-  double best = 1e300;
-  // Widths: powers of two; with more tiles than the chip holds at once also the multiples of 16 above 128, which fill the last
-  // round better (4225 x 2304 x 768 28 -> 21 us, 9000 x 3000 x 264 45 -> 37, 8192 x 3072 x 768 48.2 -> 47.4).
-  const bool fine = (long long)g.tiles_m * ((g.n + 255) / 256) > 2 * sms;
-  for (int bn = 256; bn >= 16; bn = fine && bn > 128 ? bn - 16 : bn >> 1)
-    for (int ks = 1; ks <= 8 && (ks == 1 || (bn >= 32 * ks && nkb >= 2 * ks)); ks <<= 1) {
-      if (ks > 1 && 128 * (bn / ks) * (ks - 1) * 4 > linear_stages(g.bm, bn) * (g.bm + bn) * GEMM_BK * 2) continue;
-      const long long tiles = (long long)g.tiles_m * ((g.n + bn - 1) / bn), ctas = tiles * ks;
-      if (ks > 1 && ctas > 2 * sms) continue;                                                   // (a split tile is a cluster of its own)
-      const bool pair = ctas > sms;
-      const double bytes = (double)(g.bm + bn) * GEMM_BK * 2, mma = bn <= 64 ? 200 : 2.0 * bn;
-      const double kb = pair ? (2 * bytes / 90 > 2 * mma ? 2 * bytes / 90 : 2 * mma) : (bytes / 47 > mma ? bytes / 47 : mma);
-      const double rounds = (double)((ctas + 2 * sms - 1) / (2 * sms));
-      const double tail = 1500 + 16.0 * bn / ks;
-      const double t = rounds * ((nkb + ks - 1) / ks) * kb + (bn <= 128 ? 1 : rounds) * tail + 2500 + (ks > 1 ? 2500 + 8.0 * bn : 0);
-      if (t < best) { best = t; g.bn = bn; g.ks = ks; }
-    }
-  g.tiles = g.tiles_m * ((g.n + g.bn - 1) / g.bn);
-  g.stages = linear_stages(g.bm, g.bn);
-}
 // Features a store may cover: what every row's start and the width allow.  Eight go out as 16 bytes of bf16 or four pairs of
 // fp32, two as a pair, and an odd width (or address) leaves single elements.  8192 tokens, K = 768, GELU, bf16: 3072 features 40 us,
 // 3076 in pairs 47 (96 in single elements), 3073 105; K = 64 without GELU 13.7, 24 (71), 87.  A kernel for each: chosen at run time

@@ -195,7 +195,8 @@ int vla_op_linear(const void* a, const void* w, float* out32, void* out16, int32
   LinearArgs g;
   g.m = m; g.n = n; g.kp = (int)op_pad(k, GEMM_BK); g.act = act;
   g.out32 = out32; g.out16 = static_cast<unsigned short*>(out16);
-  linear_plan(g, dev->sms);
+  const LinearPlan p = linear_plan(m, n, k, out32 != nullptr, dev->sms);
+  g.bm = p.bm; g.bn = p.bn; g.ks = p.ks; g.tiles_m = p.tiles_m; g.tiles = p.tiles; g.stages = p.stages;
   g.err = dev->error.load(std::memory_order_relaxed);
   OpMaps maps;
   if (!op_encode(&maps.m[0], w, n, k, k, g.bn) || !op_encode(&maps.m[1], a, m, k, k, g.bm)) return VLA_ERR_CUDA;

@@ -1,0 +1,7 @@
+// Host build of the linear layer's tile plan for the CPU tests.
+#include "../paper_2609_22335_b200/csrc/linear_plan.h"
+
+extern "C" void linear_plan_host(int m, int n, int k, int f32, int sms, int* out /*[6]: bm, bn, ks, tiles_m, tiles, stages*/) {
+  const vla::LinearPlan p = vla::linear_plan(m, n, k, f32 != 0, sms);
+  out[0] = p.bm; out[1] = p.bn; out[2] = p.ks; out[3] = p.tiles_m; out[4] = p.tiles; out[5] = p.stages;
+}

@@ -30,3 +30,19 @@ def test_widths_and_addresses(m, n, k):
         assert torch.equal(o16[off:off + m * n].reshape(m, n), got.to(torch.bfloat16))
         for o in (o32, o16):
             assert (o[:off] == 7).all() and (o[off + m * n:] == 7).all()
+
+
+@pytest.mark.parametrize("m,n,k", [
+    (129, 4833, 64), (129, 4790, 64), (129, 5925, 64), (129, 7154, 64),               # widths 48, 80, 96, 112
+    (300, 6284, 72), (4000, 578, 64), (300, 8038, 64), (4000, 733, 72), (4000, 784, 72), (800, 4388, 72), (4000, 923, 72),   # 144 .. 240
+    (129, 4756, 1992), (257, 2370, 2056)])                                            # K shared by two and four CTAs, for fp32 results only
+def test_widths_that_are_no_power_of_two(m, n, k):
+    import torch
+    from paper_2609_22335_b200 import api
+    g = torch.Generator(device="cuda").manual_seed(n)
+    a = torch.randn(m, k, device="cuda", generator=g).to(torch.bfloat16)
+    w = (k ** -0.5 * torch.randn(n, k, device="cuda", generator=g)).to(torch.bfloat16)
+    ref = a.double() @ w.double().T
+    sums = 2.0 ** -23 * (k / 16 + 2) * float(ref.abs().max())          # a unit in the last place per 16 products
+    assert float((api.op_linear(a, w).double() - ref).abs().max()) <= sums
+    assert bool(((api.op_linear(a, w, out_bf16=True).double() - ref).abs() <= 2.0 ** -8 * ref.abs() + 2 * sums).all())

@@ -1,0 +1,55 @@
+"""The tile plan of the stand-alone linear layer (csrc/linear_plan.h, compiled for the host): whatever the shape, the tiles cover
+the result, the stages fit half an SM, and a split's partial sums fit the stages and its clusters the chip."""
+import ctypes as C
+import os
+import random
+import subprocess
+
+import pytest
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+
+
+@pytest.fixture(scope="module")
+def plan(tmp_path_factory):
+    out = tmp_path_factory.mktemp("plan") / "libplan_host.so"
+    subprocess.run(["g++", "-std=c++17", "-O1", "-shared", "-fPIC", "-x", "c++", os.path.join(HERE, "linear_plan_host_shim.cc"),
+                    "-o", str(out)], check=True)
+    lib = C.CDLL(str(out))
+
+    def call(m, n, k, f32=False, sms=148):
+        o = (C.c_int * 6)()
+        lib.linear_plan_host(m, n, k, int(f32), sms, o)
+        return dict(zip(("bm", "bn", "ks", "tiles_m", "tiles", "stages"), o))
+    return call
+
+
+def test_every_plan_is_one_the_kernel_can_run(plan):
+    rnd = random.Random(3)
+    shapes = [(m, n, k) for m in (1, 16, 17, 64, 127, 128, 129, 100000) for n in (1, 7, 16, 255, 256, 257, 70000) for k in (8, 64, 72, 4096, 20000)]
+    shapes += [(int(2 ** rnd.uniform(0, 14)), int(2 ** rnd.uniform(0, 15)), 8 * int(2 ** rnd.uniform(0, 11))) for _ in range(3000)]
+    for m, n, k in shapes:
+        for sms, f32 in ((148, False), (148, True), (132, False), (7, False), (7, True)):
+            p = plan(m, n, k, f32, sms)
+            bm, bn, ks, stages = p["bm"], p["bn"], p["ks"], p["stages"]
+            assert bm % 16 == 0 and 16 <= bm <= 128 and p["tiles_m"] * bm >= m > (p["tiles_m"] - 1) * bm
+            assert bn % 16 == 0 and 16 <= bn <= 256 and p["tiles"] == p["tiles_m"] * -(-n // bn)
+            stage = (bm + bn) * 128
+            assert 2 <= stages <= 12 and stages * stage + max(0, 16384 - stage) <= 110 * 1024
+            assert ks in (1, 2, 4, 8)
+            if ks > 1:
+                assert bn in (32, 64, 128, 256) and bn % (32 * ks) == 0 and -(-k // 64) >= 2 * ks and p["tiles"] * ks <= 2 * sms
+                assert 128 * (bn // ks) * (ks - 1) * 4 <= stages * stage
+
+
+def test_widths_that_fill_the_chip(plan):
+    """Shapes where a power of two leaves a second CTA to a few SMs, or a second round to a few CTAs."""
+    pairs = [(p["bn"], p["ks"]) for p in (plan(3455, 1392, 8448), plan(1441, 4360, 6256), plan(653, 7782, 2248), plan(452, 6648, 6024),
+                                          plan(8192, 3072, 768), plan(50, 2048, 720))]
+    assert pairs == [(144, 1), (192, 1), (160, 1), (192, 1), (240, 1), (16, 1)]
+
+
+def test_fp32_results_keep_their_split(plan):
+    """Sums are split where they are long and the chip has room, whatever a width without a split would gain."""
+    for shape, ks in (((288, 11008, 4096), 2), ((452, 6648, 6024), 2), ((938, 1352, 6144), 4), ((91, 9152, 1344), 4), ((8192, 3072, 768), 1)):
+        assert plan(*shape, f32=True)["ks"] == ks
