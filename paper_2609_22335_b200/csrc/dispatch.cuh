@@ -160,9 +160,6 @@ constexpr unsigned RETIRE_SLEEP_NS = 4000;   // retire warp: longest sleep witho
 // length: the SM where the next tile ends is the better place, a second tile beside a first makes both of them late.  1, 4, 8,
 // 16 us: 4 streams x 3 43.4, 41.7, 40.3, 39.5 ms; 8 x 3 GR00T 40.1, 38.6, 37.1, 36.3; 64 us brings nothing more.
 constexpr unsigned long long SPREAD_WAIT_NS = 16000;
-// A node whose predecessors' tiles have all been taken may be queued before they finish (its workers wait holding their
-// weights) as long as everything queued or running still fits one tile per SM.
-constexpr int EARLY_MAX_TILES = 148;
 constexpr unsigned long long HEAD_WAIT_NS = 1500;   // an action-head tile nobody took for this long may go to a running worker
 
 static_assert(sizeof(NodeDesc) % 16 == 0 && sizeof(NodeDesc) <= 512, "a node's description is copied by one warp, 16 bytes a lane");
@@ -307,12 +304,12 @@ __device__ __forceinline__ void retire_loop(const DeviceCtx& ctx, SmState* sm, i
       continue;
     }
     // ---- starts.  The last tile of a node has been taken by a worker: tiles of a class are claimed in queue order, so all of
-    // them have been claimed.  Where that was the last predecessor of a successor, and the GPU has idle SMs for it, the successor
-    // is queued now: its tiles are taken, fetch their weights and wait for the release, instead of going through the queues
-    // after it (hand-over 3 us instead of 9).  No cycle can arise: a waiting tile waits only for tiles claimed before it, a
-    // worker takes tiles that may have to wait in the order of their claims (see priority_goes_first), and such a tile holds
-    // shared memory while it waits only on an SM where nothing claimed before it still needs some (see the worker's
-    // allocation).
+    // them have been claimed.  Where that was the last predecessor of a successor, and everything queued or running still fits
+    // one tile per SM (up to two per SM: 4 x 3 cfg2 43.3 -> 42.0 ms, but CogACT 18.8 -> 19.7), the successor is queued now: its
+    // tiles are taken, fetch their weights and wait for the release, instead of going through the queues after it (hand-over 3 us
+    // instead of 9).  No cycle can arise: a waiting tile waits only for tiles claimed before it, a worker takes tiles that may
+    // have to wait in the order of their claims (see priority_goes_first), and such a tile holds shared memory while it waits
+    // only on an SM where nothing claimed before it still needs some (see the worker's allocation).
     if (__any_sync(0xffffffffu, started)) {
       uint32_t inst = 0;
       int succ0 = 0, n_succ = 0;
@@ -332,7 +329,7 @@ __device__ __forceinline__ void retire_loop(const DeviceCtx& ctx, SmState* sm, i
           const size_t at = (size_t)inst * ctx.n_nodes + si.node;
           if (atomicSub(ctx.start_count + at, 1) == 1) {
             ctx.start_count[at] = (int)((uint32_t)si.cls_res >> 20);
-            early = sm->outstanding + si.n_tiles <= EARLY_MAX_TILES;
+            early = sm->outstanding + si.n_tiles <= (int)gridDim.x;
             // marked before this SM reports the tile finished, so whoever releases the node sees the mark
             if (early) atomicOr(ctx.dep_word + at, 1ull << 63);
           }
