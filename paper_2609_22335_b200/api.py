@@ -275,7 +275,12 @@ class Engine:
         self._check(self.lib.vla_wait_idle(self.ctx, timeout_ms))
 
     def run(self, frames, timeout_s=600.0):
-        """frames[r][n] -> chunks[r][n]; submits as fast as the rings accept and polls in frame order."""
+        """frames[r][n] -> chunks[r][n]; submits as fast as the rings accept and polls in frame order.
+
+        The calling thread polls without a pause until nothing has come for 0.1 s (a chunk is usually milliseconds away, and a
+        sleep would add its 60 us and more): it keeps one host core busy while frames are in flight.  A program that cannot
+        spare the core calls ``submit`` and ``poll`` in its own rhythm.
+        """
         import time
         R = len(frames)
         base = list(self._frames_done)
@@ -305,7 +310,7 @@ class Engine:
                 last = now
             elif now - t0 > timeout_s:
                 raise TimeoutError("no progress")
-            elif now - last > 0.1:        # a chunk is usually milliseconds away: a sleep would add its 60 us and more
+            elif now - last > 0.1:
                 time.sleep(0.0002)
         return got
 

@@ -443,7 +443,10 @@ __device__ __forceinline__ void gemm_epilogue(const TileCtx& c, const GemmArgs& 
 }
 
 // Addends of the warp's tokens (`live` from `tok` on) into the accumulators (fragment layout; columns past the last feature
-// get zero).  Two fragments at a time, all loads of an addend before the first use: 32 tokens x 32 columns, or with up to 64
+// get zero).  The tensor core then sums from them, in fp32 but without the rounding that an addition behind the product has:
+// next to an exact result, rel-L2 4.9e-6 instead of 2.3e-6 for an addend of the product's size and K = 3072, 6.4e-6 instead of
+// 5.7e-8 for one 64 times as large -- in streams whose bf16 mirror is what the next GEMM reads; whole frames are as close to the
+// fp64 oracle as with the addition (cfg1 3.17e-4, 3.26e-4 before; cfg2 layers 1.39e-3, 1.41e-3).  Two fragments at a time, all loads of an addend before the first use: 32 tokens x 32 columns, or with up to 64
 // tokens in the tile (16 per warp) 16 x 64.
 __device__ __forceinline__ void preload_rows(const TileCtx& c, const GemmArgs& g, uint32_t tmem, int tok, int live, int tpw, int lane, int r0) {
   const int q = lane & 3, cols = min(GEMM_BM, g.N - r0), under = g.under;
