@@ -42,10 +42,10 @@ CLASS_TAGS = None        # profiled intensity tags (--tags), else the library's 
 HEAD_PASSES = 1          # action-head passes per VLM pass (--head-passes): asynchronous inference
 METRIC = "action_chunks_per_sec"
 UNIT = "chunks/s"
-# DRAM bytes per action chunk of the persistent kernel, from the one-launch ncu capture of 32 request streams x 2 frames
-# summarised in profiles/cosched_kernel_cfg2_dram_and_pipes.md (109.08 GB read + 49.88 GB written for 64 chunks; the
-# 8-stream capture gives 2.41 GB per chunk, so traffic grows in proportion to the chunks and is scaled by them)
-MEASURED_DRAM_BYTES_PER_CHUNK = {"cfg2_smolvla": (109.08e9 + 49.88e9) / 64}
+# DRAM bytes per action chunk of the persistent kernel, from two one-launch ncu captures of 32 request streams x 2 frames
+# summarised in profiles/cosched_kernel_cfg2_dram_and_pipes.md (309.27 GB read + 96.73 GB written for 2 x 64 chunks; scaled by the
+# chunks of the step)
+MEASURED_DRAM_BYTES_PER_CHUNK = {"cfg2_smolvla": (309.27e9 + 96.73e9) / 128}
 
 
 def measured_peaks():

@@ -49,7 +49,7 @@ inline int perm_feature(int p) { return 8 * ((p >> 1) & 3) + 2 * (p >> 3) + (p &
 constexpr int GEMM_SMEM_BUDGET = 64 * 1024;  // stage memory a token-rich GEMM tile aims for (at least two stages are always taken)
 constexpr int GEMM_SMEM_BUDGET_SMALL = 84 * 1024;  // token-poor tiles (<= 64 tokens) are bound by TMA latency and get deeper
                                                    // pipelines, but must fit the room one finished token-rich tile leaves
-                                                   // on an SM that runs three of them (3 x 18 of 55 four-KB units)
+                                                   // on an SM that runs three of them (3 x 18 of 54 four-KB units)
 // TMA pipeline depth of a GEMM tile with `bt` tokens per tile (a 128-row weight tile plus the activation tile per stage).
 inline int gemm_stage_bytes(int bt) { return GEMM_BM * GEMM_BK * 2 + bt * GEMM_BK * 2; }
 inline int gemm_stages(int bt, int Kp) {

@@ -1,4 +1,4 @@
-"""Times the stand-alone operators (the engine's GEMM and attention tile bodies as ordinary kernels).
+"""Times the stand-alone operators (linear layer and fused attention on caller-owned tensors).
 
     python -m paper_2609_22335_b200.opbench linear M N K [--act 0|1|2] [--f32] [--iters 20]
     python -m paper_2609_22335_b200.opbench attention TQ TKV HQ HKV HD [--causal] [--iters 20]

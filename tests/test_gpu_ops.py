@@ -1,6 +1,6 @@
-"""Operator-level GPU parity: the GEMM and fused-attention tile bodies, called through the C ABI on
-their own, against the CPU oracle's `linear`, activations and `attention` (fp64) on the same
-bf16-representable inputs.  Shapes span several tiles, ragged tails and the degenerate cases."""
+"""Operator-level GPU parity: the stand-alone linear layer and fused attention (kernels of their own; the engine's tile
+bodies have test_gpu_tile_bodies.py), called through the C ABI, against the CPU oracle's `linear`, activations and
+`attention` (fp64) on the same bf16-representable inputs.  Shapes span several tiles, ragged tails and the degenerate cases."""
 import numpy as np
 import pytest
 

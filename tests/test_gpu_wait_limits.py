@@ -109,7 +109,7 @@ def test_operator_wait_runs_out_and_status_reports_it():
 
 
 def test_tiles_of_mixed_sizes_never_starve_for_room():
-    """Head-dimension-256 attention tiles (36 of an SM's 55 shared-memory units) next to 16-18-unit GEMM tiles:
+    """Head-dimension-256 attention tiles (48 of an SM's 54 shared-memory units) next to 16-18-unit GEMM tiles:
     a worker that waits for room is served before its SM's other workers get new tiles, so with a wait limit far
     below the default the run completes without a timeout, bit-identical to the serial mode."""
     from paper_2609_22335_b200 import Engine
