@@ -5,7 +5,7 @@
 
 Prints one JSON line: microseconds per call (CUDA events around `iters` back-to-back calls after three
 warm-up calls) and the achieved TFLOP/s (2 M N K, or 4 TQ TKV HQ HD).  Also the command to put under ncu
-when a tile body is profiled on its own.
+when an operator is profiled.
 """
 from __future__ import annotations
 
