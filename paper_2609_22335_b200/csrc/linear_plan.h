@@ -9,10 +9,24 @@ constexpr int LIN_SMEM = 110 * 1024;          // half an SM
 
 struct LinearPlan { int bm, bn, ks, tiles_m, tiles, stages; };   // tokens and features of a tile, CTAs that share its K, tiles, pipeline depth
 
-inline int linear_stages(int bm, int bn) {
-  const int stage = (bm + bn) * GEMM_BK * 2, tail = stage < 16384 ? 16384 - stage : 0;        // the MMA always reads 128 rows
-  const int s = (LIN_SMEM - tail) / stage;
-  return s > LIN_MAX_STAGES ? LIN_MAX_STAGES : s;
+// (Every call of the operator pays for this arithmetic, and divisions are most of it: bm and bn are multiples of 16, so what is
+// divided by them comes from tables.)
+struct LinearTables {
+  int stages[25] = {};            // by (bm + bn) / 16
+  uint64_t recip[17] = {};        // by j: x * recip >> 36 = x / j for x below 2^32
+  constexpr LinearTables() {
+    for (int i = 2; i <= 24; ++i) {
+      const int stage = i * 16 * GEMM_BK * 2, tail = stage < 16384 ? 16384 - stage : 0;       // the MMA always reads 128 rows
+      const int s = (LIN_SMEM - tail) / stage;
+      stages[i] = s > LIN_MAX_STAGES ? LIN_MAX_STAGES : s;
+    }
+    for (int j = 1; j <= 16; ++j) recip[j] = ((1ull << 36) + j - 1) / j;
+  }
+};
+constexpr LinearTables kLinearTables;
+inline int linear_stages(int bm, int bn) { return kLinearTables.stages[(bm + bn) >> 4]; }
+inline long long linear_tiles_n(int n, int bn) {                              // features / bn, rounded up
+  return (long long)(((uint64_t)((unsigned)(n - 1) >> 4) * kLinearTables.recip[bn >> 4]) >> 36) + 1;
 }
 // Whether a cluster of `ks` CTAs can share the K range of a tile of `bn` features: each finishes a whole number of 32-column
 // groups, and the others' partial sums of those have to fit its stages.
@@ -28,7 +42,7 @@ inline void linear_split_f32(LinearPlan& g, int n, int nkb, int sms) {
   double best = 1e300;
   for (int bn = 256; bn >= 16; bn >>= 1)
     for (int ks = 1; ks <= 8; ks <<= 1) {
-      const long long ctas = (long long)g.tiles_m * ((n - 1) / bn + 1) * ks, rounds = (ctas + 2 * sms - 1) / (2 * sms);
+      const long long ctas = g.tiles_m * linear_tiles_n(n, bn) * ks, rounds = ctas <= 2 * sms ? 1 : (ctas - 1) / (2 * sms) + 1;
       if (!linear_split_fits(g.bm, bn, ks, nkb) || (ks > 1 && ctas > 2 * sms)) continue;         // (a split tile is a cluster of its own)
       const double bytes = (double)(g.bm + bn) * GEMM_BK * 2, mma = bn <= 64 ? 200 : 2.0 * bn;
       const double kb = ctas > sms ? (2 * bytes / 90 > 2 * mma ? 2 * bytes / 90 : 2 * mma) : (bytes / 47 > mma ? bytes / 47 : mma);
@@ -54,9 +68,9 @@ inline LinearPlan linear_plan(int m, int n, int k, bool f32, int sms) {
   if (g.ks == 1) {
     const double operand_rate = k % GEMM_BK == 0 ? 2.0 / 58 : 2.0 / 42;      // cycles a byte of two CTAs' operands takes
     double best = 1e300;
-    for (int ks = 1; ks <= (f32 ? 1 : 8); ks <<= 1)
+    for (int ks = 1, shift = 0; ks <= (f32 ? 1 : 8) && nkb >= ks; ks <<= 1, ++shift)
       for (int bn = ks == 1 ? 16 : 32 * ks; bn <= 256 && (ks > 1 || bn < n + 16); bn += ks == 1 ? 16 : bn) {       // (of equals the narrowest)
-        const long long ctas = (long long)g.tiles_m * ((n - 1) / bn + 1) * ks;
+        const long long ctas = g.tiles_m * linear_tiles_n(n, bn) * ks;
         if (!linear_split_fits(g.bm, bn, ks, nkb) || (ks > 1 && ctas > 2 * sms)) continue;
         const long long rounds = ctas <= 2 * sms ? 1 : (ctas - 1) / (2 * sms) + 1;
         const double own = bn > 100 ? 4.0 * bn : 400.0, operands = (g.bm + bn) * GEMM_BK * 2 * operand_rate;
@@ -65,11 +79,11 @@ inline LinearPlan linear_plan(int m, int n, int k, bool f32, int sms) {
           const double trip = 2600.0 / linear_stages(g.bm, bn);
           kb = own > trip ? own : (trip < kb ? trip : kb);
         }
-        const double t = (double)(rounds * ((nkb + ks - 1) / ks)) * kb + (bn <= 128 ? 1 : rounds) * 2400.0 + (ks > 1 ? 50.0 * bn : 0);
+        const double t = (double)(rounds * ((nkb + ks - 1) >> shift)) * kb + (bn <= 128 ? 1 : rounds) * 2400.0 + (ks > 1 ? 50.0 * bn : 0);
         if (t < best) { best = t; g.bn = bn; g.ks = ks; }
       }
   }
-  g.tiles = g.tiles_m * ((n - 1) / g.bn + 1);
+  g.tiles = (int)(g.tiles_m * linear_tiles_n(n, g.bn));
   g.stages = linear_stages(g.bm, g.bn);
   return g;
 }
