@@ -341,6 +341,74 @@ __device__ __forceinline__ void epi_stream(const TileCtx& c, const EpiPlace& e, 
     }
   });
 }
+// Residual rows, fp32, in the fragment layout: this lane's two tokens of a half, eight features of each, of two groups of 32
+// columns.  The first two groups are asked for in front of the main loop, each later one in the place of a group just added: half
+// the round trips lie under the loop, where laying the rows under the accumulators had all four of a 128-token tile in front of it,
+// and the sum is rounded once, not once per MMA (32 streams x 4 178.8 -> 177.4 ms, GR00T 8 x 3 36.3 -> 36.0, CogACT 18.73 -> 18.52).
+// Four groups held at once need 440 bytes of spills.
+struct ResidRows { float4 v[2][2][2]; };
+__device__ __forceinline__ void resid_load(const float* x, int ldx, int tok, int live, int half, int lane, int cols, int c, float4 (&v)[2][2]) {
+  const int q = lane & 3;
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    const float4* p = reinterpret_cast<const float4*>(x + (size_t)(tok + min(16 * half + 8 * k + (lane >> 2), live - 1)) * ldx + min(32 * c + 8 * q, cols - 8));
+    v[k][0] = __ldcg(p); v[k][1] = __ldcg(p + 1);
+  }
+}
+// epi_stream with such rows (x: the tile's columns of them).
+template <bool MIRROR>
+__device__ __forceinline__ void epi_resid(const EpiPlace& e, const GemmArgs& g, const float* x, ResidRows& r, float* out32, unsigned short* out16, float* ssq, int ft) {
+  const int q = e.lane & 3;
+#pragma unroll 1
+  for (int h = 0; h < 2 && 16 * h < e.live; ++h) {
+    const int row = 16 * h + (e.lane >> 2);
+    const uint32_t tmem = e.tmem + ((uint32_t)(16 * h) << 16);
+    float* pa = out32 + (size_t)(e.tok + row) * g.ldo32 + e.r0 + 8 * q;
+    float* pb = pa + (size_t)8 * g.ldo32;
+    unsigned short* ha = MIRROR ? out16 + (size_t)(e.tok + row) * g.ldo16 + e.r0 + 8 * q : nullptr;
+    unsigned short* hb = MIRROR ? ha + (size_t)8 * g.ldo16 : nullptr;
+    float sa = 0.f, sb = 0.f;
+    uint32_t nx[EPI];
+#pragma unroll 1
+    for (int c2 = 0; c2 < GEMM_BM / 32; c2 += 2) {
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        const int c = c2 + i;
+        float v[EPI];
+        tmem_ld_frag(tmem + 32u * (uint32_t)c, nx);
+        tmem_ld_wait();
+#pragma unroll
+        for (int j = 0; j < EPI; ++j) v[j] = __uint_as_float(nx[j]);
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+          const float4 lo = r.v[i][k][0], hi = r.v[i][k][1];
+          float* u = v + 2 * k;
+          u[0] += lo.x; u[1] += lo.y; u[4] += lo.z; u[5] += lo.w;
+          u[8] += hi.x; u[9] += hi.y; u[12] += hi.z; u[13] += hi.w;
+        }
+        if (c2 == 0 || 16 * (h + 1) < e.live) resid_load(x, g.ldx, e.tok, e.live, c2 == 0 ? h : h + 1, e.lane, e.cols, c2 == 0 ? c + 2 : c - 2, r.v[i]);
+        const bool fok = 32 * c + 8 * q < e.cols;
+        if (MIRROR && fok) {
+#pragma unroll
+          for (int b = 0; b < 4; ++b) {
+            sa = fmaf(v[4 * b], v[4 * b], sa); sa = fmaf(v[4 * b + 1], v[4 * b + 1], sa);
+            sb = fmaf(v[4 * b + 2], v[4 * b + 2], sb); sb = fmaf(v[4 * b + 3], v[4 * b + 3], sb);
+          }
+        }
+        if (fok && row < e.live) { st_row8(pa + 32 * c, v); if (MIRROR) st_row8(ha + 32 * c, v); }
+        if (fok && row + 8 < e.live) { st_row8(pb + 32 * c, v + 2); if (MIRROR) st_row8(hb + 32 * c, v + 2); }
+      }
+    }
+    tmem_ld_wait();
+    if (MIRROR && ssq) {
+      sa += __shfl_xor_sync(0xffffffffu, sa, 1); sb += __shfl_xor_sync(0xffffffffu, sb, 1);
+      sa += __shfl_xor_sync(0xffffffffu, sa, 2); sb += __shfl_xor_sync(0xffffffffu, sb, 2);
+      float* sp = ssq + (size_t)(e.tok + row) * g.ss_out_ld + ft;
+      if (q == 0 && row < e.live) sp[0] = sa;
+      if (q == 0 && row + 8 < e.live) sp[(size_t)8 * g.ss_out_ld] = sb;
+    }
+  }
+}
 // Rows of V^T: a token per lane, so that a warp writes 32 consecutive tokens of a feature.
 __device__ __forceinline__ void epi_vt(const EpiPlace& e, const GemmArgs& g, unsigned short* outT, int split) {
   unsigned short* const base = outT + e.tok + e.lane;
@@ -409,7 +477,7 @@ __device__ __forceinline__ void epi_general(const TileCtx& c, const GemmArgs& g,
 
 // This warp's tokens of the tile: `live` of them from `tok` on.  r0: the tile's first weight row, rs: row scale of the token
 // in this lane.
-__device__ __forceinline__ void gemm_epilogue(const TileCtx& c, const GemmArgs& g, uint32_t tmem, int tok, int live, int lane, int r0, float rs, int ft) {
+__device__ __forceinline__ void gemm_epilogue(const TileCtx& c, const GemmArgs& g, uint32_t tmem, int tok, int live, int lane, int r0, float rs, int ft, ResidRows& resid) {
   EpiPlace e;
   e.tmem = tmem; e.tok = tok; e.live = live; e.lane = lane; e.r0 = r0; e.rs = rs;
   e.cols = min(GEMM_BM, (g.dual ? 2 * g.N : g.N) - r0);
@@ -421,7 +489,11 @@ __device__ __forceinline__ void gemm_epilogue(const TileCtx& c, const GemmArgs& 
     else epi_gated<ACT_NONE>(e, g, out16);
   } else if (g.out32 != 0) {
     float* const out32 = resolve<float>(c, g.out32);
-    if (g.fast == 2) {
+    if (g.resid) {
+      const float* const x = resolve<const float>(c, g.X) + r0;
+      if (out16) epi_resid<true>(e, g, x, resid, out32, out16, resolve<float>(c, g.ss_out), ft);
+      else epi_resid<false>(e, g, x, resid, out32, nullptr, nullptr, ft);
+    } else if (g.fast == 2) {
       if (out16) epi_stream<true, true>(c, e, g, out32, out16, nullptr, ft);
       else epi_stream<false, true>(c, e, g, out32, nullptr, nullptr, ft);
     } else if (out16) epi_stream<true, false>(c, e, g, out32, out16, resolve<float>(c, g.ss_out), ft);
@@ -442,12 +514,10 @@ __device__ __forceinline__ void gemm_epilogue(const TileCtx& c, const GemmArgs& 
   }
 }
 
-// Addends of the warp's tokens (`live` from `tok` on) into the accumulators (fragment layout; columns past the last feature
-// get zero).  The tensor core then sums from them, in fp32 but without the rounding that an addition behind the product has:
-// next to an exact result, rel-L2 4.9e-6 instead of 2.3e-6 for an addend of the product's size and K = 3072, 6.4e-6 instead of
-// 5.7e-8 for one 64 times as large -- in streams whose bf16 mirror is what the next GEMM reads; whole frames are as close to the
-// fp64 oracle as with the addition (cfg1 3.17e-4, 3.26e-4 before; cfg2 layers 1.39e-3, 1.41e-3).  Two fragments at a time, all loads of an addend before the first use: 32 tokens x 32 columns, or with up to 64
-// tokens in the tile (16 per warp) 16 x 64.
+// Biases, broadcast vectors and tables of the warp's tokens (`live` from `tok` on) into the accumulators (fragment layout; columns
+// past the last feature get zero).  The tensor core then sums from them, in fp32 but without the rounding that an addition behind
+// the product has; residual rows are added behind it (epi_resid).  Two fragments at a time, all loads of an addend before the first
+// use: 32 tokens x 32 columns, or with up to 64 tokens in the tile (16 per warp) 16 x 64.
 __device__ __forceinline__ void preload_rows(const TileCtx& c, const GemmArgs& g, uint32_t tmem, int tok, int live, int tpw, int lane, int r0) {
   const int q = lane & 3, cols = min(GEMM_BM, g.N - r0), under = g.under;
   const int dcol = tpw == 16 ? 32 : 0;                 // second fragment: that many columns on, or (0) 16 tokens on
@@ -479,13 +549,10 @@ __device__ __forceinline__ void preload_rows(const TileCtx& c, const GemmArgs& g
           v[k][4] += t[k][1].x; v[k][5] += t[k][1].y; v[k][6] += t[k][1].z; v[k][7] += t[k][1].w;
         }
       };
-      if (under & 4) add(g.X, g.ldx);
-      if (under & 27) {
 #pragma unroll 1
-        for (int m = under & 27; m != 0; m &= m - 1) {
-          const int which = m & -m;
-          add(which == 1 ? g.bias : (which == 2 ? g.vec : (which == 8 ? g.tab : g.tab2)), which == 8 ? g.ldtab : (which == 16 ? g.ldtab2 : 0));
-        }
+      for (int m = under; m != 0; m &= m - 1) {
+        const int which = m & -m;
+        add(which == 1 ? g.bias : (which == 2 ? g.vec : (which == 8 ? g.tab : g.tab2)), which == 8 ? g.ldtab : (which == 16 ? g.ldtab2 : 0));
       }
       if (!in2) {
 #pragma unroll
@@ -600,12 +667,22 @@ __device__ __forceinline__ void tile_gemm(const TileCtx& c, const GemmArgs& g, i
   const int tpw = bt <= 64 ? 16 : 32;
   const bool warp_live = warp * tpw < nt;
   const uint32_t my_tmem = c.tmem + ((uint32_t)(warp * 32) << 16);
-  // What is added to the product goes into the accumulators before the first MMA: its round trip then lies beside that of
-  // the first operand stages, and the epilogue neither reads nor adds anything.
+  // Biases and tables go into the accumulators before the first MMA, beside the round trip of the first operand stages; residual
+  // rows are asked for now and added in the epilogue.
   const bool under = g.under != 0;
   if (under) {
     if (warp_live) preload_rows(c, g, my_tmem, t0 + tpw * warp, min(tpw, nt - tpw * warp), tpw, lane, r0);
     tc_fence_before();
+  }
+  ResidRows resid;                                     // (set in every case: left open where there are none, 120 bytes of it were spilled)
+#pragma unroll
+  for (int j = 0; j < 2; ++j)
+#pragma unroll
+    for (int k = 0; k < 2; ++k) resid.v[j][k][0] = resid.v[j][k][1] = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (g.resid && warp_live) {
+    const float* const x = resolve<const float>(c, g.X) + r0;
+#pragma unroll
+    for (int j = 0; j < 2; ++j) resid_load(x, g.ldx, t0 + tpw * warp, min(tpw, nt - tpw * warp), 0, lane, min(GEMM_BM, g.N - r0), j, resid.v[j]);
   }
   // Folded RMSNorm: the partial sums of squares of this lane's token are requested now and added after the main loop, in a
   // fixed order (streams wider than 1024: the rest at once).
@@ -679,7 +756,7 @@ __device__ __forceinline__ void tile_gemm(const TileCtx& c, const GemmArgs& g, i
     for (int j = 0; j < 8; ++j) ssq += part[j];
     rs = 1.0f / sqrtf(ssq / (float)g.rs_d + 1e-6f);
   }
-  if (ready && warp_live) gemm_epilogue(c, g, my_tmem, t0 + tpw * warp, min(tpw, nt - tpw * warp), lane, r0, rs, ft);
+  if (ready && warp_live) gemm_epilogue(c, g, my_tmem, t0 + tpw * warp, min(tpw, nt - tpw * warp), lane, r0, rs, ft, resid);
   tc_fence_before();
   worker_sync(c);
   if (!(c.slot && c.slot->primed) && worker_tid() <= 2 * S) mbar_inval(bar0 + 8u * worker_tid());

@@ -290,11 +290,12 @@ class Builder {
       const bool adds = g.X || g.vec || g.tab || g.tab2, scaled = g.c_acc != 1.0f || g.c_x != 1.0f;
       const bool plain_add = o.norm_gain < 0 && !scaled && g.act == ACT_NONE;           // sums may start from the addends
       if (aligned && !g.dual && (!adds || plain_add) && (!g.bias || o.norm_gain < 0))
-        g.under = (g.bias ? 1 : 0) | (g.vec ? 2 : 0) | (g.X ? 4 : 0) | (g.tab ? 8 : 0) | (g.tab2 ? 16 : 0);
-      const bool all_under = (g.bias ? 1 : 0) + (g.vec ? 2 : 0) + (g.X ? 4 : 0) + (g.tab ? 8 : 0) + (g.tab2 ? 16 : 0) == g.under;
-      g.fast = aligned && g.perm && all_under && !(scaled && !g.dual) &&
+        g.under = (g.bias ? 1 : 0) | (g.vec ? 2 : 0) | (g.tab ? 8 : 0) | (g.tab2 ? 16 : 0);
+      g.resid = aligned && !g.dual && g.X && g.out32 && plain_add;
+      const bool placed = (g.bias ? 1 : 0) + (g.vec ? 2 : 0) + (g.tab ? 8 : 0) + (g.tab2 ? 16 : 0) == g.under && (!g.X || g.resid);
+      g.fast = aligned && g.perm && placed && !(scaled && !g.dual) &&
                (g.dual || g.act == ACT_NONE || (g.act == ACT_GELU && !g.out32 && !g.outT && o.rope_cols == 0));
-      if (!g.fast) g.under = 0;
+      if (!g.fast) g.under = g.resid = 0;
       // the solver update: scaled product, addends behind it
       if (!g.fast && aligned && g.perm && !g.dual && g.act == ACT_NONE && !g.bias && !g.vec && !g.tab2 && g.out32 && !g.outT && g.rope_cols == 0 &&
           ss_view(o.out16).buf < 0)

@@ -70,7 +70,7 @@ int vla_debug_tile_linear(const void* a, const void* w, const float* x, float* o
   g.bt = (int)op_pad((m + g.tiles_t - 1) / g.tiles_t, 16);
   g.stages = gemm_stages(g.bt, g.Kp);
   g.fast = g.perm = fast ? 1 : 0;
-  g.under = fast && x ? 4 : 0;
+  g.resid = fast && x ? 1 : 0;
   nd.smem_bytes = gemm_smem_bytes(g.bt, g.stages);
   nd.tmem_cols = GEMM_BM;
   const int rows = gated ? 2 * n : n, per_tile = gated ? GEMM_BM / 2 : GEMM_BM;

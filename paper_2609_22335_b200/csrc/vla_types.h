@@ -103,8 +103,8 @@ struct GemmArgs {
   int32_t fast;        // straight epilogue: addresses allow whole vectors, nothing but row scale, activation, rotation, gating (2: and
                        // the solver's scaled update)
   int32_t perm;        // the weight rows stand in the accumulator's register order (see perm_feature)
-  int32_t under;       // addends lie in the accumulators before the first MMA: 1 bias, 2 vec, 4 X, 8 tab, 16 tab2
-  int32_t pad_;
+  int32_t under;       // addends lie in the accumulators before the first MMA: 1 bias, 2 vec, 8 tab, 16 tab2
+  int32_t resid;       // X joins behind the product, from registers that were filled in front of it (straight epilogue)
   int32_t act, dual;   // activation; dual (gated): out = act(A Wgate^T) * (A Wup^T), 64 output features per tile
   float c_acc, c_x;    // out = c_x * X + c_acc * acc + vec + tab + tab2
   int32_t wmap, amap;         // tensor-map indices: shared weight maps, activation map relative to the slot's first
