@@ -475,54 +475,42 @@ __device__ __forceinline__ void epi_general(const TileCtx& c, const GemmArgs& g,
   if (ssq && live) ssq[tok * g.ss_out_ld + ft] = sq;
 }
 
-// What the epilogue needs from the node's description, read before the accumulators are waited for.
-enum : int { EPI_GENERAL, EPI_GATED, EPI_GATED_GELU, EPI_GATED_SILU, EPI_RESID, EPI_POST, EPI_STREAM, EPI_PLAIN, EPI_GELU, EPI_ROPE };
-struct EpiPlan { int kind, cols, split; float* out32; unsigned short* out16; float* ssq; };
-__device__ __forceinline__ EpiPlan epi_plan(const TileCtx& c, const GemmArgs& g, int r0) {
-  EpiPlan p;
-  p.cols = min(GEMM_BM, (g.dual ? 2 * g.N : g.N) - r0);
-  p.split = g.outT != 0 ? max(0, min(p.cols, g.t_col0 - r0)) : p.cols;      // columns from here on are V features
-  p.out32 = resolve<float>(c, g.out32); p.out16 = resolve<unsigned short>(c, g.out16); p.ssq = resolve<float>(c, g.ss_out);
-  if (!g.fast) p.kind = EPI_GENERAL;
-  else if (g.dual) p.kind = g.act == ACT_SILU ? EPI_GATED_SILU : (g.act == ACT_GELU ? EPI_GATED_GELU : EPI_GATED);
-  else if (p.out32) p.kind = g.resid ? EPI_RESID : (g.fast == 2 ? EPI_POST : EPI_STREAM);
-  else p.kind = g.act == ACT_GELU ? EPI_GELU : (g.rope_cols > 0 ? EPI_ROPE : EPI_PLAIN);
-  return p;
-}
 // This warp's tokens of the tile: `live` of them from `tok` on.  r0: the tile's first weight row, rs: row scale of the token
 // in this lane.
-__device__ __forceinline__ void gemm_epilogue(const TileCtx& c, const GemmArgs& g, const EpiPlan& p, uint32_t tmem, int tok, int live, int lane, int r0, float rs, int ft, ResidRows& resid) {
+__device__ __forceinline__ void gemm_epilogue(const TileCtx& c, const GemmArgs& g, uint32_t tmem, int tok, int live, int lane, int r0, float rs, int ft, ResidRows& resid) {
   EpiPlace e;
-  e.tmem = tmem; e.tok = tok; e.live = live; e.lane = lane; e.r0 = r0; e.rs = rs; e.cols = p.cols;
-  switch (p.kind) {
-    case EPI_GENERAL: epi_general(c, g, e, ft); return;
-    case EPI_GATED_SILU: epi_gated<ACT_SILU>(e, g, p.out16); return;
-    case EPI_GATED_GELU: epi_gated<ACT_GELU>(e, g, p.out16); return;
-    case EPI_GATED: epi_gated<ACT_NONE>(e, g, p.out16); return;
-    case EPI_RESID: {
+  e.tmem = tmem; e.tok = tok; e.live = live; e.lane = lane; e.r0 = r0; e.rs = rs;
+  e.cols = min(GEMM_BM, (g.dual ? 2 * g.N : g.N) - r0);
+  if (!g.fast) { epi_general(c, g, e, ft); return; }
+  unsigned short* const out16 = resolve<unsigned short>(c, g.out16);
+  if (g.dual) {
+    if (g.act == ACT_SILU) epi_gated<ACT_SILU>(e, g, out16);
+    else if (g.act == ACT_GELU) epi_gated<ACT_GELU>(e, g, out16);
+    else epi_gated<ACT_NONE>(e, g, out16);
+  } else if (g.out32 != 0) {
+    float* const out32 = resolve<float>(c, g.out32);
+    if (g.resid) {
       const float* const x = resolve<const float>(c, g.X) + r0;
-      if (p.out16) epi_resid<true>(e, g, x, resid, p.out32, p.out16, p.ssq, ft);
-      else epi_resid<false>(e, g, x, resid, p.out32, nullptr, nullptr, ft);
-      return;
+      if (out16) epi_resid<true>(e, g, x, resid, out32, out16, resolve<float>(c, g.ss_out), ft);
+      else epi_resid<false>(e, g, x, resid, out32, nullptr, nullptr, ft);
+    } else if (g.fast == 2) {
+      if (out16) epi_stream<true, true>(c, e, g, out32, out16, nullptr, ft);
+      else epi_stream<false, true>(c, e, g, out32, nullptr, nullptr, ft);
+    } else if (out16) epi_stream<true, false>(c, e, g, out32, out16, resolve<float>(c, g.ss_out), ft);
+    else epi_stream<false, false>(c, e, g, out32, nullptr, nullptr, ft);
+  } else {
+    const int all = e.cols;
+    if (g.outT != 0) e.cols = max(0, min(all, g.t_col0 - r0));              // columns from here on are V features
+    if (e.cols > 0) {
+      if (g.act == ACT_GELU) epi_bf16<ACT_GELU, false>(e, g, out16, nullptr);
+      else if (g.rope_cols > 0) epi_bf16<ACT_NONE, true>(e, g, out16, resolve<const float>(c, g.rope_tab));
+      else epi_bf16<ACT_NONE, false>(e, g, out16, nullptr);
     }
-    case EPI_POST:
-      if (p.out16) epi_stream<true, true>(c, e, g, p.out32, p.out16, nullptr, ft);
-      else epi_stream<false, true>(c, e, g, p.out32, nullptr, nullptr, ft);
-      return;
-    case EPI_STREAM:
-      if (p.out16) epi_stream<true, false>(c, e, g, p.out32, p.out16, p.ssq, ft);
-      else epi_stream<false, false>(c, e, g, p.out32, nullptr, nullptr, ft);
-      return;
-  }
-  e.cols = p.split;
-  if (e.cols > 0) {
-    if (p.kind == EPI_GELU) epi_bf16<ACT_GELU, false>(e, g, p.out16, nullptr);
-    else if (p.kind == EPI_ROPE) epi_bf16<ACT_NONE, true>(e, g, p.out16, resolve<const float>(c, g.rope_tab));
-    else epi_bf16<ACT_NONE, false>(e, g, p.out16, nullptr);
-  }
-  if (p.split < p.cols) {
-    e.cols = p.cols;
-    epi_vt(e, g, resolve<unsigned short>(c, g.outT), p.split);
+    if (e.cols < all) {
+      const int split = e.cols;
+      e.cols = all;
+      epi_vt(e, g, resolve<unsigned short>(c, g.outT), split);
+    }
   }
 }
 
@@ -759,17 +747,16 @@ __device__ __forceinline__ void tile_gemm(const TileCtx& c, const GemmArgs& g, i
     }
   }
 
-  const EpiPlan plan = epi_plan(c, g, r0);             // (this and the scale: under the MMAs)
+  const bool ready = mbar_wait(c, accum_bar, acc_ph);
+  __syncwarp();
+  tc_fence_after();
   float rs = 1.0f;
   if (scaled) {
 #pragma unroll
     for (int j = 0; j < 8; ++j) ssq += part[j];
     rs = 1.0f / sqrtf(ssq / (float)g.rs_d + 1e-6f);
   }
-  const bool ready = mbar_wait(c, accum_bar, acc_ph);
-  __syncwarp();
-  tc_fence_after();
-  if (ready && warp_live) gemm_epilogue(c, g, plan, my_tmem, t0 + tpw * warp, min(tpw, nt - tpw * warp), lane, r0, rs, ft, resid);
+  if (ready && warp_live) gemm_epilogue(c, g, my_tmem, t0 + tpw * warp, min(tpw, nt - tpw * warp), lane, r0, rs, ft, resid);
   tc_fence_before();
   worker_sync(c);
   if (!(c.slot && c.slot->primed) && worker_tid() <= 2 * S) mbar_inval(bar0 + 8u * worker_tid());
