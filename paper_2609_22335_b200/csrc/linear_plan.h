@@ -7,7 +7,10 @@ namespace vla {
 constexpr int LIN_MAX_STAGES = 12;
 constexpr int LIN_SMEM = 110 * 1024;          // half an SM
 
-struct LinearPlan { int bm, bn, ks, tiles_m, tiles, stages; };   // tokens and features of a tile, CTAs that share its K, tiles, pipeline depth
+struct LinearPlan {
+  int bm, bn, ks, tiles_m, tiles, stages;   // tokens and features of a tile, CTAs that share its K, tiles, pipeline depth
+  double cost;                              // the estimate it was chosen by (cycles; where K is not split)
+};
 
 // (Every call of the operator pays for this arithmetic, and divisions are most of it: bm and bn are multiples of 16, so what is
 // divided by them comes from tables.)
@@ -62,7 +65,7 @@ inline LinearPlan linear_plan(int m, int n, int k, bool f32, int sms) {
   LinearPlan g;
   g.tiles_m = (m - 1) / 128 + 1;
   g.bm = ((m - 1) / g.tiles_m / 16 + 1) * 16;
-  g.bn = 16; g.ks = 1;
+  g.bn = 16; g.ks = 1; g.cost = 0;
   const int nkb = (k - 1) / GEMM_BK + 1;
   if (f32) linear_split_f32(g, n, nkb, sms);
   if (g.ks == 1) {
@@ -82,9 +85,42 @@ inline LinearPlan linear_plan(int m, int n, int k, bool f32, int sms) {
         const double t = (double)(rounds * ((nkb + ks - 1) >> shift)) * kb + (bn <= 128 ? 1 : rounds) * 2400.0 + (ks > 1 ? 50.0 * bn : 0);
         if (t < best) { best = t; g.bn = bn; g.ks = ks; }
       }
+    g.cost = best;
   }
   g.tiles = (int)(g.tiles_m * linear_tiles_n(n, g.bn));
   g.stages = linear_stages(g.bm, g.bn);
+  return g;
+}
+
+
+// The same call as tiles of two SMs (op_linear_pair.cuh): bm tokens and half of bn features a CTA; bn = 0 where the plan above is
+// the faster one or has to stay.  Under 129 tokens one of the CTAs would idle, and a plan that splits K for an fp32 result is kept
+// for its shorter sums.  A k-block of a pair's tile costs max(350, 2 x width, its CTA's operands at 50 B/clk -- what a lone CTA of an
+// SM gets from L2; 42 where K is no multiple of 64), a tile 2000 cycles more (its first loads and what of its epilogue the next one's
+// MMAs do not cover), and a call 6000 more than the other kernel's: two CTAs have to meet, and the last epilogue stands alone.
+// Fitted to 70 shapes of 129..8192 x 64..16384 x 64..12288, nine widths each and the other kernel timed: 34 go this way, at 0.62 to
+// 0.99 of the other kernel's time (2077 x 4944 x 7144 227 -> 145 us, 4096 x 4096 x 4096 114 -> 96, 8192 x 3072 x 768 40 -> 35, 1747 x 2064 x
+// 2288 28 -> 18), none is slower, and the choice is 1.4 % behind the best of the ten on average.
+constexpr int LINP_SMEM = 224 * 1024;         // a CTA of a pair has its SM to itself
+struct LinearPairPlan { int bm, bn, tiles_m, tiles, stages; };
+inline LinearPairPlan linear_pair_plan(int m, int n, int k, const LinearPlan& single, int sms) {
+  LinearPairPlan g = {0, 0, 0, 0, 0};
+  if (m <= 128 || n <= 112 || sms < 2 || single.cost <= 6000.0) return g;
+  g.tiles_m = (m - 1) / 256 + 1;
+  g.bm = ((m - 1) / (2 * g.tiles_m) / 16 + 1) * 16;
+  const int nkb = (k - 1) / GEMM_BK + 1, pairs = sms / 2;
+  const double operand_rate = k % GEMM_BK == 0 ? 1.0 / 50 : 1.0 / 42;
+  double best = single.cost - 6000.0;
+  for (int bn = 128; bn <= 256 && bn < n + 16; bn += 16) {
+    const long long tiles = g.tiles_m * linear_tiles_n(n, bn), rounds = tiles <= pairs ? 1 : (tiles - 1) / pairs + 1;
+    const double mma = bn > 175 ? 2.0 * bn : 350.0, operands = (g.bm + bn / 2) * GEMM_BK * 2 * operand_rate;
+    const double t = (double)rounds * (nkb * (mma > operands ? mma : operands) + 2000.0);
+    if (t < best) { best = t; g.bn = bn; g.tiles = (int)tiles; }
+  }
+  if (g.bn > 0) {     // (behind the start of the last stage there are the 16 KB that the MMA reads of any token tile)
+    const int stage = (g.bm + g.bn / 2) * GEMM_BK * 2, s = (LINP_SMEM - 16384) / stage;
+    g.stages = s > LIN_MAX_STAGES ? LIN_MAX_STAGES : s;
+  }
   return g;
 }
 

@@ -72,6 +72,7 @@ __device__ __forceinline__ void op_let_next_start() { asm volatile("griddepcontr
 
 #include "op_attention.cuh"
 #include "op_linear.cuh"
+#include "op_linear_pair.cuh"
 
 namespace vla {
 
@@ -98,6 +99,8 @@ inline OpDevice* op_device() {
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return nullptr;
     for (auto* kernel : {vla_op_linear_kernel<1>, vla_op_linear_kernel<2>, vla_op_linear_kernel<8>})
       if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, LIN_SMEM) != cudaSuccess) return nullptr;
+    for (auto* kernel : {vla_op_linear_pair_kernel<1>, vla_op_linear_pair_kernel<2>, vla_op_linear_pair_kernel<8>})
+      if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, LINP_SMEM) != cudaSuccess) return nullptr;
     if (cudaFuncSetAttribute(vla_op_attention_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 224 * 1024) != cudaSuccess) return nullptr;
     d.sms = sms;
     d.error.store(static_cast<unsigned*>(a), std::memory_order_release);
@@ -195,13 +198,21 @@ int vla_op_linear(const void* a, const void* w, float* out32, void* out16, int32
   LinearArgs g;
   g.m = m; g.n = n; g.kp = (int)op_pad(k, GEMM_BK); g.act = act;
   g.out32 = out32; g.out16 = static_cast<unsigned short*>(out16);
-  const LinearPlan p = linear_plan(m, n, k, out32 != nullptr, dev->sms);
-  g.bm = p.bm; g.bn = p.bn; g.ks = p.ks; g.tiles_m = p.tiles_m; g.tiles = p.tiles; g.stages = p.stages;
   g.err = dev->error.load(std::memory_order_relaxed);
+  const LinearPlan p = linear_plan(m, n, k, out32 != nullptr, dev->sms);
+  const LinearPairPlan pp = p.ks == 1 ? linear_pair_plan(m, n, k, p, dev->sms) : LinearPairPlan{};
+  const int vec = linear_vec(n, out32, out16);
   OpMaps maps;
+  if (pp.bn > 0) {
+    g.bm = pp.bm; g.bn = pp.bn; g.ks = 1; g.tiles_m = pp.tiles_m; g.tiles = pp.tiles; g.stages = pp.stages;
+    if (!op_encode(&maps.m[0], w, n, k, k, g.bn / 2) || !op_encode(&maps.m[1], a, m, k, k, g.bm)) return VLA_ERR_CUDA;
+    const int pairs = g.tiles < dev->sms / 2 ? g.tiles : dev->sms / 2;
+    const auto kernel = vec == 8 ? vla_op_linear_pair_kernel<8> : (vec == 2 ? vla_op_linear_pair_kernel<2> : vla_op_linear_pair_kernel<1>);
+    return op_launch(kernel, 2 * pairs, LIN_THREADS, LINP_SMEM, 2, static_cast<cudaStream_t>(stream), g, maps, op_fault());
+  }
+  g.bm = p.bm; g.bn = p.bn; g.ks = p.ks; g.tiles_m = p.tiles_m; g.tiles = p.tiles; g.stages = p.stages;
   if (!op_encode(&maps.m[0], w, n, k, k, g.bn) || !op_encode(&maps.m[1], a, m, k, k, g.bm)) return VLA_ERR_CUDA;
   const int grid = g.ks > 1 ? g.tiles * g.ks : (g.tiles < 2 * dev->sms ? g.tiles : 2 * dev->sms);
-  const int vec = linear_vec(n, out32, out16);
   const auto kernel = vec == 8 ? vla_op_linear_kernel<8> : (vec == 2 ? vla_op_linear_kernel<2> : vla_op_linear_kernel<1>);
   return op_launch(kernel, grid, LIN_THREADS, linear_smem(g), g.ks, static_cast<cudaStream_t>(stream), g, maps, op_fault());
 }

@@ -5,3 +5,8 @@ extern "C" void linear_plan_host(int m, int n, int k, int f32, int sms, int* out
   const vla::LinearPlan p = vla::linear_plan(m, n, k, f32 != 0, sms);
   out[0] = p.bm; out[1] = p.bn; out[2] = p.ks; out[3] = p.tiles_m; out[4] = p.tiles; out[5] = p.stages;
 }
+extern "C" void linear_pair_plan_host(int m, int n, int k, int f32, int sms, int* out /*[5]: bm, bn, tiles_m, tiles, stages*/) {
+  const vla::LinearPlan p = vla::linear_plan(m, n, k, f32 != 0, sms);
+  const vla::LinearPairPlan q = p.ks == 1 ? vla::linear_pair_plan(m, n, k, p, sms) : vla::LinearPairPlan{};
+  out[0] = q.bm; out[1] = q.bn; out[2] = q.tiles_m; out[3] = q.tiles; out[4] = q.stages;
+}

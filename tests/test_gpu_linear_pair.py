@@ -1,0 +1,48 @@
+"""The linear layer's tiles of two SMs (csrc/op_linear_pair.cuh) at their edges: token tiles whose second half is ragged or empty,
+widths between 128 and 256 and their remainders, K that ends inside a block, every activation, both result types, stores of
+eight, two and one feature; and a call whose operand loads never come."""
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+SHAPES = [(2077, 4944, 712), (1747, 2064, 2288), (4645, 3040, 1000), (7744, 2824, 472), (2936, 1496, 1160), (5125, 440, 2048),
+          (978, 14489, 792), (3000, 4902, 520), (129, 16384, 4096)]
+
+
+@pytest.mark.parametrize("m,n,k", SHAPES)
+@pytest.mark.parametrize("act", [0, 1, 2])
+def test_against_64_bit_sums(m, n, k, act):
+    import torch
+    from paper_2609_22335_b200 import api
+    g = torch.Generator(device="cuda").manual_seed(m + act)
+    a = torch.randn(m, k, device="cuda", generator=g).to(torch.bfloat16)
+    w = (k ** -0.5 * torch.randn(n, k, device="cuda", generator=g)).to(torch.bfloat16)
+    ref = a.double() @ w.double().T
+    sums = 2.0 ** -23 * (k / 16 + 2) * float(ref.abs().max())          # a unit in the last place per 16 products
+    if act:
+        ref = torch.nn.functional.gelu(ref, approximate="tanh") if act == 1 else torch.nn.functional.silu(ref)
+        sums = 2 * sums + 2.0 ** -10 * float(ref.abs().max())          # (the activations' approximations)
+    assert float((api.op_linear(a, w, act=act).double() - ref).abs().max()) <= sums
+    assert bool(((api.op_linear(a, w, act=act, out_bf16=True).double() - ref).abs() <= 2.0 ** -8 * ref.abs() + 2 * sums).all())
+    assert api.op_status(api.OP_LINEAR) == api.VLA_OK
+
+
+def test_calls_that_follow_one_another_and_a_wait_that_runs_out():
+    import torch
+    from paper_2609_22335_b200 import api
+    g = torch.Generator(device="cuda").manual_seed(0)
+    a = torch.randn(2048, 4096, device="cuda", generator=g).to(torch.bfloat16)
+    w = (4096 ** -0.5 * torch.randn(4096, 4096, device="cuda", generator=g)).to(torch.bfloat16)
+    x = a
+    for i in range(12):                                                # tiles of two SMs and of one in turn, each reading the last result
+        x = api.op_linear(x if i % 2 else x[:64].repeat(32, 1), w, out_bf16=True)
+        y = api.op_linear(x[:64], w, out_bf16=True)
+    assert torch.equal(api.op_linear(x[:64].contiguous(), w, out_bf16=True), y)
+    good = api.op_linear(a, w, out_bf16=True)
+    api.debug_op_fault(True, 2_000_000)
+    try:
+        api.op_linear(a, w, out_bf16=True)
+        assert api.op_status(api.OP_LINEAR) == api.VLA_ERR_TIMEOUT
+    finally:
+        api.debug_op_fault(False)
+    assert torch.equal(api.op_linear(a, w, out_bf16=True), good) and api.op_status(api.OP_LINEAR) == api.VLA_OK

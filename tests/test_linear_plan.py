@@ -21,6 +21,12 @@ def plan(tmp_path_factory):
         o = (C.c_int * 6)()
         lib.linear_plan_host(m, n, k, int(f32), sms, o)
         return dict(zip(("bm", "bn", "ks", "tiles_m", "tiles", "stages"), o))
+
+    def pair(m, n, k, f32=False, sms=148):
+        o = (C.c_int * 5)()
+        lib.linear_pair_plan_host(m, n, k, int(f32), sms, o)
+        return list(o)
+    call.pair = pair
     return call
 
 
@@ -53,3 +59,23 @@ def test_fp32_results_keep_their_split(plan):
     """Sums are split where they are long and the chip has room, whatever a width without a split would gain."""
     for shape, ks in (((288, 11008, 4096), 2), ((452, 6648, 6024), 2), ((938, 1352, 6144), 4), ((91, 9152, 1344), 4), ((8192, 3072, 768), 1)):
         assert plan(*shape, f32=True)["ks"] == ks
+
+
+def test_every_plan_of_two_sm_tiles_is_one_the_kernel_can_run(plan):
+    rnd = random.Random(5)
+    shapes = [(m, n, k) for m in (1, 128, 129, 256, 257, 100000) for n in (7, 112, 113, 255, 257, 70000) for k in (8, 72, 4096, 20000)]
+    shapes += [(int(2 ** rnd.uniform(6, 14)), int(2 ** rnd.uniform(4, 15)), 8 * int(2 ** rnd.uniform(0, 11))) for _ in range(3000)]
+    used = 0
+    for m, n, k in shapes:
+        for sms, f32 in ((148, False), (148, True), (132, False), (7, True), (1, False)):
+            bm, bn, tiles_m, tiles, stages = plan.pair(m, n, k, f32, sms)
+            if bn == 0:
+                continue
+            used += 1
+            assert m > 128 and sms > 1 and plan(m, n, k, f32, sms)["ks"] == 1
+            assert bm % 16 == 0 and 16 <= bm <= 128 and tiles_m * 2 * bm >= m > (tiles_m - 1) * 2 * bm
+            assert bn % 16 == 0 and 128 <= bn <= 256 and tiles == tiles_m * -(-n // bn)
+            stage = (bm + bn // 2) * 128                       # whole 1024-byte swizzle groups, and the MMA reads 128 rows of tokens
+            assert bm * 128 % 1024 == 0 and stage % 1024 == 0
+            assert 2 <= stages <= 12 and (stages - 1) * stage + max(stage, 16384) <= 224 * 1024
+    assert used > 1000
