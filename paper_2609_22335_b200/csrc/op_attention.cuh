@@ -5,37 +5,52 @@
 // results meet in distributed shared memory -- a call of few tiles (96 heads x query blocks, or the action head's 4) is
 // bound by the length of a tile's chain of key blocks, not by throughput, and this cuts the chain.
 //
-// Inside a CTA: a TMA warp, an MMA warp and four softmax warps (a query row per thread).  S has two tensor-memory buffers, so
-// the scores of block i + 1 are computed under the softmax of block i; the probabilities go back into the front of their
-// scores' buffer and are the first operand of P V.  V is read as it lies, [key, head dim] (MN-major second operand), so
-// nothing is transposed in front of the kernel.
+// Inside a CTA: a TMA warp, a warp that issues Q K^T, one that issues P V, and four softmax warps (a query row per thread).  S
+// has three tensor-memory buffers where the output leaves room for them (two elsewhere), so scores are computed up to two blocks ahead
+// of the softmax; the probabilities go back into the front of their scores' buffer and are the first operand of P V.  V is read as it lies,
+// [key, head dim] (MN-major second operand), so nothing is transposed in front of the kernel.
 #pragma once
 #include "dispatch.cuh"
 
 namespace vla {
 
-constexpr int OPA_THREADS = 192;
+constexpr int OPA_THREADS = 224;
+constexpr int OPA_MAX_S = 3;             // score buffers
+constexpr int OPA_MAX_SPLIT = 8;         // CTAs of a cluster
+constexpr int OPA_MAX_SMEM = 208 * 1024;
 constexpr int OPA_MAX_STAGES = 4;
 
-struct OpAttnLaunch { int split, stages, smem, tmem_cols; };
+struct OpAttnLaunch { int split, stages, smem, tmem_cols, s_bufs; };
 
 inline int opa_smem(int hs, int stages) {
   const int nbox = (hs + 63) / 64;
   return nbox * (128 * 128 + stages * 2 * 64 * 128);
 }
-// Two CTAs share an SM up to a head width of 128 (tensor memory 128 + hs columns of 512); the keys are split while that
-// still gives every CTA a slot of its own and at least one block of 64 keys.
-inline OpAttnLaunch opa_plan(int tiles, int tkv, int hs, int sms) {
+// The split of the keys is the one with the least estimated time, in units of a key block of a CTA that has its SM to itself (0.7 us
+// up to a head width of 128, 1.05 at 256): its CTAs' blocks, 1.55 times that where two share an SM (up to a width of 128), 7 for a call
+// and 4 for every further wave, 1.8 (3 above 128) for meeting in the cluster.  `clusters[s]`: clusters of s CTAs the chip holds, one CTA per SM -- from
+// three CTAs on a cluster is not given an SM that has one already (288 CTAs in clusters of three take two waves, in pairs one).
+// Fitted to 60 shapes of 16..2048 queries and keys with every split timed: the split chosen is at most 6 % behind the best.  (Powers of
+// two up to the chip's two CTAs per SM: 725 x 687, 12 heads of 128, 19.6 us split four ways and 12.2 two ways; 87 x 956, 36 heads over 12
+// of 128, 20.6 eight and 10.7 three ways.)
+inline OpAttnLaunch opa_plan(int tiles, int tkv, int hs, int sms, const int* clusters) {
   OpAttnLaunch p;
-  const int per_sm = hs <= 128 ? 2 : 1, budget = per_sm == 2 ? 112 * 1024 : 224 * 1024, blocks = (tkv + 63) / 64, chunks = hs / 16;
+  const int per_sm = hs <= 128 ? 2 : 1, budget = per_sm == 2 ? OPA_MAX_SMEM / 2 : OPA_MAX_SMEM, blocks = (tkv + 63) / 64, chunks = hs / 16;
   p.stages = OPA_MAX_STAGES;
   while (p.stages > 2 && opa_smem(hs, p.stages) > budget) --p.stages;
   p.smem = opa_smem(hs, p.stages);
   p.split = 1;
-  while (p.split < 8 && tiles * p.split * 2 <= per_sm * sms && blocks >= p.split * 2 &&
-         ((chunks + 2 * p.split - 1) / (2 * p.split)) * 2 * p.split * 8192 <= p.smem)
-    p.split *= 2;
+  double best = 1e300;
+  for (int s = 1; s <= OPA_MAX_SPLIT && s <= blocks; ++s) {
+    if ((chunks + s - 1) / s * s * 8192 > p.smem) continue;                       // (the partial rows meet in the stages)
+    const long long ctas = (long long)tiles * s, room = s > 2 ? (long long)clusters[s] * s : (long long)per_sm * sms;
+    const long long waves = room > 0 ? (ctas - 1) / room + 1 : ctas;
+    const double block = per_sm == 2 && s <= 2 && ctas > sms ? 1.55 : 1.0;
+    const double t = (double)waves * ((blocks + s - 1) / s * block + 4.0) + 3.0 + (s == 1 ? 0.0 : (hs <= 128 ? 1.8 : 3.0));
+    if (t < best) { best = t; p.split = s; }
+  }
   p.tmem_cols = hs <= 128 ? 256 : 512;
+  p.s_bufs = (p.tmem_cols - hs) / ATTN_BN < OPA_MAX_S ? (p.tmem_cols - hs) / ATTN_BN : OPA_MAX_S;
   return p;
 }
 
@@ -55,10 +70,8 @@ __device__ __forceinline__ uint32_t cluster_addr(uint32_t saddr, uint32_t rank) 
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(saddr), "r"(rank));
   return r;
 }
-__device__ __forceinline__ float2 ld_cluster_f2(uint32_t a) {
-  float2 v;
-  asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(a) : "memory");
-  return v;
+__device__ __forceinline__ void st_cluster_f2(uint32_t a, float x, float y) {
+  asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(a), "f"(x), "f"(y) : "memory");
 }
 __device__ __forceinline__ void st_cluster_f4(uint32_t a, const float* v) {
   asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(a), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]) : "memory");
@@ -73,11 +86,11 @@ __global__ void __launch_bounds__(OPA_THREADS) vla_op_attention_kernel(const __g
                                                                        const __grid_constant__ OpAttnLaunch p, unsigned* err, OpFault fault) {
   extern __shared__ __align__(1024) char smem_raw[];
   __shared__ uint32_t tmem_base_s;
-  __shared__ __align__(8) uint64_t bars[4 * OPA_MAX_STAGES + 6];
-  __shared__ __align__(8) float2 row_ml[ATTN_BQ];
+  __shared__ __align__(8) uint64_t bars[4 * OPA_MAX_STAGES + 3 * OPA_MAX_S + 1];
+  __shared__ __align__(8) float2 row_ml[OPA_MAX_SPLIT][ATTN_BQ];       // each CTA's maximum and sum of a row
   __shared__ unsigned failed_s;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int split = p.split, rank = (int)blockIdx.x % split, tile = (int)blockIdx.x / split, NS = p.stages;
+  const int split = p.split, rank = (int)blockIdx.x % split, tile = (int)blockIdx.x / split, NS = p.stages, NB = p.s_bufs;
   const AttnPlace at = attn_place(a, tile);
   const int g = (at.head * a.hkv) / a.hq, hs = a.hs, nbox = (hs + 63) / 64;
   int nb = (a.t0 + ATTN_BN - 1) / ATTN_BN;
@@ -85,12 +98,12 @@ __global__ void __launch_bounds__(OPA_THREADS) vla_op_attention_kernel(const __g
   const int b0 = nb * rank / split, n = nb * (rank + 1) / split - b0;          // this CTA's key blocks
   const uint32_t bar0 = smem_u32(bars);
   const uint32_t kfull = bar0, kempty = bar0 + 8 * OPA_MAX_STAGES, vfull = kempty + 8 * OPA_MAX_STAGES, vempty = vfull + 8 * OPA_MAX_STAGES;
-  const uint32_t bar_s = vempty + 8 * OPA_MAX_STAGES, bar_p = bar_s + 16, bar_o = bar_p + 16, bar_q = bar_o + 8;
+  const uint32_t bar_s = vempty + 8 * OPA_MAX_STAGES, bar_p = bar_s + 8 * OPA_MAX_S, bar_o = bar_p + 8 * OPA_MAX_S, bar_q = bar_o + 8 * OPA_MAX_S;   // (s, p, o: one per score buffer)
   const uint32_t kv_bytes = (uint32_t)nbox * (ATTN_BN * 128);
   const uint32_t Qs = smem_u32(smem_raw), Ks = Qs + (uint32_t)nbox * (ATTN_BQ * 128), Vs = Ks + (uint32_t)NS * kv_bytes;
   if (warp == 4) {
-    if (lane < 4 * OPA_MAX_STAGES + 6) {
-      const bool is_p = lane == 4 * OPA_MAX_STAGES + 2 || lane == 4 * OPA_MAX_STAGES + 3;
+    if (lane < 4 * OPA_MAX_STAGES + 3 * OPA_MAX_S + 1) {
+      const bool is_p = lane >= 4 * OPA_MAX_STAGES + OPA_MAX_S && lane < 4 * OPA_MAX_STAGES + 2 * OPA_MAX_S;
       mbar_init(bar0 + 8u * lane, is_p ? 4 : 1);
       asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -107,23 +120,11 @@ __global__ void __launch_bounds__(OPA_THREADS) vla_op_attention_kernel(const __g
   __syncthreads();
   op_let_next_start();
   tc_fence_after();
-  const uint32_t tmem = tmem_base_s, tmem_o = tmem + 2u * ATTN_BN;     // two score buffers, then O
+  const uint32_t tmem = tmem_base_s, tmem_o = tmem + (uint32_t)(NB * ATTN_BN);     // score buffers, then O
 
   if (warp == 4) {
     // ---------------- loads
     if (lane == 0 && !fault.drop_loads && n > 0) {
-      if (a.hpt <= 1) {
-        mbar_expect_tx(bar_q, (uint32_t)nbox * (ATTN_BQ * 128));
-#pragma unroll 1
-        for (int b = 0; b < nbox; ++b) tma_load_2d(Qs + (uint32_t)b * (ATTN_BQ * 128), &maps.m[0], bar_q, at.head * hs + b * 64, at.q0);
-      } else {
-        mbar_expect_tx(bar_q, (uint32_t)(at.nh * nbox * a.rph * 128));
-#pragma unroll 1
-        for (int i = 0; i < at.nh; ++i)
-#pragma unroll 1
-          for (int b = 0; b < nbox; ++b)
-            tma_load_2d(Qs + (uint32_t)b * (ATTN_BQ * 128) + (uint32_t)(i * a.rph * 128), &maps.m[0], bar_q, (at.head + i) * hs + b * 64, 0);
-      }
       uint32_t s = 0, ph = 1u;
       bool ok = true;
 #pragma unroll 1
@@ -142,48 +143,71 @@ __global__ void __launch_bounds__(OPA_THREADS) vla_op_attention_kernel(const __g
     }
     __syncwarp();
   } else if (warp == 5) {
-    // ---------------- MMAs
-    const uint32_t idesc_s = umma_idesc_bf16(ATTN_BN), idesc_o = umma_idesc_bf16(hs) | (1u << 16);       // second operand MN-major
+    // ---------------- S = Q K^T, into a buffer as soon as P V has read the probabilities that were in it.  (The commit that somebody
+    // waits for goes first: each costs its thread 150 cycles.)
+    const uint32_t idesc_s = umma_idesc_bf16(ATTN_BN);
     const uint64_t qdesc = umma_desc_sw128(Qs);
-    uint32_t ks = 0, kph = 0u, vs = 0, vph = 0u;
-    auto issue_s = [&](int i) -> bool {
-      if (!mbar_wait(c, kfull + 8u * ks, kph)) return false;
+    uint32_t s = 0, ph = 0u, buf = 0, bph = 1u;
+    bool ok = n > 0 && mbar_wait(c, bar_q, 0u);
+#pragma unroll 1
+    for (int i = 0; i < n && ok; ++i) {
+      if (i >= NB && !(ok = mbar_wait(c, bar_o + 8u * buf, bph))) break;
+      if (!(ok = mbar_wait(c, kfull + 8u * s, ph))) break;
       tc_fence_after();
-      uint64_t qd = qdesc, kd = umma_desc_sw128(Ks + ks * kv_bytes);
+      uint64_t qd = qdesc, kd = umma_desc_sw128(Ks + s * kv_bytes);
+      const uint32_t ts = tmem + ATTN_BN * buf;
       if (elect_one()) {
         int kc = 0;
 #pragma unroll 1
         for (; kc + 4 <= hs / 16; kc += 4) {
 #pragma unroll
-          for (int k = 0; k < 4; ++k) umma_bf16(tmem + ATTN_BN * (uint32_t)(i & 1), qd + 2u * k, kd + 2u * k, idesc_s, (kc | k) != 0 ? 1u : 0u);
+          for (int k = 0; k < 4; ++k) umma_bf16(ts, qd + 2u * k, kd + 2u * k, idesc_s, (kc | k) != 0 ? 1u : 0u);
           qd += (ATTN_BQ * 128) >> 4; kd += (ATTN_BN * 128) >> 4;
         }
 #pragma unroll 1
-        for (int k = 0; kc < hs / 16; ++kc, ++k) umma_bf16(tmem + ATTN_BN * (uint32_t)(i & 1), qd + 2u * k, kd + 2u * k, idesc_s, kc != 0 ? 1u : 0u);
-        umma_commit(kempty + 8u * ks);
-        umma_commit(bar_s + 8u * (uint32_t)(i & 1));
+        for (int k = 0; kc < hs / 16; ++kc, ++k) umma_bf16(ts, qd + 2u * k, kd + 2u * k, idesc_s, kc != 0 ? 1u : 0u);
+        umma_commit(bar_s + 8u * buf);
+        umma_commit(kempty + 8u * s);
       }
       __syncwarp();
-      if (++ks == (uint32_t)NS) { ks = 0; kph ^= 1u; }
-      return true;
-    };
-    bool ok = n > 0 && mbar_wait(c, bar_q, 0u) && issue_s(0);
-    if (ok && n > 1) ok = issue_s(1);
+      if (++s == (uint32_t)NS) { s = 0; ph ^= 1u; }
+      if (++buf == (uint32_t)NB) { buf = 0; bph ^= 1u; }
+    }
+  } else if (warp == 6) {
+    // ---------------- the queries (beside the first keys, which warp 4 asks for), then O += P V
+    if (lane == 0 && !fault.drop_loads && n > 0) {
+      if (a.hpt <= 1) {
+        mbar_expect_tx(bar_q, (uint32_t)nbox * (ATTN_BQ * 128));
 #pragma unroll 1
-    for (int i = 0; i < n && ok; ++i) {
-      if (!(ok = mbar_wait(c, bar_p + 8u * (uint32_t)(i & 1), ((uint32_t)i >> 1) & 1u) && mbar_wait(c, vfull + 8u * vs, vph))) break;
+        for (int b = 0; b < nbox; ++b) tma_load_2d(Qs + (uint32_t)b * (ATTN_BQ * 128), &maps.m[0], bar_q, at.head * hs + b * 64, at.q0);
+      } else {
+        mbar_expect_tx(bar_q, (uint32_t)(at.nh * nbox * a.rph * 128));
+#pragma unroll 1
+        for (int i = 0; i < at.nh; ++i)
+#pragma unroll 1
+          for (int b = 0; b < nbox; ++b)
+            tma_load_2d(Qs + (uint32_t)b * (ATTN_BQ * 128) + (uint32_t)(i * a.rph * 128), &maps.m[0], bar_q, (at.head + i) * hs + b * 64, 0);
+      }
+    }
+    __syncwarp();
+    const uint32_t idesc_o = umma_idesc_bf16(hs) | (1u << 16);       // second operand MN-major
+    uint32_t s = 0, ph = 0u, buf = 0, bph = 0u;
+#pragma unroll 1
+    for (int i = 0; i < n; ++i) {
+      if (!mbar_wait(c, vfull + 8u * s, ph) || !mbar_wait(c, bar_p + 8u * buf, bph)) break;
       tc_fence_after();
-      const uint64_t vd = umma_desc_mn_sw128(Vs + vs * kv_bytes, ATTN_BN * 128);
+      const uint64_t vd = umma_desc_mn_sw128(Vs + s * kv_bytes, ATTN_BN * 128);
+      const uint32_t tp = tmem + ATTN_BN * buf;
       if (elect_one()) {
 #pragma unroll
         for (int k = 0; k < ATTN_BN / 16; ++k)      // 16 keys = 16 rows of 128 bytes = 32 words of P pairs / 4
-          umma_bf16_ta(tmem_o, tmem + ATTN_BN * (uint32_t)(i & 1) + 8u * k, vd + (uint64_t)(k * (16 * 128 >> 4)), idesc_o, (i | k) != 0 ? 1u : 0u);
-        umma_commit(vempty + 8u * vs);
-        umma_commit(bar_o);
+          umma_bf16_ta(tmem_o, tp + 8u * k, vd + (uint64_t)(k * (16 * 128 >> 4)), idesc_o, (i | k) != 0 ? 1u : 0u);
+        umma_commit(bar_o + 8u * buf);
+        umma_commit(vempty + 8u * s);
       }
       __syncwarp();
-      if (++vs == (uint32_t)NS) { vs = 0; vph ^= 1u; }
-      if (i + 2 < n) ok = mbar_wait(c, bar_o, (uint32_t)i & 1u) && issue_s(i + 2);     // (its scores go where P(i) was read from)
+      if (++s == (uint32_t)NS) { s = 0; ph ^= 1u; }
+      if (++buf == (uint32_t)NB) { buf = 0; bph ^= 1u; }
     }
   }
   float m_run = -INFINITY, l_run = 0.f;
@@ -191,11 +215,13 @@ __global__ void __launch_bounds__(OPA_THREADS) vla_op_attention_kernel(const __g
   const int row = a.hpt > 1 ? (int)threadIdx.x % a.rph : at.q0 + (int)threadIdx.x;            // this thread's query (softmax warps)
   const float sl2 = a.scale_log2e;
   if (warp < 4) {
-    // ---------------- softmax: one thread per query row
+    // ---------------- softmax: one thread per query row.  A wait on a buffer's barriers never sees one more than a phase behind: S(i)
+    // was issued after P V of the block that had the buffer before.
+    uint32_t b = 0, bph = 0u, last = 0, lph = 0u;           // this block's score buffer and its phase; those of the block before
 #pragma unroll 1
     for (int i = 0; i < n; ++i) {
-      const uint32_t buf = tmem + my_lanes + ATTN_BN * (uint32_t)(i & 1);
-      if (!mbar_wait(c, bar_s + 8u * (uint32_t)(i & 1), ((uint32_t)i >> 1) & 1u)) break;
+      const uint32_t buf = tmem + my_lanes + ATTN_BN * b;
+      if (!mbar_wait(c, bar_s + 8u * b, bph)) break;
       __syncwarp();
       tc_fence_after();
       uint32_t sr[ATTN_BN];
@@ -211,23 +237,23 @@ __global__ void __launch_bounds__(OPA_THREADS) vla_op_attention_kernel(const __g
       }
       float alpha;
       attn_softmax_block(sr, sl2, m_run, l_run, alpha);
-      // O follows a moved maximum (rarely); everything before has been added by then.  The last block waits for P V of the one
-      // before it in any case: the wait behind the loop tells phases apart by parity, and this warp may be a whole block ahead
-      // of another one, whose part of that P V is still to come.  (P V of this block cannot start before this warp arrives.)
-      const bool moved = __any_sync(0xffffffffu, alpha != 1.0f);
-      if (i > 0 && (moved || i == n - 1)) {
-        mbar_wait(c, bar_o, (uint32_t)(i - 1) & 1u);
+      // O follows a moved maximum (rarely); everything before has been added by then.  (P V of this block cannot start before this
+      // warp arrives.)
+      if (i > 0 && __any_sync(0xffffffffu, alpha != 1.0f)) {
+        mbar_wait(c, bar_o + 8u * last, lph);
         __syncwarp();
         tc_fence_after();
-        if (moved) attn_rescale(tmem_o + my_lanes, hs, alpha);
+        attn_rescale(tmem_o + my_lanes, hs, alpha);
       }
       tmem_st16u(buf, sr);
       tmem_st16u(buf + 16u, sr + 16);
       tmem_st_wait();
       tc_fence_before();
-      arrive_warp(bar_p + 8u * (uint32_t)(i & 1), lane);
+      arrive_warp(bar_p + 8u * b, lane);
+      last = b; lph = bph;
+      if (++b == (uint32_t)NB) { b = 0; bph ^= 1u; }
     }
-    if (n > 0) mbar_wait(c, bar_o, (uint32_t)(n - 1) & 1u);
+    if (n > 0) mbar_wait(c, bar_o + 8u * last, lph);
     __syncwarp();
     tc_fence_after();
   }
@@ -247,48 +273,67 @@ __global__ void __launch_bounds__(OPA_THREADS) vla_op_attention_kernel(const __g
       }
     }
   } else {
-    // ---------------- the cluster's partial rows: maxima and sums first, then each CTA adds up its share of the columns
-    if (warp < 4) row_ml[threadIdx.x] = make_float2(m_run, l_run);
-    cluster_sync();                       // (and: every CTA has done its last load and MMA, so shared memory is free)
-    const uint32_t slab = smem_u32(smem_raw);
+    // ---------------- the cluster's partial rows go to the CTA that finishes their columns as they are, with every CTA's maxima and
+    // sums, so that they are weighted there and one exchange does
+    cluster_sync();                       // every CTA has done its last load and MMA, so shared memory is free
     if (warp < 4) {
-      float M = -INFINITY, L = 0.f;
-      float2 ml[8];
-#pragma unroll
-      for (int r = 0; r < 8; ++r)
-        if (r < split) { ml[r] = ld_cluster_f2(cluster_addr(smem_u32(&row_ml[threadIdx.x]), (uint32_t)r)); M = fmaxf(M, ml[r].x); }
-#pragma unroll
-      for (int r = 0; r < 8; ++r)
-        if (r < split && ml[r].x != -INFINITY) L = fmaf(ml[r].y, exp2_fast((ml[r].x - M) * sl2), L);
-      const float f = (m_run == -INFINITY || L == 0.f) ? 0.f : exp2_fast((m_run - M) * sl2) / L;
+      const uint32_t ml = smem_u32(&row_ml[rank][threadIdx.x]);
+#pragma unroll 1
+      for (int r = 0; r < split; ++r) st_cluster_f2(cluster_addr(ml, (uint32_t)r), m_run, l_run);
+    }
+    const uint32_t slab = smem_u32(smem_raw);
+    if (warp < 4 && n > 0) {
+      int to = 0, own = 0;                // chunk ch = own * split + to
+      uint32_t nx[16];
+      tmem_ld16_nowait(tmem_o + my_lanes, nx);
 #pragma unroll 1
       for (int ch = 0; ch < hs / 16; ++ch) {
         float o[16];
-        tmem_ld16(tmem_o + my_lanes + 16u * (uint32_t)ch, o);
+        tmem_ld_wait();
 #pragma unroll
-        for (int j = 0; j < 16; ++j) o[j] = f != 0.f ? o[j] * f : 0.f;
+        for (int j = 0; j < 16; ++j) o[j] = __uint_as_float(nx[j]);
+        tmem_ld16_nowait(tmem_o + my_lanes + 16u * (uint32_t)min(ch + 1, hs / 16 - 1), nx);
         // [owned chunk][source CTA][quarter][row] of four floats
-        const uint32_t at_ = cluster_addr(slab + (uint32_t)(((ch / split) * split + rank) * 4 * ATTN_BQ + (int)threadIdx.x) * 16u, (uint32_t)(ch % split));
+        const uint32_t at_ = cluster_addr(slab + (uint32_t)((own * split + rank) * 4 * ATTN_BQ + (int)threadIdx.x) * 16u, (uint32_t)to);
+        if (row_ok) {                     // (rows that nobody stores are not sent: the exchange is most of a short call of wide heads)
 #pragma unroll
-        for (int q = 0; q < 4; ++q) st_cluster_f4(at_ + (uint32_t)(q * ATTN_BQ * 16), o + 4 * q);
+          for (int q = 0; q < 4; ++q) st_cluster_f4(at_ + (uint32_t)(q * ATTN_BQ * 16), o + 4 * q);
+        }
+        if (++to == split) { to = 0; ++own; }
       }
+      tmem_ld_wait();
     }
     cluster_sync();
     if (row_ok) {
-      const float4* part = reinterpret_cast<const float4*>(smem_raw);
+      float M = -INFINITY, L = 0.f, f[OPA_MAX_SPLIT];
+#pragma unroll
+      for (int r = 0; r < OPA_MAX_SPLIT; ++r)
+        if (r < split) M = fmaxf(M, row_ml[r][threadIdx.x].x);
+#pragma unroll
+      for (int r = 0; r < OPA_MAX_SPLIT; ++r) {
+        const float2 v = r < split ? row_ml[r][threadIdx.x] : make_float2(-INFINITY, 0.f);
+        f[r] = v.x == -INFINITY ? 0.f : exp2_fast((v.x - M) * sl2);
+        if (f[r] != 0.f) L = fmaf(v.y, f[r], L);
+      }
+      const float inv = L > 0.f ? 1.0f / L : 0.f;
+      const float4* part = reinterpret_cast<const float4*>(smem_raw) + threadIdx.x;
 #pragma unroll 1
-      for (int ch = rank; ch < hs / 16; ch += split) {
+      for (int ch = rank; ch < hs / 16; ch += split, part += split * 4 * ATTN_BQ) {
         float o[16];
 #pragma unroll
         for (int j = 0; j < 16; ++j) o[j] = 0.f;
-#pragma unroll 1
-        for (int r = 0; r < split; ++r) {
+#pragma unroll
+        for (int r = 0; r < OPA_MAX_SPLIT; ++r) {
+          if (f[r] == 0.f) continue;      // (a CTA without keys of this row: whatever lies there)
 #pragma unroll
           for (int q = 0; q < 4; ++q) {
-            const float4 v = part[(((ch / split) * split + r) * 4 + q) * ATTN_BQ + (int)threadIdx.x];
-            o[4 * q] += v.x; o[4 * q + 1] += v.y; o[4 * q + 2] += v.z; o[4 * q + 3] += v.w;
+            const float4 v = part[(r * 4 + q) * ATTN_BQ];
+            o[4 * q] = fmaf(f[r], v.x, o[4 * q]); o[4 * q + 1] = fmaf(f[r], v.y, o[4 * q + 1]);
+            o[4 * q + 2] = fmaf(f[r], v.z, o[4 * q + 2]); o[4 * q + 3] = fmaf(f[r], v.w, o[4 * q + 3]);
           }
         }
+#pragma unroll
+        for (int j = 0; j < 16; ++j) o[j] *= inv;
         put16(O + 16 * ch, o);
       }
     }
