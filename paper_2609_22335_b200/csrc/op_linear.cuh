@@ -97,10 +97,11 @@ __device__ __forceinline__ void linear_store(const LinearArgs& g, float* v, int 
   }
 }
 // This warp's share of a tile's columns: groups of 32, [lo, hi), for its 32 lanes.  `part` (split K): the other CTAs'
-// fragments of the same group, written by the threads that hold the same place.
+// fragments of the same group, written by the threads that hold the same place.  `n_acc`: accumulators of the same columns,
+// `acc_stride` apart, that add up to the result.
 template <int ACT, int VEC>
 __device__ __forceinline__ void linear_rows(const LinearArgs& g, uint32_t tmem, int lane, int row0, int rows, int n0, int lo, int hi, const float4* part,
-                                            int n_part, int part_stride) {
+                                            int n_part, int part_stride, int n_acc = 1, uint32_t acc_stride = 0) {
   const int q = lane & 3;
 #pragma unroll 1
   for (int h = 0; h < 2 && 16 * h < rows; ++h) {
@@ -115,6 +116,14 @@ __device__ __forceinline__ void linear_rows(const LinearArgs& g, uint32_t tmem, 
 #pragma unroll
       for (int j = 0; j < EPI; ++j) v[j] = __uint_as_float(nx[j]);
       tmem_ld_frag(th + 32u * (uint32_t)(c + 1 < hi ? c + 1 : c), nx);
+#pragma unroll 1
+      for (int r = 1; r < n_acc; ++r) {
+        uint32_t t[EPI];
+        tmem_ld_frag(th + (uint32_t)r * acc_stride + 32u * (uint32_t)c, t);
+        tmem_ld_wait();
+#pragma unroll
+        for (int j = 0; j < EPI; ++j) v[j] += __uint_as_float(t[j]);
+      }
 #pragma unroll 1
       for (int r = 0; r < n_part; ++r) {
         const float4* p = part + (size_t)r * part_stride + ((c - lo) * 2 + h) * (4 * 128);

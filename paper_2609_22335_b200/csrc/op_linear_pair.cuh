@@ -4,7 +4,8 @@
 // stages its own 128 tokens and its own half of the weight rows, the leader issues MMAs that read both SMs' shared memory, and
 // each CTA's tensor memory receives its own tokens' rows.  An SM so loads 32 KB per 256 x 256 x 64 block where two separate
 // 128 x 256 tiles load 48 KB, and the L2-to-shared-memory path is what bounds the layer.  Two accumulators of 256 columns: the
-// eight epilogue warps store one tile while the MMAs of the next run.  Persistent, one CTA per SM.  4096 x 4096 x 4096 114 -> 96 us
+// eight epilogue warps store one tile while the MMAs of the next run (or two to four accumulators that take a part of K each, where the
+// sums of an fp32 result are kept short).  Persistent, one CTA per SM.  4096 x 4096 x 4096 114 -> 96 us
 // (1.43 PFLOP/s), 8192 x 3072 x 768 with GELU 47.7 -> 42.2 called from Python on new inputs: 700 cycles a k-block of 512 cycles of MMA,
 // since a lone CTA gets 47 B/clk from L2 whichever warps ask (two of them loading one operand each changed nothing).
 #pragma once
@@ -12,8 +13,7 @@
 
 namespace vla {
 
-constexpr int LINP_ACC_COLS = 256;             // tensor-memory columns of an accumulator (two of them: all there is)
-constexpr int LINP_MMA_ROWS_BYTES = 128 * GEMM_BK * 2;      // what the MMA reads of a CTA's token tile, however high its box is
+constexpr int LINP_TMEM_COLS = 512;            // all there is
 
 __device__ __forceinline__ void tmem_alloc_pair(uint32_t* smem_dst, uint32_t cols) {
   asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(smem_dst)), "r"(cols) : "memory");
@@ -61,7 +61,7 @@ __global__ void __launch_bounds__(LIN_THREADS, 1) vla_op_linear_pair_kernel(cons
     }
     if (lane == 0) failed_s = 0;
   } else if (warp == 1) {
-    tmem_alloc_pair(&tmem_base_s, 2 * LINP_ACC_COLS);
+    tmem_alloc_pair(&tmem_base_s, LINP_TMEM_COLS);
   }
   tc_fence_before();
   __syncthreads();
@@ -74,6 +74,9 @@ __global__ void __launch_bounds__(LIN_THREADS, 1) vla_op_linear_pair_kernel(cons
   c.deadline = gtimer() + fault.wait_limit_ns;
   op_let_next_start();
   const uint32_t tmem = tmem_base_s;
+  // An accumulator for each of the parts K is summed in, and where there is room two sets of them.
+  const int parts = g.ks;
+  const uint32_t sets = 2 * parts * g.bn <= LINP_TMEM_COLS ? 2u : 1u, part_cols = LINP_TMEM_COLS / (sets * (uint32_t)parts), set_cols = part_cols * (uint32_t)parts;
   bool ok = true;
   if (warp == 0) {
     if (lane == 0 && !fault.drop_loads) {
@@ -100,35 +103,38 @@ __global__ void __launch_bounds__(LIN_THREADS, 1) vla_op_linear_pair_kernel(cons
     if (rank == 0) {
       const uint32_t idesc = umma_idesc_bf16(g.bn, 256);
       const uint64_t desc0 = umma_desc_sw128(stage0);
-      uint32_t s = 0, ph = 0u, i = 0;
-      for (int t = first_tile; t < g.tiles && ok; t += step, ++i) {
-        const uint32_t buf = i & 1u;
-        if (!(ok = mbar_wait(c, acce0 + 8u * buf, ((i >> 1) & 1u) ^ 1u))) break;
+      uint32_t s = 0, ph = 0u, buf = 0, bph = 1u;
+      for (int t = first_tile; t < g.tiles && ok; t += step) {
+        if (!(ok = mbar_wait(c, acce0 + 8u * buf, bph))) break;
         tc_fence_after();
+        int part = 0, from = 0, to = nkb / parts;                     // k-blocks of this part
 #pragma unroll 1
         for (int kb = 0; kb < nkb; ++kb) {
+          if (kb == to) { ++part; from = to; to = nkb * (part + 1) / parts; }
           if (!(ok = mbar_wait(c, full0 + 8u * s, ph))) break;
           tc_fence_after();
           const uint64_t ad = desc0 + s * (stage_bytes >> 4), wd = ad + (a_bytes >> 4);
+          const uint32_t acc = tmem + set_cols * buf + part_cols * (uint32_t)part;
           if (elect_one()) {
 #pragma unroll
-            for (int k = 0; k < GEMM_BK / 16; ++k) umma_bf16_pair(tmem + LINP_ACC_COLS * buf, ad + 2u * k, wd + 2u * k, idesc, (kb | k) != 0 ? 1u : 0u);
+            for (int k = 0; k < GEMM_BK / 16; ++k) umma_bf16_pair(acc, ad + 2u * k, wd + 2u * k, idesc, kb != from || k != 0 ? 1u : 0u);
             umma_commit_pair(empty0 + 8u * s);
             if (kb == nkb - 1) umma_commit_pair(accf0 + 8u * buf);
           }
           __syncwarp();
           if (++s == (uint32_t)S) { s = 0; ph ^= 1u; }
         }
+        if (++buf == sets) { buf = 0; bph ^= 1u; }
       }
     }
   } else {
     const int quarter = warp & 3, half = warp >= 6 ? 1 : 0;           // (epilogue warps 2..9: a quarter of the lanes is fixed by warp % 4)
     const uint32_t lanes = (uint32_t)(quarter * 32) << 16, acce_leader = cluster_addr(acce0, 0u);
     const int groups = (g.bn + 31) / 32, mid = (groups + 1) / 2, lo = half ? mid : 0, hi = half ? groups : mid;
-    uint32_t i = 0;
-    for (int t = first_tile; t < g.tiles; t += step, ++i) {
-      const uint32_t buf = i & 1u, acc = tmem + LINP_ACC_COLS * buf + lanes;
-      if (!mbar_wait(c, accf0 + 8u * buf, (i >> 1) & 1u)) break;
+    uint32_t buf = 0, bph = 0u;
+    for (int t = first_tile; t < g.tiles; t += step) {
+      const uint32_t acc = tmem + set_cols * buf + lanes;
+      if (!mbar_wait(c, accf0 + 8u * buf, bph)) break;
       __syncwarp();
       tc_fence_after();
       const int cta_row = (2 * (t % g.tiles_m) + rank) * g.bm, row0 = cta_row + 32 * quarter, rows = min(g.bm, g.m - cta_row) - 32 * quarter;
@@ -136,18 +142,19 @@ __global__ void __launch_bounds__(LIN_THREADS, 1) vla_op_linear_pair_kernel(cons
       LinearArgs gg = g;
       gg.m = row0 + max(rows, 0);                                     // (this tile's rows and features only)
       gg.n_end = min(g.n, n0 + g.bn);
-      if (g.act == ACT_GELU) linear_rows<ACT_GELU, VEC>(gg, acc, lane, row0, rows, n0, lo, hi, nullptr, 0, 0);
-      else if (g.act == ACT_SILU) linear_rows<ACT_SILU, VEC>(gg, acc, lane, row0, rows, n0, lo, hi, nullptr, 0, 0);
-      else linear_rows<ACT_NONE, VEC>(gg, acc, lane, row0, rows, n0, lo, hi, nullptr, 0, 0);
+      if (g.act == ACT_GELU) linear_rows<ACT_GELU, VEC>(gg, acc, lane, row0, rows, n0, lo, hi, nullptr, 0, 0, parts, part_cols);
+      else if (g.act == ACT_SILU) linear_rows<ACT_SILU, VEC>(gg, acc, lane, row0, rows, n0, lo, hi, nullptr, 0, 0, parts, part_cols);
+      else linear_rows<ACT_NONE, VEC>(gg, acc, lane, row0, rows, n0, lo, hi, nullptr, 0, 0, parts, part_cols);
       tc_fence_before();
       __syncwarp();
       if (lane == 0) asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(acce_leader + 8u * buf) : "memory");
+      if (++buf == sets) { buf = 0; bph ^= 1u; }
     }
   }
   tc_fence_before();
   __syncthreads();
   cluster_sync();                              // nobody reads or signals the other CTA any more
-  if (warp == 1) tmem_dealloc_pair(tmem, 2 * LINP_ACC_COLS);
+  if (warp == 1) tmem_dealloc_pair(tmem, LINP_TMEM_COLS);
   if (threadIdx.x == 0 && *reinterpret_cast<volatile unsigned*>(&failed_s) != 0u) *g.err = (unsigned)DEV_ERR_WAIT_MBAR;
   cluster_sync();                              // (both have given their columns back)
 }

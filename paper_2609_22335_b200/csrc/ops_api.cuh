@@ -213,11 +213,11 @@ int vla_op_linear(const void* a, const void* w, float* out32, void* out16, int32
   g.out32 = out32; g.out16 = static_cast<unsigned short*>(out16);
   g.err = dev->error.load(std::memory_order_relaxed);
   const LinearPlan p = linear_plan(m, n, k, out32 != nullptr, dev->sms);
-  const LinearPairPlan pp = p.ks == 1 ? linear_pair_plan(m, n, k, p, dev->sms) : LinearPairPlan{};
+  const LinearPairPlan pp = linear_pair_plan(m, n, k, p, dev->sms);
   const int vec = linear_vec(n, out32, out16);
   OpMaps maps;
   if (pp.bn > 0) {
-    g.bm = pp.bm; g.bn = pp.bn; g.ks = 1; g.tiles_m = pp.tiles_m; g.tiles = pp.tiles; g.stages = pp.stages;
+    g.bm = pp.bm; g.bn = pp.bn; g.ks = p.ks; g.tiles_m = pp.tiles_m; g.tiles = pp.tiles; g.stages = pp.stages;
     if (!op_encode(&maps.m[0], w, n, k, k, g.bn / 2) || !op_encode(&maps.m[1], a, m, k, k, g.bm)) return VLA_ERR_CUDA;
     const int pairs = g.tiles < dev->sms / 2 ? g.tiles : dev->sms / 2;
     const auto kernel = vec == 8 ? vla_op_linear_pair_kernel<8> : (vec == 2 ? vla_op_linear_pair_kernel<2> : vla_op_linear_pair_kernel<1>);

@@ -7,6 +7,6 @@ extern "C" void linear_plan_host(int m, int n, int k, int f32, int sms, int* out
 }
 extern "C" void linear_pair_plan_host(int m, int n, int k, int f32, int sms, int* out /*[5]: bm, bn, tiles_m, tiles, stages*/) {
   const vla::LinearPlan p = vla::linear_plan(m, n, k, f32 != 0, sms);
-  const vla::LinearPairPlan q = p.ks == 1 ? vla::linear_pair_plan(m, n, k, p, sms) : vla::LinearPairPlan{};
+  const vla::LinearPairPlan q = vla::linear_pair_plan(m, n, k, p, sms);
   out[0] = q.bm; out[1] = q.bn; out[2] = q.tiles_m; out[3] = q.tiles; out[4] = q.stages;
 }

@@ -72,7 +72,8 @@ def test_every_plan_of_two_sm_tiles_is_one_the_kernel_can_run(plan):
             if bn == 0:
                 continue
             used += 1
-            assert m > 128 and sms > 1 and plan(m, n, k, f32, sms)["ks"] == 1
+            parts = plan(m, n, k, f32, sms)["ks"]              # accumulators in the 512 columns of tensor memory
+            assert m > 128 and sms > 1 and parts * bn <= 512 and -(-k // 64) >= parts
             assert bm % 16 == 0 and 16 <= bm <= 128 and tiles_m * 2 * bm >= m > (tiles_m - 1) * 2 * bm
             assert bn % 16 == 0 and 128 <= bn <= 256 and tiles == tiles_m * -(-n // bn)
             stage = (bm + bn // 2) * 128                       # whole 1024-byte swizzle groups, and the MMA reads 128 rows of tokens
