@@ -315,7 +315,7 @@ __global__ void __launch_bounds__(OPA_THREADS) vla_op_attention_kernel(const __g
         f[r] = v.x == -INFINITY ? 0.f : exp2_fast((v.x - M) * sl2);
         if (f[r] != 0.f) L = fmaf(v.y, f[r], L);
       }
-      const float inv = L > 0.f ? 1.0f / L : 0.f;
+      const float inv = L == 0.f ? 0.f : 1.0f / L;
       const float4* part = reinterpret_cast<const float4*>(smem_raw) + threadIdx.x;
 #pragma unroll 1
       for (int ch = rank; ch < hs / 16; ch += split, part += split * 4 * ATTN_BQ) {

@@ -100,7 +100,8 @@ inline OpDevice* op_device() {
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return nullptr;
     for (auto* kernel : {vla_op_linear_kernel<1>, vla_op_linear_kernel<2>, vla_op_linear_kernel<8>})
       if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, LIN_SMEM) != cudaSuccess) return nullptr;
-    for (auto* kernel : {vla_op_linear_pair_kernel<1>, vla_op_linear_pair_kernel<2>, vla_op_linear_pair_kernel<8>})
+    for (auto* kernel : {vla_op_linear_pair_kernel<1, false>, vla_op_linear_pair_kernel<2, false>, vla_op_linear_pair_kernel<8, false>,
+                         vla_op_linear_pair_kernel<1, true>, vla_op_linear_pair_kernel<2, true>, vla_op_linear_pair_kernel<8, true>})
       if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, LINP_SMEM) != cudaSuccess) return nullptr;
     if (cudaFuncSetAttribute(vla_op_attention_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, OPA_MAX_SMEM) != cudaSuccess) return nullptr;
     for (int s = 1; s <= OPA_MAX_SPLIT; ++s) {
@@ -220,7 +221,8 @@ int vla_op_linear(const void* a, const void* w, float* out32, void* out16, int32
     g.bm = pp.bm; g.bn = pp.bn; g.ks = p.ks; g.tiles_m = pp.tiles_m; g.tiles = pp.tiles; g.stages = pp.stages;
     if (!op_encode(&maps.m[0], w, n, k, k, g.bn / 2) || !op_encode(&maps.m[1], a, m, k, k, g.bm)) return VLA_ERR_CUDA;
     const int pairs = g.tiles < dev->sms / 2 ? g.tiles : dev->sms / 2;
-    const auto kernel = vec == 8 ? vla_op_linear_pair_kernel<8> : (vec == 2 ? vla_op_linear_pair_kernel<2> : vla_op_linear_pair_kernel<1>);
+    const auto kernel = g.ks > 1 ? (vec == 8 ? vla_op_linear_pair_kernel<8, true> : (vec == 2 ? vla_op_linear_pair_kernel<2, true> : vla_op_linear_pair_kernel<1, true>))
+                                 : (vec == 8 ? vla_op_linear_pair_kernel<8, false> : (vec == 2 ? vla_op_linear_pair_kernel<2, false> : vla_op_linear_pair_kernel<1, false>));
     return op_launch(kernel, 2 * pairs, LIN_THREADS, LINP_SMEM, 2, static_cast<cudaStream_t>(stream), g, maps, op_fault());
   }
   g.bm = p.bm; g.bn = p.bn; g.ks = p.ks; g.tiles_m = p.tiles_m; g.tiles = p.tiles; g.stages = p.stages;

@@ -47,3 +47,30 @@ def test_calls_that_follow_one_another_and_a_wait_that_runs_out():
     finally:
         api.debug_op_fault(False)
     assert torch.equal(api.op_linear(a, w, out_bf16=True), good) and api.op_status(api.OP_LINEAR) == api.VLA_OK
+
+
+def test_captured_calls_follow_their_inputs():
+    """Tiles of two SMs and attention over clusters of three CTAs in one graph: a replay computes from what the inputs hold then."""
+    import torch
+    from paper_2609_22335_b200 import api
+    g = torch.Generator(device="cuda").manual_seed(1)
+    a = torch.randn(1747, 2288, device="cuda", generator=g).to(torch.bfloat16)
+    w = (2288 ** -0.5 * torch.randn(2064, 2288, device="cuda", generator=g)).to(torch.bfloat16)
+    q, k, v = (torch.randn(n, 36 * 128, device="cuda", generator=g).to(torch.bfloat16)[:, :c].contiguous() for n, c in ((87, 4608), (956, 1536), (956, 1536)))
+    scratch = torch.empty(api.op_attention_scratch_bytes(956, 12, 128), dtype=torch.uint8, device="cuda")
+
+    def calls(stream=None):
+        return (api.op_linear(a, w, act=1, out_bf16=True, stream=stream), api.op_linear(a, w, stream=stream),
+                api.op_attention(q, k, v, 36, 12, 128, scratch=scratch, stream=stream))
+    calls()
+    side, graph = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=side):
+        out = calls(side)
+    for _ in range(2):
+        for x in (a, q, k):
+            x.copy_(x.flip(0))
+        want = calls()
+        graph.replay()
+        torch.cuda.synchronize()
+        assert all(torch.equal(x, y) for x, y in zip(out, want))
+    assert api.op_status(api.OP_LINEAR) == api.VLA_OK and api.op_status(api.OP_ATTENTION, scratch) == api.VLA_OK
