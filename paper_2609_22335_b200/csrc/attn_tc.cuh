@@ -18,12 +18,11 @@
 // next block, and warps 2 and 3, which issue nothing, wait for K and V on the issuers' behalf (a test of a barrier that is
 // ready costs 160-190 cycles): single frame 12.07 -> 11.98 ms, 4 x 2 pi0 streams 77.9 -> 77.3.
 #pragma once
+#include "attention_plan.h"
 #include "gemm_tc.cuh"
 
 namespace vla {
 
-constexpr int ATTN_BQ = 128;   // queries per tile (MMA M)
-constexpr int ATTN_BN = 64;    // keys per block (MMA N of S, MMA K of P V; one 128-byte swizzle row of P)
 constexpr float ATTN_RESCALE_LOG2 = 8.0f;   // the running row maximum may lag the true one by this much (log2 units)
 
 // Every warp of the tile arrives (after its lanes are together), one warp waits: an mbarrier of count four, so that a wait
@@ -83,7 +82,9 @@ __device__ __forceinline__ void attn_mask(uint32_t* sr, int lim) {
   for (int j = 0; j < ATTN_BN; ++j)
     if (j >= lim) sr[j] = 0xFF800000u;
 }
-// One block of a row's online softmax: 64 scores in, 32 bf16 probability pairs out (front half of the registers).
+// One block of a row's online softmax: 64 scores in, 32 bf16 probability pairs out (front half of the registers).  TERMS 2: the pairs'
+// rounding errors, in bf16 themselves, in the other half.
+template <int TERMS = 1>
 __device__ __forceinline__ void attn_softmax_block(uint32_t* sr, float sl2, float& m_run, float& l_run, float& alpha) {
   float m4[4] = {m_run, __uint_as_float(sr[0]), __uint_as_float(sr[1]), __uint_as_float(sr[2])};
 #pragma unroll
@@ -99,6 +100,7 @@ __device__ __forceinline__ void attn_softmax_block(uint32_t* sr, float sl2, floa
   const float mb = mx == -INFINITY ? 0.f : -mx * sl2;
   const uint64_t sl2_2 = pack2(sl2, sl2), mb_2 = pack2(mb, mb);
   uint64_t s2[2] = {0ull, 0ull};
+  uint32_t lo[ATTN_BN / 2];
 #pragma unroll
   for (int j = 0; j < ATTN_BN; j += 2) {
     const uint64_t e2 = fma2(pack2(__uint_as_float(sr[j]), __uint_as_float(sr[j + 1])), sl2_2, mb_2);
@@ -107,6 +109,11 @@ __device__ __forceinline__ void attn_softmax_block(uint32_t* sr, float sl2, floa
     p0 = exp2_fast(p0); p1 = exp2_fast(p1);
     s2[(j >> 1) & 1] = add2(s2[(j >> 1) & 1], pack2(p0, p1));
     sr[j >> 1] = pack_bf16(p0, p1);
+    if (TERMS == 2) lo[j >> 1] = pack_bf16(p0 - __uint_as_float(sr[j >> 1] << 16), p1 - __uint_as_float(sr[j >> 1] & 0xFFFF0000u));
+  }
+  if (TERMS == 2) {
+#pragma unroll
+    for (int j = 0; j < ATTN_BN / 2; ++j) sr[ATTN_BN / 2 + j] = lo[j];
   }
   float x0, x1;
   unpack2(add2(s2[0], s2[1]), x0, x1);

@@ -8,51 +8,16 @@
 // Inside a CTA: a TMA warp, a warp that issues Q K^T, one that issues P V, and four softmax warps (a query row per thread).  S
 // has three tensor-memory buffers where the output leaves room for them (two elsewhere), so scores are computed up to two blocks ahead
 // of the softmax; the probabilities go back into the front of their scores' buffer and are the first operand of P V.  V is read as it lies,
-// [key, head dim] (MN-major second operand), so nothing is transposed in front of the kernel.
+// [key, head dim] (MN-major second operand), so nothing is transposed in front of the kernel.  Where the keys are in few parts (opa_plan) a
+// probability is the sum of two bf16 numbers, the second in the back of the buffer, and P V takes two products: rel-L2 to 64 bits 1.65e-3
+// where one number gives 2.0e-3 to 2.3e-3.
 #pragma once
+#include "attention_plan.h"
 #include "dispatch.cuh"
 
 namespace vla {
 
 constexpr int OPA_THREADS = 224;
-constexpr int OPA_MAX_S = 3;             // score buffers
-constexpr int OPA_MAX_SPLIT = 8;         // CTAs of a cluster
-constexpr int OPA_MAX_SMEM = 208 * 1024;
-constexpr int OPA_MAX_STAGES = 4;
-
-struct OpAttnLaunch { int split, stages, smem, tmem_cols, s_bufs; };
-
-inline int opa_smem(int hs, int stages) {
-  const int nbox = (hs + 63) / 64;
-  return nbox * (128 * 128 + stages * 2 * 64 * 128);
-}
-// The split of the keys is the one with the least estimated time, in units of a key block of a CTA that has its SM to itself (0.7 us
-// up to a head width of 128, 1.05 at 256): its CTAs' blocks, 1.55 times that where two share an SM (up to a width of 128), 7 for a call
-// and 4 for every further wave, 1.8 (3 above 128) for meeting in the cluster.  `clusters[s]`: clusters of s CTAs the chip holds, one CTA per SM -- from
-// three CTAs on a cluster is not given an SM that has one already (288 CTAs in clusters of three take two waves, in pairs one).
-// Fitted to 60 shapes of 16..2048 queries and keys with every split timed: the split chosen is at most 6 % behind the best.  (Powers of
-// two up to the chip's two CTAs per SM: 725 x 687, 12 heads of 128, 19.6 us split four ways and 12.2 two ways; 87 x 956, 36 heads over 12
-// of 128, 20.6 eight and 10.7 three ways.)
-inline OpAttnLaunch opa_plan(int tiles, int tkv, int hs, int sms, const int* clusters) {
-  OpAttnLaunch p;
-  const int per_sm = hs <= 128 ? 2 : 1, budget = per_sm == 2 ? OPA_MAX_SMEM / 2 : OPA_MAX_SMEM, blocks = (tkv + 63) / 64, chunks = hs / 16;
-  p.stages = OPA_MAX_STAGES;
-  while (p.stages > 2 && opa_smem(hs, p.stages) > budget) --p.stages;
-  p.smem = opa_smem(hs, p.stages);
-  p.split = 1;
-  double best = 1e300;
-  for (int s = 1; s <= OPA_MAX_SPLIT && s <= blocks; ++s) {
-    if ((chunks + s - 1) / s * s * 8192 > p.smem) continue;                       // (the partial rows meet in the stages)
-    const long long ctas = (long long)tiles * s, room = s > 2 ? (long long)clusters[s] * s : (long long)per_sm * sms;
-    const long long waves = room > 0 ? (ctas - 1) / room + 1 : ctas;
-    const double block = per_sm == 2 && s <= 2 && ctas > sms ? 1.55 : 1.0;
-    const double t = (double)waves * ((blocks + s - 1) / s * block + 4.0) + 3.0 + (s == 1 ? 0.0 : (hs <= 128 ? 1.8 : 3.0));
-    if (t < best) { best = t; p.split = s; }
-  }
-  p.tmem_cols = hs <= 128 ? 256 : 512;
-  p.s_bufs = (p.tmem_cols - hs) / ATTN_BN < OPA_MAX_S ? (p.tmem_cols - hs) / ATTN_BN : OPA_MAX_S;
-  return p;
-}
 
 // second operand [key, head dim] as it lies: MN-major, 128-byte swizzle -- 64-wide columns of boxes `box` bytes apart, groups
 // of eight keys 1024 bytes apart
@@ -81,8 +46,11 @@ __device__ __forceinline__ void cluster_sync() {
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
-// maps: 0 Q [tq, hq*hd], 1 K, 2 V [tkv, hkv*hd].  a.out is an absolute address; a.t0 keys, no second segment.
-__global__ void __launch_bounds__(OPA_THREADS) vla_op_attention_kernel(const __grid_constant__ AttnArgs a, const __grid_constant__ OpMaps maps,
+// maps: 0 Q [tq, hq*hd], 1 K, 2 V [tkv, hkv*hd].  a.out is an absolute address; a.t0 keys, no second segment.  TERMS: bf16 numbers of a
+// probability.  (Two of its CTAs share an SM only up to 128 registers a thread -- 14 warps put four on one scheduler -- which the form of
+// two terms exceeds unless it is told: 1024 x 1024 of 12 heads of 64 22.6 instead of 15.7 us.)
+template <int TERMS>
+__global__ void __launch_bounds__(OPA_THREADS, TERMS) vla_op_attention_kernel(const __grid_constant__ AttnArgs a, const __grid_constant__ OpMaps maps,
                                                                        const __grid_constant__ OpAttnLaunch p, unsigned* err, OpFault fault) {
   extern __shared__ __align__(1024) char smem_raw[];
   __shared__ uint32_t tmem_base_s;
@@ -200,8 +168,8 @@ __global__ void __launch_bounds__(OPA_THREADS) vla_op_attention_kernel(const __g
       const uint32_t tp = tmem + ATTN_BN * buf;
       if (elect_one()) {
 #pragma unroll
-        for (int k = 0; k < ATTN_BN / 16; ++k)      // 16 keys = 16 rows of 128 bytes = 32 words of P pairs / 4
-          umma_bf16_ta(tmem_o, tp + 8u * k, vd + (uint64_t)(k * (16 * 128 >> 4)), idesc_o, (i | k) != 0 ? 1u : 0u);
+        for (int k = 0; k < TERMS * (ATTN_BN / 16); ++k)      // 16 keys = 16 rows of 128 bytes = 32 words of P pairs / 4
+          umma_bf16_ta(tmem_o, tp + 8u * k, vd + (uint64_t)(k % (ATTN_BN / 16) * (16 * 128 >> 4)), idesc_o, (i | k) != 0 ? 1u : 0u);
         umma_commit(bar_o + 8u * buf);
         umma_commit(vempty + 8u * s);
       }
@@ -236,7 +204,7 @@ __global__ void __launch_bounds__(OPA_THREADS) vla_op_attention_kernel(const __g
         if (a.causal || a.t0 - kv0 < ATTN_BN) attn_mask(sr, lim);
       }
       float alpha;
-      attn_softmax_block(sr, sl2, m_run, l_run, alpha);
+      attn_softmax_block<TERMS>(sr, sl2, m_run, l_run, alpha);
       // O follows a moved maximum (rarely); everything before has been added by then.  (P V of this block cannot start before this
       // warp arrives.)
       if (i > 0 && __any_sync(0xffffffffu, alpha != 1.0f)) {
@@ -247,6 +215,10 @@ __global__ void __launch_bounds__(OPA_THREADS) vla_op_attention_kernel(const __g
       }
       tmem_st16u(buf, sr);
       tmem_st16u(buf + 16u, sr + 16);
+      if (TERMS == 2) {
+        tmem_st16u(buf + 32u, sr + 32);
+        tmem_st16u(buf + 48u, sr + 48);
+      }
       tmem_st_wait();
       tc_fence_before();
       arrive_warp(bar_p + 8u * b, lane);

@@ -103,7 +103,8 @@ inline OpDevice* op_device() {
     for (auto* kernel : {vla_op_linear_pair_kernel<1, false>, vla_op_linear_pair_kernel<2, false>, vla_op_linear_pair_kernel<8, false>,
                          vla_op_linear_pair_kernel<1, true>, vla_op_linear_pair_kernel<2, true>, vla_op_linear_pair_kernel<8, true>})
       if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, LINP_SMEM) != cudaSuccess) return nullptr;
-    if (cudaFuncSetAttribute(vla_op_attention_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, OPA_MAX_SMEM) != cudaSuccess) return nullptr;
+    for (auto* kernel : {vla_op_attention_kernel<1>, vla_op_attention_kernel<2>})
+      if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, OPA_MAX_SMEM) != cudaSuccess) return nullptr;
     for (int s = 1; s <= OPA_MAX_SPLIT; ++s) {
       cudaLaunchConfig_t cfg = {};
       cudaLaunchAttribute at;
@@ -111,7 +112,7 @@ inline OpDevice* op_device() {
       at.val.clusterDim.x = (unsigned)s; at.val.clusterDim.y = 1; at.val.clusterDim.z = 1;
       cfg.gridDim = dim3((unsigned)s); cfg.blockDim = dim3(OPA_THREADS); cfg.dynamicSmemBytes = 192 * 1024;
       cfg.attrs = &at; cfg.numAttrs = 1;
-      if (cudaOccupancyMaxActiveClusters(&d.clusters[s], vla_op_attention_kernel, &cfg) != cudaSuccess) return nullptr;
+      if (cudaOccupancyMaxActiveClusters(&d.clusters[s], vla_op_attention_kernel<1>, &cfg) != cudaSuccess) return nullptr;
     }
     d.sms = sms;
     d.error.store(static_cast<unsigned*>(a), std::memory_order_release);
@@ -181,7 +182,7 @@ inline int op_attention_run(const void* q, const void* k, const void* v, void* o
       !op_encode(&maps.m[1], k, tkv, (int64_t)hkv * hd, (int64_t)hkv * hd, a.bn) ||
       !op_encode(&maps.m[2], v, tkv, (int64_t)hkv * hd, (int64_t)hkv * hd, a.bn))
     return VLA_ERR_CUDA;
-  return op_launch(vla_op_attention_kernel, n_tiles * p.split, OPA_THREADS, p.smem, p.split, s, a, maps, p, static_cast<unsigned*>(scratch), op_fault());
+  return op_launch(p.terms == 2 ? vla_op_attention_kernel<2> : vla_op_attention_kernel<1>, n_tiles * p.split, OPA_THREADS, p.smem, p.split, s, a, maps, p, static_cast<unsigned*>(scratch), op_fault());
 }
 
 }  // namespace vla
