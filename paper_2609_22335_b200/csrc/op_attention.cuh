@@ -284,7 +284,8 @@ __global__ void __launch_bounds__(OPA_THREADS, TERMS) vla_op_attention_kernel(co
 #pragma unroll
       for (int r = 0; r < OPA_MAX_SPLIT; ++r) {
         const float2 v = r < split ? row_ml[r][threadIdx.x] : make_float2(-INFINITY, 0.f);
-        f[r] = v.x == -INFINITY ? 0.f : exp2_fast((v.x - M) * sl2);
+        // (no maximum: a part without keys of this row, or one whose scores are all NaN -- its sum is then, and the row is as it would be unsplit)
+        f[r] = v.x == -INFINITY ? (v.y == 0.f ? 0.f : v.y) : exp2_fast((v.x - M) * sl2);
         if (f[r] != 0.f) L = fmaf(v.y, f[r], L);
       }
       const float inv = L == 0.f ? 0.f : 1.0f / L;

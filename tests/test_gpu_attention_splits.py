@@ -32,3 +32,27 @@ def test_against_64_bit(tq, tkv, hq, hkv, hd, causal, scale):
     assert err <= 2.0 ** -8, err
     assert torch.isfinite(got.float()).all()
     assert torch.equal(got, api.op_attention(q, k, v, hq, hkv, hd, causal=causal))
+
+
+@pytest.mark.parametrize("tq,tkv,hq,hkv,hd", [
+    (1024, 512, 48, 48, 64), (90, 900, 4, 4, 64), (51, 867, 8, 1, 256), (87, 956, 36, 12, 128), (9, 300, 4, 2, 64)])
+def test_nan_is_not_lost(tq, tkv, hq, hkv, hd):
+    """A row whose scores are NaN is NaN whether its keys are split or not, and where only some of the parts hold a NaN; others are as without it."""
+    import torch
+    from paper_2609_22335_b200 import api
+    g = torch.Generator(device="cuda").manual_seed(tq)
+    q, k, v = ((torch.randn(n, h * hd, device="cuda", generator=g)).to(torch.bfloat16) for n, h in ((tq, hq), (tkv, hkv), (tkv, hkv)))
+    clean = api.op_attention(q, k, v, hq, hkv, hd).view(tq, hq, hd)
+    bad = q.clone()
+    bad.view(tq, hq, hd)[tq // 2, hq - 1] = float("nan")
+    got = api.op_attention(bad, k, v, hq, hkv, hd).view(tq, hq, hd)
+    assert torch.isnan(got[tq // 2, hq - 1]).all()
+    keep = torch.ones(tq, hq, dtype=torch.bool, device="cuda")
+    keep[tq // 2, hq - 1] = False
+    assert torch.equal(got[keep], clean[keep])
+    for keys in (slice(0, 64), slice(0, tkv // 2), slice(tkv - 1, tkv)):
+        bad = k.clone()
+        bad.view(tkv, hkv, hd)[keys, 0] = float("nan")
+        got = api.op_attention(q, bad, v, hq, hkv, hd).view(tq, hq, hd)
+        assert torch.isnan(got[:, :hq // hkv]).all(), keys
+        assert torch.equal(got[:, hq // hkv:], clean[:, hq // hkv:])
