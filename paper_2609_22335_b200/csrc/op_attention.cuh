@@ -112,7 +112,8 @@ __global__ void __launch_bounds__(OPA_THREADS, TERMS) vla_op_attention_kernel(co
     __syncwarp();
   } else if (warp == 5) {
     // ---------------- S = Q K^T, into a buffer as soon as P V has read the probabilities that were in it.  (The commit that somebody
-    // waits for goes first: each costs its thread 150 cycles.)
+    // waits for goes first: each costs its thread 150 cycles.  A stage that no later block is loaded into is not released: nobody would
+    // wait for that arrival, and it could come after the CTA's end.)
     const uint32_t idesc_s = umma_idesc_bf16(ATTN_BN);
     const uint64_t qdesc = umma_desc_sw128(Qs);
     uint32_t s = 0, ph = 0u, buf = 0, bph = 1u;
@@ -135,7 +136,7 @@ __global__ void __launch_bounds__(OPA_THREADS, TERMS) vla_op_attention_kernel(co
 #pragma unroll 1
         for (int k = 0; kc < hs / 16; ++kc, ++k) umma_bf16(ts, qd + 2u * k, kd + 2u * k, idesc_s, kc != 0 ? 1u : 0u);
         umma_commit(bar_s + 8u * buf);
-        umma_commit(kempty + 8u * s);
+        if (i + NS < n) umma_commit(kempty + 8u * s);
       }
       __syncwarp();
       if (++s == (uint32_t)NS) { s = 0; ph ^= 1u; }
@@ -171,7 +172,7 @@ __global__ void __launch_bounds__(OPA_THREADS, TERMS) vla_op_attention_kernel(co
         for (int k = 0; k < TERMS * (ATTN_BN / 16); ++k)      // 16 keys = 16 rows of 128 bytes = 32 words of P pairs / 4
           umma_bf16_ta(tmem_o, tp + 8u * k, vd + (uint64_t)(k % (ATTN_BN / 16) * (16 * 128 >> 4)), idesc_o, (i | k) != 0 ? 1u : 0u);
         umma_commit(bar_o + 8u * buf);
-        umma_commit(vempty + 8u * s);
+        if (i + NS < n) umma_commit(vempty + 8u * s);
       }
       __syncwarp();
       if (++s == (uint32_t)NS) { s = 0; ph ^= 1u; }

@@ -105,12 +105,15 @@ __global__ void __launch_bounds__(LIN_THREADS, 1) vla_op_linear_pair_kernel(cons
       const uint32_t idesc = umma_idesc_bf16(g.bn, 256);
       const uint64_t desc0 = umma_desc_sw128(stage0);
       uint32_t s = 0, ph = 0u, buf = 0, bph = 1u;
+      // A stage is released where a later k-block is loaded into it (in both CTAs, whose producers wait for that): an arrival that
+      // nobody waits for could come when the other CTA has ended and its shared memory is somebody else's.
+      int left = first_tile < g.tiles ? ((g.tiles - 1 - first_tile) / step + 1) * nkb : 0;
       for (int t = first_tile; t < g.tiles && ok; t += step) {
         if (!(ok = mbar_wait(c, acce0 + 8u * buf, bph))) break;
         tc_fence_after();
         int part = 0, from = 0, to = nkb / parts;                     // k-blocks of this part
 #pragma unroll 1
-        for (int kb = 0; kb < nkb; ++kb) {
+        for (int kb = 0; kb < nkb; ++kb, --left) {
           if (PARTS && kb == to) { ++part; from = to; to = nkb * (part + 1) / parts; }
           if (!(ok = mbar_wait(c, full0 + 8u * s, ph))) break;
           tc_fence_after();
@@ -119,7 +122,7 @@ __global__ void __launch_bounds__(LIN_THREADS, 1) vla_op_linear_pair_kernel(cons
           if (elect_one()) {
 #pragma unroll
             for (int k = 0; k < GEMM_BK / 16; ++k) umma_bf16_pair(acc, ad + 2u * k, wd + 2u * k, idesc, kb != from || k != 0 ? 1u : 0u);
-            umma_commit_pair(empty0 + 8u * s);
+            if (left > S) umma_commit_pair(empty0 + 8u * s);
             if (kb == nkb - 1) umma_commit_pair(accf0 + 8u * buf);
           }
           __syncwarp();

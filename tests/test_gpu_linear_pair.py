@@ -49,6 +49,30 @@ def test_calls_that_follow_one_another_and_a_wait_that_runs_out():
     assert torch.equal(api.op_linear(a, w, out_bf16=True), good) and api.op_status(api.OP_LINEAR) == api.VLA_OK
 
 
+def test_what_starts_behind_a_call_finds_its_own_barriers():
+    """Calls whose CTAs take the shared memory of the CTAs before them at once (each starts while the one in front ends): tiles of two SMs
+    whose k-blocks are few more than the stages and not, tiles of one SM, attention of one to eight blocks a CTA.  An arrival that came
+    after its CTA's end would land on one of their barriers."""
+    import torch
+    from paper_2609_22335_b200 import api
+    g = torch.Generator(device="cuda").manual_seed(3)
+
+    def rand(rows, cols, s):
+        return (s * torch.randn(rows, cols, device="cuda", generator=g)).to(torch.bfloat16)
+    linear = [(rand(m, k, 1.0), rand(n, k, k ** -0.5), f32) for m, n, k, f32 in
+              ((2048, 16384, 64, False), (1747, 2064, 2288, False), (64, 4096, 720, False), (294, 8512, 2952, True), (3000, 4902, 520, True))]
+    attn = [(rand(tq, hq * hd, 1.0), rand(tkv, hkv * hd, 1.0), rand(tkv, hkv * hd, 1.0), hq, hkv, hd) for tq, tkv, hq, hkv, hd in
+            ((87, 956, 36, 12, 128), (1024, 1024, 12, 12, 64), (51, 867, 8, 1, 256), (300, 64, 16, 16, 128))]
+    calls = [lambda a=a, w=w, f=f: api.op_linear(a, w, out_bf16=not f) for a, w, f in linear] + [lambda x=x: api.op_attention(*x) for x in attn]
+    want = [f() for f in calls]
+    torch.cuda.synchronize()
+    for i in range(40):
+        order = torch.randperm(len(calls), generator=torch.Generator().manual_seed(i)).tolist()
+        got = [calls[j]() for j in order]
+        assert all(torch.equal(x, want[j]) for x, j in zip(got, order)), i
+    assert api.op_status(api.OP_LINEAR) == api.VLA_OK
+
+
 def test_captured_calls_follow_their_inputs():
     """Tiles of two SMs and attention over clusters of three CTAs in one graph: a replay computes from what the inputs hold then."""
     import torch
