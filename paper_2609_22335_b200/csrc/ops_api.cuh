@@ -5,10 +5,9 @@
 #include <cuda.h>
 #include <cuda_runtime.h>
 
-#include <atomic>
-
 #include "../../include/vla.h"
 #include "dispatch.cuh"
+#include "per_device.h"
 
 namespace vla {
 
@@ -83,41 +82,37 @@ constexpr size_t OP_ATTN_HEADER = 256;   // error word + padding (behind it: roo
 // that was captured into a graph reports on its latest replay like any other.
 static __device__ __align__(256) unsigned g_op_linear_error[64];
 struct OpDevice {
-  std::atomic<unsigned*> error{nullptr};
+  unsigned* error = nullptr;
   int sms = 0;
   int clusters[OPA_MAX_SPLIT + 1] = {};       // attention: clusters of so many CTAs that the chip holds
 };
-inline OpDevice* op_device() {
-  constexpr int kMax = 64;
-  static OpDevice devices[kMax];
-  int dev = -1;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMax) return nullptr;
-  OpDevice& d = devices[dev];
-  if (!d.error.load(std::memory_order_acquire)) {
-    void* a = nullptr;
-    int sms = 0;
-    if (cudaGetSymbolAddress(&a, g_op_linear_error) != cudaSuccess || !a) return nullptr;
-    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return nullptr;
-    for (auto* kernel : {vla_op_linear_kernel<1>, vla_op_linear_kernel<2>, vla_op_linear_kernel<8>})
-      if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, LIN_SMEM) != cudaSuccess) return nullptr;
-    for (auto* kernel : {vla_op_linear_pair_kernel<1, false>, vla_op_linear_pair_kernel<2, false>, vla_op_linear_pair_kernel<8, false>,
-                         vla_op_linear_pair_kernel<1, true>, vla_op_linear_pair_kernel<2, true>, vla_op_linear_pair_kernel<8, true>})
-      if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, LINP_SMEM) != cudaSuccess) return nullptr;
-    for (auto* kernel : {vla_op_attention_kernel<1>, vla_op_attention_kernel<2>})
-      if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, OPA_MAX_SMEM) != cudaSuccess) return nullptr;
-    for (int s = 1; s <= OPA_MAX_SPLIT; ++s) {
-      cudaLaunchConfig_t cfg = {};
-      cudaLaunchAttribute at;
-      at.id = cudaLaunchAttributeClusterDimension;
-      at.val.clusterDim.x = (unsigned)s; at.val.clusterDim.y = 1; at.val.clusterDim.z = 1;
-      cfg.gridDim = dim3((unsigned)s); cfg.blockDim = dim3(OPA_THREADS); cfg.dynamicSmemBytes = 192 * 1024;
-      cfg.attrs = &at; cfg.numAttrs = 1;
-      if (cudaOccupancyMaxActiveClusters(&d.clusters[s], vla_op_attention_kernel<1>, &cfg) != cudaSuccess) return nullptr;
-    }
-    d.sms = sms;
-    d.error.store(static_cast<unsigned*>(a), std::memory_order_release);
+inline bool op_look_up(int dev, OpDevice* d) {
+  void* a = nullptr;
+  if (cudaGetSymbolAddress(&a, g_op_linear_error) != cudaSuccess || !a) return false;
+  d->error = static_cast<unsigned*>(a);
+  if (cudaDeviceGetAttribute(&d->sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return false;
+  for (auto* kernel : {vla_op_linear_kernel<1>, vla_op_linear_kernel<2>, vla_op_linear_kernel<8>})
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, LIN_SMEM) != cudaSuccess) return false;
+  for (auto* kernel : {vla_op_linear_pair_kernel<1, false>, vla_op_linear_pair_kernel<2, false>, vla_op_linear_pair_kernel<8, false>,
+                       vla_op_linear_pair_kernel<1, true>, vla_op_linear_pair_kernel<2, true>, vla_op_linear_pair_kernel<8, true>})
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, LINP_SMEM) != cudaSuccess) return false;
+  for (auto* kernel : {vla_op_attention_kernel<1>, vla_op_attention_kernel<2>})
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, OPA_MAX_SMEM) != cudaSuccess) return false;
+  for (int s = 1; s <= OPA_MAX_SPLIT; ++s) {
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = (unsigned)s; at.val.clusterDim.y = 1; at.val.clusterDim.z = 1;
+    cfg.gridDim = dim3((unsigned)s); cfg.blockDim = dim3(OPA_THREADS); cfg.dynamicSmemBytes = 192 * 1024;
+    cfg.attrs = &at; cfg.numAttrs = 1;
+    if (cudaOccupancyMaxActiveClusters(&d->clusters[s], vla_op_attention_kernel<1>, &cfg) != cudaSuccess) return false;
   }
-  return &d;
+  return true;
+}
+inline bool op_device(OpDevice* d) {
+  static PerDevice<OpDevice> devices;
+  int dev = -1;
+  return cudaGetDevice(&dev) == cudaSuccess && devices.get(dev, d, [dev](OpDevice* r) { return op_look_up(dev, r); });
 }
 
 // Reads an operator's error word back after the stream has drained.
@@ -160,8 +155,8 @@ inline size_t op_attention_scratch_bytes(int tkv, int hkv, int hd) {
 // Shared implementation of the two attention entry points: the first word of `scratch` is the call's error word.
 inline int op_attention_run(const void* q, const void* k, const void* v, void* out, int tq, int tkv, int hq, int hkv, int hd,
                             int causal, void* scratch, cudaStream_t s) {
-  OpDevice* dev = op_device();
-  if (!dev) return VLA_ERR_CUDA;
+  OpDevice dev;
+  if (!op_device(&dev)) return VLA_ERR_CUDA;
   AttnArgs a;
   memset(&a, 0, sizeof a);
   a.out = reinterpret_cast<Ref>(out);
@@ -172,10 +167,10 @@ inline int op_attention_run(const void* q, const void* k, const void* v, void* o
   a.q_blocks = (tq + 127) / 128;
   a.hpt = attn_fold(tq, hq, hkv, &a.rph);
   int n_tiles = a.hpt > 1 ? hkv * (((hq / hkv) + a.hpt - 1) / a.hpt) : hq * a.q_blocks;
-  OpAttnLaunch p = opa_plan(n_tiles, tkv, hd, dev->sms, dev->clusters);
+  OpAttnLaunch p = opa_plan(n_tiles, tkv, hd, dev.sms, dev.clusters);
   // Folded heads share the loads of their keys, but a split tile of several heads also has several heads' rows to exchange: where
   // the chip has the room, each head is a tile of its own (51 x 867, 8 heads of 256 over one: 11.9 -> 9.2 us).
-  if (a.hpt > 1 && p.split > 2 && hq <= dev->clusters[p.split]) { a.hpt = 1; n_tiles = hq; }
+  if (a.hpt > 1 && p.split > 2 && hq <= dev.clusters[p.split]) { a.hpt = 1; n_tiles = hq; }
   a.scale_log2e = 1.4426950408889634f / sqrtf((float)hd);
   OpMaps maps;
   if (!op_encode(&maps.m[0], q, tq, (int64_t)hq * hd, (int64_t)hq * hd, a.hpt > 1 ? a.rph : 128) ||
@@ -208,27 +203,27 @@ int vla_op_linear(const void* a, const void* w, float* out32, void* out16, int32
                   void* stream) {
   using namespace vla;
   if (!a || !w || (!out32 && !out16) || m < 1 || n < 1 || k < 8 || k % 8 || act < 0 || act > 2) return VLA_ERR_INVALID;
-  OpDevice* dev = op_device();
-  if (!dev) return VLA_ERR_CUDA;
+  OpDevice dev;
+  if (!op_device(&dev)) return VLA_ERR_CUDA;
   LinearArgs g;
   g.m = m; g.n = n; g.kp = (int)op_pad(k, GEMM_BK); g.act = act;
   g.out32 = out32; g.out16 = static_cast<unsigned short*>(out16);
-  g.err = dev->error.load(std::memory_order_relaxed);
-  const LinearPlan p = linear_plan(m, n, k, out32 != nullptr, dev->sms);
-  const LinearPairPlan pp = linear_pair_plan(m, n, k, p, dev->sms);
+  g.err = dev.error;
+  const LinearPlan p = linear_plan(m, n, k, out32 != nullptr, dev.sms);
+  const LinearPairPlan pp = linear_pair_plan(m, n, k, p, dev.sms);
   const int vec = linear_vec(n, out32, out16);
   OpMaps maps;
   if (pp.bn > 0) {
     g.bm = pp.bm; g.bn = pp.bn; g.ks = p.ks; g.tiles_m = pp.tiles_m; g.tiles = pp.tiles; g.stages = pp.stages;
     if (!op_encode(&maps.m[0], w, n, k, k, g.bn / 2) || !op_encode(&maps.m[1], a, m, k, k, g.bm)) return VLA_ERR_CUDA;
-    const int pairs = g.tiles < dev->sms / 2 ? g.tiles : dev->sms / 2;
+    const int pairs = g.tiles < dev.sms / 2 ? g.tiles : dev.sms / 2;
     const auto kernel = g.ks > 1 ? (vec == 8 ? vla_op_linear_pair_kernel<8, true> : (vec == 2 ? vla_op_linear_pair_kernel<2, true> : vla_op_linear_pair_kernel<1, true>))
                                  : (vec == 8 ? vla_op_linear_pair_kernel<8, false> : (vec == 2 ? vla_op_linear_pair_kernel<2, false> : vla_op_linear_pair_kernel<1, false>));
     return op_launch(kernel, 2 * pairs, LIN_THREADS, LINP_SMEM, 2, static_cast<cudaStream_t>(stream), g, maps, op_fault());
   }
   g.bm = p.bm; g.bn = p.bn; g.ks = p.ks; g.tiles_m = p.tiles_m; g.tiles = p.tiles; g.stages = p.stages;
   if (!op_encode(&maps.m[0], w, n, k, k, g.bn) || !op_encode(&maps.m[1], a, m, k, k, g.bm)) return VLA_ERR_CUDA;
-  const int grid = g.ks > 1 ? g.tiles * g.ks : (g.tiles < 2 * dev->sms ? g.tiles : 2 * dev->sms);
+  const int grid = g.ks > 1 ? g.tiles * g.ks : (g.tiles < 2 * dev.sms ? g.tiles : 2 * dev.sms);
   const auto kernel = vec == 8 ? vla_op_linear_kernel<8> : (vec == 2 ? vla_op_linear_kernel<2> : vla_op_linear_kernel<1>);
   return op_launch(kernel, grid, LIN_THREADS, linear_smem(g), g.ks, static_cast<cudaStream_t>(stream), g, maps, op_fault());
 }

@@ -911,8 +911,8 @@ int vla_op_attention_static(const void* q, const void* k, const void* v, void* o
 int vla_op_status(int32_t op, const void* scratch, void* stream) {
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   if (op == VLA_OP_LINEAR) {
-    vla::OpDevice* d = vla::op_device();
-    return d ? vla::op_status_of(d->error.load(), s) : VLA_ERR_CUDA;
+    vla::OpDevice d;
+    return vla::op_device(&d) ? vla::op_status_of(d.error, s) : VLA_ERR_CUDA;
   }
   if (op == VLA_OP_ATTENTION) {
     if (!scratch) return VLA_ERR_INVALID;
