@@ -105,7 +105,10 @@ inline bool op_look_up(int dev, OpDevice* d) {
     at.val.clusterDim.x = (unsigned)s; at.val.clusterDim.y = 1; at.val.clusterDim.z = 1;
     cfg.gridDim = dim3((unsigned)s); cfg.blockDim = dim3(OPA_THREADS); cfg.dynamicSmemBytes = 192 * 1024;
     cfg.attrs = &at; cfg.numAttrs = 1;
-    if (cudaOccupancyMaxActiveClusters(&d->clusters[s], vla_op_attention_kernel<1>, &cfg) != cudaSuccess) return false;
+    if (cudaOccupancyMaxActiveClusters(&d->clusters[s], vla_op_attention_kernel<1>, &cfg) != cudaSuccess) {
+      d->clusters[s] = 0;                     // not known: attention then stays at one or two CTAs, and nothing fails for it
+      cudaGetLastError();
+    }
   }
   return true;
 }
