@@ -84,8 +84,24 @@ static __device__ __align__(256) unsigned g_op_linear_error[64];
 struct OpDevice {
   unsigned* error = nullptr;
   int sms = 0;
-  int clusters[OPA_MAX_SPLIT + 1] = {};       // attention: clusters of so many CTAs that the chip holds
+  OpRoom room = {};
 };
+// The occupancy query answers one CTA per SM for a kernel that allocates tensor memory, where the hardware runs two once the first has
+// allocated; so it is asked for a kernel that does not, with the shared memory of the operators' CTAs.  What it does not answer stays 0, and
+// calls then use one or two CTAs a tile.
+__global__ void vla_op_room_kernel() {}
+inline int op_clusters(int s, int smem) {
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = (unsigned)s; at.val.clusterDim.y = 1; at.val.clusterDim.z = 1;
+  cfg.gridDim = dim3((unsigned)s); cfg.blockDim = dim3(LIN_THREADS); cfg.dynamicSmemBytes = (size_t)smem;
+  cfg.attrs = &at; cfg.numAttrs = 1;
+  int n = 0;
+  if (cudaOccupancyMaxActiveClusters(&n, vla_op_room_kernel, &cfg) == cudaSuccess) return n;
+  cudaGetLastError();
+  return 0;
+}
 inline bool op_look_up(int dev, OpDevice* d) {
   void* a = nullptr;
   if (cudaGetSymbolAddress(&a, g_op_linear_error) != cudaSuccess || !a) return false;
@@ -98,18 +114,8 @@ inline bool op_look_up(int dev, OpDevice* d) {
     if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, LINP_SMEM) != cudaSuccess) return false;
   for (auto* kernel : {vla_op_attention_kernel<1>, vla_op_attention_kernel<2>})
     if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, OPA_MAX_SMEM) != cudaSuccess) return false;
-  for (int s = 1; s <= OPA_MAX_SPLIT; ++s) {
-    cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute at;
-    at.id = cudaLaunchAttributeClusterDimension;
-    at.val.clusterDim.x = (unsigned)s; at.val.clusterDim.y = 1; at.val.clusterDim.z = 1;
-    cfg.gridDim = dim3((unsigned)s); cfg.blockDim = dim3(OPA_THREADS); cfg.dynamicSmemBytes = 192 * 1024;
-    cfg.attrs = &at; cfg.numAttrs = 1;
-    if (cudaOccupancyMaxActiveClusters(&d->clusters[s], vla_op_attention_kernel<1>, &cfg) != cudaSuccess) {
-      d->clusters[s] = 0;                     // not known: attention then stays at one or two CTAs, and nothing fails for it
-      cudaGetLastError();
-    }
-  }
+  const bool asked = cudaFuncSetAttribute(vla_op_room_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, OPA_MAX_SMEM) == cudaSuccess;
+  for (int s = 1; s <= OPA_MAX_SPLIT && asked; ++s) { d->room.alone[s] = op_clusters(s, OPA_MAX_SMEM); d->room.two[s] = op_clusters(s, LIN_SMEM); }
   return true;
 }
 inline bool op_device(OpDevice* d) {
@@ -170,10 +176,10 @@ inline int op_attention_run(const void* q, const void* k, const void* v, void* o
   a.q_blocks = (tq + 127) / 128;
   a.hpt = attn_fold(tq, hq, hkv, &a.rph);
   int n_tiles = a.hpt > 1 ? hkv * (((hq / hkv) + a.hpt - 1) / a.hpt) : hq * a.q_blocks;
-  OpAttnLaunch p = opa_plan(n_tiles, tkv, hd, dev.sms, dev.clusters);
+  OpAttnLaunch p = opa_plan(n_tiles, tkv, hd, causal != 0, dev.sms, dev.room);
   // Folded heads share the loads of their keys, but a split tile of several heads also has several heads' rows to exchange: where
   // the chip has the room, each head is a tile of its own (51 x 867, 8 heads of 256 over one: 11.9 -> 9.2 us).
-  if (a.hpt > 1 && p.split > 2 && hq <= dev.clusters[p.split]) { a.hpt = 1; n_tiles = hq; }
+  if (a.hpt > 1 && p.split > 2 && hq <= dev.room.alone[p.split]) { a.hpt = 1; n_tiles = hq; }
   a.scale_log2e = 1.4426950408889634f / sqrtf((float)hd);
   OpMaps maps;
   if (!op_encode(&maps.m[0], q, tq, (int64_t)hq * hd, (int64_t)hq * hd, a.hpt > 1 ? a.rph : 128) ||
