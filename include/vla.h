@@ -302,10 +302,16 @@ int vla_debug_op_fault(int32_t drop_operand_loads, uint64_t wait_limit_ns);
  * one, for which n is a multiple of 8 (gated: 4), the rows of w are padded to a multiple of 32 and reordered within each
  * 32 as the engine's are (row p holds feature 8 * ((p >> 1) & 3) + 2 * (p >> 3) + (p & 1)), x comes with out32 and
  * without act, and act = 1 with out16 alone.
+ * Addends, straight epilogue: bias and vec [n], tab and tab_b [m,n] (each optional, fp32) under the accumulators, x behind the
+ * product (may be out32 itself); act = 1 with out16 alone and no addend but bias.  ss (optional, fp32 [m, n / 128 rounded
+ * up], with out32 and out16): sums of squares of each row's features, 128 at a time.
  * Attention: q [tq, hq*hd] and k0 [t0, hkv*hd] bf16, vt0 [hkv*hd, t0 rounded up to 64] bf16, V transposed; an optional
  * second segment of t1 keys, of which the queries below sfx see only the first sfx; out [tq, hq*hd] bf16. */
 int vla_debug_tile_linear(const void* a, const void* w, const float* x, float* out32, void* out16, int32_t m, int32_t n,
                           int32_t k, int32_t act, int32_t gated, int32_t fast);
+int vla_debug_tile_addends(const void* a, const void* w, const float* x, const float* bias, const float* vec, const float* tab,
+                           const float* tab_b, float* out32, void* out16, float* ss, int32_t m, int32_t n, int32_t k,
+                           int32_t act);
 int vla_debug_tile_attention(const void* q, const void* k0, const void* vt0, const void* k1, const void* vt1, void* out,
                              int32_t tq, int32_t t0, int32_t t1, int32_t hq, int32_t hkv, int32_t hd, int32_t causal,
                              int32_t sfx);

@@ -26,7 +26,7 @@ _SOLVER = {"euler": 0, "ddim": 1}
 EXPORTS = ["vla_required_arena_bytes", "vla_init", "vla_load_weights", "vla_submit_frame", "vla_submit_frame_device",
            "vla_poll_actions", "vla_hold_launches", "vla_wait_idle", "vla_get_trace", "vla_reset_trace", "vla_program_info", "vla_debug_fetch",
            "vla_get_counters", "vla_set_class_tags", "vla_get_class_tags", "vla_policy_probe", "vla_policy_probe_ex", "vla_debug_bump_dependency", "vla_debug_guards", "vla_last_error",
-           "vla_destroy", "vla_op_status", "vla_debug_op_fault", "vla_debug_tile_linear", "vla_debug_tile_attention",
+           "vla_destroy", "vla_op_status", "vla_debug_op_fault", "vla_debug_tile_linear", "vla_debug_tile_addends", "vla_debug_tile_attention",
            "vla_op_attention_scratch_bytes", "vla_op_attention", "vla_op_linear",
            "vla_op_attention_static_capacity", "vla_op_attention_static"]
 
@@ -102,6 +102,7 @@ def load_library() -> C.CDLL:
     lib.vla_op_status.argtypes = [C.c_int32, C.c_void_p, C.c_void_p]
     lib.vla_debug_op_fault.argtypes = [C.c_int32, C.c_uint64]
     lib.vla_debug_tile_linear.argtypes = [C.c_void_p] * 5 + [C.c_int32] * 6
+    lib.vla_debug_tile_addends.argtypes = [C.c_void_p] * 10 + [C.c_int32] * 4
     lib.vla_debug_tile_attention.argtypes = [C.c_void_p] * 6 + [C.c_int32] * 8
     lib.vla_op_attention_scratch_bytes.argtypes = [C.c_int32, C.c_int32, C.c_int32, P(C.c_size_t)]
     lib.vla_op_attention.argtypes = [C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p] + [C.c_int32] * 6 + [C.c_void_p, C.c_size_t, C.c_void_p]
@@ -497,6 +498,22 @@ def debug_tile_linear(a, w, n, x=None, act=0, gated=False, fast=False, out32=Tru
     if rc != VLA_OK:
         raise VlaError(rc, "vla_debug_tile_linear failed")
     return o32, o16
+
+
+def debug_tile_addends(a, w, n, x=None, bias=None, vec=None, tab=None, tab2=None, act=0, out32=True, out16=False, ss=False, in_place=False):
+    """Test hook: the GEMM tile body with addends (see vla_debug_tile_addends).  Returns (fp32 [m,n], bf16 [m,n], sums of squares), None
+    where not asked for; ``in_place``: the fp32 rows take the place of ``x``."""
+    import torch
+    m, k = a.shape
+    o32 = x if in_place else a.new_empty((m, n), dtype=torch.float32) if out32 else None
+    o16 = a.new_empty((m, n), dtype=torch.bfloat16) if out16 else None
+    sums = a.new_empty((m, (n + 127) // 128), dtype=torch.float32) if ss else None
+    ptr = lambda t: None if t is None else t.data_ptr()
+    rc = load_library().vla_debug_tile_addends(a.data_ptr(), w.data_ptr(), ptr(x), ptr(bias), ptr(vec), ptr(tab), ptr(tab2), ptr(o32), ptr(o16),
+                                               ptr(sums), m, n, k, act)
+    if rc != VLA_OK:
+        raise VlaError(rc, "vla_debug_tile_addends failed")
+    return o32, o16, sums
 
 
 def debug_tile_attention(q, k0, v0, hq, hkv, hd, k1=None, v1=None, causal=False, sfx=0):

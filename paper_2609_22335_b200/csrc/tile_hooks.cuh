@@ -43,40 +43,66 @@ inline int run_tile_hook(TileHookBlock& h, int n_maps) {
 
 inline bool hook_aligned(const void* p, uintptr_t bytes) { return (reinterpret_cast<uintptr_t>(p) & (bytes - 1)) == 0; }
 
-}  // namespace vla
-
-extern "C" {
-
-int vla_debug_tile_linear(const void* a, const void* w, const float* x, float* out32, void* out16, int32_t m, int32_t n, int32_t k,
-                          int32_t act, int32_t gated, int32_t fast) {
-  using namespace vla;
-  if (!a || !w || (!out32 && !out16) || m < 1 || n < 1 || k < 8 || k % 8 || act < 0 || act > 2) return VLA_ERR_INVALID;
-  if (gated && (x || out32)) return VLA_ERR_INVALID;
+// The GEMM node of a hook; `bias` .. `tab2` and `ss` with the straight epilogue only.
+struct TileLinear {
+  const void *a, *w;
+  const float *x, *bias, *vec, *tab, *tab2;
+  float* out32;
+  void* out16;
+  float* ss;
+  int m, n, k, act, gated, fast;
+};
+inline int run_tile_linear(const TileLinear& t) {
+  const bool under = t.bias || t.vec || t.tab || t.tab2, adds = t.x || t.vec || t.tab || t.tab2;
+  if (!t.a || !t.w || (!t.out32 && !t.out16) || t.m < 1 || t.n < 1 || t.k < 8 || t.k % 8 || t.act < 0 || t.act > 2) return VLA_ERR_INVALID;
+  if (t.gated && (t.x || under || t.out32)) return VLA_ERR_INVALID;
+  if ((under || t.ss) && !t.fast) return VLA_ERR_INVALID;
+  if (t.ss && (!t.out32 || !t.out16)) return VLA_ERR_INVALID;
   // what the straight epilogue takes (see the rule in program.cc): whole vectors, and no activation behind an addend or in fp32 rows
-  if (fast && (n % (gated ? 4 : 8) || !hook_aligned(x, 16) || !hook_aligned(out32, 32) || !hook_aligned(out16, 16) ||
-               (!gated && act != ACT_NONE && (act != ACT_GELU || out32 || x)) || (x && !out32)))
+  if (t.fast && (t.n % (t.gated ? 4 : 8) || !hook_aligned(t.x, 16) || !hook_aligned(t.bias, 16) || !hook_aligned(t.vec, 16) || !hook_aligned(t.tab, 16) ||
+                 !hook_aligned(t.tab2, 16) || !hook_aligned(t.out32, 32) || !hook_aligned(t.out16, 16) ||
+                 (!t.gated && t.act != ACT_NONE && (t.act != ACT_GELU || t.out32 || adds)) || (t.x && !t.out32)))
     return VLA_ERR_INVALID;
   TileHookBlock h;
   memset(&h, 0, sizeof h);
   NodeDesc& nd = h.node;
   GemmArgs& g = nd.u.gemm;
   nd.op = OP_GEMM;
-  g.M = m; g.N = n; g.Kp = (int)op_pad(k, GEMM_BK);
-  g.X = reinterpret_cast<Ref>(x); g.ldx = n;
-  g.out32 = reinterpret_cast<Ref>(out32); g.ldo32 = n;
-  g.out16 = reinterpret_cast<Ref>(out16); g.ldo16 = n;
-  g.act = act; g.dual = gated ? 1 : 0; g.c_acc = 1.f; g.c_x = 1.f;
-  g.tiles_t = (m + GEMM_MAX_BT - 1) / GEMM_MAX_BT;
-  g.bt = (int)op_pad((m + g.tiles_t - 1) / g.tiles_t, 16);
+  g.M = t.m; g.N = t.n; g.Kp = (int)op_pad(t.k, GEMM_BK);
+  g.X = reinterpret_cast<Ref>(t.x); g.ldx = t.n;
+  g.bias = reinterpret_cast<Ref>(t.bias); g.vec = reinterpret_cast<Ref>(t.vec);
+  g.tab = reinterpret_cast<Ref>(t.tab); g.ldtab = t.n;
+  g.tab2 = reinterpret_cast<Ref>(t.tab2); g.ldtab2 = t.n;
+  g.out32 = reinterpret_cast<Ref>(t.out32); g.ldo32 = t.n;
+  g.out16 = reinterpret_cast<Ref>(t.out16); g.ldo16 = t.n;
+  g.act = t.act; g.dual = t.gated ? 1 : 0; g.c_acc = 1.f; g.c_x = 1.f;
+  g.tiles_t = (t.m + GEMM_MAX_BT - 1) / GEMM_MAX_BT;
+  g.bt = (int)op_pad((t.m + g.tiles_t - 1) / g.tiles_t, 16);
   g.stages = gemm_stages(g.bt, g.Kp);
-  g.fast = g.perm = fast ? 1 : 0;
-  g.resid = fast && x ? 1 : 0;
+  g.fast = g.perm = t.fast ? 1 : 0;
+  g.resid = t.fast && t.x ? 1 : 0;
+  g.under = (t.bias ? 1 : 0) | (t.vec ? 2 : 0) | (t.tab ? 8 : 0) | (t.tab2 ? 16 : 0);
   nd.smem_bytes = gemm_smem_bytes(g.bt, g.stages);
   nd.tmem_cols = GEMM_BM;
-  const int rows = gated ? 2 * n : n, per_tile = gated ? GEMM_BM / 2 : GEMM_BM;
-  nd.n_tiles = (n + per_tile - 1) / per_tile * g.tiles_t;
-  if (!op_encode(h.maps, w, fast ? op_pad(rows, 32) : rows, k, k, GEMM_BM) || !op_encode(h.maps + 1, a, m, k, k, g.bt)) return VLA_ERR_CUDA;
+  const int rows = t.gated ? 2 * t.n : t.n, per_tile = t.gated ? GEMM_BM / 2 : GEMM_BM, tiles_n = (t.n + per_tile - 1) / per_tile;
+  g.ss_out = reinterpret_cast<Ref>(t.ss); g.ss_out_ld = tiles_n;
+  nd.n_tiles = tiles_n * g.tiles_t;
+  if (!op_encode(h.maps, t.w, t.fast ? op_pad(rows, 32) : rows, t.k, t.k, GEMM_BM) || !op_encode(h.maps + 1, t.a, t.m, t.k, t.k, g.bt)) return VLA_ERR_CUDA;
   return run_tile_hook(h, 2);
+}
+
+}  // namespace vla
+
+extern "C" {
+
+int vla_debug_tile_linear(const void* a, const void* w, const float* x, float* out32, void* out16, int32_t m, int32_t n, int32_t k,
+                          int32_t act, int32_t gated, int32_t fast) {
+  return vla::run_tile_linear({a, w, x, nullptr, nullptr, nullptr, nullptr, out32, out16, nullptr, m, n, k, act, gated, fast});
+}
+
+int vla_debug_tile_addends(const void* a, const void* w, const float* x, const float* bias, const float* vec, const float* tab,
+                           const float* tab_b, float* out32, void* out16, float* ss, int32_t m, int32_t n, int32_t k, int32_t act) {
+  return vla::run_tile_linear({a, w, x, bias, vec, tab, tab_b, out32, out16, ss, m, n, k, act, 0, 1});
 }
 
 int vla_debug_tile_attention(const void* q, const void* k0, const void* vt0, const void* k1, const void* vt1, void* out, int32_t tq,

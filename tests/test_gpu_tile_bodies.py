@@ -1,6 +1,6 @@
 """The engine's GEMM and attention tile bodies, operator by operator, against the CPU oracle (fp64) on the same
 bf16-representable inputs: the stand-alone operators are kernels of their own and say nothing about these.  Both epilogues of
-the GEMM tile, gated rows, addends under the accumulators; attention over one and two key segments, folded heads, causal and
+the GEMM tile, gated rows, addends under the accumulators and behind the product; attention over one and two key segments, folded heads, causal and
 suffix masks; and the waits inside the bodies, which run out and are reported."""
 import numpy as np
 import pytest
@@ -90,9 +90,9 @@ def test_gemm_tile_gated(m, n, k, act, fast):
 @pytest.mark.parametrize("scale", [1.0, 64.0])
 @pytest.mark.parametrize("fast", [False, True])
 def test_gemm_tile_addend(m, n, k, scale, fast):
-    """out = a w^T + x: added behind the product (general epilogue), or lying under the accumulators (straight one).  An fp32 sum
-    of k products of two bf16 values next to an addend of up to `scale` times their size: every step may lose one unit in the
-    last place of the larger, 2^-23 of it, and the tensor core adds 16 products a step."""
+    """out = a w^T + x: both epilogues add behind the product.  An fp32 sum of k products of two bf16 values next to an addend of up to
+    `scale` times their size: every step may lose one unit in the last place of the larger, 2^-23 of it, and the tensor core adds 16
+    products a step; the straight epilogue's single rounding is what test_gemm_tile_residual_is_rounded_once holds it to."""
     import torch
     from paper_2609_22335_b200 import api
     rng = np.random.default_rng(m + n + k)
@@ -101,8 +101,69 @@ def test_gemm_tile_addend(m, n, k, scale, fast):
     ref = O.linear(a.astype(np.float64), w.astype(np.float64)) + x
     got = api.debug_tile_linear(_dev(a), _dev(_engine_rows(w) if fast else w), n, x=torch.from_numpy(x).cuda(), fast=fast)[0]
     err = np.abs(got.cpu().numpy() - ref)
-    print(f"addend {scale:g} x product, k = {k}, {'under the accumulators' if fast else 'behind the product'}: rel-L2 {np.linalg.norm(err) / np.linalg.norm(ref):.3g}")
+    print(f"addend {scale:g} x product, k = {k}, {'straight' if fast else 'general'} epilogue: rel-L2 {np.linalg.norm(err) / np.linalg.norm(ref):.3g}")
     assert err.max() <= 2.0 ** -23 * (k / 16 + 2) * np.abs(ref).max()
+
+
+ADDEND_SHAPES = [(1, 8, 64), (17, 136, 64), (50, 720, 960), (64, 136, 2048), (65, 40, 192), (129, 72, 64), (300, 384, 512), (1024, 768, 3072)]
+
+
+def _f32(rng, shape, scale=1.0):
+    return (scale * rng.standard_normal(shape)).astype(np.float32)
+
+
+@pytest.mark.parametrize("m,n,k", ADDEND_SHAPES)
+@pytest.mark.parametrize("scale", [1.0, 64.0])
+@pytest.mark.parametrize("in_place", [False, True])
+@pytest.mark.parametrize("mirror", [False, True])
+def test_gemm_tile_residual_is_rounded_once(m, n, k, scale, in_place, mirror):
+    """x + a w^T with the straight epilogue, into rows of its own and in place, alone and with the bf16 mirror and the sums of squares that the
+    next norm reads.  The product's sums are exact to a unit in the last place per 16 products at the product's own size, however large x is,
+    and the one addition behind them rounds by half a unit of the result; the mirror is the fp32 rows' rounding, and a partial sum of 128
+    squares (32 in a lane, two exchanges, all positive) loses at most 36 half units."""
+    import torch
+    from paper_2609_22335_b200 import api
+    rng = np.random.default_rng(m + n + k)
+    a, w, x = _rand(rng, (m, k)), _rand(rng, (n, k), k ** -0.5), _f32(rng, (m, n), scale)
+    product = O.linear(a.astype(np.float64), w.astype(np.float64))
+    ref = product + x
+    o32, o16, ss = api.debug_tile_addends(_dev(a), _dev(_engine_rows(w)), n, x=torch.from_numpy(x).cuda(), out16=mirror, ss=mirror, in_place=in_place)
+    got = o32.cpu().numpy().astype(np.float64)
+    assert (np.abs(got - ref) <= 2.0 ** -23 * (k / 16 + 2) * np.abs(product).max() + 2.0 ** -24 * np.abs(ref)).all()
+    if mirror:
+        assert torch.equal(o16, o32.to(torch.bfloat16))
+        squares = np.add.reduceat(got ** 2, np.arange(0, n, 128), axis=1)
+        assert (np.abs(ss.cpu().numpy() - squares) <= 36 * 2.0 ** -24 * squares).all()
+
+
+@pytest.mark.parametrize("m,n,k", ADDEND_SHAPES)
+@pytest.mark.parametrize("terms", ["b", "v", "t", "u", "bv", "tu", "bvtu"])
+def test_gemm_tile_addends_under_the_accumulators(m, n, k, terms):
+    """Bias, broadcast vector and tables lie in the accumulators before the first MMA: alone, together, and with residual rows behind the
+    product.  The sums then start from them: a unit in the last place of the largest partial sum per 16 products and per addend."""
+    import torch
+    from paper_2609_22335_b200 import api
+    rng = np.random.default_rng(m + n + k + len(terms))
+    a, w, x = _rand(rng, (m, k)), _rand(rng, (n, k), k ** -0.5), _f32(rng, (m, n), 4.0)
+    under = {"b": _f32(rng, n), "v": _f32(rng, n), "t": _f32(rng, (m, n)), "u": _f32(rng, (m, n))}
+    names = {"b": "bias", "v": "vec", "t": "tab", "u": "tab2"}
+    args = {names[t]: torch.from_numpy(under[t]).cuda() for t in terms}
+    product = O.linear(a.astype(np.float64), w.astype(np.float64))
+    added = sum(under[t].astype(np.float64) for t in terms)
+    ref = product + added
+    sums = 2.0 ** -23 * (k / 16 + 2 + len(terms)) * (np.abs(product).max() + np.abs(added).max())
+    da, dw = _dev(a), _dev(_engine_rows(w))
+    o32, o16, ss = api.debug_tile_addends(da, dw, n, out16=True, ss=True, **args)
+    got = o32.cpu().numpy().astype(np.float64)
+    assert (np.abs(got - ref) <= sums).all()
+    assert torch.equal(o16, o32.to(torch.bfloat16))
+    squares = np.add.reduceat(got ** 2, np.arange(0, n, 128), axis=1)
+    assert (np.abs(ss.cpu().numpy() - squares) <= 36 * 2.0 ** -24 * squares).all()
+    assert torch.equal(api.debug_tile_addends(da, dw, n, out32=False, out16=True, **args)[1], o16)
+    both = api.debug_tile_addends(da, dw, n, x=torch.from_numpy(x).cuda(), **args)[0].cpu().numpy()
+    assert (np.abs(both - (ref + x)) <= sums + 2.0 ** -24 * np.abs(ref + x)).all()
+    if terms == "b":
+        _check(api.debug_tile_addends(da, dw, n, act=1, out32=False, out16=True, **args)[1], _act(1, ref), True)
 
 
 ATTENTION_SHAPES = [
@@ -179,5 +240,8 @@ def test_hooks_refuse_what_the_straight_epilogue_cannot_take():
     assert lib.vla_debug_tile_linear(t, t, o, o, None, 64, 64, 64, 1, 0, 1) == bad           # activation behind an addend
     assert lib.vla_debug_tile_linear(t, t, o, None, t, 64, 64, 64, 0, 0, 1) == bad           # addend without fp32 rows
     assert lib.vla_debug_tile_linear(t, t, None, o, None, 64, 64, 64, 0, 1, 0) == bad        # gated rows are bf16
+    assert lib.vla_debug_tile_addends(t, t, None, o, o, None, None, None, t, None, 64, 64, 64, 1) == bad     # activation behind a broadcast vector
+    assert lib.vla_debug_tile_addends(t, t, None, o + 4, None, None, None, o, None, None, 8, 64, 64, 0) == bad    # bias that is not 16-byte aligned
+    assert lib.vla_debug_tile_addends(t, t, None, None, None, None, None, o, None, o, 64, 64, 64, 0) == bad  # sums of squares without the mirror
     assert lib.vla_debug_tile_attention(t, t, t, None, None, t, 64, 64, 8, 1, 1, 64, 0, 0) == bad    # a second segment without its keys
     assert lib.vla_debug_tile_attention(t, t, t, None, None, t, 32, 64, 0, 1, 1, 64, 1, 0) == bad    # causal needs tq == t0
