@@ -218,7 +218,7 @@ int vla_op_linear(const void* a, const void* w, float* out32, void* out16, int32
   g.m = m; g.n = n; g.kp = (int)op_pad(k, GEMM_BK); g.act = act;
   g.out32 = out32; g.out16 = static_cast<unsigned short*>(out16);
   g.err = dev.error;
-  const LinearPlan p = linear_plan(m, n, k, out32 != nullptr, dev.sms);
+  const LinearPlan p = linear_plan(m, n, k, out32 != nullptr, dev.sms, LinearRoom{dev.room.alone[4], dev.room.two[4]});
   const LinearPairPlan pp = linear_pair_plan(m, n, k, p, dev.sms);
   const int vec = linear_vec(n, out32, out16);
   OpMaps maps;

@@ -7,7 +7,8 @@ pytestmark = pytest.mark.gpu
 
 SHAPES = [(2077, 4944, 712), (1747, 2064, 2288), (4645, 3040, 1000), (7744, 2824, 472), (2936, 1496, 1160), (5125, 440, 2048),
           (978, 14489, 792), (3000, 4902, 520), (129, 16384, 4096),
-          (294, 8512, 2952), (452, 6648, 6024), (3261, 392, 1424), (823, 2105, 2000), (3104, 592, 1992)]       # (fp32: K in two and four parts)
+          (294, 8512, 2952), (452, 6648, 6024), (3261, 392, 1424), (823, 2105, 2000), (3104, 592, 1992), (729, 3139, 3160),       # (fp32: K in two and four parts)
+          (300, 5144, 4264), (983, 1626, 3912), (326, 5053, 4064), (935, 1456, 3616), (453, 3482, 3024), (929, 1601, 4064)]      # (bf16 too)
 
 
 @pytest.mark.parametrize("m,n,k", SHAPES)

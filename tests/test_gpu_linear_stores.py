@@ -35,7 +35,8 @@ def test_widths_and_addresses(m, n, k):
 @pytest.mark.parametrize("m,n,k", [
     (129, 4833, 64), (129, 4790, 64), (129, 5925, 64), (129, 7154, 64),               # widths 48, 80, 96, 112
     (300, 6284, 72), (4000, 578, 64), (300, 8038, 64), (4000, 733, 72), (4000, 784, 72), (800, 4388, 72), (4000, 923, 72),   # 144 .. 240
-    (129, 4756, 1992), (257, 2370, 2056)])                                            # K shared by two and four CTAs, for fp32 results only
+    (129, 4756, 1992),                                                                # (fp32: tiles of two SMs)
+    (288, 11008, 4096), (572, 6298, 1616), (257, 2370, 2056)])                        # K shared by two and four CTAs, for fp32 results only
 def test_widths_that_are_no_power_of_two(m, n, k):
     import torch
     from paper_2609_22335_b200 import api

@@ -61,6 +61,20 @@ def test_fp32_results_keep_their_split(plan):
         assert plan(*shape, f32=True)["ks"] == ks
 
 
+def test_a_call_goes_where_it_is_faster(plan):
+    """Shapes that a plan which took clusters of four for one CTA per SM, their late ones for a whole wave, and a pair's k-block for 350 cycles
+    sent to two-SM tiles or a wider split at up to 1.5 times the time; and ones that gain from two SMs."""
+    def choice(*shape):
+        pair = plan.pair(*shape)[1]
+        p = plan(*shape)
+        return (pair or p["bn"], p["ks"], pair > 0)
+    for shape, best in (((948, 786, 6656, False), (128, 4, False)), ((719, 1056, 5472, False), (128, 4, False)), ((286, 2435, 4640, False), (128, 4, False)),
+                        ((4390, 149, 6736, True), (128, 4, False)), ((1215, 810, 10616, True), (128, 4, False)), ((931, 1072, 11040, True), (128, 4, False)),
+                        ((4917, 1076, 7296, True), (160, 1, False)), ((360, 10776, 5888, False), (112, 1, False)),
+                        ((489, 4487, 2928, True), (128, 4, True)), ((983, 1626, 3912, False), (128, 2, True)), ((4096, 4096, 4096, False), (240, 1, True))):
+        assert choice(*shape) == best, shape
+
+
 def test_every_plan_of_two_sm_tiles_is_one_the_kernel_can_run(plan):
     rnd = random.Random(5)
     shapes = [(m, n, k) for m in (1, 128, 129, 256, 257, 100000) for n in (7, 112, 113, 255, 257, 70000) for k in (8, 72, 4096, 20000)]
@@ -80,3 +94,21 @@ def test_every_plan_of_two_sm_tiles_is_one_the_kernel_can_run(plan):
             assert bm * 128 % 1024 == 0 and stage % 1024 == 0
             assert 2 <= stages <= 12 and (stages - 1) * stage + max(stage, 16384) <= 224 * 1024
     assert used > 1000
+
+
+def test_the_gpu_tests_reach_what_they_are_for(plan):
+    """The shapes of the tests of two-SM tiles go to them, with K in one, two and four parts for both result types, stores of eight, two and
+    one feature, and widths that end inside 32 columns; those of the exchange between CTAs go to that."""
+    from test_gpu_linear_pair import SHAPES
+    reached = set()
+    for m, n, k in SHAPES:
+        for f32 in (False, True):
+            width = plan.pair(m, n, k, f32)[1]
+            assert width > 0 or (m, n, k, f32) in ((3261, 392, 1424, False), (326, 5053, 4064, True))
+            if width:
+                reached.add((f32, plan(m, n, k, f32)["ks"], 8 if n % 8 == 0 else 2 if n % 2 == 0 else 1))
+                reached.add((f32, width % 32))
+    assert reached >= {(False, p, v) for p in (1, 2, 4) for v in (8, 2, 1)} | {(True, 1, v) for v in (8, 2, 1)} | {(True, 2, 8), (True, 2, 1), (True, 4, 8), (True, 4, 1)}
+    assert reached >= {(f32, w) for f32 in (False, True) for w in (0, 16)}
+    for shape, ks in (((288, 11008, 4096), 2), ((572, 6298, 1616), 2), ((257, 2370, 2056), 4)):
+        assert plan(*shape, f32=True)["ks"] == ks and plan(*shape, f32=True)["bn"] == (256 if ks == 2 else 128) and plan.pair(*shape, True)[1] == 0
