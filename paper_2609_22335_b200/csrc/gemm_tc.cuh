@@ -344,8 +344,9 @@ __device__ __forceinline__ void epi_stream(const TileCtx& c, const EpiPlace& e, 
 // Residual rows, fp32, in the fragment layout: this lane's two tokens of a half, eight features of each, of two groups of 32
 // columns.  The first two groups are asked for in front of the main loop, each later one in the place of a group just added: half
 // the round trips lie under the loop, where laying the rows under the accumulators had all four of a 128-token tile in front of it,
-// and the sum is rounded once, not once per MMA (32 streams x 4 178.8 -> 177.4 ms, GR00T 8 x 3 36.3 -> 36.0, CogACT 18.73 -> 18.52).
-// Four groups held at once need 440 bytes of spills.
+// and the sum is rounded once, not once per MMA (CogACT 18.74 -> 18.57 ms; the other workloads 0.4 to 1.4 %, which is what their runs differ by).
+// Two groups in flight cost 44 bytes of spills in the persistent kernel, one group 16 and 1 % of CogACT, GR00T and 4 x 3 (18.53 -> 18.76,
+// 36.06 -> 36.43, 40.28 -> 40.71 ms); four groups 440 bytes.
 struct ResidRows { float4 v[2][2][2]; };
 __device__ __forceinline__ void resid_load(const float* x, int ldx, int tok, int live, int half, int lane, int cols, int c, float4 (&v)[2][2]) {
   const int q = lane & 3;
@@ -674,7 +675,7 @@ __device__ __forceinline__ void tile_gemm(const TileCtx& c, const GemmArgs& g, i
     if (warp_live) preload_rows(c, g, my_tmem, t0 + tpw * warp, min(tpw, nt - tpw * warp), tpw, lane, r0);
     tc_fence_before();
   }
-  ResidRows resid;                                     // (set in every case: left open where there are none, 120 bytes of it were spilled)
+  ResidRows resid;                                     // (set in every case: left open where there are none, 120 more bytes are spilled)
 #pragma unroll
   for (int j = 0; j < 2; ++j)
 #pragma unroll
